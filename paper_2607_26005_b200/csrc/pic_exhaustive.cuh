@@ -1,13 +1,10 @@
-// Exhaustive tile renderer shared by the cross-check kernel (PIC_OPT_BRUTE_FORCE) and by
-// pic_render_static (internal).
+// Exhaustive tile renderer of the cross-check kernel (PIC_OPT_BRUTE_FORCE; internal).
 //
 // One CTA renders one 64 x 64 tile of one view: every map item and every face of every other
 // agent's box against every pixel (a thread per primitive, a shared-memory atomic max per
 // fragment) -- no hierarchy, no frustum or pixel-box culling, no size classes.  It shares only the
 // per-primitive arithmetic of pic_device.cuh (and the per-call camera and ray tables) with the
 // production kernels, so comparing the images checks everything the production kernels add.
-// The two users differ in where a map item comes from, which `fetch` hides: the scene's
-// preprocessed primitives, or the caller's raw triangles.
 #pragma once
 #include "pic_device.cuh"
 

@@ -219,8 +219,8 @@ __device__ __forceinline__ int tally_value(const NoCount&) { return 0; }
 struct NoTally { NoCount grp, leaf, tested, setup, tiny, recs, fallback, classified, cells, jobs, coop; };
 
 // Cooperative kernel, phase 2b body: set a surviving primitive up, rasterize it (tiny) or leave a record.
-template <class TL>
-__device__ __forceinline__ void setup_prim(TileSmem& s, const TileCtx& t, const V3 (&V)[4], bool quad, uint32_t flags,
+template <class S, class TL>
+__device__ __forceinline__ void setup_prim(S& s, const TileCtx& t, const V3 (&V)[4], bool quad, uint32_t flags,
                                            const V3 Pn, uint32_t key_lo, uint32_t box, int rec_cap, TL& n) {
     PrimEq q;
     if (!prim_equations(V, quad, flags, Pn, q)) return;
@@ -402,7 +402,8 @@ __device__ __forceinline__ void store_tile(S& s, const TileCtx& t, const RenderP
     uint8_t* oc = P.out_class + view * img;
     uint16_t* od = P.out_depth + view * img;
     float* o32 = P.out_depth32 ? P.out_depth32 + view * img : nullptr;
-    const bool vec_ok = FULL || ((P.W % 16 == 0) && o32 == nullptr);
+    // (pic_render_static takes outputs of any alignment)
+    const bool vec_ok = FULL || ((P.W % 16 == 0) && o32 == nullptr && ((reinterpret_cast<uintptr_t>(P.out_class) | reinterpret_cast<uintptr_t>(P.out_depth)) & 15u) == 0);
     const int segs_per_row = FULL ? TILE / 16 : (t.tw + 15) >> 4;
     const int n_seg = t.th * segs_per_row;
     // consecutive threads take consecutive 16-pixel segments of a row, then the next row: a warp's
@@ -472,7 +473,8 @@ struct Job {
 };
 
 // Job `id` of the launch: tiles of a view are consecutive, views follow P.view_first.
-__device__ __forceinline__ Job decode_job(const RenderParams& P, unsigned id) {
+// (tile_h: rows of a tile, for the kernel that cuts views into lower pieces.)
+__device__ __forceinline__ Job decode_job(const RenderParams& P, unsigned id, int tile_h = TILE) {
     const unsigned tiles = (unsigned)(P.tiles_x * P.tiles_y);
     const unsigned vrel = id / tiles;
     const unsigned long long v = (unsigned long long)P.view_first + vrel;
@@ -483,8 +485,8 @@ __device__ __forceinline__ Job decode_job(const RenderParams& P, unsigned id) {
     j.k = (int)((unsigned)v - va * (unsigned)P.K);
     j.e = (int)(va / (unsigned)P.A);
     j.a = (int)(va - (unsigned)j.e * (unsigned)P.A);
-    j.t.x0 = (j.tile % P.tiles_x) * TILE; j.t.y0 = (j.tile / P.tiles_x) * TILE;
-    j.t.tw = min(TILE, P.W - j.t.x0); j.t.th = min(TILE, P.H - j.t.y0);
+    j.t.x0 = (j.tile % P.tiles_x) * TILE; j.t.y0 = (j.tile / P.tiles_x) * tile_h;
+    j.t.tw = min(TILE, P.W - j.t.x0); j.t.th = min(tile_h, P.H - j.t.y0);
     j.t.w_near = P.w_near; j.t.w_far = P.w_far; j.t.near_z = P.near_z; j.t.far_z = P.far_z;
     return j;
 }
@@ -1785,6 +1787,7 @@ __global__ void __launch_bounds__(NTHREADS) coverage_kernel(const __grid_constan
 #include "pic_coverage.cuh"
 namespace pic {
 #include "pic_colour.cuh"
+#include "pic_static.cuh"
 
 size_t survivor_bytes_per_tile() { return sizeof(uint2) * SURV_STRIDE; }
 

@@ -17,12 +17,14 @@
 #include <mutex>
 
 #include "../../include/pictura.h"
-#include "pic_exhaustive.cuh"
+#include "pic_types.h"
 
 namespace pic {
 cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses, float* state, const float* actions,
                          const float* dims, const uint8_t* active, const uint8_t* agent_cls, AgentGeom* agents_out, ViewCam* cams_out,
                          float* tables, uint32_t* status, float dt, float wheelbase, float v_max, cudaStream_t stream);
+cudaError_t configure_static_kernel();            // pic_static.cuh (part of pic_render.cu)
+cudaError_t launch_static_kernel(const RenderParams& P, const float* tri_xyz, const uint8_t* tri_class, int n_tris, int sm_count, cudaStream_t stream);
 void set_last_error(const char* msg);
 }  // namespace pic
 
@@ -48,46 +50,7 @@ static __device__ __align__(256) unsigned char g_static_scratch[kScratchBytes];
 
 std::mutex g_mutex;
 unsigned char* g_scratch_ptr[kMaxDevices] = {};     // device address of g_static_scratch, per device
-
-struct StaticParams {
-    RenderParams P;
-    const float* tri_xyz;        // dev [N,3,3]
-    const uint8_t* tri_class;    // dev [N]
-    uint32_t n_tris;
-};
-
-__device__ __forceinline__ bool lex_less(float ax, float ay, float az, float bx, float by, float bz) {
-    if (ax != bx) return ax < bx;
-    if (ay != by) return ay < by;
-    return az < bz;
-}
-
-// The exhaustive tile renderer over the caller's raw triangles.
-__global__ void __launch_bounds__(EXH_THREADS) render_static_kernel(const __grid_constant__ StaticParams S) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    ExhaustiveSmem& s = *reinterpret_cast<ExhaustiveSmem*>(smem_raw);
-    const float* tri_xyz = S.tri_xyz;
-    const uint8_t* tri_class = S.tri_class;
-    exhaustive_tile(s, S.P, blockIdx.x, S.n_tris, S.n_tris,
-                    [tri_xyz, tri_class](uint32_t i, const Cam& c, V3 (&V)[4], V3& Pn, bool& quad, uint32_t& flags, uint32_t& key_lo) {
-                        const float* p = tri_xyz + 9 * (size_t)i;
-                        float v[9];
-#pragma unroll
-                        for (int j = 0; j < 9; ++j) v[j] = __ldg(p + j);
-#pragma unroll
-                        for (int j = 0; j < 3; ++j) V[j] = to_camera(c, v[3 * j], v[3 * j + 1], v[3 * j + 2]);
-                        V[3] = V[2];
-                        const float v12[12] = {v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], v[8], v[6], v[7], v[8]};
-                        Pn = plane_normal_world(c, v12, false);
-                        quad = false;
-                        flags = 0u;
-                        // an edge shared by two triangles is evaluated in the same direction by both
-                        if (!lex_less(v[0], v[1], v[2], v[3], v[4], v[5])) flags |= 1u << 4;
-                        if (!lex_less(v[3], v[4], v[5], v[6], v[7], v[8])) flags |= 1u << 5;
-                        if (!lex_less(v[6], v[7], v[8], v[0], v[1], v[2])) flags |= 1u << 6;
-                        key_lo = ((0xFFFFFFu - i) << 8) | __ldg(tri_class + i);
-                    });
-}
+int g_sm_count[kMaxDevices] = {};
 
 pic_status fail(pic_status st, const char* fmt, ...) {
     char buf[384];
@@ -144,16 +107,17 @@ extern "C" pic_status pic_render_static(const pic_static_desc* d, const float* t
             void* p = nullptr;
             ce = cudaGetSymbolAddress(&p, g_static_scratch);
             if (ce != cudaSuccess) return fail(PIC_ERR_CUDA, "cudaGetSymbolAddress: %s", cudaGetErrorString(ce));
-            ce = cudaFuncSetAttribute(render_static_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(ExhaustiveSmem));
+            ce = pic::configure_static_kernel();
             if (ce != cudaSuccess) return fail(PIC_ERR_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(ce));
+            ce = cudaDeviceGetAttribute(&g_sm_count[dev], cudaDevAttrMultiProcessorCount, dev);
+            if (ce != cudaSuccess) return fail(PIC_ERR_CUDA, "cudaDeviceGetAttribute: %s", cudaGetErrorString(ce));
             g_scratch_ptr[dev] = static_cast<unsigned char*>(p);
         }
         scratch = g_scratch_ptr[dev];
     }
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    StaticParams S;
-    memset(&S, 0, sizeof(S));
-    RenderParams& P = S.P;
+    RenderParams P;
+    memset(&P, 0, sizeof(P));
     P.E = d->E; P.A = d->A; P.K = d->K; P.H = d->H; P.W = d->W;
     P.tiles_x = (d->W + TILE - 1) / TILE; P.tiles_y = (d->H + TILE - 1) / TILE;
     P.near_z = d->near_z; P.far_z = d->far_z; P.w_near = 1.0f / d->near_z; P.w_far = 1.0f / d->far_z;
@@ -175,13 +139,10 @@ extern "C" pic_status pic_render_static(const pic_static_desc* d, const float* t
         o.cphi = (float)std::cos((double)rig[k].pitch); o.sphi = (float)std::sin((double)rig[k].pitch);
         o.fx = rig[k].fx; o.fy = rig[k].fy;
     }
-    S.tri_xyz = tri_xyz; S.tri_class = tri_class; S.n_tris = (uint32_t)d->n_tris;
     // (the status word is sticky across calls, like a scene's: pic_static_status reads and clears it)
     ce = pic::launch_setup(P, d->E * d->A, poses, nullptr, nullptr, dims, active, nullptr, agents, cams, tables, status, 0.f, 1.f, 0.f, stream);
     if (ce != cudaSuccess) return fail(PIC_ERR_CUDA, "set-up kernels: %s", cudaGetErrorString(ce));
-    const unsigned blocks = (unsigned)(d->E * d->A * d->K * P.tiles_x * P.tiles_y);
-    render_static_kernel<<<blocks, EXH_THREADS, sizeof(ExhaustiveSmem), stream>>>(S);
-    ce = cudaGetLastError();
+    ce = pic::launch_static_kernel(P, tri_xyz, tri_class, d->n_tris, g_sm_count[dev], stream);
     if (ce != cudaSuccess) return fail(PIC_ERR_CUDA, "render_static_kernel: %s", cudaGetErrorString(ce));
     return PIC_OK;
 }

@@ -1,0 +1,49 @@
+"""Branches that depend on the size of a call, at the sizes where they change: the piece height of
+pic_render_static, its list of survivors and its batches of records."""
+import numpy as np
+import pytest
+
+from scenes import custom_scene, make_rig
+
+pytestmark = pytest.mark.gpu
+CAR = (4.5, 1.9, 1.5)
+
+
+def soup(seed, n_tris, E, A, H, W, K=2, spread=25.0):
+    """E x A agents in a soup of n_tris small triangles; camera 1 looks back from another mount."""
+    rng = np.random.default_rng(seed)
+    c = np.stack([rng.uniform(-spread, spread, n_tris), rng.uniform(-spread, spread, n_tris), rng.uniform(0.0, 4.0, n_tris)], axis=1)
+    tris = (c[:, None, :] + rng.uniform(-3, 3, size=(n_tris, 3, 3))).astype(np.float32)
+    rig = make_rig(tuple(np.arange(K) * 170.0), 80.0, 70.0, W, H, mount=(1.0, 0.2, 1.4))
+    poses = rng.uniform(-10, 10, size=(E, A, 3)).astype(np.float32)
+    return custom_scene(tris, rng.integers(0, 200, n_tris).astype(np.uint8), poses, np.tile(np.array(CAR, np.float32), (E, A, 1)), rig, H, W)
+
+
+@pytest.mark.parametrize("n_tris,E,A,H,W,offset", [
+    (1, 1, 1, 17, 33, 0),            # one triangle, pieces of 16 rows, the last of one row
+    (127, 1, 2, 64, 64, 0),          # one round of tests less a thread
+    (257, 1, 3, 70, 100, 1),         # two rounds and a thread; outputs that allow no vector store
+    (1500, 1, 2, 64, 80, 0),         # several hundred survivors per tile: the list is emptied more than once
+    (300, 2, 60, 96, 64, 0),         # more CTAs than two per multiprocessor: pieces of 64 rows
+])
+def test_static_pieces_lists_and_alignment(n_tris, E, A, H, W, offset):
+    import torch
+    import paper_2607_26005_b200 as pic
+    from tests.gpu_util import CudaRun
+    s = soup(n_tris, n_tris, E, A, H, W)
+    dev = torch.device("cuda", 0)
+    g = CudaRun(s)
+    try:
+        want = g.render(brute=True)
+    finally:
+        g.close()
+    n = E * A * s.K * H * W
+    cls = torch.full((n + offset,), 255, dtype=torch.uint8, device=dev)[offset:]
+    dep = torch.full((n + offset,), -1.0, dtype=torch.float16, device=dev)[offset:]
+    put = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(dev)
+    pic.render_static(E, A, s.K, H, W, s.near, s.far, put(s.tri_xyz), put(s.tri_class), put(s.poses), put(s.dims), s.rig, cls, dep)
+    V = E * A * s.K
+    c, d = cls.cpu().numpy().reshape(V, H, W), dep.cpu().numpy().reshape(V, H, W)
+    assert (c == want[0]).all()
+    assert (np.abs(d.view(np.uint16).astype(int) - want[1].view(np.uint16).astype(int)) <= 1).all()
+    assert pic.static_status() == 0
