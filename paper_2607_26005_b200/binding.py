@@ -54,6 +54,16 @@ class pic_static_desc(C.Structure):
 
 
 _lib = None
+_torch_module = None
+
+
+def _torch():
+    """torch, imported when it is first needed."""
+    global _torch_module
+    if _torch_module is None:
+        import torch
+        _torch_module = torch
+    return _torch_module
 
 
 def load(path: Optional[str] = None):
@@ -69,20 +79,20 @@ def load(path: Optional[str] = None):
     vp = C.c_void_p
     lib.pic_scene_create.argtypes = [C.POINTER(pic_scene_desc), C.POINTER(vp)]
     lib.pic_scene_destroy.argtypes = [vp]
-    lib.pic_render.argtypes = [vp, vp, vp, vp, C.POINTER(pic_camera), vp, vp, vp]
-    lib.pic_render_host.argtypes = [vp, vp, vp, vp, C.POINTER(pic_camera), vp, vp, vp]
+    lib.pic_render.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp]
+    lib.pic_render_host.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp]
     lib.pic_set_state.argtypes = [vp, vp, vp, vp, vp]
     lib.pic_get_state.argtypes = [vp, vp, vp]
     lib.pic_set_agent_classes.argtypes = [vp, vp, vp]
     lib.pic_set_palette.argtypes = [vp, vp, vp]
-    lib.pic_render_rgb.argtypes = [vp, vp, vp, vp, C.POINTER(pic_camera), C.c_int32, vp, vp]
-    lib.pic_step_rgb.argtypes = [vp, vp, C.POINTER(pic_camera), C.c_int32, vp, vp]
-    lib.pic_step.argtypes = [vp, vp, C.POINTER(pic_camera), vp, vp, vp]
+    lib.pic_render_rgb.argtypes = [vp, vp, vp, vp, vp, C.c_int32, vp, vp]
+    lib.pic_step_rgb.argtypes = [vp, vp, vp, C.c_int32, vp, vp]
+    lib.pic_step.argtypes = [vp, vp, vp, vp, vp, vp]
     lib.pic_get_status.argtypes = [vp, C.POINTER(C.c_uint32), vp]
     lib.pic_scene_set_option.argtypes = [vp, C.c_int32, C.c_uint64]
     lib.pic_get_kernel_times.argtypes = [vp, C.POINTER(C.c_float), C.c_int32, C.POINTER(C.c_int32)]
     lib.pic_map_stats.argtypes = [C.POINTER(pic_scene_desc), C.POINTER(C.c_int64)]
-    lib.pic_render_static.argtypes = [C.POINTER(pic_static_desc), vp, vp, vp, vp, vp, C.POINTER(pic_camera), vp, vp, vp]
+    lib.pic_render_static.argtypes = [C.POINTER(pic_static_desc), vp, vp, vp, vp, vp, vp, vp, vp, vp]
     lib.pic_static_status.argtypes = [C.POINTER(C.c_uint32), vp]
     lib.pic_probe_fill.argtypes = [vp, C.c_uint64, vp]
     lib.pic_probe_ffma.argtypes = [vp, C.c_uint64, C.c_int32, C.POINTER(C.c_uint64), vp]
@@ -101,19 +111,20 @@ def _check(lib, status: int):
         raise PicError(status, lib.pic_last_error().decode("utf-8", "replace"))
 
 
-def _rig_array(rig) -> "C.Array":
-    rig = np.asarray(rig, dtype=np.float32).reshape(-1, 7)
-    arr = (pic_camera * rig.shape[0])()
-    for k in range(rig.shape[0]):
-        arr[k] = pic_camera(*[float(v) for v in rig[k]])
-    return arr
+def _rig_ptr(rig):
+    """The rig as the library reads it: K rows of 7 float32, which is how numpy lays out a C-contiguous [K, 7] array.  Returns (address, the
+    array that has to outlive the call)."""
+    if not (type(rig) is np.ndarray and rig.dtype == np.float32 and rig.flags.c_contiguous):
+        rig = np.ascontiguousarray(rig, dtype=np.float32)
+    if rig.size % 7:
+        raise ValueError("a rig has 7 values per camera")
+    return rig.__array_interface__["data"][0], rig
 
 
 def _dev_ptr(t, dtype, numel: Optional[int] = None) -> int:
-    import torch
     if t is None:
         return 0
-    if not isinstance(t, torch.Tensor) or not t.is_cuda:
+    if not isinstance(t, _torch().Tensor) or not t.is_cuda:
         raise TypeError("expected a CUDA torch tensor")
     if t.dtype != dtype or not t.is_contiguous():
         raise TypeError(f"expected a contiguous {dtype} tensor, got {t.dtype}")
@@ -123,10 +134,11 @@ def _dev_ptr(t, dtype, numel: Optional[int] = None) -> int:
 
 
 def _stream_ptr(stream) -> int:
-    import torch
     if stream is None:
-        stream = torch.cuda.current_stream()
-    return int(stream.cuda_stream)
+        torch = _torch()
+        # (the handle alone: torch.cuda.current_stream() builds a Stream object, a microsecond of a small call)
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream
 
 
 def map_stats(tri_xyz, tri_class, map_tri_offset=None, A: int = 0) -> dict:
@@ -157,7 +169,7 @@ def render_static(E: int, A: int, K: int, H: int, W: int, near: float, far: floa
     """pic_render_static: render on the current device without a scene and without allocating.
     tri_xyz (f32 [N,3,3]), tri_class (u8 [N]), poses, dims, active and the outputs are CUDA tensors
     the caller already owns; nothing is allocated here either."""
-    import torch
+    torch = _torch()
     lib = load()
     n, npx = E * A, E * A * K * H * W
     n_tris = 0 if tri_xyz is None else int(tri_xyz.shape[0])
@@ -166,11 +178,12 @@ def render_static(E: int, A: int, K: int, H: int, W: int, near: float, far: floa
     d.E, d.A, d.K, d.H, d.W, d.n_tris = int(E), int(A), int(K), int(H), int(W), n_tris
     d.near_z, d.far_z = float(near), float(far)
     d.agent_class, d.sky_class, d.ground_class = int(agent_class), int(sky_class), int(ground_class)
+    rig_ptr, rig = _rig_ptr(rig)
     _check(lib, lib.pic_render_static(
         C.byref(d), _dev_ptr(tri_xyz, torch.float32, 9 * n_tris) if n_tris else None,
         _dev_ptr(tri_class, torch.uint8, n_tris) if n_tris else None, _dev_ptr(poses, torch.float32, 3 * n),
         _dev_ptr(dims, torch.float32, 3 * n), _dev_ptr(active, torch.uint8, n) if active is not None else None,
-        _rig_array(rig), _dev_ptr(out_class, torch.uint8, npx), _dev_ptr(out_depth, torch.float16, npx),
+        rig_ptr, _dev_ptr(out_class, torch.uint8, npx), _dev_ptr(out_depth, torch.float16, npx),
         _stream_ptr(stream)))
     return out_class, out_depth
 
@@ -185,7 +198,7 @@ def probe_fill(dst, stream=None) -> int:
 
 def probe_ffma(out, iters: int, stream=None) -> int:
     """pic_probe_ffma (register-only FFMA loop); `out` is a float32 CUDA tensor; returns the per-lane FMA count."""
-    import torch
+    torch = _torch()
     lib = load()
     n = C.c_uint64(0)
     _check(lib, lib.pic_probe_ffma(_dev_ptr(out, torch.float32, out.numel()), out.numel(), int(iters), C.byref(n), _stream_ptr(stream)))
@@ -206,7 +219,7 @@ class Scene:
     def __init__(self, E: int, A: int, K: int, H: int, W: int, near: float, far: float, tri_xyz, tri_class,
                  map_tri_offset=None, env_map_id=None, agent_class: int = 4, sky_class: int = 0,
                  ground_class: int = 1, device: int = 0, tri_vis_cos=None):
-        import torch
+        torch = _torch()
         if not torch.cuda.is_available():
             raise RuntimeError("no CUDA device: the rasterizer has no CPU path")
         self._lib = load()
@@ -248,20 +261,21 @@ class Scene:
         return (self.E, self.A, self.K, self.H, self.W)
 
     def alloc_outputs(self):
-        import torch
+        torch = _torch()
         cls = torch.empty(self.image_shape, dtype=torch.uint8, device=self.device)
         depth = torch.empty(self.image_shape, dtype=torch.float16, device=self.device)
         return cls, depth
 
     # -- calls ----------------------------------------------------------------------------------
     def render(self, poses, dims, rig, active=None, out_class=None, out_depth=None, stream=None):
-        import torch
+        torch = _torch()
         if out_class is None or out_depth is None:
             out_class, out_depth = self.alloc_outputs()
         n, npx = self.n_agents, self.n_agents * self.K * self.H * self.W
+        rig_ptr, rig = _rig_ptr(rig)
         _check(self._lib, self._lib.pic_render(
             self._h, _dev_ptr(poses, torch.float32, 3 * n), _dev_ptr(dims, torch.float32, 3 * n),
-            _dev_ptr(active, torch.uint8, n) if active is not None else None, _rig_array(rig),
+            _dev_ptr(active, torch.uint8, n) if active is not None else None, rig_ptr,
             _dev_ptr(out_class, torch.uint8, npx), _dev_ptr(out_depth, torch.float16, npx), _stream_ptr(stream)))
         return out_class, out_depth
 
@@ -275,13 +289,14 @@ class Scene:
     def render_rgb(self, poses, dims, rig, active=None, out_rgb=None, antialias=False, stream=None):
         """Colour images, u8 [E,A,K,H,W,3] (with OPT_OUT_RELATIVE: [views rendered,H,W,3], which the caller sizes);
         antialias: analytic coverage at one sample per pixel."""
-        import torch
+        torch = _torch()
         if out_rgb is None:
             out_rgb = torch.empty(self.image_shape + (3,), dtype=torch.uint8, device=self.device)
         n, npx = self.n_agents, self.n_agents * self.K * self.H * self.W
+        rig_ptr, rig = _rig_ptr(rig)
         _check(self._lib, self._lib.pic_render_rgb(
             self._h, _dev_ptr(poses, torch.float32, 3 * n), _dev_ptr(dims, torch.float32, 3 * n),
-            _dev_ptr(active, torch.uint8, n) if active is not None else None, _rig_array(rig),
+            _dev_ptr(active, torch.uint8, n) if active is not None else None, rig_ptr,
             1 if antialias else 0, _dev_ptr(out_rgb, torch.uint8), _stream_ptr(stream)))
         return out_rgb
 
@@ -291,13 +306,14 @@ class Scene:
         called with views of the buffers (shape [n_views, H, W]); the device is synchronised before it runs, and
         the next pass overwrites the buffers.  Returns the number of passes.  Argument marshalling only: every
         pass is one pic_render call with PIC_OPT_VIEW_FIRST / VIEW_COUNT / OUT_RELATIVE set."""
-        import torch
+        torch = _torch()
         total = self.n_agents * self.K
         per_view = 3 * self.H * self.W
         n_pass_views = max(1, min(total, int(max_bytes) // per_view))
         out_c = torch.empty((n_pass_views, self.H, self.W), dtype=torch.uint8, device=self.device)
         out_d = torch.empty((n_pass_views, self.H, self.W), dtype=torch.float16, device=self.device)
         n, passes = self.n_agents, 0
+        rig_ptr, rig = _rig_ptr(rig)
         try:
             self.set_option(OPT_OUT_RELATIVE, 1)
             for first in range(0, total, n_pass_views):
@@ -306,7 +322,7 @@ class Scene:
                 self.set_option(OPT_VIEW_COUNT, cnt)
                 _check(self._lib, self._lib.pic_render(
                     self._h, _dev_ptr(poses, torch.float32, 3 * n), _dev_ptr(dims, torch.float32, 3 * n),
-                    _dev_ptr(active, torch.uint8, n) if active is not None else None, _rig_array(rig),
+                    _dev_ptr(active, torch.uint8, n) if active is not None else None, rig_ptr,
                     out_c.data_ptr(), out_d.data_ptr(), _stream_ptr(stream)))
                 torch.cuda.synchronize(self.device)
                 consume(first, cnt, out_c[:cnt], out_d[:cnt])
@@ -327,13 +343,14 @@ class Scene:
                 raise TypeError(f"expected contiguous {dtype} array of {numel} elements")
             return a.ctypes.data
         n, npx = self.n_agents, self.n_agents * self.K * self.H * self.W
+        rig_ptr, rig = _rig_ptr(rig)
         _check(self._lib, self._lib.pic_render_host(
             self._h, hp(poses, np.float32, 3 * n), hp(dims, np.float32, 3 * n), hp(active, np.uint8, n),
-            _rig_array(rig), hp(out_class, np.uint8, npx), hp(out_depth, np.float16, npx), _stream_ptr(stream)))
+            rig_ptr, hp(out_class, np.uint8, npx), hp(out_depth, np.float16, npx), _stream_ptr(stream)))
         return out_class, out_depth
 
     def set_state(self, state, dims, active=None, stream=None):
-        import torch
+        torch = _torch()
         n = self.n_agents
         _check(self._lib, self._lib.pic_set_state(
             self._h, _dev_ptr(state, torch.float32, 4 * n), _dev_ptr(dims, torch.float32, 3 * n),
@@ -341,12 +358,12 @@ class Scene:
 
     def set_agent_classes(self, classes, stream=None):
         """classes: CUDA u8 tensor [E,A] (class of each agent's box), or None for the scene-wide agent class."""
-        import torch
+        torch = _torch()
         _check(self._lib, self._lib.pic_set_agent_classes(
             self._h, _dev_ptr(classes, torch.uint8, self.n_agents) if classes is not None else None, _stream_ptr(stream)))
 
     def get_state(self, out=None, stream=None):
-        import torch
+        torch = _torch()
         if out is None:
             out = torch.empty((self.E, self.A, 4), dtype=torch.float32, device=self.device)
         _check(self._lib, self._lib.pic_get_state(self._h, _dev_ptr(out, torch.float32, 4 * self.n_agents),
@@ -354,22 +371,24 @@ class Scene:
         return out
 
     def step(self, actions, rig, out_class=None, out_depth=None, stream=None):
-        import torch
+        torch = _torch()
         if out_class is None or out_depth is None:
             out_class, out_depth = self.alloc_outputs()
         n, npx = self.n_agents, self.n_agents * self.K * self.H * self.W
+        rig_ptr, rig = _rig_ptr(rig)
         _check(self._lib, self._lib.pic_step(
-            self._h, _dev_ptr(actions, torch.float32, 2 * n), _rig_array(rig), _dev_ptr(out_class, torch.uint8, npx),
+            self._h, _dev_ptr(actions, torch.float32, 2 * n), rig_ptr, _dev_ptr(out_class, torch.uint8, npx),
             _dev_ptr(out_depth, torch.float16, npx), _stream_ptr(stream)))
         return out_class, out_depth
 
     def step_rgb(self, actions, rig, out_rgb=None, antialias=False, stream=None):
         """One simulator step, then colour images u8 [E,A,K,H,W,3] from the new state."""
-        import torch
+        torch = _torch()
         if out_rgb is None:
             out_rgb = torch.empty(self.image_shape + (3,), dtype=torch.uint8, device=self.device)
+        rig_ptr, rig = _rig_ptr(rig)
         _check(self._lib, self._lib.pic_step_rgb(
-            self._h, _dev_ptr(actions, torch.float32, 2 * self.n_agents), _rig_array(rig), 1 if antialias else 0,
+            self._h, _dev_ptr(actions, torch.float32, 2 * self.n_agents), rig_ptr, 1 if antialias else 0,
             _dev_ptr(out_rgb, torch.uint8), _stream_ptr(stream)))
         return out_rgb
 
@@ -386,7 +405,7 @@ class Scene:
         return np.array(buf[:min(int(n.value), 1024)], dtype=np.float64)
 
     def set_option(self, option: int, value) -> None:
-        import torch
+        torch = _torch()
         if isinstance(value, torch.Tensor):
             self._keep.append(value)
             value = value.data_ptr()
