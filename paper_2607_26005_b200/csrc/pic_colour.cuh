@@ -385,7 +385,8 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
     extern __shared__ __align__(16) unsigned char smem_raw[];
     ColourSmem& s = *reinterpret_cast<ColourSmem*>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned id = blockIdx.x * (unsigned)NW + warp;
+    launch_dependents();
+    const unsigned id = await_previous(blockIdx.x) * (unsigned)NW + warp;
     const bool valid = id < P.n_jobs;
     const uint2* blk = P.surv + (size_t)id * SURV_STRIDE;
     int ns = -2, n_big = 0;
@@ -626,11 +627,7 @@ cudaError_t launch_colour_kernel(const RenderParams& P0, long long n_views, bool
     P.debug_flags = 0;
     P.counters = nullptr;
     const unsigned grid = (unsigned)((jobs + NW - 1) / NW);
-    if (antialias) cull_kernel<NoTally, true><<<grid, NTHREADS, sizeof(CullSmem), stream>>>(P);
-    else cull_kernel<NoTally, false><<<grid, NTHREADS, sizeof(CullSmem), stream>>>(P);
-    cudaError_t err = cudaGetLastError();
+    const cudaError_t err = launch_next(antialias ? cull_kernel<NoTally, true> : cull_kernel<NoTally, false>, grid, sizeof(CullSmem), stream, P);
     if (err != cudaSuccess) return err;
-    if (antialias) colour_kernel<true><<<grid, NTHREADS, sizeof(ColourSmem), stream>>>(P);
-    else colour_kernel<false><<<grid, NTHREADS, sizeof(ColourSmem), stream>>>(P);
-    return cudaGetLastError();
+    return launch_next(antialias ? colour_kernel<true> : colour_kernel<false>, grid, sizeof(ColourSmem), stream, P);
 }

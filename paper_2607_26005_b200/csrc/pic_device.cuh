@@ -15,6 +15,16 @@ namespace pic {
 
 constexpr float ZPROJ_FRAC = 0.5f;     // vertices nearer than this * near are not projected
 
+// Programmatic dependent launch: the kernels of a call are launched so that the next one is brought onto the
+// multiprocessors while the last blocks of the previous one still run.  A kernel that reads what its predecessor wrote
+// first waits for it with await_previous, which passes a value through (the thread's job number): every address derived
+// from that value, read-only loads included, is ordered after the wait.
+__device__ __forceinline__ void launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ unsigned await_previous(unsigned id) {
+    asm volatile("griddepcontrol.wait;" : "+r"(id)::"memory");
+    return id;
+}
+
 // Geometry of the tile being rendered.
 struct TileCtx {
     int x0, y0, tw, th;          // tile origin and size in pixels

@@ -1,10 +1,12 @@
-// Agent kernel, rig-table kernel, exhaustive cross-check kernel and host-side launchers.
+// Set-up kernel (agents, rig tables), exhaustive cross-check kernel and host-side launchers.
 //
 // The exhaustive kernel (see pic_exhaustive.cuh) is the cross-check of the production kernels in
 // pic_render.cu.
 #include "pic_exhaustive.cuh"
 
 namespace pic {
+
+constexpr int SETUP_THREADS = 128;
 
 struct RigParams {
     int32_t K, W, H;
@@ -14,15 +16,33 @@ struct RigParams {
 };
 
 // ------------------------------------------------------------------------------------------------
-// agent kernel: poses/dims/active -> AgentGeom + one ViewCam per camera (optionally after one
+// set-up kernel, agents: poses/dims/active -> AgentGeom + one ViewCam per camera (optionally after one
 // kinematic-bicycle step of the scene's own state)
 // ------------------------------------------------------------------------------------------------
-__global__ void agent_kernel(int n, const float* __restrict__ poses, float* state, const float* __restrict__ actions,
-                             const float* __restrict__ dims, const uint8_t* __restrict__ active,
-                             const uint8_t* __restrict__ agent_cls, uint32_t default_cls, AgentGeom* __restrict__ out, ViewCam* __restrict__ cams, uint32_t* status,
-                             const __grid_constant__ RigParams R, float dt, float wheelbase, float v_max) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
+struct AgentArgs {
+    int n;
+    const float* poses;
+    float* state;
+    const float* actions;
+    const float* dims;
+    const uint8_t* active;
+    const uint8_t* agent_cls;
+    uint32_t default_cls;
+    AgentGeom* out;
+    ViewCam* cams;
+    uint32_t* status;
+    float dt, wheelbase, v_max;
+};
+
+// One agent: its kinematic step, geometry and camera records.
+__device__ __forceinline__ void agent_setup(const AgentArgs& G, const RigParams& R, int i) {
+    const float* __restrict__ poses = G.poses;
+    const float* __restrict__ actions = G.actions;
+    const float* __restrict__ dims = G.dims;
+    float* state = G.state;
+    const float dt = G.dt, wheelbase = G.wheelbase, v_max = G.v_max;
+    const uint8_t* __restrict__ active = G.active;
+    uint32_t* status = G.status;
     bool act = active ? active[i] != 0 : true;
     float x, y, th;
     if (state) {                                   // pic_step: update the scene's own state in place
@@ -59,22 +79,20 @@ __global__ void agent_kernel(int n, const float* __restrict__ poses, float* stat
     g.x = x; g.y = y;
     sincosf(th, &g.s, &g.c);
     g.hl = 0.5f * l; g.hw = 0.5f * w; g.h = h;
-    g.active = act ? (1u | ((agent_cls ? (uint32_t)agent_cls[i] : default_cls) << 8)) : 0u;
-    out[i] = g;
+    g.active = act ? (1u | ((G.agent_cls ? (uint32_t)G.agent_cls[i] : G.default_cls) << 8)) : 0u;
+    G.out[i] = g;
     for (int k = 0; k < R.K; ++k) {
         ViewCam vc;
         make_view_cam(vc, g, R.cam[k]);
-        float4* dst = reinterpret_cast<float4*>(cams + (size_t)i * R.K + k);
+        float4* dst = reinterpret_cast<float4*>(G.cams + (size_t)i * R.K + k);
         const float4* src = reinterpret_cast<const float4*>(&vc);
         dst[0] = src[0]; dst[1] = src[1]; dst[2] = src[2]; dst[3] = src[3];
     }
 }
 
 // Per-camera tables: ray coordinates of every pixel column / row and the background of every row.
-__global__ void rig_kernel(const __grid_constant__ RigParams R, float* __restrict__ ray_x, float* __restrict__ ray_y,
-                           float* __restrict__ bg_z, uint32_t* __restrict__ bg_cls, uint32_t* overflow) {
-    const int k = blockIdx.x;
-    if (overflow && k == 0 && threadIdx.x == 0) overflow[0] = 0u;   // the render kernels' list of left-out tiles starts empty (absent for callers that do not use them)
+__device__ __forceinline__ void rig_setup(const RigParams& R, int k, float* __restrict__ ray_x, float* __restrict__ ray_y,
+                                          float* __restrict__ bg_z, uint32_t* __restrict__ bg_cls) {
     const CamConst c = R.cam[k];
     const float cx = 0.5f * (float)R.W, cy = 0.5f * (float)R.H;
     for (int u = threadIdx.x; u < R.W; u += blockDim.x)
@@ -86,6 +104,20 @@ __global__ void rig_kernel(const __grid_constant__ RigParams R, float* __restric
         background(c.cphi, c.sphi, c.mz, ry, R.far_z, R.cls_sky, R.cls_ground, cls, z);
         bg_z[(size_t)k * R.H + v] = z;
         bg_cls[(size_t)k * R.H + v] = cls;
+    }
+}
+
+// One launch prepares a call: the first K blocks write a camera's tables each, the others set up an agent per thread.
+__global__ void __launch_bounds__(SETUP_THREADS) setup_kernel(const __grid_constant__ AgentArgs G, const __grid_constant__ RigParams R,
+                                                              float* __restrict__ ray_x, float* __restrict__ ray_y, float* __restrict__ bg_z,
+                                                              uint32_t* __restrict__ bg_cls, uint32_t* overflow) {
+    launch_dependents();
+    if (overflow && blockIdx.x == 0 && threadIdx.x == 0) overflow[0] = 0u;   // the render kernels' list of left-out tiles starts empty (absent for callers that do not use them)
+    if ((int)blockIdx.x < R.K) {
+        rig_setup(R, (int)blockIdx.x, ray_x, ray_y, bg_z, bg_cls);
+    } else {
+        const int i = ((int)blockIdx.x - R.K) * SETUP_THREADS + (int)threadIdx.x;
+        if (i < G.n) agent_setup(G, R, i);
     }
 }
 
@@ -137,7 +169,7 @@ static RigParams rig_params(const RenderParams& P) {
     return R;
 }
 
-// Per call: rig tables, then agents (+ optional bicycle step) and their cameras.
+// Per call: rig tables, agents (+ optional bicycle step) and their cameras.
 cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses, float* state, const float* actions,
                          const float* dims, const uint8_t* active, const uint8_t* agent_cls, AgentGeom* agents_out, ViewCam* cams_out,
                          float* tables, uint32_t* status, float dt, float wheelbase, float v_max, cudaStream_t stream) {
@@ -146,11 +178,11 @@ cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses
     float* ray_y = ray_x + (size_t)P.K * P.W;
     float* bg_z = ray_y + (size_t)P.K * P.H;
     uint32_t* bg_cls = reinterpret_cast<uint32_t*>(bg_z + (size_t)P.K * P.H);
-    rig_kernel<<<P.K, 256, 0, stream>>>(R, ray_x, ray_y, bg_z, bg_cls, P.overflow);
-    cudaError_t err = cudaGetLastError();
-    if (err != cudaSuccess || n_agents <= 0) return err;
-    agent_kernel<<<(n_agents + 127) / 128, 128, 0, stream>>>(n_agents, poses, state, actions, dims, active, agent_cls, P.cls_agent, agents_out,
-                                                              cams_out, status, R, dt, wheelbase, v_max);
+    AgentArgs G;
+    G.n = n_agents; G.poses = poses; G.state = state; G.actions = actions; G.dims = dims; G.active = active;
+    G.agent_cls = agent_cls; G.default_cls = P.cls_agent; G.out = agents_out; G.cams = cams_out; G.status = status;
+    G.dt = dt; G.wheelbase = wheelbase; G.v_max = v_max;
+    setup_kernel<<<P.K + (n_agents + SETUP_THREADS - 1) / SETUP_THREADS, SETUP_THREADS, 0, stream>>>(G, R, ray_x, ray_y, bg_z, bg_cls, P.overflow);
     return cudaGetLastError();
 }
 

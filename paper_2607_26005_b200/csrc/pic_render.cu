@@ -5,33 +5,30 @@
 // so "nearest fragment wins, exact ties go to the lower index" is an unsigned max that does not
 // depend on the order in which primitives arrive; 0 means "no fragment" (background).
 //
-// A unit of work is a tile: up to 64 x 64 pixels of one view.  Two kernels share the work.
+// A unit of work is a tile: up to 64 x 64 pixels of one view.
 //
-// render_kernel (the fused kernel).  A CTA of 4 warps takes 4 consecutive tiles.
-//   front   (a) cull, (c) set-up -- one warp per tile, warp-level synchronisation only.  The warp
-//           tests the map's group boxes and the leaf boxes of the visible groups against the tile
-//           frustum (a lane per box), culls the other agents' boxes as spheres and keeps their
-//           camera-facing faces, then tests the candidates 32 at a time (camera-space vertices,
-//           pixel box) and compacts the survivors with ballots.  Its lists live in the key buffer,
-//           which is idle until the back end starts.  After one CTA barrier the survivors of the 4
-//           tiles get consecutive ranges of a shared record pool and are set up, a lane per
+// cull_kernel.  A warp per tile finds the primitives and box faces that can touch a pixel centre and leaves them as a
+// list in device memory.
+//
+// render_full_kernel (images of full tiles, the workloads) and render_kernel (ragged tiles, options).  A CTA of 4 warps
+// takes 4 consecutive tiles.
+//   set-up  the survivors of the 4 tiles get consecutive ranges of a shared record pool and are set up, a lane per
 //           survivor: 3-4 edge functions + 1/z plane in a 17-word record.
-//   back    (b) raster, (c), (d) store -- after a second CTA barrier the 16 strips of 16 pixel rows
-//           (4 per tile) are tasks that the warps draw from a counter.  A warp owns one strip of
-//           keys (8 KB).  Per strip it looks at the tile's records 32 at a time (a lane each: does
-//           the box reach the strip?), rasterizes primitives of <= 4 pixels from their lane with
-//           atomic max, then walks the other hits together: a lane per pixel pair of a 16 x 4
-//           pixel cell, plain loads and stores; boxes of >= 256 pixels first classify the strip's
-//           16 cells (trivial reject / trivial accept / which edges still need testing) from the
-//           same float32 edge functions.  The store converts keys to class u8 + depth binary16
-//           with 128-bit stores, resets the keys it read, and writes 8 x 8 blocks that nothing
-//           touched without reading keys.
-//   Tiles whose lists overflow, or whose records do not fit the pool beside their fellows', are
-//   appended to a list in device memory.
+//   raster  the 16 strips of 16 pixel rows (4 per tile) are tasks that the warps draw from a counter.  A warp owns one
+//           strip of keys (8 KB).  Per strip it looks at the tile's records 32 at a time (a lane each: does the box
+//           reach the strip?), rasterizes primitives of <= 4 pixels from their lane with atomic max, then walks the
+//           other hits together: a lane per pixel pair of a 16 x 4 pixel cell, plain loads and stores; boxes of >= 256
+//           pixels first classify the strip's 16 cells (trivial reject / trivial accept / which edges still need
+//           testing) from the same float32 edge functions.
+//   store   converts keys to class u8 + depth binary16 with 128- and 256-bit stores, resets the keys it read, and
+//           writes 8 x 8 blocks that nothing touched without reading keys.
+//   Tiles whose lists overflow, or whose records do not fit the pool, are appended to a list in device memory.
 //
 // cooperative_kernel.  One wave of CTAs walks that list; a whole CTA renders a tile in
 // barrier-separated phases with per-round lists (any number of groups, boxes, survivors and
-// records): the general path, and the one the fused kernel is checked against in the tests.
+// records): the general path, and the one the others are checked against in the tests.
+//
+// render_small_kernel (pic_small.cuh).  Calls with few tiles: a CTA of 8 warps takes one tile from culling to store.
 //
 // Cameras (one 64-byte record per view) and per-camera ray / background tables are prepared by
 // the agent and rig kernels, so the prologues are a few loads.
@@ -323,7 +320,7 @@ __device__ __forceinline__ bool raster_cell(S& s, const TileCtx& t, const PrimEq
 // Cooperative kernel, phase 3: every warp walks all records but rasterizes only the bands (4 pixel rows) it owns --
 // band b belongs to warp b % NW -- so keys are updated without atomics and the bands of a large
 // primitive are shared out evenly.
-template <class S, class TL>
+template <int NWARPS, class S, class TL>
 __device__ __forceinline__ void raster_records(S& s, const float4* rec, uint32_t* touched_out, const TileCtx& t, int n_rec, bool classify, TL& n) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     unsigned long long touched = 0ull;     // 8x8 blocks
@@ -334,7 +331,7 @@ __device__ __forceinline__ void raster_records(S& s, const float4* rec, uint32_t
         const int bx0 = bw & 63, by0 = (bw >> 6) & 63, bx1 = (bw >> 12) & 63, by1 = (bw >> 18) & 63;
         // first band of this warp at or after the box's first band
         const int band0 = by0 >> 2, band1 = by1 >> 2;
-        int first = band0 + ((warp - band0) & (NW - 1));
+        int first = band0 + ((warp - band0) & (NWARPS - 1));
         if (first > band1) continue;
         PrimEq q;
         const float4 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3];
@@ -349,7 +346,7 @@ __device__ __forceinline__ void raster_records(S& s, const float4* rec, uint32_t
         if (classify && (bx1 - bx0 + 1) * (by1 - by0 + 1) >= CLASSIFY_MIN_PIXELS) {
             // (b) lanes 0..15 classify this warp's 16 cells: reject / partly covered / inside
             if (warp == 0) ++n.classified;
-            const int band = (lane >> 2) * NW + warp, col = lane & 3;
+            const int band = (lane >> 2) * NWARPS + warp, col = lane & 3;
             const int xa = col * 16, xb = xa + 15, ya = band * 4, yb = ya + 3;
             bool reject = lane >= 16 || xb < bx0 || xa > bx1 || yb < by0 || ya > by1;
             uint32_t need = 0u;
@@ -373,13 +370,13 @@ __device__ __forceinline__ void raster_records(S& s, const float4* rec, uint32_t
             }
             for (unsigned m = __ballot_sync(0xffffffffu, !reject); m; m &= m - 1) {
                 const int cell = __ffs(m) - 1;
-                const int xx = (cell & 3) * 16, yy = ((cell >> 2) * NW + warp) * 4;
+                const int xx = (cell & 3) * 16, yy = ((cell >> 2) * NWARPS + warp) * 4;
                 const uint32_t need_c = __shfl_sync(0xffffffffu, need, cell);
                 ++n.cells;
                 if (raster_cell(s, t, q, thr, key_lo, xx, yy, need_c, lane)) touched |= 3ull << ((yy >> 3) * 8 + (xx >> 3));
             }
         } else {
-            for (int band = first; band <= band1; band += NW)
+            for (int band = first; band <= band1; band += NWARPS)
                 for (int xx = bx0 & ~15; xx <= bx1; xx += 16) {
                     ++n.cells;
                     if (raster_cell(s, t, q, thr, key_lo, xx, band * 4, 0xFu, lane)) touched |= 3ull << ((band >> 1) * 8 + (xx >> 3));
@@ -504,8 +501,8 @@ __device__ __forceinline__ void load_rays(S& s, const RenderParams& P, const Job
 }
 
 // A whole tile rendered by the CTA in barrier-separated phases with per-round lists: any number of
-// groups, boxes, survivors and records.  It serves the tiles that the fused kernel leaves out.
-template <class TL, bool FULL>
+// groups, boxes, survivors and records.  It serves the tiles that a render kernel's lists cannot hold.
+template <class TL, bool FULL, int NT>
 __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams& P, unsigned job_id, TL& n) {
     const Job job = decode_job(P, job_id);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -534,12 +531,12 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
         } else {
             tile_planes(s, threadIdx.x, c, t);
         }
-    } else if (threadIdx.x >= 64) {
+    } else if (threadIdx.x >= 64 && threadIdx.x < 64 + TILE) {
         load_rays(s, P, job, threadIdx.x - 64);
     }
 #pragma unroll
-    for (int i = 0; i < TILE * TILE / 2 / NTHREADS; ++i)
-        reinterpret_cast<ulonglong2*>(s.key)[i * NTHREADS + threadIdx.x] = make_ulonglong2(0ull, 0ull);
+    for (int i = 0; i < TILE * TILE / 2 / NT; ++i)
+        reinterpret_cast<ulonglong2*>(s.key)[i * NT + threadIdx.x] = make_ulonglong2(0ull, 0ull);
     __syncthreads();
 
     if (ego_active && stop != 1) {
@@ -555,9 +552,9 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
                 Node gn;
                 if (lane < GROUP_BATCH && g < mi.group_end) { gn = (round == 0) ? gn0 : P.groups[g]; vis = box_visible(s, gn); if (warp == 0) ++n.grp; }
                 unsigned gm = __ballot_sync(0xffffffffu, vis);
-                // warp w takes the visible groups w, w + NW, ...
+                // warp w takes the visible groups w, w + NT / 32, ...
                 for (int i = 0; gm; gm &= gm - 1, ++i) {
-                    if ((i & (NW - 1)) != warp) continue;
+                    if ((i & (NT / 32 - 1)) != warp) continue;
                     const int src = __ffs(gm) - 1;
                     const uint32_t first = __shfl_sync(0xffffffffu, gn.first, src);
                     const uint32_t cnt = __shfl_sync(0xffffffffu, gn.count, src);
@@ -572,7 +569,7 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
                 }
             }
             // boxes are taken from the last thread down: the first warps are busier with the visible groups
-            for (int b = round * BOX_ROUND + (NTHREADS - 1 - (int)threadIdx.x); b < min(P.A, (round + 1) * BOX_ROUND); b += NTHREADS) {
+            for (int b = round * BOX_ROUND + (NT - 1 - (int)threadIdx.x); b < min(P.A, (round + 1) * BOX_ROUND); b += NT) {
                 if (b == a) continue;
                 const AgentGeom g = P.agents[(size_t)e * P.A + b];
                 if (!g.active) continue;
@@ -585,7 +582,7 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
             // ---- phase 2a (a): one thread per candidate: camera space, pixel box; survivors are compacted
             const int nl = s.n_leaf, nf = s.n_face;
             const int n_items = (stop == 2) ? 0 : nl * LEAF_PRIMS + nf;
-            for (int i0 = 0; i0 < n_items; i0 += NTHREADS) {
+            for (int i0 = 0; i0 < n_items; i0 += NT) {
                 const int i = i0 + threadIdx.x;
                 V3 V[4], Pn;
                 uint32_t key_lo, flags, box = 0;
@@ -610,7 +607,7 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
             __syncthreads();
             // ---- phase 2b (c): one thread per survivor: edge functions, 1/z plane, tiny raster or record
             const int ns = (stop == 3) ? 0 : min(s.n_surv, SCAP);
-            for (int j = threadIdx.x; j < ns; j += NTHREADS) {
+            for (int j = threadIdx.x; j < ns; j += NT) {
                 const uint2 sv = s.surv[j];
                 V3 V[4], Pn;
                 uint32_t key_lo, flags;
@@ -621,19 +618,19 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
             if (round + 1 < n_rounds) {
                 // the lists are reused by the next round; records are rasterized now if they might overflow
                 const int n_rec = min(s.n_rec, rec_cap);
-                if (n_rec > rec_cap / 2) raster_records(s, s.rec, s.touched, t, n_rec, classify, n);
+                if (n_rec > rec_cap / 2) raster_records<NT / 32>(s, s.rec, s.touched, t, n_rec, classify, n);
                 __syncthreads();
                 if (threadIdx.x == 0) { s.n_leaf = 0; s.n_face = 0; s.n_surv = 0; if (n_rec > rec_cap / 2) s.n_rec = 0; }
                 __syncthreads();
             }
         }
         // ---- phase 3 (b)+(c): one warp per record
-        if (stop == 0 || stop > 5) raster_records(s, s.rec, s.touched, t, min(s.n_rec, rec_cap), classify, n);
+        if (stop == 0 || stop > 5) raster_records<NT / 32>(s, s.rec, s.touched, t, min(s.n_rec, rec_cap), classify, n);
         if (stop == 5 && threadIdx.x == 0) { s.touched[0] = 0xffffffffu; s.touched[1] = 0xffffffffu; }
         __syncthreads();
     }
     // ---- phase 4 (d)
-    store_tile<FULL>(s, t, P, view, k, ego_active, ((unsigned long long)s.touched[1] << 32) | s.touched[0], false, threadIdx.x, NTHREADS, mi.n_tris);
+    store_tile<FULL>(s, t, P, view, k, ego_active, ((unsigned long long)s.touched[1] << 32) | s.touched[0], false, threadIdx.x, NT, mi.n_tris);
     if (threadIdx.x == 0) { ++n.jobs; ++n.coop; }
 }
 
@@ -654,15 +651,7 @@ __device__ __forceinline__ void flush_counters(const RenderParams& P, const Tall
 }
 
 // ---------------------------------------------------------------------------------------------
-// Fused kernel: a CTA takes NW consecutive tiles (see the head of this file).
-//
-//   front   warp w culls tile w on its own (hierarchy, boxes, candidate tests), with warp-level
-//           synchronisation only and its lists in its (still unused) strip of keys; after a CTA
-//           barrier the survivors of the NW tiles get consecutive ranges of one record pool and
-//           are set up, one lane per survivor.  Dense passes.
-//   back    after a second CTA barrier, 16-row strips are tasks drawn from a counter: a warp
-//           rasterizes a strip of some tile into its own strip of keys and stores it (back_strip).
-//   rest    tiles whose lists or records did not fit are appended to the cooperative kernel's list.
+// Cull kernel, and the render kernels over its survivor lists (see the head of this file).
 // ---------------------------------------------------------------------------------------------
 constexpr int POOL = 128;         // records shared by the NW tiles of a CTA
 constexpr int STRIP = 16;         // pixel rows a warp rasterizes at a time
@@ -680,19 +669,25 @@ constexpr uint32_t REC_TINY = 1u << 28, REC_DEAD = 1u << 29;   // flags in the b
 constexpr uint32_t REC_INRANGE = 1u << 30;   // every covered pixel is within [near, far]: no per-pixel range test
 
 constexpr int W_LARGE = 64;       // visible leaves of the large-primitive list
-struct __align__(16) FrontLists {
+// A tile's frustum and its footprint on the ground plane.
+struct __align__(16) Frustum {
     float plane[6][4];                        // (read as float4: kept first, 16-byte aligned)
     float side[4][4];
     Cam cam;
     float seg[10][6];                         // footprint segments: x, y, dx, dy, 1 / dy, unused
     float pt[5][2];                           // footprint corners (ego-relative xy): apex, four far corners
+    int n_seg;                                // segments to look at: 3 for a camera without pitch (the corners coincide in pairs), else 10
+};
+static_assert(offsetof(Frustum, plane) % 16 == 0 && offsetof(Frustum, side) % 16 == 0, "planes are read with 128-bit loads");
+
+struct __align__(16) FrontLists {
+    Frustum f;
     uint32_t face[W_FACE];                    // agent << 3 | face
     uint32_t lleaf[W_LARGE];                  // visible large-primitive leaves: first << 3 | count
     uint32_t row_first[32];                   // grid rows of a pass: first entry of the row's range in cell_prims
     uint32_t row_off[33];                     //   and the number of candidates before the row (the total at [32])
     int n_face;
 };
-static_assert(offsetof(FrontLists, plane) % 16 == 0 && offsetof(FrontLists, side) % 16 == 0, "planes are read with 128-bit loads");
 
 struct __align__(16) FusedSmem {
     unsigned long long key[NW][STRIP_KEYS];   // warp w's strip of keys; during the front end, its FrontLists
@@ -783,6 +778,83 @@ __device__ __forceinline__ void append_survivor(uint2* __restrict__ surv, bool k
     n_tiny += __popc(mt);
 }
 
+// Camera, frustum planes and footprint of a tile, by one warp.  The footprint is the convex hull of the apex and the
+// four far corners, kept as the segments between them (the hull's edges are among them, the others lie inside it).
+__device__ __forceinline__ void frustum_setup(Frustum& f, const RenderParams& P, const Job& job, int lane) {
+    const TileCtx& t = job.t;
+    if (lane < 7) {
+        Cam c;
+        load_camera(c, P.cams[job.view], P.cam[job.k], P.W, P.H);
+        if (lane == 6) {
+            f.cam = c;
+            f.n_seg = (c.dx == 0.f && c.dy == 0.f) ? 3 : 10;     // no pitch: corners 1, 3 and 2, 4 have the same x, y
+        } else {
+            tile_planes(f, lane, c, t);
+        }
+        if (lane < 5) {
+            // footprint corner `lane`: the apex, or a corner of the tile's frustum at depth far (a little beyond)
+            const float F = lane ? t.far_z * 1.001f : 0.f;
+            const float xc = ((float)((lane & 1) ? t.x0 + t.tw : t.x0) - c.cx) / c.focx * F;
+            const float yc = ((float)((lane & 2) ? t.y0 + t.th : t.y0) - c.cy) / c.focy * F;
+            f.pt[lane][0] = c.mwx + c.rx * xc + c.dx * yc + c.fx_ * F;
+            f.pt[lane][1] = c.mwy + c.ry * xc + c.dy * yc + c.fy_ * F;
+        }
+    }
+    __syncwarp();
+    if (lane < 10) {
+        const int i = (int)((0x3221100100ull >> (4 * lane)) & 15u), j = (int)((0x4434343221ull >> (4 * lane)) & 15u);   // (0,1) (0,2) (1,2) (0,3) (0,4) (1,3) (1,4) (2,3) (2,4) (3,4)
+        const float px = f.pt[i][0], py = f.pt[i][1], dx = f.pt[j][0] - px, dy = f.pt[j][1] - py;
+        f.seg[lane][0] = px; f.seg[lane][1] = py; f.seg[lane][2] = dx; f.seg[lane][3] = dy;
+        f.seg[lane][4] = dy != 0.f ? 1.f / dy : 0.f; f.seg[lane][5] = 0.f;
+    }
+    __syncwarp();
+}
+
+// The grid rows crossed by the footprint, widened by the map's margin.
+struct GridRows {
+    int lo, hi;             // (hi < lo if the footprint misses the grid)
+    float gx0, gy0;         // the grid's corner, ego-relative
+};
+__device__ __forceinline__ GridRows grid_rows(const Frustum& f, const MapInfo& mi) {
+    GridRows g;
+    g.gx0 = sub(mi.gx0, f.cam.px); g.gy0 = sub(mi.gy0, f.cam.py);
+    float ylo = f.pt[0][1], yhi = ylo;
+#pragma unroll
+    for (int k = 1; k < 5; ++k) { ylo = fminf(ylo, f.pt[k][1]); yhi = fmaxf(yhi, f.pt[k][1]); }
+    const float fr0 = floorf((ylo - mi.margin - g.gy0) * mi.inv_cell), fr1 = floorf((yhi + mi.margin - g.gy0) * mi.inv_cell);
+    g.lo = (int)fmaxf(fr0, 0.f); g.hi = (int)fminf(fr1, (float)mi.ny - 1.f);
+    return g;
+}
+
+// The range of grid_prims under the part of grid row `row` that the widened footprint crosses.
+__device__ __forceinline__ void row_range(const Frustum& f, const RenderParams& P, const MapInfo& mi, const GridRows& g, int row, uint32_t& first, uint32_t& cnt) {
+    first = 0u; cnt = 0u;
+    if (row > g.hi) return;
+    const float margin = mi.margin, blo = g.gy0 + (float)row * mi.cell - margin, bhi = blo + mi.cell + 2.f * margin;
+    float xlo = 3e38f, xhi = -3e38f;
+    const int n_seg = f.n_seg;
+#pragma unroll 1
+    for (int k = 0; k < n_seg; ++k) {
+        const float px = f.seg[k][0], py = f.seg[k][1], dx = f.seg[k][2], dy = f.seg[k][3], idy = f.seg[k][4];
+        const float ya = fminf(py, py + dy), yb = fmaxf(py, py + dy);
+        if (yb >= blo && ya <= bhi) {
+            const float ta = (blo - py) * idy, tb = (bhi - py) * idy;
+            const float t0 = dy != 0.f ? fminf(fmaxf(fminf(ta, tb), 0.f), 1.f) : 0.f, t1 = dy != 0.f ? fminf(fmaxf(fmaxf(ta, tb), 0.f), 1.f) : 1.f;
+            const float xa = px + t0 * dx, xb = px + t1 * dx;
+            xlo = fminf(xlo, fminf(xa, xb)); xhi = fmaxf(xhi, fmaxf(xa, xb));
+        }
+    }
+    if (xlo <= xhi) {
+        const float fx0 = floorf((xlo - margin - g.gx0) * mi.inv_cell), fx1 = floorf((xhi + margin - g.gx0) * mi.inv_cell);
+        if (fx1 >= 0.f && fx0 <= (float)mi.nx - 1.f) {
+            const uint32_t ix0 = (uint32_t)fmaxf(fx0, 0.f), ix1 = (uint32_t)fminf(fx1, (float)mi.nx - 1.f);
+            const uint32_t* cs = P.cell_start + mi.cell_begin + (uint32_t)row * mi.nx;
+            first = __ldg(cs + ix0);
+            cnt = __ldg(cs + ix1 + 1) - first;
+        }
+    }
+}
+
 // Front end of one tile by one warp: fills the survivor list.  Returns the survivor counts
 // (front | back << 16), or -1 if a list overflowed (the tile then goes to the cooperative kernel).
 //
@@ -808,75 +880,24 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
     ag0.active = 0u; ag1.active = 0u;
     if (lane < P.A) ag0 = load_agent(env_agents + lane);
     if (lane + 32 < P.A) ag1 = load_agent(env_agents + lane + 32);
-    if (lane < 7) {
-        Cam c;
-        load_camera(c, P.cams[job.view], P.cam[job.k], P.W, P.H);
-        if (lane == 6) { f.cam = c; f.n_face = 0; }
-        else tile_planes(f, lane, c, t);
-        if (lane < 5) {
-            // footprint corner `lane`: the apex, or a corner of the tile's frustum at depth far (a little beyond)
-            const float F = lane ? t.far_z * 1.001f : 0.f;
-            const float xc = ((float)((lane & 1) ? t.x0 + t.tw : t.x0) - c.cx) / c.focx * F;
-            const float yc = ((float)((lane & 2) ? t.y0 + t.th : t.y0) - c.cy) / c.focy * F;
-            f.pt[lane][0] = c.mwx + c.rx * xc + c.dx * yc + c.fx_ * F;
-            f.pt[lane][1] = c.mwy + c.ry * xc + c.dy * yc + c.fy_ * F;
-        }
-    }
-    __syncwarp();
-    if (lane < 10) {
-        // segment between two of the five corners (every pair: the hull's edges are among them, the others lie inside it)
-        const int i = lane < 4 ? 0 : lane < 7 ? 1 : lane < 9 ? 2 : 3, j = lane < 4 ? lane + 1 : lane < 7 ? lane - 2 : lane < 9 ? lane - 4 : 4;
-        const float px = f.pt[i][0], py = f.pt[i][1], dx = f.pt[j][0] - px, dy = f.pt[j][1] - py;
-        f.seg[lane][0] = px; f.seg[lane][1] = py; f.seg[lane][2] = dx; f.seg[lane][3] = dy;
-        f.seg[lane][4] = dy != 0.f ? 1.f / dy : 0.f; f.seg[lane][5] = 0.f;
-    }
-    __syncwarp();
+    Frustum& fr = f.f;
+    if (lane == 0) f.n_face = 0;
+    frustum_setup(fr, P, job, lane);
     if (stop == 11) return 0;
-    const Cam& c = f.cam;
+    const Cam& c = fr.cam;
     int n_big = 0, n_tiny = 0;
     // ---- the grid rows crossed by the widened footprint; the range of a row's cells in grid_prims
-    const float margin = mi.margin, gx0 = sub(mi.gx0, c.px), gy0 = sub(mi.gy0, c.py);
-    float ylo = f.pt[0][1], yhi = ylo;
-#pragma unroll
-    for (int k = 1; k < 5; ++k) { ylo = fminf(ylo, f.pt[k][1]); yhi = fmaxf(yhi, f.pt[k][1]); }
-    const float fr0 = floorf((ylo - margin - gy0) * mi.inv_cell), fr1 = floorf((yhi + margin - gy0) * mi.inv_cell);
-    const int row_lo = (int)fmaxf(fr0, 0.f), row_hi = (int)fminf(fr1, (float)mi.ny - 1.f);     // (empty if the footprint misses the grid)
-    auto row_range = [&](int row, uint32_t& first, uint32_t& cnt) {
-        first = 0u; cnt = 0u;
-        if (row > row_hi) return;
-        ++n.grp;
-        const float blo = gy0 + (float)row * mi.cell - margin, bhi = blo + mi.cell + 2.f * margin;
-        float xlo = 3e38f, xhi = -3e38f;
-#pragma unroll 1
-        for (int k = 0; k < 10; ++k) {
-            const float px = f.seg[k][0], py = f.seg[k][1], dx = f.seg[k][2], dy = f.seg[k][3], idy = f.seg[k][4];
-            const float ya = fminf(py, py + dy), yb = fmaxf(py, py + dy);
-            if (yb >= blo && ya <= bhi) {
-                const float ta = (blo - py) * idy, tb = (bhi - py) * idy;
-                const float t0 = dy != 0.f ? fminf(fmaxf(fminf(ta, tb), 0.f), 1.f) : 0.f, t1 = dy != 0.f ? fminf(fmaxf(fmaxf(ta, tb), 0.f), 1.f) : 1.f;
-                const float xa = px + t0 * dx, xb = px + t1 * dx;
-                xlo = fminf(xlo, fminf(xa, xb)); xhi = fmaxf(xhi, fmaxf(xa, xb));
-            }
-        }
-        if (xlo <= xhi) {
-            const float fx0 = floorf((xlo - margin - gx0) * mi.inv_cell), fx1 = floorf((xhi + margin - gx0) * mi.inv_cell);
-            if (fx1 >= 0.f && fx0 <= (float)mi.nx - 1.f) {
-                const uint32_t ix0 = (uint32_t)fmaxf(fx0, 0.f), ix1 = (uint32_t)fminf(fx1, (float)mi.nx - 1.f);
-                const uint32_t* cs = P.cell_start + mi.cell_begin + (uint32_t)row * mi.nx;
-                first = __ldg(cs + ix0);
-                cnt = __ldg(cs + ix1 + 1) - first;
-            }
-        }
-    };
+    const GridRows rows = grid_rows(fr, mi);
     // the first 32 rows' ranges are requested now; the boxes below are tested while the loads are under way
     uint32_t first0, cnt0;
-    row_range(row_lo + lane, first0, cnt0);
+    row_range(fr, P, mi, rows, rows.lo + lane, first0, cnt0);
+    if (rows.lo + lane <= rows.hi) ++n.grp;
     // ---- the large primitives' leaves: a lane per leaf box against the six frustum planes
     int n_ll = 0;
     {
         float4 pl[6];
 #pragma unroll
-        for (int p = 0; p < 6; ++p) pl[p] = *reinterpret_cast<const float4*>(f.plane[p]);
+        for (int p = 0; p < 6; ++p) pl[p] = *reinterpret_cast<const float4*>(fr.plane[p]);
         for (uint32_t l0 = mi.large_begin; l0 < mi.large_end; l0 += 32) {
             const uint32_t l = l0 + lane;
             bool vis = false;
@@ -904,7 +925,7 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
             const AgentGeom g = u ? ag1 : ag0;
             const int b = b0 + lane + 32 * u;
             uint32_t faces = 0u;
-            if (b < P.A && b != job.a && g.active) faces = box_faces(f, c, t, g);
+            if (b < P.A && b != job.a && g.active) faces = box_faces(fr, c, t, g);
             if (faces) {
                 int slot = atomicAdd(&f.n_face, __popc(faces));
                 for (; faces; faces &= faces - 1, ++slot)
@@ -914,9 +935,12 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
     }
     if (stop == 12) return 0;
     // ---- candidates of the grid rows, 32 rows per pass: camera space, pixel box; survivors are compacted
-    for (int r0 = row_lo; r0 <= row_hi; r0 += 32) {
+    for (int r0 = rows.lo; r0 <= rows.hi; r0 += 32) {
         uint32_t first = first0, cnt = cnt0;
-        if (r0 != row_lo) row_range(r0 + lane, first, cnt);
+        if (r0 != rows.lo) {
+            row_range(fr, P, mi, rows, r0 + lane, first, cnt);
+            if (r0 + lane <= rows.hi) ++n.grp;
+        }
         uint32_t incl = cnt;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
@@ -1189,10 +1213,6 @@ struct __align__(16) CullSmem {
 #ifndef PIC_CULL_CTAS
 #define PIC_CULL_CTAS 6
 #endif
-#ifndef PIC_CULL_ROUNDS
-#define PIC_CULL_ROUNDS 1
-#endif
-constexpr int CULL_ROUNDS = PIC_CULL_ROUNDS;   // rounds of NW tiles per CTA of the cull kernel
 #ifndef PIC_RENDER_CTAS
 #define PIC_RENDER_CTAS 5
 #endif
@@ -1202,26 +1222,24 @@ __global__ void __launch_bounds__(NTHREADS, PIC_CULL_CTAS) cull_kernel(const __g
     CullSmem& s = *reinterpret_cast<CullSmem*>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int stop = PIC_STOP(P);
-    // a CTA takes CULL_ROUNDS x NW consecutive tiles, NW at a time: consecutive tiles belong to the
-    // same or to neighbouring agents, so the map data a round pulls in serves the next from L1
-#pragma unroll 1
-    for (int round = 0; round < CULL_ROUNDS; ++round) {
-        const unsigned id = (blockIdx.x * (unsigned)CULL_ROUNDS + round) * (unsigned)NW + warp;
-        if (id >= P.n_jobs) return;
-        TL n = {};
-        const Job job = decode_job(P, id);
-        const MapInfo mi = P.env_maps[job.e];
-        const bool ego_active = P.agents[(size_t)job.e * P.A + job.a].active != 0;
-        uint2* blk = P.surv + (size_t)id * SURV_STRIDE;
-        int ns = 0;
-        if (P.debug_flags & 4) ns = -1;             // test aid: every tile through cooperative_job
-        else if (ego_active && stop != 1 && !(stop >= 8 && stop <= 10)) ns = front_cull<TL, CONS>(s.lists[warp], blk + 2, P, job, mi, lane, n);
-        // (the work counts are summed over the warp's lanes; without counters they are constants)
-        const uint32_t c_grp = __reduce_add_sync(0xffffffffu, (uint32_t)tally_value(n.grp)), c_leaf = __reduce_add_sync(0xffffffffu, (uint32_t)tally_value(n.leaf)),
-                       c_tested = __reduce_add_sync(0xffffffffu, (uint32_t)tally_value(n.tested));
-        if (lane == 0) *reinterpret_cast<uint4*>(blk) = make_uint4((uint32_t)ns, c_grp, c_leaf, c_tested);
-        __syncwarp();
-    }
+    const unsigned cta = await_previous(blockIdx.x);
+    const unsigned id = cta * (unsigned)NW + warp;
+    if (id >= P.n_jobs) return;
+    TL n = {};
+    const Job job = decode_job(P, id);
+    const MapInfo mi = P.env_maps[job.e];
+    const bool ego_active = P.agents[(size_t)job.e * P.A + job.a].active != 0;
+    uint2* blk = P.surv + (size_t)id * SURV_STRIDE;
+    int ns = 0;
+    if (P.debug_flags & 4) ns = -1;             // test aid: every tile through cooperative_job
+    else if (ego_active && stop != 1 && !(stop >= 8 && stop <= 10)) ns = front_cull<TL, CONS>(s.lists[warp], blk + 2, P, job, mi, lane, n);
+    // (the work counts are summed over the warp's lanes; without counters they are constants)
+    const uint32_t c_grp = __reduce_add_sync(0xffffffffu, (uint32_t)tally_value(n.grp)), c_leaf = __reduce_add_sync(0xffffffffu, (uint32_t)tally_value(n.leaf)),
+                   c_tested = __reduce_add_sync(0xffffffffu, (uint32_t)tally_value(n.tested));
+    if (lane == 0) *reinterpret_cast<uint4*>(blk) = make_uint4((uint32_t)ns, c_grp, c_leaf, c_tested);
+    // (only now: blocks of the next kernel that came in earlier would crowd the multiprocessors that still have room
+    // instead of spreading over all of them)
+    launch_dependents();
 }
 
 // Render kernel.  FULL: every tile is 64 x 64, rows allow 128-bit stores, no float32 depth image (the
@@ -1232,7 +1250,8 @@ __global__ void __launch_bounds__(NTHREADS, 5) render_kernel(const __grid_consta
     FusedSmem& s = *reinterpret_cast<FusedSmem*>(smem_raw);
     if (PIC_STOP(P) == 15) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned first = blockIdx.x * (unsigned)NW, n_jobs = P.n_jobs;
+    launch_dependents();
+    const unsigned first = await_previous(blockIdx.x) * (unsigned)NW, n_jobs = P.n_jobs;
     TL n = {};
     const bool classify = !(P.debug_flags & 1);
     const int stop = PIC_STOP(P);
@@ -1354,13 +1373,15 @@ static_assert(FSTRIP == 16 || FSTRIP == 8, "strips of 16 or 8 rows");
 
 // The record pool of the full-tile kernel, one array per 16-byte part of a record: 17 words per
 // record instead of the 20 of an array of padded records, so more records fit beside the keys.
+template <int N>
 struct __align__(16) RecordPool {
-    float4 nx[FPOOL], ny[FPOOL], nz[FPOOL];   // edge functions E_i = nx[i] rx + ny[i] ry + nz[i]
-    float4 w[FPOOL];                          // 1/z plane wx, wy, wz; key low word
-    uint32_t box[FPOOL];                      // pixel box (6 bits per coordinate), top-left bits, flags
+    float4 nx[N], ny[N], nz[N];               // edge functions E_i = nx[i] rx + ny[i] ry + nz[i]
+    float4 w[N];                              // 1/z plane wx, wy, wz; key low word
+    uint32_t box[N];                          // pixel box (6 bits per coordinate), top-left bits, flags
 };
 
-__device__ __forceinline__ void write_record(RecordPool& pool, int slot, const PrimEq& q, uint32_t key_lo, uint32_t box, uint32_t extra) {
+template <int N>
+__device__ __forceinline__ void write_record(RecordPool<N>& pool, int slot, const PrimEq& q, uint32_t key_lo, uint32_t box, uint32_t extra) {
     const uint32_t bx0 = box & 0xff, by0 = (box >> 8) & 0xff, bx1 = (box >> 16) & 0xff, by1 = box >> 24;
     pool.nx[slot] = make_float4(q.nx[0], q.nx[1], q.nx[2], q.nx[3]);
     pool.ny[slot] = make_float4(q.ny[0], q.ny[1], q.ny[2], q.ny[3]);
@@ -1369,7 +1390,8 @@ __device__ __forceinline__ void write_record(RecordPool& pool, int slot, const P
     pool.box[slot] = bx0 | (by0 << 6) | (bx1 << 12) | (by1 << 18) | (q.tl << 24) | extra;
 }
 
-__device__ __forceinline__ void read_record(const RecordPool& pool, int slot, PrimEq& q, uint32_t& key_lo) {
+template <int N>
+__device__ __forceinline__ void read_record(const RecordPool<N>& pool, int slot, PrimEq& q, uint32_t& key_lo) {
     const float4 r0 = pool.nx[slot], r1 = pool.ny[slot], r2 = pool.nz[slot], r3 = pool.w[slot];
     q.nx[0] = r0.x; q.nx[1] = r0.y; q.nx[2] = r0.z; q.nx[3] = r0.w;
     q.ny[0] = r1.x; q.ny[1] = r1.y; q.ny[2] = r1.z; q.ny[3] = r1.w;
@@ -1386,7 +1408,7 @@ struct __align__(16) TileRef {
 
 struct __align__(16) FullSmem {
     unsigned long long key[NW][FSTRIP_KEYS];  // warp w's strip of keys
-    RecordPool pool;
+    RecordPool<FPOOL> pool;
     float ray_x[NW][TILE], ray_y[NW][TILE];   // ray tables of tile w
     Cam cam[NW];
     TileRef tile[NW];
@@ -1470,7 +1492,8 @@ __device__ __forceinline__ void store_strip_full(unsigned long long* key, uint8_
 
 // One strip (rows ys .. of the tile) by one warp: the tile's fragments that fall into it, then
 // the records that reach it, cell by cell.  Returns the touched 8 x 8 blocks.
-__device__ __forceinline__ uint32_t raster_strip_full(StripView& s, const RecordPool& pool, int first, int n_rec, int ys, float w_near,
+template <int ROWS, int N>
+__device__ __forceinline__ uint32_t raster_strip(StripView& s, const RecordPool<N>& pool, int first, int n_rec, int ys, float w_near,
                                                       float w_far, int stop, int lane) {
     uint32_t touched = 0u;                       // bit (row >> 3) * 8 + (column >> 3)
     const int kbase = (lane >> 3) << 6, lsw = (lane & 7) ^ (((lane >> 3) & 1) << 2);   // see strip_cell
@@ -1481,11 +1504,11 @@ __device__ __forceinline__ uint32_t raster_strip_full(StripView& s, const Record
             const int slot = first + base + lane;
             bw_lane = pool.box[slot];
             const int by0 = (bw_lane >> 6) & 63, by1 = (bw_lane >> 18) & 63;
-            hit = !(bw_lane & REC_DEAD) && by1 >= ys && by0 < ys + FSTRIP;
+            hit = !(bw_lane & REC_DEAD) && by1 >= ys && by0 < ys + ROWS;
             if (hit && (bw_lane & REC_TINY)) {           // a few pixels: rasterized by this lane (atomic max)
                 hit = false;
                 const int bx0 = bw_lane & 63, bx1 = (bw_lane >> 12) & 63;
-                const int y0 = max(by0, ys) - ys, y1 = min(by1, ys + FSTRIP - 1) - ys;
+                const int y0 = max(by0, ys) - ys, y1 = min(by1, ys + ROWS - 1) - ys;
                 PrimEq q;
                 uint32_t key_lo;
                 read_record(pool, slot, q, key_lo);
@@ -1512,7 +1535,7 @@ __device__ __forceinline__ uint32_t raster_strip_full(StripView& s, const Record
             const uint32_t bw = __shfl_sync(0xffffffffu, bw_lane, src);
             const int by0 = (bw >> 6) & 63, by1 = (bw >> 18) & 63;
             const int bx0 = bw & 63, bx1 = (bw >> 12) & 63;
-            const int ly0 = max(by0, ys) - ys, ly1 = min(by1, ys + FSTRIP - 1) - ys;
+            const int ly0 = max(by0, ys) - ys, ly1 = min(by1, ys + ROWS - 1) - ys;
             PrimEq q;
             uint32_t key_lo;
             read_record(pool, first + base + src, q, key_lo);
@@ -1520,10 +1543,10 @@ __device__ __forceinline__ uint32_t raster_strip_full(StripView& s, const Record
             float thr[4];
             edge_thresholds(q.tl, thr);
             const bool range = !(bw & REC_INRANGE);
-            if (stop != 3 && (bx1 - bx0 + 1) * (ly1 - ly0 + 1) >= CLASSIFY_MIN_STRIP * FSTRIP / 16) {
+            if (stop != 3 && (bx1 - bx0 + 1) * (ly1 - ly0 + 1) >= CLASSIFY_MIN_STRIP * ROWS / 16) {
                 // a lane per 16 x 4 pixel cell of the strip classifies it: reject / partly covered / inside
                 const int xa = (lane & 3) * 16, xb = xa + 15, ya = ((lane >> 2) & 3) * 4, yb = ya + 3;
-                bool reject = lane >= FSTRIP || xb < bx0 || xa > bx1 || yb < ly0 || ya > ly1;
+                bool reject = lane >= ROWS || xb < bx0 || xa > bx1 || yb < ly0 || ya > ly1;
                 uint32_t need = 0u;
                 if (!reject) {
                     const float rxa = s.ray_x[xa], rxb = s.ray_x[xb], rya = s.ray_y[ya], ryb = s.ray_y[yb];   // rxa < rxb, rya < ryb
@@ -1568,7 +1591,8 @@ __global__ void __launch_bounds__(NTHREADS, PIC_RENDER_CTAS) render_full_kernel(
     const int stop = PIC_STOP(P);
     if (stop == 15) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const unsigned id = blockIdx.x * (unsigned)NW + warp;
+    launch_dependents();
+    const unsigned id = await_previous(blockIdx.x) * (unsigned)NW + warp;
     const bool valid = id < P.n_jobs;
     // ---- the cull kernel's survivors of tile first + w, and everything that does not depend on them
     const uint2* blk = P.surv + (size_t)id * SURV_STRIDE;
@@ -1662,7 +1686,7 @@ __global__ void __launch_bounds__(NTHREADS, PIC_RENDER_CTAS) render_full_kernel(
                 if (FSTRIP == 16) { bgc[1] = __ldg(bg_cls + 8); bgz[1] = __ldg(bg_z + 8); }
             }
             sv.ray_x = s.ray_x[j]; sv.ray_y = s.ray_y[j] + ys;
-            uint32_t touched = raster_strip_full(sv, s.pool, (int)((bases >> (8 * j)) & 0xffu), (stop == 14) ? 0 : cj, ys, P.w_near, P.w_far, stop, lane);
+            uint32_t touched = raster_strip<FSTRIP>(sv, s.pool, (int)((bases >> (8 * j)) & 0xffu), (stop == 14) ? 0 : cj, ys, P.w_near, P.w_far, stop, lane);
             if (stop == 5) touched = 0xffffu;
             if (stop == 6) touched |= 0x80000000u;
             const size_t o = tr.pixel0 + (size_t)ys * P.W;
@@ -1677,15 +1701,17 @@ __global__ void __launch_bounds__(NTHREADS, PIC_RENDER_CTAS) render_full_kernel(
         P.overflow[1u + atomicAdd(&P.overflow[0], 1u)] = blockIdx.x * (unsigned)NW + threadIdx.x;
 }
 
-// The tiles the fused kernel left out, a CTA at a time.
+// The tiles the render kernels left out, a CTA at a time.  (Called from the end of those kernels instead, the same code
+// costs them 2 % -- a call bounds their registers -- which is more than a launch that overlaps their last blocks.)
 template <class TL, bool FULL>
 __global__ void __launch_bounds__(NTHREADS, 5) cooperative_kernel(const __grid_constant__ RenderParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TileSmem& cs = *reinterpret_cast<TileSmem*>(smem_raw);
+    const unsigned cta = await_previous(blockIdx.x);
     TL n = {};
     const unsigned count = __ldcg(&P.overflow[0]);
-    for (unsigned i = blockIdx.x; i < count; i += gridDim.x) {
-        cooperative_job<TL, FULL>(cs, P, __ldcg(&P.overflow[1u + i]), n);
+    for (unsigned i = cta; i < count; i += gridDim.x) {
+        cooperative_job<TL, FULL, NTHREADS>(cs, P, __ldcg(&P.overflow[1u + i]), n);
         __syncthreads();
     }
     flush_counters(P, n);
@@ -1703,9 +1729,12 @@ static size_t smem_pad() { const char* e = getenv("PIC_SMEM_PAD"); return e ? (s
 #endif
 #define FULL_SMEM (sizeof(FullSmem) + (RENDER_SMEM - RENDER_SMEM_BASE))
 size_t render_smem_bytes() { return RENDER_SMEM; }
+cudaError_t configure_small_kernel();
 
 cudaError_t configure_render_kernel() {
-    cudaError_t err = cudaFuncSetAttribute(render_full_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FULL_SMEM);
+    cudaError_t err = configure_small_kernel();
+    if (err != cudaSuccess) return err;
+    err = cudaFuncSetAttribute(render_full_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FULL_SMEM);
     if (err != cudaSuccess) return err;
     err = cudaFuncSetAttribute(render_kernel<NoTally, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RENDER_SMEM);
     if (err != cudaSuccess) return err;
@@ -1783,11 +1812,25 @@ __global__ void __launch_bounds__(NTHREADS) coverage_kernel(const __grid_constan
     }
 }
 
+// Launches the next kernel of a call: its blocks may be brought in while the last blocks of the kernel before it still
+// run (it waits for that kernel itself, see await_previous).
+template <class K>
+cudaError_t launch_next(K kernel, unsigned grid, size_t smem, cudaStream_t stream, const RenderParams& P, unsigned threads = NTHREADS) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr; cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P);
+}
+
 }  // namespace pic
 #include "pic_coverage.cuh"
 namespace pic {
 #include "pic_colour.cuh"
 #include "pic_static.cuh"
+#include "pic_small.cuh"
 
 size_t survivor_bytes_per_tile() { return sizeof(uint2) * SURV_STRIDE; }
 
@@ -1798,27 +1841,27 @@ cudaError_t launch_render_kernel(const RenderParams& P0, long long n_views, int 
     if (jobs <= 0) return cudaSuccess;
     P.n_jobs = (uint32_t)jobs;
     const unsigned grid = (unsigned)((jobs + NW - 1) / NW);
+    // few tiles: one CTA takes a tile from culling to store.  Measured (a call on 16 agents per environment, both image
+    // shapes of the workloads): 64 tiles 37.0 -> 20.7 us, 256 tiles 44.6 -> 22.7, 768 tiles 47.3 -> 44.8, 1024 tiles
+    // 48.4 -> 53.7, so the line lies at five tiles per multiprocessor.
+    if (jobs <= 5LL * sm_count && !P.counters && !P.occlusion && (P.debug_flags & 15) == 0)
+        return launch_next(render_small_kernel, (unsigned)jobs, SMALL_SMEM, stream, P, SMALL_THREADS);
     const bool full = P.W % TILE == 0 && P.H % TILE == 0 && P.out_depth32 == nullptr && P.occlusion == nullptr && (P.debug_flags & 15) == 0 &&
                       (reinterpret_cast<uintptr_t>(P.out_depth) & 31u) == 0;   // 256-bit depth stores
     // (a) cull: survivors per tile
-    const unsigned cull_grid = (unsigned)((jobs + NW * CULL_ROUNDS - 1) / (NW * CULL_ROUNDS));
-    if (P.counters) cull_kernel<Tally, false><<<cull_grid, NTHREADS, sizeof(CullSmem), stream>>>(P);
-    else cull_kernel<NoTally, false><<<cull_grid, NTHREADS, sizeof(CullSmem), stream>>>(P);
-    cudaError_t err = cudaGetLastError();
+    cudaError_t err = launch_next(P.counters ? cull_kernel<Tally, false> : cull_kernel<NoTally, false>, grid, sizeof(CullSmem), stream, P);
     if (err != cudaSuccess) return err;
     // (b)-(d) set-up, raster, store
-    if (P.counters) render_kernel<Tally, false><<<grid, NTHREADS, RENDER_SMEM, stream>>>(P);
-    else if (full) render_full_kernel<<<grid, NTHREADS, FULL_SMEM, stream>>>(P);
-    else render_kernel<NoTally, false><<<grid, NTHREADS, RENDER_SMEM, stream>>>(P);
-    err = cudaGetLastError();
+    err = P.counters ? launch_next(render_kernel<Tally, false>, grid, RENDER_SMEM, stream, P)
+          : full     ? launch_next(render_full_kernel, grid, FULL_SMEM, stream, P)
+                     : launch_next(render_kernel<NoTally, false>, grid, RENDER_SMEM, stream, P);
     if (err != cudaSuccess) return err;
     // the tiles left out (their number is only known on the device): one wave of CTAs walks the list
-    const long long wave = (long long)(sm_count > 0 ? sm_count : 148) * 5;
+    const long long wave = (long long)sm_count * 5;
     const unsigned cgrid = (unsigned)(jobs < wave ? jobs : wave);
-    if (P.counters) cooperative_kernel<Tally, false><<<cgrid, NTHREADS, sizeof(TileSmem), stream>>>(P);
-    else if (full) cooperative_kernel<NoTally, true><<<cgrid, NTHREADS, sizeof(TileSmem), stream>>>(P);
-    else cooperative_kernel<NoTally, false><<<cgrid, NTHREADS, sizeof(TileSmem), stream>>>(P);
-    err = cudaGetLastError();
+    err = P.counters ? launch_next(cooperative_kernel<Tally, false>, cgrid, sizeof(TileSmem), stream, P)
+          : full     ? launch_next(cooperative_kernel<NoTally, true>, cgrid, sizeof(TileSmem), stream, P)
+                     : launch_next(cooperative_kernel<NoTally, false>, cgrid, sizeof(TileSmem), stream, P);
     if (err != cudaSuccess || !P.occlusion) return err;
     coverage_kernel<<<grid, NTHREADS, 0, stream>>>(P);
     return cudaGetLastError();

@@ -121,7 +121,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) render_static_kernel(const __grid
                     setup_prim(s, t, V, flags & 1u, flags, Pn, key_lo, sv.y, STATIC_RCAP, n);
                 }
                 __syncthreads();
-                raster_records(s, s.rec, s.touched, t, s.n_rec, true, n);
+                raster_records<NW>(s, s.rec, s.touched, t, s.n_rec, true, n);
                 __syncthreads();
                 if (threadIdx.x == 0) { s.n_rec = 0; s.n_surv = 0; }
                 __syncthreads();

@@ -47,3 +47,29 @@ def test_static_pieces_lists_and_alignment(n_tris, E, A, H, W, offset):
     assert (c == want[0]).all()
     assert (np.abs(d.view(np.uint16).astype(int) - want[1].view(np.uint16).astype(int)) <= 1).all()
     assert pic.static_status() == 0
+
+
+@pytest.mark.parametrize("n_tris,E,A,H,W,K,spread", [
+    (40, 1, 1, 8, 16, 1, 25.0),           # one tile of one strip
+    (300, 1, 3, 17, 33, 2, 25.0),         # ragged in both directions
+    (300, 5, 37, 64, 64, 4, 200.0),       # 740 tiles: the most that take one CTA each (on 148 multiprocessors) ...
+    (300, 57, 13, 64, 64, 1, 200.0),      # ... and one more
+    (3000, 1, 2, 130, 70, 2, 12.0),       # more survivors than the record pool holds
+    (20, 1, 120, 64, 64, 1, 25.0),        # more visible box faces than their list holds, all around the cameras
+    (4000, 1, 4, 64, 64, 2, 90.0),        # a map of small cells: more grid rows in view than one pass takes
+])
+def test_calls_with_few_tiles(n_tris, E, A, H, W, K, spread):
+    from tests.gpu_util import CudaRun
+    from tests.util import assert_same_as_exhaustive
+    s = soup(n_tris + A, n_tris, E, A, H, W, K=K, spread=spread)
+    g = CudaRun(s)
+    try:
+        V = E * A * K
+        n = min(V, 300)
+        a = g.render()
+        b = g.render(brute=True, view_first=V - n, view_count=n)
+        assert_same_as_exhaustive(a, b, slice(V - n, V))
+        c = g.render(depth32=False)
+        assert (a[0] == c[0]).all() and (a[1].view(np.uint16) == c[1].view(np.uint16)).all()
+    finally:
+        g.close()
