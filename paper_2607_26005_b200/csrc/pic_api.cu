@@ -15,7 +15,7 @@ size_t max_smem_bytes();
 cudaError_t configure_kernels();
 cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses, float* state, const float* actions,
                          const float* dims, const uint8_t* active, const uint8_t* agent_cls, AgentGeom* agents_out, ViewCam* cams_out,
-                         float* tables, uint32_t* status, float dt, float wheelbase, float v_max, cudaStream_t stream);
+                         uint32_t* status, float dt, float wheelbase, float v_max, cudaStream_t stream);
 cudaError_t launch_render(const RenderParams& P, long long n_views, bool brute, int sm_count, cudaStream_t stream);
 cudaError_t launch_colour(const RenderParams& P, long long n_views, bool antialias, cudaStream_t stream);
 size_t survivor_bytes_per_tile();
@@ -70,13 +70,14 @@ struct pic_scene {
     pic::Prim* d_prims = nullptr;
     uint32_t* d_cell_start = nullptr;
     pic::Prim* d_grid_prims = nullptr;
+    pic::Bound* d_grid_bounds = nullptr;
     pic::Node* d_large_leaves = nullptr;
     pic::AgentGeom* d_agents = nullptr;
     pic::ViewCam* d_cams = nullptr;   // [E*A*K]
     uint32_t* d_overflow = nullptr;   // [1 + E*A*K*tiles] tiles handed from the render kernel to the cooperative kernel
     uint2* d_surv = nullptr;          // per tile: survivors of the cull kernel, read by the render kernel
     int sm_count = 0;
-    float* d_tables = nullptr;        // per-camera ray and background tables, K*(W+3H) words
+    float* d_tables = nullptr;        // per-camera ray and background tables (rig_tables)
     float* d_state = nullptr;       // [E*A*4]
     float* d_dims = nullptr;        // [E*A*3]
     uint8_t* d_active = nullptr;    // [E*A]
@@ -118,7 +119,7 @@ struct DeviceGuard {
 };
 
 void free_scene(pic_scene* s) {
-    cudaFree(s->d_env_map); cudaFree(s->d_env_maps); cudaFree(s->d_maps); cudaFree(s->d_groups); cudaFree(s->d_leaves); cudaFree(s->d_prims); cudaFree(s->d_cell_start); cudaFree(s->d_grid_prims); cudaFree(s->d_large_leaves);
+    cudaFree(s->d_env_map); cudaFree(s->d_env_maps); cudaFree(s->d_maps); cudaFree(s->d_groups); cudaFree(s->d_leaves); cudaFree(s->d_prims); cudaFree(s->d_cell_start); cudaFree(s->d_grid_prims); cudaFree(s->d_grid_bounds); cudaFree(s->d_large_leaves);
     cudaFree(s->d_agents); cudaFree(s->d_cams); cudaFree(s->d_overflow); cudaFree(s->d_surv); cudaFree(s->d_tables); cudaFree(s->d_state); cudaFree(s->d_dims); cudaFree(s->d_active); cudaFree(s->d_agent_cls); cudaFree(s->d_status); cudaFree(s->d_palette);
     cudaFree(s->d_in_poses); cudaFree(s->d_in_dims); cudaFree(s->d_in_active); cudaFree(s->d_out_class);
     cudaFree(s->d_out_depth);
@@ -139,21 +140,19 @@ pic_status fill_params(const pic_scene* s, const pic_camera* rig, uint8_t* out_c
     P.E = s->E; P.A = s->A; P.K = s->K; P.H = s->H; P.W = s->W;
     P.tiles_x = (s->W + pic::TILE - 1) / pic::TILE;
     P.tiles_y = (s->H + pic::TILE - 1) / pic::TILE;
+    pic::set_divisors(P);
     P.near_z = s->near_z; P.far_z = s->far_z;
     P.w_near = 1.0f / s->near_z; P.w_far = 1.0f / s->far_z;
     P.cls_agent = s->cls_agent; P.cls_sky = s->cls_sky; P.cls_ground = s->cls_ground;
     P.env_map = s->d_env_map; P.env_maps = s->d_env_maps; P.maps = s->d_maps; P.groups = s->d_groups; P.leaves = s->d_leaves; P.prims = s->d_prims;
-    P.cell_start = s->d_cell_start; P.grid_prims = s->d_grid_prims; P.large_leaves = s->d_large_leaves;
+    P.cell_start = s->d_cell_start; P.grid_prims = s->d_grid_prims; P.grid_bounds = s->d_grid_bounds; P.large_leaves = s->d_large_leaves;
     P.agents = s->d_agents;
     P.cams = s->d_cams;
     P.overflow = s->d_overflow;
     P.surv = s->d_surv;
     P.palette = s->d_palette;
     P.status = s->d_status;
-    P.rig.ray_x = s->d_tables;
-    P.rig.ray_y = P.rig.ray_x + (size_t)s->K * s->W;
-    P.rig.bg_z = P.rig.ray_y + (size_t)s->K * s->H;
-    P.rig.bg_cls = reinterpret_cast<const uint32_t*>(P.rig.bg_z + (size_t)s->K * s->H);
+    P.rig = pic::rig_tables(s->d_tables, s->K, s->H, s->W);
     P.out_class = out_class; P.out_depth = out_depth; P.out_depth32 = s->depth32; P.counters = s->counters; P.occlusion = s->occlusion;
     P.view_first = 0;
     P.debug_flags = s->debug_flags;
@@ -239,7 +238,8 @@ pic_status pic_scene_create(const pic_scene_desc* d, pic_scene** out) {
     const pic::Node* leaves = pic::hierarchy_leaves(hh, &nl);
     const pic::Node* groups = pic::hierarchy_groups(hh, &ng);
     const pic::MapInfo* maps = pic::hierarchy_maps(hh, &nm);
-    size_t ncs, ngp, nll;
+    size_t ncs, ngp, ngb, nll;
+    const pic::Bound* grid_bounds = pic::hierarchy_grid_bounds(hh, &ngb);
     const uint32_t* cell_start = pic::hierarchy_cell_start(hh, &ncs);
     const pic::Prim* grid_prims = pic::hierarchy_grid_prims(hh, &ngp);
     const pic::Node* large_leaves = pic::hierarchy_large_leaves(hh, &nll);
@@ -262,12 +262,13 @@ pic_status pic_scene_create(const pic_scene_desc* d, pic_scene** out) {
     dmalloc((void**)&s->d_prims, sizeof(pic::Prim) * np);
     dmalloc((void**)&s->d_cell_start, sizeof(uint32_t) * ncs);
     dmalloc((void**)&s->d_grid_prims, sizeof(pic::Prim) * ngp);
+    dmalloc((void**)&s->d_grid_bounds, sizeof(pic::Bound) * ngb);
     dmalloc((void**)&s->d_large_leaves, sizeof(pic::Node) * nll);
     dmalloc((void**)&s->d_agents, sizeof(pic::AgentGeom) * n_agents);
     dmalloc((void**)&s->d_cams, sizeof(pic::ViewCam) * n_agents * d->K);
     dmalloc((void**)&s->d_overflow, sizeof(uint32_t) * (1 + (size_t)n_agents * d->K * ((d->W + pic::TILE - 1) / pic::TILE) * ((d->H + pic::TILE - 1) / pic::TILE)));
     dmalloc((void**)&s->d_surv, pic::survivor_bytes_per_tile() * (size_t)n_agents * d->K * ((d->W + pic::TILE - 1) / pic::TILE) * ((d->H + pic::TILE - 1) / pic::TILE));
-    dmalloc((void**)&s->d_tables, sizeof(float) * (size_t)d->K * ((size_t)d->W + 3 * (size_t)d->H));
+    dmalloc((void**)&s->d_tables, pic::table_bytes(d->K, d->H, d->W));
     dmalloc((void**)&s->d_state, sizeof(float) * 4 * n_agents);
     dmalloc((void**)&s->d_dims, sizeof(float) * 3 * n_agents);
     dmalloc((void**)&s->d_active, n_agents);
@@ -290,6 +291,7 @@ pic_status pic_scene_create(const pic_scene_desc* d, pic_scene** out) {
     upload(s->d_prims, prims, sizeof(pic::Prim) * np);
     upload(s->d_cell_start, cell_start, sizeof(uint32_t) * ncs);
     upload(s->d_grid_prims, grid_prims, sizeof(pic::Prim) * ngp);
+    upload(s->d_grid_bounds, grid_bounds, sizeof(pic::Bound) * ngb);
     upload(s->d_large_leaves, large_leaves, sizeof(pic::Node) * nll);
     if (ce == cudaSuccess) ce = cudaMemset(s->d_status, 0, sizeof(uint32_t));
     if (ce == cudaSuccess) {          // until pic_set_palette: class c is the grey (c, c, c)
@@ -402,7 +404,7 @@ static pic_status render_from(pic_scene* s, const float* poses, float* state, co
     DeviceGuard guard(s->device);
     if (!guard.ok) return fail(PIC_ERR_CUDA, "cannot select device %d", s->device);
     const int n_agents = s->E * s->A;
-    CUDA_TRY(pic::launch_setup(P, n_agents, poses, state, actions, dims, active, s->have_agent_cls ? s->d_agent_cls : nullptr, s->d_agents, s->d_cams, s->d_tables,
+    CUDA_TRY(pic::launch_setup(P, n_agents, poses, state, actions, dims, active, s->have_agent_cls ? s->d_agent_cls : nullptr, s->d_agents, s->d_cams,
                                s->d_status, kDt, kWheelbase, kVMax, stream));
     const long long total = (long long)s->E * s->A * s->K;
     long long count = total - s->view_first;

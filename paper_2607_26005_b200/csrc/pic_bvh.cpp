@@ -32,6 +32,7 @@ struct HostHierarchy {
     std::vector<MapInfo> maps;
     std::vector<uint32_t> cell_start;
     std::vector<Prim> grid_prims;             // the same primitives once more, in grid order
+    std::vector<Bound> grid_bounds;           // their bounding cylinders
     std::vector<Node> large_leaves;
 };
 
@@ -105,6 +106,31 @@ void box_of_prim(const Prim& p, float lo[3], float hi[3]) {
             lo[c] = std::min(lo[c], p.v[3 * k + c]);
             hi[c] = std::max(hi[c], p.v[3 * k + c]);
         }
+}
+
+// Upper half of the float32 not below x: how a Bound stores a size.
+uint32_t up16(double x) {
+    const float f = (float)(x * 1.000001);
+    uint32_t b;
+    std::memcpy(&b, &f, 4);
+    return (b + 0xffffu) >> 16;
+}
+
+// The upright cylinder around a primitive, widened by what float32 arithmetic on its coordinates can lose.
+Bound bound_of_prim(const Prim& p) {
+    float lo[3], hi[3];
+    box_of_prim(p, lo, hi);
+    Bound b;
+    b.x = 0.5f * (lo[0] + hi[0]); b.y = 0.5f * (lo[1] + hi[1]); b.z = 0.5f * (lo[2] + hi[2]);
+    double r = 0.0, hz = 0.0;
+    for (int k = 0; k < 4; ++k) {
+        const double dx = (double)p.v[3 * k] - b.x, dy = (double)p.v[3 * k + 1] - b.y;
+        r = std::max(r, std::sqrt(dx * dx + dy * dy));
+        hz = std::max(hz, std::fabs((double)p.v[3 * k + 2] - b.z));
+    }
+    const double slack = 2e-3 + 1e-6 * (std::fabs((double)b.x) + std::fabs((double)b.y) + std::fabs((double)b.z) + r);
+    b.size = (up16(r + slack) << 16) | up16(hz + slack);
+    return b;
 }
 
 // The uniform grid and the large-primitive leaves of one map (primitives mi.prim_begin .. mi.prim_end of h.prims).
@@ -305,6 +331,7 @@ HostHierarchy* build_hierarchy(int num_maps, const int64_t* tri_offset, const fl
         }
         mi.group_end = (uint32_t)h->groups.size();
         build_grid(*h, mi);
+        for (size_t g = h->grid_bounds.size(); g < h->grid_prims.size(); ++g) h->grid_bounds.push_back(bound_of_prim(h->grid_prims[g]));
         if (h->prims.size() >= (1ull << 28)) {
             std::snprintf(err, err_len, "more than 2^28 primitives in one scene");
             delete h;
@@ -321,6 +348,7 @@ const Node* hierarchy_groups(const HostHierarchy* h, size_t* n) { *n = h->groups
 const MapInfo* hierarchy_maps(const HostHierarchy* h, size_t* n) { *n = h->maps.size(); return h->maps.data(); }
 const uint32_t* hierarchy_cell_start(const HostHierarchy* h, size_t* n) { *n = h->cell_start.size(); return h->cell_start.data(); }
 const Prim* hierarchy_grid_prims(const HostHierarchy* h, size_t* n) { *n = h->grid_prims.size(); return h->grid_prims.data(); }
+const Bound* hierarchy_grid_bounds(const HostHierarchy* h, size_t* n) { *n = h->grid_bounds.size(); return h->grid_bounds.data(); }
 const Node* hierarchy_large_leaves(const HostHierarchy* h, size_t* n) { *n = h->large_leaves.size(); return h->large_leaves.data(); }
 
 }  // namespace pic

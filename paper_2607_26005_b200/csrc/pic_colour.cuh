@@ -389,7 +389,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
     const unsigned id = await_previous(blockIdx.x) * (unsigned)NW + warp;
     const bool valid = id < P.n_jobs;
     const uint2* blk = P.surv + (size_t)id * SURV_STRIDE;
-    int ns = -2, n_big = 0;
+    int ns = -2;
     Job job;
     uint32_t n_map_tris = 0u;
     if (valid) {
@@ -404,11 +404,10 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
             s.job[warp] = job;
             s.active[warp] = ego_active ? 1 : 0;
         }
-        n_big = (int)(head.x & 0xffffu);
-        ns = n_big + (int)(head.x >> 16);
+        ns = (int)head.x;
         if (head.x == SURV_OVERFLOW) {
             // more visible primitives than the tile's list holds: the tile shows only the background, and the call says so
-            ns = 0; n_big = 0;
+            ns = 0;
             if (lane == 0) atomicOr(P.status, STATUS_COLOUR_INCOMPLETE);
         }
     }
@@ -444,7 +443,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
             const int my_base = (int)((bases >> (8 * warp)) & 0xffu);
             const Cam& c = s.cam[warp];
             for (int i = lane; i < ns; i += 32) {
-                const uint2 svi = __ldcg(blk + 2 + (i < n_big ? i : W_SURV - 1 - (i - n_big)));
+                const uint2 svi = __ldcg(blk + 2 + i);
                 V3 V[4], Pn;
                 uint32_t key_lo, flags;
                 fetch_survivor(c, P, svi.x, job.e, n_map_tris, V, Pn, key_lo, flags);

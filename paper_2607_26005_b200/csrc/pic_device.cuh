@@ -50,6 +50,8 @@ struct PrimEq {
 
 struct V3 { float x, y, z; };
 
+__device__ __forceinline__ unsigned divide(unsigned n, const FastDiv& f) { return (__umulhi(n, f.m) + n) >> f.s; }
+
 __device__ __forceinline__ float fm(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float sub(float a, float b) { return __fsub_rn(a, b); }
@@ -128,30 +130,22 @@ __device__ __forceinline__ V3 plane_normal_world(const Cam& c, const float (&v)[
 // normal P (same orientation as the vertex order).
 // Returns false for degenerate / edge-on primitives (D == 0), which cover nothing.
 __device__ __forceinline__ bool prim_equations(const V3 (&V)[4], bool quad, uint32_t flags, const V3 P, PrimEq& q) {
-    const int n = quad ? 4 : 3;
-    V3 N[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        if (i < n) {
-            const V3 a = V[i];
-            const V3 b = (i == 3 || (i == 2 && !quad)) ? V[0] : V[(i + 1) & 3];
-            if ((flags >> (4 + i)) & 1u) {       // evaluate in the canonical direction b -> a, then negate
-                V3 t = vcross(b, vsub(a, b));
-                N[i] = {-t.x, -t.y, -t.z};
-            } else {
-                N[i] = vcross(a, vsub(b, a));
-            }
-        } else {
-            N[i] = {0.f, 0.f, 1.f};              // triangles: a fourth edge that is always inside
-        }
-    }
-    float D = vdot(P, V[0]);
+    const float D = vdot(P, V[0]);
     if (!(D != 0.f)) return false;               // also drops NaN
     const float s = D < 0.f ? -1.f : 1.f;
     uint32_t tl = 0;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-        float sx = (i < n) ? mul(s, N[i].x) : 0.f, sy = (i < n) ? mul(s, N[i].y) : 0.f, sz = (i < n) ? mul(s, N[i].z) : 1.f;
+        const V3 a = V[i];
+        const V3 b = i == 3 ? V[0] : (i == 2 && !quad) ? V[0] : V[(i + 1) & 3];
+        // an edge that runs against its canonical direction is evaluated in that direction, then negated (selects, not
+        // branches: the lanes of a warp do not agree)
+        const bool rev = (flags >> (4 + i)) & 1u;
+        const V3 p = {rev ? b.x : a.x, rev ? b.y : a.y, rev ? b.z : a.z}, r = {rev ? a.x : b.x, rev ? a.y : b.y, rev ? a.z : b.z};
+        const V3 N = vcross(p, vsub(r, p));
+        const float sg = rev ? -s : s;
+        float sx = mul(sg, N.x), sy = mul(sg, N.y), sz = mul(sg, N.z);
+        if (i == 3 && !quad) { sx = 0.f; sy = 0.f; sz = 1.f; }     // triangles: a fourth edge that is always inside
         q.nx[i] = sx; q.ny[i] = sy; q.nz[i] = sz;
         if (sx > 0.f || (sx == 0.f && sy > 0.f)) tl |= 1u << i;
     }

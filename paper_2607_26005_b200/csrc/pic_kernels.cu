@@ -91,8 +91,12 @@ __device__ __forceinline__ void agent_setup(const AgentArgs& G, const RigParams&
 }
 
 // Per-camera tables: ray coordinates of every pixel column / row and the background of every row.
-__device__ __forceinline__ void rig_setup(const RigParams& R, int k, float* __restrict__ ray_x, float* __restrict__ ray_y,
-                                          float* __restrict__ bg_z, uint32_t* __restrict__ bg_cls) {
+__device__ __forceinline__ void rig_setup(const RigParams& R, int k, const RigTables& T) {
+    float* ray_x = const_cast<float*>(T.ray_x);
+    float* ray_y = const_cast<float*>(T.ray_y);
+    float* bg_z = const_cast<float*>(T.bg_z);
+    uint32_t* bg_cls = const_cast<uint32_t*>(T.bg_cls);
+    uint2* bg_fill = const_cast<uint2*>(T.bg_fill);
     const CamConst c = R.cam[k];
     const float cx = 0.5f * (float)R.W, cy = 0.5f * (float)R.H;
     for (int u = threadIdx.x; u < R.W; u += blockDim.x)
@@ -104,17 +108,18 @@ __device__ __forceinline__ void rig_setup(const RigParams& R, int k, float* __re
         background(c.cphi, c.sphi, c.mz, ry, R.far_z, R.cls_sky, R.cls_ground, cls, z);
         bg_z[(size_t)k * R.H + v] = z;
         bg_cls[(size_t)k * R.H + v] = cls;
+        const __half2 h = __floats2half2_rn(z, z);
+        bg_fill[(size_t)k * R.H + v] = make_uint2(cls * 0x01010101u, *reinterpret_cast<const uint32_t*>(&h));
     }
 }
 
 // One launch prepares a call: the first K blocks write a camera's tables each, the others set up an agent per thread.
 __global__ void __launch_bounds__(SETUP_THREADS) setup_kernel(const __grid_constant__ AgentArgs G, const __grid_constant__ RigParams R,
-                                                              float* __restrict__ ray_x, float* __restrict__ ray_y, float* __restrict__ bg_z,
-                                                              uint32_t* __restrict__ bg_cls, uint32_t* overflow) {
+                                                              const __grid_constant__ RigTables T, uint32_t* overflow) {
     launch_dependents();
     if (overflow && blockIdx.x == 0 && threadIdx.x == 0) overflow[0] = 0u;   // the render kernels' list of left-out tiles starts empty (absent for callers that do not use them)
     if ((int)blockIdx.x < R.K) {
-        rig_setup(R, (int)blockIdx.x, ray_x, ray_y, bg_z, bg_cls);
+        rig_setup(R, (int)blockIdx.x, T);
     } else {
         const int i = ((int)blockIdx.x - R.K) * SETUP_THREADS + (int)threadIdx.x;
         if (i < G.n) agent_setup(G, R, i);
@@ -172,17 +177,13 @@ static RigParams rig_params(const RenderParams& P) {
 // Per call: rig tables, agents (+ optional bicycle step) and their cameras.
 cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses, float* state, const float* actions,
                          const float* dims, const uint8_t* active, const uint8_t* agent_cls, AgentGeom* agents_out, ViewCam* cams_out,
-                         float* tables, uint32_t* status, float dt, float wheelbase, float v_max, cudaStream_t stream) {
+                         uint32_t* status, float dt, float wheelbase, float v_max, cudaStream_t stream) {
     const RigParams R = rig_params(P);
-    float* ray_x = tables;
-    float* ray_y = ray_x + (size_t)P.K * P.W;
-    float* bg_z = ray_y + (size_t)P.K * P.H;
-    uint32_t* bg_cls = reinterpret_cast<uint32_t*>(bg_z + (size_t)P.K * P.H);
     AgentArgs G;
     G.n = n_agents; G.poses = poses; G.state = state; G.actions = actions; G.dims = dims; G.active = active;
     G.agent_cls = agent_cls; G.default_cls = P.cls_agent; G.out = agents_out; G.cams = cams_out; G.status = status;
     G.dt = dt; G.wheelbase = wheelbase; G.v_max = v_max;
-    setup_kernel<<<P.K + (n_agents + SETUP_THREADS - 1) / SETUP_THREADS, SETUP_THREADS, 0, stream>>>(G, R, ray_x, ray_y, bg_z, bg_cls, P.overflow);
+    setup_kernel<<<P.K + (n_agents + SETUP_THREADS - 1) / SETUP_THREADS, SETUP_THREADS, 0, stream>>>(G, R, P.rig, P.overflow);
     return cudaGetLastError();
 }
 

@@ -59,10 +59,7 @@ constexpr int SCAP = 128;         // candidates that survive the pixel-box test,
 constexpr int TINY_MAX_PIXELS = 4;         // pixel centres in the box of a primitive rasterized by its own thread
 static_assert(TINY_MAX_PIXELS == 4, "the strip back end enumerates the pixels of such a box for at most 4");
 constexpr int CLASSIFY_MIN_PIXELS = 192;   // pixel boxes at least this large classify cells before rasterizing
-#ifndef PIC_CLASSIFY_MIN
-#define PIC_CLASSIFY_MIN 256
-#endif
-constexpr int CLASSIFY_MIN_STRIP = PIC_CLASSIFY_MIN;    // the same for the part of a box inside a 16-row strip
+constexpr int CLASSIFY_MIN_STRIP = 256;    // the same for the part of a box inside a 16-row strip
 
 struct __align__(16) TileSmem {
     unsigned long long key[TILE * TILE];      // 32 KB, 16-byte chunks XOR-swizzled by row (key_index)
@@ -210,6 +207,7 @@ struct Tally { int grp, leaf, tested, setup, tiny, recs, fallback, classified, c
 struct NoCount {
     __device__ __forceinline__ NoCount& operator++() { return *this; }
     __device__ __forceinline__ NoCount& operator=(int) { return *this; }
+    __device__ __forceinline__ NoCount& operator+=(int) { return *this; }
 };
 __device__ __forceinline__ int tally_value(int v) { return v; }
 __device__ __forceinline__ int tally_value(const NoCount&) { return 0; }
@@ -472,17 +470,17 @@ struct Job {
 // Job `id` of the launch: tiles of a view are consecutive, views follow P.view_first.
 // (tile_h: rows of a tile, for the kernel that cuts views into lower pieces.)
 __device__ __forceinline__ Job decode_job(const RenderParams& P, unsigned id, int tile_h = TILE) {
-    const unsigned tiles = (unsigned)(P.tiles_x * P.tiles_y);
-    const unsigned vrel = id / tiles;
-    const unsigned long long v = (unsigned long long)P.view_first + vrel;
+    const unsigned vrel = divide(id, P.div_tiles);
+    const unsigned v = (unsigned)P.view_first + vrel;         // E * A * K < 2^31 (checked by the launcher)
     Job j;
-    j.tile = (int)(id - vrel * tiles);
+    j.tile = (int)(id - vrel * (unsigned)(P.tiles_x * P.tiles_y));
     j.view = (size_t)v;
-    const unsigned va = (unsigned)(v / (unsigned)P.K);        // E * A * K < 2^31 (checked by the launcher)
-    j.k = (int)((unsigned)v - va * (unsigned)P.K);
-    j.e = (int)(va / (unsigned)P.A);
+    const unsigned va = divide(v, P.div_K);
+    j.k = (int)(v - va * (unsigned)P.K);
+    j.e = (int)divide(va, P.div_A);
     j.a = (int)(va - (unsigned)j.e * (unsigned)P.A);
-    j.t.x0 = (j.tile % P.tiles_x) * TILE; j.t.y0 = (j.tile / P.tiles_x) * tile_h;
+    const int ty = (int)divide((unsigned)j.tile, P.div_tiles_x);
+    j.t.x0 = (j.tile - ty * P.tiles_x) * TILE; j.t.y0 = ty * tile_h;
     j.t.tw = min(TILE, P.W - j.t.x0); j.t.th = min(tile_h, P.H - j.t.y0);
     j.t.w_near = P.w_near; j.t.w_far = P.w_far; j.t.near_z = P.near_z; j.t.far_z = P.far_z;
     return j;
@@ -653,14 +651,9 @@ __device__ __forceinline__ void flush_counters(const RenderParams& P, const Tall
 // ---------------------------------------------------------------------------------------------
 // Cull kernel, and the render kernels over its survivor lists (see the head of this file).
 // ---------------------------------------------------------------------------------------------
-constexpr int POOL = 128;         // records shared by the NW tiles of a CTA
-constexpr int STRIP = 16;         // pixel rows a warp rasterizes at a time
-constexpr int STRIP_KEYS = TILE * STRIP;
-constexpr int W_FACE = 384;        // box-face items of a tile in the cull kernel
-// Survivor buffer, SURV_STRIDE uint2 per tile: a 16-byte head (counts; work counts), then W_SURV
-// entries (id, pixel box).  Survivors whose pixel box holds more than TINY_MAX_PIXELS pixel centres
-// fill the list from the front, the others from the back; head.x = front count | back count << 16,
-// or all ones if a list overflowed.
+constexpr int W_ITEM = 448;        // items of a tile in the cull kernel at a time; the large primitives and box faces must fit at once
+// Survivor buffer, SURV_STRIDE uint2 per tile: a 16-byte head (number of survivors, or all ones if a list overflowed;
+// work counts), then W_SURV entries (id, pixel box).
 constexpr int SURV_STRIDE = 256;
 constexpr int W_SURV = SURV_STRIDE - 2;
 constexpr uint32_t SURV_OVERFLOW = 0xffffffffu;
@@ -668,7 +661,6 @@ constexpr uint32_t SURV_FACE = 0x80000000u;   // survivor id: index into grid_pr
 constexpr uint32_t REC_TINY = 1u << 28, REC_DEAD = 1u << 29;   // flags in the box word of a record
 constexpr uint32_t REC_INRANGE = 1u << 30;   // every covered pixel is within [near, far]: no per-pixel range test
 
-constexpr int W_LARGE = 64;       // visible leaves of the large-primitive list
 // A tile's frustum and its footprint on the ground plane.
 struct __align__(16) Frustum {
     float plane[6][4];                        // (read as float4: kept first, 16-byte aligned)
@@ -682,53 +674,18 @@ static_assert(offsetof(Frustum, plane) % 16 == 0 && offsetof(Frustum, side) % 16
 
 struct __align__(16) FrontLists {
     Frustum f;
-    uint32_t face[W_FACE];                    // agent << 3 | face
-    uint32_t lleaf[W_LARGE];                  // visible large-primitive leaves: first << 3 | count
+    uint32_t item[W_ITEM];                    // survivor ids to be tested
     uint32_t row_first[32];                   // grid rows of a pass: first entry of the row's range in cell_prims
     uint32_t row_off[33];                     //   and the number of candidates before the row (the total at [32])
-    int n_face;
+    int n_item;
 };
 
-struct __align__(16) FusedSmem {
-    unsigned long long key[NW][STRIP_KEYS];   // warp w's strip of keys; during the front end, its FrontLists
-    float4 pool[POOL * REC / 4];
-    float ray_x[NW][TILE], ray_y[NW][STRIP];  // ray tables of the strip a warp works on
-    int n_surv[NW];                           // survivors of tile w; -1: lists overflowed, -2: no such tile
-    int next_task;
-    int tile_active[NW];                      // is the ego agent of tile w active
-    uint32_t tile_ntris[NW];                  // triangles of its environment's map as given (box primitive indices start there)
-    Job tile_job[NW];                         // tile w, decoded by its warp
-    Cam cam[NW];                              // its camera
-};
-static_assert(sizeof(FusedSmem) <= 44 * 1024 && sizeof(TileSmem) <= 44 * 1024,
-              "shared memory must leave room for 5 CTAs per SM (228 KB, 1 KB reserved per CTA)");
 // What the raster and store templates need of a warp's strip: rows are counted from the strip's first.
 struct StripView {
     unsigned long long* key;
     const float* ray_x;
     const float* ray_y;
 };
-constexpr size_t RENDER_SMEM_BASE = sizeof(FusedSmem) > sizeof(TileSmem) ? sizeof(FusedSmem) : sizeof(TileSmem);
-
-__device__ __forceinline__ void write_record(float4* r, const PrimEq& q, uint32_t key_lo, uint32_t box, uint32_t extra) {
-    const uint32_t bx0 = box & 0xff, by0 = (box >> 8) & 0xff, bx1 = (box >> 16) & 0xff, by1 = box >> 24;
-    r[0] = make_float4(q.nx[0], q.nx[1], q.nx[2], q.nx[3]);
-    r[1] = make_float4(q.ny[0], q.ny[1], q.ny[2], q.ny[3]);
-    r[2] = make_float4(q.nz[0], q.nz[1], q.nz[2], q.nz[3]);
-    r[3] = make_float4(q.wx, q.wy, q.wz, __uint_as_float(key_lo));
-    // the pixel box needs 6 bits per coordinate; the top-left bits and the flags ride along
-    r[4].x = __uint_as_float(bx0 | (by0 << 6) | (bx1 << 12) | (by1 << 18) | (q.tl << 24) | extra);
-}
-
-__device__ __forceinline__ void read_record(const float4* r, PrimEq& q, uint32_t& key_lo) {
-    const float4 r0 = r[0], r1 = r[1], r2 = r[2], r3 = r[3];
-    q.nx[0] = r0.x; q.nx[1] = r0.y; q.nx[2] = r0.z; q.nx[3] = r0.w;
-    q.ny[0] = r1.x; q.ny[1] = r1.y; q.ny[2] = r1.z; q.ny[3] = r1.w;
-    q.nz[0] = r2.x; q.nz[1] = r2.y; q.nz[2] = r2.z; q.nz[3] = r2.w;
-    q.wx = r3.x; q.wy = r3.y; q.wz = r3.z;
-    key_lo = __float_as_uint(r3.w);
-}
-
 // Box test against planes held in registers (see box_visible).
 __device__ __forceinline__ bool box_visible_reg(const float4 (&pl)[6], float px, float py, const Node& b) {
     const float ax = sub(b.lo[0], px), bx = sub(b.hi[0], px);
@@ -766,16 +723,11 @@ __device__ __forceinline__ bool tiny_box(uint32_t box) {
     return (bx1 - bx0 + 1) * (by1 - by0 + 1) <= TINY_MAX_PIXELS;
 }
 
-// Warp-wide append to the two-ended survivor list (see SURV_STRIDE).
-__device__ __forceinline__ void append_survivor(uint2* __restrict__ surv, bool keep, uint32_t id, uint32_t box, int& n_big, int& n_tiny, int lane) {
-    const bool tiny = keep && tiny_box(box), big = keep && !tiny;
-    const unsigned mb = __ballot_sync(0xffffffffu, big), mt = __ballot_sync(0xffffffffu, tiny);
-    const unsigned below = (1u << lane) - 1u;
-    // (a slot is written only while front and back have not met; the caller checks the total)
-    if (big) { const int slot = n_big + __popc(mb & below); if (slot + n_tiny < W_SURV) surv[slot] = make_uint2(id, box); }
-    if (tiny) { const int slot = n_tiny + __popc(mt & below); if (slot + n_big + __popc(mb) < W_SURV) surv[W_SURV - 1 - slot] = make_uint2(id, box); }
-    n_big += __popc(mb);
-    n_tiny += __popc(mt);
+// Warp-wide append to the survivor list (a slot past the end is not written; the caller checks the total).
+__device__ __forceinline__ void append_survivor(uint2* __restrict__ surv, bool keep, uint32_t id, uint32_t box, int& n, int lane) {
+    const unsigned m = __ballot_sync(0xffffffffu, keep);
+    if (keep) { const int slot = n + __popc(m & ((1u << lane) - 1u)); if (slot < W_SURV) surv[slot] = make_uint2(id, box); }
+    n += __popc(m);
 }
 
 // Camera, frustum planes and footprint of a tile, by one warp.  The footprint is the convex hull of the apex and the
@@ -855,16 +807,44 @@ __device__ __forceinline__ void row_range(const Frustum& f, const RenderParams& 
     }
 }
 
-// Front end of one tile by one warp: fills the survivor list.  Returns the survivor counts
-// (front | back << 16), or -1 if a list overflowed (the tile then goes to the cooperative kernel).
+// Can the primitive inside bound `b` touch a pixel centre of the tile (margin m: see pixel_box)?  Conservative: the
+// bound's camera-space box is projected as a whole.  On flat maps this decides most candidates: a lane marking beyond
+// some twenty metres projects to a sliver between two rows of pixel centres.
+__device__ __forceinline__ bool bound_visible(const Cam& c, const TileCtx& t, const float4 b, const float m) {
+    const uint32_t size = __float_as_uint(b.w);
+    const float r = __uint_as_float(size & 0xffff0000u), hz = __uint_as_float(size << 16);
+    const V3 q = to_camera(c, b.x, b.y, b.z);
+    const float cphi = fabsf(c.dz), sphi = fabsf(c.fz_);                       // pitch
+    const float rz = cphi * r + sphi * hz, ry = sphi * r + cphi * hz;
+    const float z0 = q.z - rz, z1 = q.z + rz;
+    bool ok = z1 >= t.near_z * 0.9999f && z0 <= t.far_z * 1.0001f;
+    if (z0 >= t.near_z * ZPROJ_FRAC) {                                         // (else a vertex may not project: pixel_box looks closer)
+        const float i0 = __fdividef(1.f, z0), i1 = __fdividef(1.f, z1);
+        const float xa = q.x - r, xb = q.x + r, ya = q.y - ry, yb = q.y + ry;
+        const float mm = m + 0.015625f;                                        // 1/64 pixel for the rounding above
+        const float sx0 = fm(c.focx, xa * (xa < 0.f ? i0 : i1), c.cx), sx1 = fm(c.focx, xb * (xb < 0.f ? i1 : i0), c.cx);
+        const float sy0 = fm(c.focy, ya * (ya < 0.f ? i0 : i1), c.cy), sy1 = fm(c.focy, yb * (yb < 0.f ? i1 : i0), c.cy);
+        const float fx0 = fmaxf(ceilf(sx0 - 0.5f - mm), (float)t.x0), fx1 = fminf(floorf(sx1 - 0.5f + mm), (float)(t.x0 + t.tw - 1));
+        const float fy0 = fmaxf(ceilf(sy0 - 0.5f - mm), (float)t.y0), fy1 = fminf(floorf(sy1 - 0.5f + mm), (float)(t.y0 + t.th - 1));
+        ok = ok && fx0 <= fx1 && fy0 <= fy1;
+    }
+    return ok;
+}
+
+// Front end of one tile by one warp: fills the survivor list.  Returns the number of survivors,
+// or -1 if a list overflowed (the tile then goes to the cooperative kernel).
 //
 // Map primitives come from the uniform grid: the footprint of the tile's frustum on the ground
 // plane is the convex hull of the apex and the four far corners; for every grid row the footprint
 // (widened by the map's margin) crosses, the small primitives of the cells it covers are one
-// contiguous range of cell_prims.  The ranges of up to 32 rows are laid end to end and tested two
-// candidates per lane at a time (camera space, pixel box).  The large primitives are found through
-// their leaves (a lane per leaf box against the six frustum planes), the other agents' boxes as
-// bounding spheres.  Loads that do not depend on one another are issued together.
+// contiguous range of grid_prims.  The ranges of up to 32 rows are laid end to end and their bounds tested two
+// candidates per lane at a time; what remains joins a list of items with the primitives of the visible
+// large-primitive leaves (a lane per leaf box against the six frustum planes) and the faces of the other agents' boxes
+// (culled as bounding spheres).  The items are then tested a lane each -- camera space, pixel box -- and the survivors
+// compacted.  Loads that do not depend on one another are issued together.
+//
+// Bound by the issue of dependent instructions at 24-32 resident warps: the full test costs some 230 instructions and 64
+// bytes a candidate, the bound's some 60 and 16, and four candidates in five die by it.
 template <class TL, bool CONS>
 __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ surv, const RenderParams& P, const Job& job,
                                           const MapInfo& mi, int lane, TL& n) {
@@ -881,37 +861,32 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
     if (lane < P.A) ag0 = load_agent(env_agents + lane);
     if (lane + 32 < P.A) ag1 = load_agent(env_agents + lane + 32);
     Frustum& fr = f.f;
-    if (lane == 0) f.n_face = 0;
+    if (lane == 0) f.n_item = 0;
     frustum_setup(fr, P, job, lane);
     if (stop == 11) return 0;
     const Cam& c = fr.cam;
-    int n_big = 0, n_tiny = 0;
-    // ---- the grid rows crossed by the widened footprint; the range of a row's cells in grid_prims
+    // ---- the grid rows crossed by the widened footprint; the first 32 rows' ranges are requested now, the boxes below
+    // are tested while the loads are under way
     const GridRows rows = grid_rows(fr, mi);
-    // the first 32 rows' ranges are requested now; the boxes below are tested while the loads are under way
-    uint32_t first0, cnt0;
-    row_range(fr, P, mi, rows, rows.lo + lane, first0, cnt0);
+    uint32_t first, cnt;
+    row_range(fr, P, mi, rows, rows.lo + lane, first, cnt);
     if (rows.lo + lane <= rows.hi) ++n.grp;
     // ---- the large primitives' leaves: a lane per leaf box against the six frustum planes
-    int n_ll = 0;
     {
         float4 pl[6];
 #pragma unroll
         for (int p = 0; p < 6; ++p) pl[p] = *reinterpret_cast<const float4*>(fr.plane[p]);
         for (uint32_t l0 = mi.large_begin; l0 < mi.large_end; l0 += 32) {
             const uint32_t l = l0 + lane;
-            bool vis = false;
-            Node ln;
-            ln.first = 0; ln.count = 0;
-            if (l < mi.large_end) { ln = (l0 == mi.large_begin) ? ln0 : load_node(P.large_leaves + l); vis = box_visible_reg(pl, c.px, c.py, ln); ++n.leaf; }
-            const unsigned m = __ballot_sync(0xffffffffu, vis);
-            if (vis) {
-                const int slot = n_ll + __popc(m & ((1u << lane) - 1u));
-                if (slot < W_LARGE) f.lleaf[slot] = (ln.first << 3) | ln.count;
+            if (l >= mi.large_end) continue;
+            const Node ln = (l0 == mi.large_begin) ? ln0 : load_node(P.large_leaves + l);
+            ++n.leaf;
+            if (box_visible_reg(pl, c.px, c.py, ln)) {
+                const int slot = atomicAdd(&f.n_item, (int)ln.count);
+                for (uint32_t k = 0; k < ln.count; ++k)
+                    if (slot + (int)k < W_ITEM) f.item[slot + k] = ln.first + k;
             }
-            n_ll += __popc(m);
         }
-        if (n_ll > W_LARGE) return -1;
     }
     // ---- other agents' boxes, two per lane at a time
     for (int b0 = 0; b0 < P.A; b0 += 64) {
@@ -927,113 +902,101 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
             uint32_t faces = 0u;
             if (b < P.A && b != job.a && g.active) faces = box_faces(fr, c, t, g);
             if (faces) {
-                int slot = atomicAdd(&f.n_face, __popc(faces));
+                int slot = atomicAdd(&f.n_item, __popc(faces));
                 for (; faces; faces &= faces - 1, ++slot)
-                    if (slot < W_FACE) f.face[slot] = ((uint32_t)b << 3) | (uint32_t)(__ffs(faces) - 1);
+                    if (slot < W_ITEM) f.item[slot] = SURV_FACE | ((uint32_t)b << 3) | (uint32_t)(__ffs(faces) - 1);
             }
         }
     }
-    if (stop == 12) return 0;
-    // ---- candidates of the grid rows, 32 rows per pass: camera space, pixel box; survivors are compacted
-    for (int r0 = rows.lo; r0 <= rows.hi; r0 += 32) {
-        uint32_t first = first0, cnt = cnt0;
-        if (r0 != rows.lo) {
-            row_range(fr, P, mi, rows, r0 + lane, first, cnt);
-            if (r0 + lane <= rows.hi) ++n.grp;
-        }
-        uint32_t incl = cnt;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-            const uint32_t up = __shfl_up_sync(0xffffffffu, incl, d);
-            if (lane >= d) incl += up;
-        }
-        const int total = (int)__shfl_sync(0xffffffffu, incl, 31);
-        __syncwarp();
-        f.row_first[lane] = first;
-        f.row_off[lane] = incl - cnt;
-        if (lane == 31) f.row_off[32] = incl;
-        __syncwarp();
-        for (int i0 = 0; i0 < total; i0 += 64) {         // two candidates per lane at a time
-            float v[2][12];
-            bool have[2];
-            uint32_t id[2] = {0u, 0u};
-#pragma unroll
-            for (int u = 0; u < 2; ++u) {
-                const int i = i0 + 32 * u + lane;
-                have[u] = i < total;
-                if (have[u]) {
-                    int r = 0;
-#pragma unroll
-                    for (int st = 16; st; st >>= 1)
-                        if (f.row_off[r + st] <= (uint32_t)i) r += st;
-                    id[u] = f.row_first[r] + ((uint32_t)i - f.row_off[r]);
-                    uint32_t key_lo, flags;
-                    load_prim(P.grid_prims + id[u], v[u], key_lo, flags);
-                }
-            }
-#pragma unroll 1
-            for (int u = 0; u < 2; ++u) {               // (one copy of the test for both candidates: less code to fetch)
-                uint32_t box = 0;
-                bool keep = false;
-                const bool hv = u ? have[1] : have[0];
-                if (hv) {
-                    V3 V[4];
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        V[q] = to_camera(c, u ? v[1][3 * q] : v[0][3 * q], u ? v[1][3 * q + 1] : v[0][3 * q + 1], u ? v[1][3 * q + 2] : v[0][3 * q + 2]);
-                    ++n.tested;
-                    keep = pixel_box(c, t, V, box, BOX_MARGIN);
-                }
-                append_survivor(surv, keep, u ? id[1] : id[0], box, n_big, n_tiny, lane);
-            }
-        }
-    }
-    // ---- the primitives of the visible large leaves
     __syncwarp();
-    for (int i0 = 0; i0 < n_ll * LARGE_LEAF_PRIMS; i0 += 32) {
-        const int i = i0 + lane;
-        uint32_t box = 0, id = 0;
-        bool keep = false;
-        if (i < n_ll * LARGE_LEAF_PRIMS) {
-            const uint32_t lf = f.lleaf[i / LARGE_LEAF_PRIMS];
-            const uint32_t j = i % LARGE_LEAF_PRIMS;
-            if (j < (lf & 7u)) {
-                id = (lf >> 3) + j;
-                float v[12];
-                uint32_t key_lo, flags;
-                load_prim(P.grid_prims + id, v, key_lo, flags);
-                V3 V[4];
+    int n_item = f.n_item;
+    if (n_item > W_ITEM) return -1;
+    if (stop == 12) return 0;
+    int n_surv = 0;
+    // ---- fill the item list with the candidates of the grid rows (32 rows per pass), test the items, until both are done
+    int row = rows.lo, i0 = 0, total = -1;         // total < 0: the ranges of the pass have not been laid out
+    bool more = row <= rows.hi;
+#pragma unroll 1
+    do {
+        while (more && n_item <= W_ITEM - 64) {
+            if (total < 0) {
+                if (row != rows.lo) {
+                    row_range(fr, P, mi, rows, row + lane, first, cnt);
+                    if (row + lane <= rows.hi) ++n.grp;
+                }
+                uint32_t incl = cnt;
 #pragma unroll
-                for (int q = 0; q < 4; ++q) V[q] = to_camera(c, v[3 * q], v[3 * q + 1], v[3 * q + 2]);
+                for (int d = 1; d < 32; d <<= 1) {
+                    const uint32_t up = __shfl_up_sync(0xffffffffu, incl, d);
+                    if (lane >= d) incl += up;
+                }
+                total = (int)__shfl_sync(0xffffffffu, incl, 31);
+                __syncwarp();
+                f.row_first[lane] = first;
+                f.row_off[lane] = incl - cnt;
+                if (lane == 31) f.row_off[32] = incl;
+                __syncwarp();
+                i0 = 0;
+            }
+            if (i0 < total) {
+                float4 b[2];
+                uint32_t id[2] = {0u, 0u};
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const int i = i0 + 32 * u + lane;
+                    b[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (i < total) {
+                        int r = 0;
+#pragma unroll
+                        for (int st = 16; st; st >>= 1)
+                            if (f.row_off[r + st] <= (uint32_t)i) r += st;
+                        id[u] = f.row_first[r] + ((uint32_t)i - f.row_off[r]);
+                        b[u] = __ldg(reinterpret_cast<const float4*>(P.grid_bounds) + id[u]);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    const bool have = i0 + 32 * u + lane < total;
+                    const bool keep = have && bound_visible(c, t, b[u], BOX_MARGIN);
+                    const unsigned m = __ballot_sync(0xffffffffu, keep);
+                    if (keep) f.item[n_item + __popc(m & ((1u << lane) - 1u))] = id[u];
+                    n_item += __popc(m);
+                }
+                i0 += 64;
+            }
+            if (i0 >= total) { row += 32; total = -1; more = row <= rows.hi; }
+        }
+        __syncwarp();
+        if (stop == 13) return 0;
+#pragma unroll 1
+        for (int i = lane; i - lane < n_item; i += 32) {
+            uint32_t box = 0, id = 0;
+            bool keep = false;
+            if (i < n_item) {
+                id = f.item[i];
+                V3 V[4];
+                if (id & SURV_FACE) {
+                    const AgentGeom g = load_agent(env_agents + ((id & ~SURV_FACE) >> 3));
+                    const uint32_t corners = face_corners((int)(id & 7u));
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) V[q] = box_corner(c, g, (corners >> (4 * q)) & 7u);
+                } else {
+                    float v[12];
+                    uint32_t key_lo, flags;
+                    load_prim(P.grid_prims + id, v, key_lo, flags);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) V[q] = to_camera(c, v[3 * q], v[3 * q + 1], v[3 * q + 2]);
+                }
                 ++n.tested;
                 keep = pixel_box(c, t, V, box, BOX_MARGIN);
             }
+            append_survivor(surv, keep, id, box, n_surv, lane);
         }
-        append_survivor(surv, keep, id, box, n_big, n_tiny, lane);
-    }
-    __syncwarp();
-    const int n_face = f.n_face;
-    if (n_face > W_FACE) return -1;
-    if (stop == 13) return 0;
-    for (int i0 = 0; i0 < n_face; i0 += 32) {
-        const int i = i0 + lane;
-        uint32_t box = 0, it = 0;
-        bool keep = false;
-        if (i < n_face) {
-            it = f.face[i];
-            const AgentGeom g = load_agent(env_agents + (it >> 3));
-            const uint32_t corners = face_corners((int)(it & 7u));
-            V3 V[4];
-#pragma unroll
-            for (int q = 0; q < 4; ++q) V[q] = box_corner(c, g, (corners >> (4 * q)) & 7u);
-            ++n.tested;
-            keep = pixel_box(c, t, V, box, BOX_MARGIN);
-        }
-        append_survivor(surv, keep, SURV_FACE | it, box, n_big, n_tiny, lane);
-    }
-    __syncwarp();
+        __syncwarp();
+        n_item = 0;
+    } while (more);
     if (stop == 14) return 0;
-    return n_big + n_tiny > W_SURV ? -1 : (n_big | (n_tiny << 16));
+    return n_surv > W_SURV ? -1 : n_surv;
 }
 
 // Survivor `id` in camera space with its plane normal.
@@ -1064,143 +1027,6 @@ __device__ __forceinline__ bool record_in_range(const V3 (&V)[4], const RenderPa
     return zlo >= P.near_z * 1.001f && zhi <= P.far_z * 0.999f;
 }
 
-// Set-up of a tile's survivors (the cull kernel's list) by its warp: survivor i becomes record i of `rec`.
-template <class TL>
-__device__ __forceinline__ void front_setup(const Cam& c, const uint2* __restrict__ surv, float4* rec, const RenderParams& P,
-                                            const Job& job, const MapInfo& mi, int ns, int n_big, int lane, TL& n) {
-    for (int i = lane; i < ns; i += 32) {
-        const uint2 sv = __ldcg(surv + (i < n_big ? i : W_SURV - 1 - (i - n_big)));
-        V3 V[4], Pn;
-        uint32_t key_lo, flags;
-        fetch_survivor(c, P, sv.x, job.e, mi.n_tris, V, Pn, key_lo, flags);
-        PrimEq q;
-        float4* r = rec + i * (REC / 4);
-        if (!prim_equations(V, flags & 1u, flags, Pn, q)) { r[4].x = __uint_as_float(REC_DEAD); continue; }
-        ++n.setup;
-        const uint32_t box = sv.y;
-        const int bx0 = box & 0xff, by0 = (box >> 8) & 0xff, bx1 = (box >> 16) & 0xff, by1 = box >> 24;
-        const bool tiny = (bx1 - bx0 + 1) * (by1 - by0 + 1) <= TINY_MAX_PIXELS;
-        if (tiny) ++n.tiny; else ++n.recs;
-        write_record(r, q, key_lo, box, (tiny ? REC_TINY : 0u) | (record_in_range(V, P) ? REC_INRANGE : 0u));
-    }
-}
-
-// Back end of one strip (rows ys .. ys + STRIP - 1 of the tile) by one warp; the strip's keys are
-// all "no fragment" on entry and on exit.
-template <bool FULL, class TL>
-__device__ __forceinline__ void back_strip(StripView& s, const RenderParams& P, const Job& job, bool ego_active, int ys,
-                                           const float4* rec, int n_rec, bool classify, int stop, int lane, uint32_t n_map_tris, TL& n) {
-    const TileCtx& t = job.t;
-    const int rows = FULL ? STRIP : min(STRIP, t.th - ys);
-    uint32_t touched = 0u;                       // 8x8 blocks of the strip: bit (row >> 3) * 8 + (column >> 3)
-    // Records are looked at 32 at a time, a lane each: which reach the strip?  Those of a few
-    // pixels are rasterized by their lane (atomic max); the warp then walks the other hits
-    // together, a lane per pixel pair.
-    for (int base = 0; base < n_rec; base += 32) {
-        uint32_t bw_lane = 0u;
-        bool hit = false;
-        if (base + lane < n_rec) {
-            const float4* r = rec + (base + lane) * (REC / 4);
-            bw_lane = __float_as_uint(r[4].x);
-            const int by0 = (bw_lane >> 6) & 63, by1 = (bw_lane >> 18) & 63;
-            hit = !(bw_lane & REC_DEAD) && by1 >= ys && by0 < ys + STRIP;
-            if (hit && (bw_lane & REC_TINY) && stop == 7) hit = false;
-            if (hit && (bw_lane & REC_TINY)) {
-                hit = false;
-                const int bx0 = bw_lane & 63, bx1 = (bw_lane >> 12) & 63;
-                const int y0 = max(by0, ys) - ys, y1 = min(by1, ys + STRIP - 1) - ys;
-                PrimEq q;
-                uint32_t key_lo;
-                read_record(r, q, key_lo);
-                q.tl = (bw_lane >> 24) & 15u;
-                // at most TINY_MAX_PIXELS pixels: one column (w == 1), two columns, or one row
-                const int w = bx1 - bx0 + 1, npx = w * (y1 - y0 + 1);
-                bool any = false;
-#pragma unroll
-                for (int px = 0; px < TINY_MAX_PIXELS; ++px) {
-                    if (px < npx) {
-                        const int x = bx0 + (w == 1 ? 0 : w == 2 ? (px & 1) : px), y = y0 + (w == 1 ? px : w == 2 ? (px >> 1) : 0);
-                        const uint32_t wb = fragment(q, s.ray_x[x], s.ray_y[y], t.w_near, t.w_far);
-                        if (wb) { put_fragment(s, x, y, wb, key_lo); any = true; }
-                    }
-                }
-                if (any) touched |= (uint32_t)block_mask(bx0, y0, bx1, y1);
-            }
-        }
-        __syncwarp();
-        unsigned hits = __ballot_sync(0xffffffffu, hit);
-        if (!(stop == 0 || stop > 5)) hits = 0u;
-        for (; hits; hits &= hits - 1) {
-            const int src = __ffs(hits) - 1;
-            const uint32_t bw = __shfl_sync(0xffffffffu, bw_lane, src);
-            const float4* r = &rec[(base + src) * (REC / 4)];
-            const int by0 = (bw >> 6) & 63, by1 = (bw >> 18) & 63;
-            const int bx0 = bw & 63, bx1 = (bw >> 12) & 63;
-            const int ly0 = max(by0, ys) - ys, ly1 = min(by1, ys + STRIP - 1) - ys;
-            PrimEq q;
-            uint32_t key_lo;
-            read_record(r, q, key_lo);
-            q.tl = (bw >> 24) & 15u;
-            float thr[4];
-            edge_thresholds(q.tl, thr);
-            if (classify && (bx1 - bx0 + 1) * (ly1 - ly0 + 1) >= CLASSIFY_MIN_STRIP) {
-                // lanes 0..15 classify the strip's 16 x 4 pixel cells: reject / partly covered / inside
-                ++n.classified;
-                const int xa = (lane & 3) * 16, xb = xa + 15, ya = ((lane >> 2) & 3) * 4, yb = ya + 3;
-                bool reject = lane >= 16 || xb < bx0 || xa > bx1 || yb < ly0 || ya > ly1;
-                uint32_t need = 0u;
-                if (!reject) {
-                    const float rxa = s.ray_x[xa], rxb = s.ray_x[xb], rya = s.ray_y[ya], ryb = s.ray_y[yb];   // rxa < rxb, rya < ryb
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        // fma is monotone in each argument, so the cell's extreme values are at its corners
-                        const float ta = fm(q.ny[e], rya, q.nz[e]), tb = fm(q.ny[e], ryb, q.nz[e]);
-                        const float emax = fm(q.nx[e], q.nx[e] >= 0.f ? rxb : rxa, fmaxf(ta, tb));
-                        const float emin = fm(q.nx[e], q.nx[e] >= 0.f ? rxa : rxb, fminf(ta, tb));
-                        reject = reject || (emax < 0.f);
-                        if (!(emin > 0.f)) need |= 1u << e;
-                    }
-                    const float wa = fm(q.wy, rya, q.wz), wb = fm(q.wy, ryb, q.wz);
-                    const float wmax = fm(q.wx, q.wx >= 0.f ? rxb : rxa, fmaxf(wa, wb));
-                    const float wmin = fm(q.wx, q.wx >= 0.f ? rxa : rxb, fminf(wa, wb));
-                    reject = reject || (wmax < t.w_far) || (wmin > t.w_near);
-                    // the depth range test rides on the edge tests: if it is still needed, so is one edge
-                    if (need == 0u && !((wmin >= t.w_far) && (wmax <= t.w_near))) need = 1u;
-                }
-                for (unsigned m = __ballot_sync(0xffffffffu, !reject); m; m &= m - 1) {
-                    const int cell = __ffs(m) - 1;
-                    const int xx = (cell & 3) * 16, yy = (cell >> 2) * 4;
-                    const uint32_t need_c = __shfl_sync(0xffffffffu, need, cell);
-                    ++n.cells;
-                    if (raster_cell(s, t, q, thr, key_lo, xx, yy, need_c, lane)) touched |= 3u << ((yy >> 3) * 8 + (xx >> 3));
-                }
-            } else {
-                for (int yy = ly0 & ~3; yy <= ly1; yy += 4)
-                    for (int xx = bx0 & ~15; xx <= bx1; xx += 16) {
-                        ++n.cells;
-                        if (raster_cell(s, t, q, thr, key_lo, xx, yy, 0xFu, lane)) touched |= 3u << ((yy >> 3) * 8 + (xx >> 3));
-                    }
-            }
-        }
-        __syncwarp();
-    }
-    touched = __reduce_or_sync(0xffffffffu, touched);
-    if (stop == 5) touched = 0xffffu;
-    // ---- store; a ragged strip may hold keys past the image edge, which the store never visits:
-    // it clears the whole strip instead of the keys it read
-    TileCtx ts = t;
-    ts.y0 = t.y0 + ys; ts.th = rows;
-    const bool ragged = !FULL && (t.tw < TILE || rows < STRIP);
-    if (stop != 8) store_tile<FULL>(s, ts, P, job.view, job.k, ego_active, (unsigned long long)touched, !ragged, lane, 32, n_map_tris);
-    __syncwarp();
-    if (ragged) {
-#pragma unroll
-        for (int i = 0; i < STRIP_KEYS / 2 / 32; ++i)
-            reinterpret_cast<ulonglong2*>(s.key)[i * 32 + lane] = make_ulonglong2(0ull, 0ull);
-        __syncwarp();
-    }
-}
-
 // Cull kernel: a warp per tile walks the hierarchy and the other agents' boxes, tests the candidates
 // and leaves the tile's survivors (id, pixel box) in device memory: a 16-byte head (count, or -1 if a
 // list overflowed; with counters, the tile's group / leaf / candidate tests), then the list.  No
@@ -1213,8 +1039,11 @@ struct __align__(16) CullSmem {
 #ifndef PIC_CULL_CTAS
 #define PIC_CULL_CTAS 6
 #endif
-#ifndef PIC_RENDER_CTAS
-#define PIC_RENDER_CTAS 5
+#ifndef PIC_SMALL_PIXELS
+#define PIC_SMALL_PIXELS 16
+#endif
+#ifndef PIC_TILE_CTAS
+#define PIC_TILE_CTAS 24
 #endif
 template <class TL, bool CONS>
 __global__ void __launch_bounds__(NTHREADS, PIC_CULL_CTAS) cull_kernel(const __grid_constant__ RenderParams P) {
@@ -1242,137 +1071,8 @@ __global__ void __launch_bounds__(NTHREADS, PIC_CULL_CTAS) cull_kernel(const __g
     launch_dependents();
 }
 
-// Render kernel.  FULL: every tile is 64 x 64, rows allow 128-bit stores, no float32 depth image (the
-// launcher checks) -- the instantiation the workloads run, without the code for ragged tiles.
-template <class TL, bool FULL>
-__global__ void __launch_bounds__(NTHREADS, 5) render_kernel(const __grid_constant__ RenderParams P) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    FusedSmem& s = *reinterpret_cast<FusedSmem*>(smem_raw);
-    if (PIC_STOP(P) == 15) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    launch_dependents();
-    const unsigned first = await_previous(blockIdx.x) * (unsigned)NW, n_jobs = P.n_jobs;
-    TL n = {};
-    const bool classify = !(P.debug_flags & 1);
-    const int stop = PIC_STOP(P);
-    // test aids: a pool of 2 records sends nearly every tile to cooperative_job, one of 40 mixes both paths
-    const int pool_cap = FULL ? POOL : (P.debug_flags & 2) ? 2 : (P.debug_flags & 8) ? 40 : POOL;   // (FULL is launched without these flags)
-    if (threadIdx.x == 0) s.next_task = 0;
-
-    // ---- the cull kernel's survivors of tile first + w
-    const bool valid = first + warp < n_jobs;
-    Job job;
-    MapInfo mi;
-    const uint2* blk = P.surv + (size_t)(first + warp) * SURV_STRIDE;
-    int ns = -2, n_big = 0;
-    if (valid) {
-        const uint4 head = __ldcg(reinterpret_cast<const uint4*>(blk));
-        job = decode_job(P, first + warp);
-        mi = P.env_maps[job.e];
-        const bool ego_active = P.agents[(size_t)job.e * P.A + job.a].active != 0;
-        if (lane == 0) {
-            s.tile_job[warp] = job; s.tile_active[warp] = ego_active; s.tile_ntris[warp] = mi.n_tris;
-            load_camera(s.cam[warp], P.cams[job.view], P.cam[job.k], P.W, P.H);
-        }
-        n_big = (int)(head.x & 0xffffu);
-        ns = head.x == SURV_OVERFLOW ? -1 : n_big + (int)(head.x >> 16);
-        if (lane == 0) { n.grp = (int)head.y; n.leaf = (int)head.z; n.tested = (int)head.w; }
-    }
-    if (lane == 0) s.n_surv[warp] = ns;
-    __syncthreads();
-    // every thread lays the record pool out alike: tiles in order, a tile that does not fit is left
-    // out.  One byte per tile: first record, and count (0xff: to cooperative_job, 0xfe: no such tile)
-    uint32_t bases = 0u, cnts = 0u;
-    {
-        int off = 0;
-#pragma unroll
-        for (int j = 0; j < NW; ++j) {
-            const int c = s.n_surv[j];
-            bases |= (uint32_t)off << (8 * j);
-            if (c >= 0 && off + c <= pool_cap) { cnts |= (uint32_t)c << (8 * j); off += c; }
-            else cnts |= ((c == -2) ? 0xfeu : 0xffu) << (8 * j);
-        }
-    }
-    {
-        const int my_base = (int)((bases >> (8 * warp)) & 0xffu), my_cnt = (int)((cnts >> (8 * warp)) & 0xffu);
-        if (my_cnt == 0xff) { n.grp = 0; n.leaf = 0; n.tested = 0; }       // counted again by cooperative_job
-        else if (my_cnt != 0xfe && my_cnt > 0 && stop != 14) front_setup(s.cam[warp], blk + 2, s.pool + my_base * (REC / 4), P, job, mi, my_cnt, n_big, lane, n);
-    }
-    __syncthreads();
-    // ---- back end: the NW tiles' strips are tasks that the warps draw from a counter; a warp's
-    // lists are dead, their memory becomes its strip of keys
-    if (stop != 9) {
-#pragma unroll
-        for (int i = 0; i < STRIP_KEYS / 2 / 32; ++i)
-            reinterpret_cast<ulonglong2*>(s.key[warp])[i * 32 + lane] = make_ulonglong2(0ull, 0ull);
-    }
-    __syncwarp();
-    if (stop == 10) return;
-    StripView sv;
-    sv.key = s.key[warp]; sv.ray_x = s.ray_x[warp]; sv.ray_y = s.ray_y[warp];
-    constexpr int STRIPS = TILE / STRIP;
-#pragma unroll 1
-    for (;;) {
-        int task = 0;
-        if (lane == 0) task = atomicAdd(&s.next_task, 1);
-        task = __shfl_sync(0xffffffffu, task, 0);
-        if (task >= NW * STRIPS) break;
-        const int j = task / STRIPS, ys = (task % STRIPS) * STRIP;
-        const int cj = (int)((cnts >> (8 * j)) & 0xffu);
-        if (cj >= 0xfe) continue;
-        const Job jb = s.tile_job[j];
-        if (!FULL && ys >= jb.t.th) continue;
-        const bool ego_active = s.tile_active[j] != 0;
-        if (FULL || (jb.t.tw == TILE && ys + STRIP <= jb.t.th)) {     // ray tables of the strip
-            const float* rx = P.rig.ray_x + (size_t)jb.k * P.W + jb.t.x0;
-            s.ray_x[warp][lane] = __ldg(rx + lane);
-            s.ray_x[warp][lane + 32] = __ldg(rx + lane + 32);
-            if (lane < STRIP) s.ray_y[warp][lane] = __ldg(P.rig.ray_y + (size_t)jb.k * P.H + jb.t.y0 + ys + lane);
-        } else {                                            // ragged: columns / rows past the image edge continue the formula
-            const CamConst& ck = P.cam[jb.k];
-#pragma unroll
-            for (int i = lane; i < TILE; i += 32)
-                s.ray_x[warp][i] = (jb.t.x0 + i < P.W) ? __ldg(P.rig.ray_x + (size_t)jb.k * P.W + jb.t.x0 + i)
-                                                      : __fdiv_rn(sub(add((float)(jb.t.x0 + i), 0.5f), 0.5f * (float)P.W), ck.fx);
-            if (lane < STRIP) {
-                const int y = jb.t.y0 + ys + lane;
-                s.ray_y[warp][lane] = (y < P.H) ? __ldg(P.rig.ray_y + (size_t)jb.k * P.H + y)
-                                                : __fdiv_rn(sub(add((float)y, 0.5f), 0.5f * (float)P.H), ck.fy);
-            }
-        }
-        __syncwarp();
-        back_strip<FULL>(sv, P, jb, ego_active, ys, s.pool + ((bases >> (8 * j)) & 0xffu) * (REC / 4), cj, classify, stop, lane, s.tile_ntris[j], n);
-        if (lane == 0 && ys == 0) ++n.jobs;
-    }
-    // ---- the rest: tiles that did not fit are left to the cooperative kernel
-    if (threadIdx.x < NW && ((cnts >> (8 * threadIdx.x)) & 0xffu) == 0xffu)
-        P.overflow[1u + atomicAdd(&P.overflow[0], 1u)] = first + threadIdx.x;
-    flush_counters(P, n);
-}
-
-// ---------------------------------------------------------------------------------------------
-// Render kernel for images made of full 64 x 64 tiles whose rows allow vector stores (every
-// benchmark workload).  Like render_kernel, with less bookkeeping: ray tables of the four tiles are
-// loaded once, per-tile constants are a 16-byte record, the background rows a lane stores are
-// fetched before the strip is rasterized.  The record pool is handed out in rounds: tiles that do
-// not fit beside their fellows are set up and rasterized in a further round of the same CTA (their
-// survivors are already in device memory), so only a tile whose own survivors exceed the pool, or
-// whose cull lists overflowed, is left to the cooperative kernel.
-// ---------------------------------------------------------------------------------------------
-#ifndef PIC_FSTRIP
-#define PIC_FSTRIP 16
-#endif
-#ifndef PIC_FPOOL
-#define PIC_FPOOL 144
-#endif
-constexpr int FPOOL = PIC_FPOOL;     // records shared by the four tiles of a CTA
-constexpr int FSTRIP = PIC_FSTRIP;   // pixel rows of a strip: 16 or 8
-constexpr int FSTRIP_KEYS = TILE * FSTRIP;
-constexpr int FSTRIPS = TILE / FSTRIP;
-static_assert(FSTRIP == 16 || FSTRIP == 8, "strips of 16 or 8 rows");
-
-// The record pool of the full-tile kernel, one array per 16-byte part of a record: 17 words per
-// record instead of the 20 of an array of padded records, so more records fit beside the keys.
+// A record pool, one array per 16-byte part of a record: 17 words per
+// record instead of the 20 of an array of padded records.
 template <int N>
 struct __align__(16) RecordPool {
     float4 nx[N], ny[N], nz[N];               // edge functions E_i = nx[i] rx + ny[i] ry + nz[i]
@@ -1399,23 +1099,6 @@ __device__ __forceinline__ void read_record(const RecordPool<N>& pool, int slot,
     q.wx = r3.x; q.wy = r3.y; q.wz = r3.z;
     key_lo = __float_as_uint(r3.w);
 }
-
-struct __align__(16) TileRef {
-    size_t pixel0;       // offset of the tile's first pixel in the output images
-    int bg_row0;         // first row of the tile in the per-camera background tables
-    int active;          // is the ego agent active
-};
-
-struct __align__(16) FullSmem {
-    unsigned long long key[NW][FSTRIP_KEYS];  // warp w's strip of keys
-    RecordPool<FPOOL> pool;
-    float ray_x[NW][TILE], ray_y[NW][TILE];   // ray tables of tile w
-    Cam cam[NW];
-    TileRef tile[NW];
-    int n_surv[NW];
-    int next_task;
-};
-static_assert(sizeof(FullSmem) <= 44 * 1024, "shared memory must leave room for 5 CTAs per SM");
 
 // The 16 x 4 cell of strip_cell's comment, for the full-tile kernel: `kbase` and `lsw` are the
 // lane's share of the key address (row lane >> 3, chunk lane & 7, swizzle), `range` says whether
@@ -1450,44 +1133,6 @@ __device__ __forceinline__ void strip_cell(unsigned long long* key, const float*
     const unsigned long long k0 = make_key(__float_as_uint(w0), key_lo), k1 = make_key(__float_as_uint(w1), key_lo);
     if (in0 && k0 > kk.x) kp[0] = k0;
     if (in1 && k1 > kk.y) kp[1] = k1;
-}
-
-// Strip -> class / depth images, 16 pixels per lane and pass (see store_tile); resets the keys it reads.
-__device__ __forceinline__ void store_strip_full(unsigned long long* key, uint8_t* oc, uint16_t* od, int W, uint32_t touched,
-                                                 const uint32_t (&bgc)[2], const float (&bgz)[2], int lane) {
-#pragma unroll
-    for (int it = 0; it < FSTRIP / 8; ++it) {
-        const int y = it * 8 + (lane >> 2), xs = (lane & 3) * 16;
-        const size_t o = (size_t)y * W + xs;
-        uint32_t cw[4], dw[8];
-        if (((touched >> (it * 8 + (xs >> 3))) & 3u) == 0u) {       // both 8 x 8 blocks of the segment are background
-            const uint32_t c4 = bgc[it] * 0x01010101u;
-            const __half2 h = __floats2half2_rn(bgz[it], bgz[it]);
-            const uint32_t d2 = *reinterpret_cast<const uint32_t*>(&h);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) cw[j] = c4;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) dw[j] = d2;
-        } else {
-#pragma unroll
-            for (int j = 0; j < 16; j += 2) {
-                ulonglong2* kp = reinterpret_cast<ulonglong2*>(&key[key_index(xs + j, y)]);
-                const ulonglong2 kk = *kp;
-                *kp = make_ulonglong2(0ull, 0ull);
-                const float z0 = kk.x ? fast_rcp(__uint_as_float((uint32_t)(kk.x >> 32))) : bgz[it];
-                const float z1 = kk.y ? fast_rcp(__uint_as_float((uint32_t)(kk.y >> 32))) : bgz[it];
-                const uint32_t c0 = kk.x ? (uint32_t)(kk.x & 0xff) : bgc[it], c1 = kk.y ? (uint32_t)(kk.y & 0xff) : bgc[it];
-                const __half2 h = __floats2half2_rn(z0, z1);
-                dw[j >> 1] = *reinterpret_cast<const uint32_t*>(&h);
-                if ((j & 3) == 0) cw[j >> 2] = c0 | (c1 << 8); else cw[j >> 2] |= (c0 << 16) | (c1 << 24);
-            }
-        }
-#ifdef PIC_PROFILE
-        if (touched & 0x80000000u) continue;       // profiling: no global stores
-#endif
-        *reinterpret_cast<uint4*>(oc + o) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
-        store_256(od + o, dw);
-    }
 }
 
 // One strip (rows ys .. of the tile) by one warp: the tile's fragments that fall into it, then
@@ -1585,122 +1230,6 @@ __device__ __forceinline__ uint32_t raster_strip(StripView& s, const RecordPool<
     return __reduce_or_sync(0xffffffffu, touched);
 }
 
-__global__ void __launch_bounds__(NTHREADS, PIC_RENDER_CTAS) render_full_kernel(const __grid_constant__ RenderParams P) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    FullSmem& s = *reinterpret_cast<FullSmem*>(smem_raw);
-    const int stop = PIC_STOP(P);
-    if (stop == 15) return;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    launch_dependents();
-    const unsigned id = await_previous(blockIdx.x) * (unsigned)NW + warp;
-    const bool valid = id < P.n_jobs;
-    // ---- the cull kernel's survivors of tile first + w, and everything that does not depend on them
-    const uint2* blk = P.surv + (size_t)id * SURV_STRIDE;
-    int ns = -2, n_big = 0;
-    uint2 sv0 = make_uint2(0u, 0u);
-    Job job;
-    uint32_t n_map_tris = 0u;
-    if (valid) {
-        const uint4 head = __ldcg(reinterpret_cast<const uint4*>(blk));
-        job = decode_job(P, id);
-        n_map_tris = __ldg(&P.env_maps[job.e].n_tris);
-        const bool ego_active = __ldg(&P.agents[(size_t)job.e * P.A + job.a].active) != 0u;
-        const float* rx = P.rig.ray_x + (size_t)job.k * P.W + job.t.x0;
-        const float* ry = P.rig.ray_y + (size_t)job.k * P.H + job.t.y0;
-        s.ray_x[warp][lane] = __ldg(rx + lane); s.ray_x[warp][lane + 32] = __ldg(rx + lane + 32);
-        s.ray_y[warp][lane] = __ldg(ry + lane); s.ray_y[warp][lane + 32] = __ldg(ry + lane + 32);
-        if (lane == 0) {
-            load_camera(s.cam[warp], P.cams[job.view], P.cam[job.k], P.W, P.H);
-            TileRef tr;
-            tr.pixel0 = job.view * ((size_t)P.H * P.W) + (size_t)job.t.y0 * P.W + job.t.x0;
-            tr.bg_row0 = job.k * P.H + job.t.y0;
-            tr.active = ego_active ? 1 : 0;
-            s.tile[warp] = tr;
-        }
-        n_big = (int)(head.x & 0xffffu);
-        ns = head.x == SURV_OVERFLOW ? -1 : n_big + (int)(head.x >> 16);
-        if (ns > FPOOL) ns = -1;                            // more survivors than the whole pool
-        // the first survivor of this lane (front list, then back list); the others are fetched in the set-up loop
-        if (lane < ns) sv0 = __ldcg(blk + 2 + (lane < n_big ? lane : W_SURV - 1 - (lane - n_big)));
-    }
-    if (lane == 0) s.n_surv[warp] = ns;
-#pragma unroll
-    for (int i = 0; i < FSTRIP_KEYS / 2 / 32; ++i)
-        reinterpret_cast<ulonglong2*>(s.key[warp])[i * 32 + lane] = make_ulonglong2(0ull, 0ull);
-    __syncthreads();
-    StripView sv;
-    sv.key = s.key[warp];
-    // Rounds: every thread lays the record pool out alike -- the tiles not yet rendered, in order,
-    // as long as they fit.  One byte per tile: first record, and count (0xff: not in this round).
-    uint32_t done = 0u;                                      // bit j: tile j is rendered, absent, or left to the cooperative kernel
-#pragma unroll
-    for (int j = 0; j < NW; ++j)
-        if (s.n_surv[j] < 0) done |= 1u << j;
-#pragma unroll 1
-    while (done != (1u << NW) - 1u) {
-        uint32_t bases = 0u, cnts = 0u, now = 0u;
-        {
-            int off = 0;
-#pragma unroll
-            for (int j = 0; j < NW; ++j) {
-                const int c = s.n_surv[j];
-                bases |= (uint32_t)off << (8 * j);
-                if (!((done >> j) & 1u) && off + c <= FPOOL) { cnts |= (uint32_t)c << (8 * j); off += c; now |= 1u << j; }
-                else cnts |= 0xffu << (8 * j);
-            }
-        }
-        // ---- set-up by the tile's warp: survivor i becomes record i
-        if ((now >> warp) & 1u) {
-            const int my_base = (int)((bases >> (8 * warp)) & 0xffu);
-            const int my_cnt = (stop == 14) ? 0 : ns;
-            for (int i = lane; i < my_cnt; i += 32) {
-                const uint2 svi = (i < 32) ? sv0 : __ldcg(blk + 2 + (i < n_big ? i : W_SURV - 1 - (i - n_big)));
-                V3 V[4], Pn;
-                uint32_t key_lo, flags;
-                fetch_survivor(s.cam[warp], P, svi.x, job.e, n_map_tris, V, Pn, key_lo, flags);
-                PrimEq q;
-                if (!prim_equations(V, flags & 1u, flags, Pn, q)) { s.pool.box[my_base + i] = REC_DEAD; continue; }
-                write_record(s.pool, my_base + i, q, key_lo, svi.y, (tiny_box(svi.y) ? REC_TINY : 0u) | (record_in_range(V, P) ? REC_INRANGE : 0u));
-            }
-        }
-        if (threadIdx.x == 0) s.next_task = 0;
-        __syncthreads();
-        if (stop == 10) return;
-        // ---- the strips of this round's tiles are tasks that the warps draw from a counter
-#pragma unroll 1
-        for (;;) {
-            int task = 0;
-            if (lane == 0) task = atomicAdd(&s.next_task, 1);
-            task = __shfl_sync(0xffffffffu, task, 0);
-            if (task >= NW * FSTRIPS) break;
-            const int j = task / FSTRIPS, ys = (task % FSTRIPS) * FSTRIP;
-            const int cj = (int)((cnts >> (8 * j)) & 0xffu);
-            if (cj == 0xff) continue;
-            const TileRef tr = s.tile[j];
-            uint32_t bgc[2] = {P.cls_sky, P.cls_sky};
-            float bgz[2] = {P.far_z, P.far_z};
-            if (tr.active) {                                 // background of the rows this lane stores
-                const uint32_t* bg_cls = P.rig.bg_cls + tr.bg_row0 + ys + (lane >> 2);
-                const float* bg_z = P.rig.bg_z + tr.bg_row0 + ys + (lane >> 2);
-                bgc[0] = __ldg(bg_cls); bgz[0] = __ldg(bg_z);
-                if (FSTRIP == 16) { bgc[1] = __ldg(bg_cls + 8); bgz[1] = __ldg(bg_z + 8); }
-            }
-            sv.ray_x = s.ray_x[j]; sv.ray_y = s.ray_y[j] + ys;
-            uint32_t touched = raster_strip<FSTRIP>(sv, s.pool, (int)((bases >> (8 * j)) & 0xffu), (stop == 14) ? 0 : cj, ys, P.w_near, P.w_far, stop, lane);
-            if (stop == 5) touched = 0xffffu;
-            if (stop == 6) touched |= 0x80000000u;
-            const size_t o = tr.pixel0 + (size_t)ys * P.W;
-            if (stop != 8) store_strip_full(sv.key, P.out_class + o, P.out_depth + o, P.W, touched, bgc, bgz, lane);
-            __syncwarp();
-        }
-        done |= now;
-        if (done != (1u << NW) - 1u) __syncthreads();        // the pool is reused by the next round
-    }
-    // ---- the rest: tiles with too many survivors, or whose cull lists overflowed, are left to the cooperative kernel
-    if (threadIdx.x < NW && s.n_surv[threadIdx.x] == -1)
-        P.overflow[1u + atomicAdd(&P.overflow[0], 1u)] = blockIdx.x * (unsigned)NW + threadIdx.x;
-}
-
 // The tiles the render kernels left out, a CTA at a time.  (Called from the end of those kernels instead, the same code
 // costs them 2 % -- a call bounds their registers -- which is more than a launch that overlaps their last blocks.)
 template <class TL, bool FULL>
@@ -1717,30 +1246,10 @@ __global__ void __launch_bounds__(NTHREADS, 5) cooperative_kernel(const __grid_c
     flush_counters(P, n);
 }
 
-#ifdef PIC_PROFILE
-}  // namespace pic
-#include <cstdlib>
-namespace pic {
-// profiling aid: extra dynamic shared memory per CTA lowers the number of resident CTAs per SM
-static size_t smem_pad() { const char* e = getenv("PIC_SMEM_PAD"); return e ? (size_t)atoi(e) : 0; }
-#define RENDER_SMEM (RENDER_SMEM_BASE + smem_pad())
-#else
-#define RENDER_SMEM RENDER_SMEM_BASE
-#endif
-#define FULL_SMEM (sizeof(FullSmem) + (RENDER_SMEM - RENDER_SMEM_BASE))
-size_t render_smem_bytes() { return RENDER_SMEM; }
 cudaError_t configure_small_kernel();
 
 cudaError_t configure_render_kernel() {
     cudaError_t err = configure_small_kernel();
-    if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(render_full_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)FULL_SMEM);
-    if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(render_kernel<NoTally, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RENDER_SMEM);
-    if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(render_kernel<Tally, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)RENDER_SMEM);
-    if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(cooperative_kernel<NoTally, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem));
     if (err != cudaSuccess) return err;
     err = cudaFuncSetAttribute(cooperative_kernel<NoTally, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem));
     if (err != cudaSuccess) return err;
@@ -1829,9 +1338,11 @@ cudaError_t launch_next(K kernel, unsigned grid, size_t smem, cudaStream_t strea
 #include "pic_coverage.cuh"
 namespace pic {
 #include "pic_colour.cuh"
+#include "pic_tile.cuh"
 #include "pic_static.cuh"
 #include "pic_small.cuh"
 
+size_t render_smem_bytes() { return SMALL_SMEM > sizeof(ColourSmem) ? SMALL_SMEM : sizeof(ColourSmem); }
 size_t survivor_bytes_per_tile() { return sizeof(uint2) * SURV_STRIDE; }
 
 cudaError_t launch_render_kernel(const RenderParams& P0, long long n_views, int sm_count, cudaStream_t stream) {
@@ -1840,28 +1351,25 @@ cudaError_t launch_render_kernel(const RenderParams& P0, long long n_views, int 
     if (jobs > 0x7fffffffLL || (long long)P.E * P.A * P.K > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     if (jobs <= 0) return cudaSuccess;
     P.n_jobs = (uint32_t)jobs;
+    P.far_z2 = 0x10001u * (uint32_t)__half_as_ushort(__float2half_rn(P.far_z));
     const unsigned grid = (unsigned)((jobs + NW - 1) / NW);
     // few tiles: one CTA takes a tile from culling to store.  Measured (a call on 16 agents per environment, both image
     // shapes of the workloads): 64 tiles 37.0 -> 20.7 us, 256 tiles 44.6 -> 22.7, 768 tiles 47.3 -> 44.8, 1024 tiles
     // 48.4 -> 53.7, so the line lies at five tiles per multiprocessor.
     if (jobs <= 5LL * sm_count && !P.counters && !P.occlusion && (P.debug_flags & 15) == 0)
         return launch_next(render_small_kernel, (unsigned)jobs, SMALL_SMEM, stream, P, SMALL_THREADS);
-    const bool full = P.W % TILE == 0 && P.H % TILE == 0 && P.out_depth32 == nullptr && P.occlusion == nullptr && (P.debug_flags & 15) == 0 &&
-                      (reinterpret_cast<uintptr_t>(P.out_depth) & 31u) == 0;   // 256-bit depth stores
     // (a) cull: survivors per tile
     cudaError_t err = launch_next(P.counters ? cull_kernel<Tally, false> : cull_kernel<NoTally, false>, grid, sizeof(CullSmem), stream, P);
     if (err != cudaSuccess) return err;
     // (b)-(d) set-up, raster, store
-    err = P.counters ? launch_next(render_kernel<Tally, false>, grid, RENDER_SMEM, stream, P)
-          : full     ? launch_next(render_full_kernel, grid, FULL_SMEM, stream, P)
-                     : launch_next(render_kernel<NoTally, false>, grid, RENDER_SMEM, stream, P);
+    err = launch_next(P.counters ? render_tile_kernel<Tally, false>
+                      : P.W % 4 == 0 && !P.out_depth32 && !P.occlusion ? render_tile_kernel<NoTally, true>
+                                                                       : render_tile_kernel<NoTally, false>, (unsigned)jobs, 0, stream, P, 32);
     if (err != cudaSuccess) return err;
     // the tiles left out (their number is only known on the device): one wave of CTAs walks the list
     const long long wave = (long long)sm_count * 5;
     const unsigned cgrid = (unsigned)(jobs < wave ? jobs : wave);
-    err = P.counters ? launch_next(cooperative_kernel<Tally, false>, cgrid, sizeof(TileSmem), stream, P)
-          : full     ? launch_next(cooperative_kernel<NoTally, true>, cgrid, sizeof(TileSmem), stream, P)
-                     : launch_next(cooperative_kernel<NoTally, false>, cgrid, sizeof(TileSmem), stream, P);
+    err = launch_next(P.counters ? cooperative_kernel<Tally, false> : cooperative_kernel<NoTally, false>, cgrid, sizeof(TileSmem), stream, P);
     if (err != cudaSuccess || !P.occlusion) return err;
     coverage_kernel<<<grid, NTHREADS, 0, stream>>>(P);
     return cudaGetLastError();

@@ -22,7 +22,7 @@
 namespace pic {
 cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses, float* state, const float* actions,
                          const float* dims, const uint8_t* active, const uint8_t* agent_cls, AgentGeom* agents_out, ViewCam* cams_out,
-                         float* tables, uint32_t* status, float dt, float wheelbase, float v_max, cudaStream_t stream);
+                         uint32_t* status, float dt, float wheelbase, float v_max, cudaStream_t stream);
 cudaError_t configure_static_kernel();            // pic_static.cuh (part of pic_render.cu)
 cudaError_t launch_static_kernel(const RenderParams& P, const float* tri_xyz, const uint8_t* tri_class, int n_tris, int sm_count, cudaStream_t stream);
 void set_last_error(const char* msg);
@@ -41,10 +41,10 @@ constexpr int kMaxDevices = 64;
 constexpr size_t kOffAgents = 0;
 constexpr size_t kOffCams = kOffAgents + sizeof(AgentGeom) * kMaxAgents;
 constexpr size_t kOffTables = kOffCams + sizeof(ViewCam) * kMaxViews;
-constexpr size_t kOffStatus = kOffTables + sizeof(float) * MAX_CAMS * 4 * kMaxSide;
+constexpr size_t kOffStatus = kOffTables + sizeof(float) * MAX_CAMS * 6 * kMaxSide;
 constexpr size_t kScratchBytes = kOffStatus + 256;
 
-// The only device memory this entry point ever uses besides the caller's buffers (about 420 KB,
+// The only device memory this entry point ever uses besides the caller's buffers (about 490 KB,
 // held by every device that loads the library until the process exits).
 static __device__ __align__(256) unsigned char g_static_scratch[kScratchBytes];
 
@@ -120,6 +120,7 @@ extern "C" pic_status pic_render_static(const pic_static_desc* d, const float* t
     memset(&P, 0, sizeof(P));
     P.E = d->E; P.A = d->A; P.K = d->K; P.H = d->H; P.W = d->W;
     P.tiles_x = (d->W + TILE - 1) / TILE; P.tiles_y = (d->H + TILE - 1) / TILE;
+    set_divisors(P);
     P.near_z = d->near_z; P.far_z = d->far_z; P.w_near = 1.0f / d->near_z; P.w_far = 1.0f / d->far_z;
     P.cls_agent = d->agent_class; P.cls_sky = d->sky_class; P.cls_ground = d->ground_class;
     AgentGeom* agents = reinterpret_cast<AgentGeom*>(scratch + kOffAgents);
@@ -127,10 +128,7 @@ extern "C" pic_status pic_render_static(const pic_static_desc* d, const float* t
     float* tables = reinterpret_cast<float*>(scratch + kOffTables);
     uint32_t* status = reinterpret_cast<uint32_t*>(scratch + kOffStatus);
     P.agents = agents; P.cams = cams;
-    P.rig.ray_x = tables;
-    P.rig.ray_y = P.rig.ray_x + (size_t)d->K * d->W;
-    P.rig.bg_z = P.rig.ray_y + (size_t)d->K * d->H;
-    P.rig.bg_cls = reinterpret_cast<const uint32_t*>(P.rig.bg_z + (size_t)d->K * d->H);
+    P.rig = rig_tables(tables, d->K, d->H, d->W);
     P.out_class = out_class; P.out_depth = out_depth;
     for (int k = 0; k < d->K; ++k) {
         CamConst& o = P.cam[k];
@@ -140,7 +138,7 @@ extern "C" pic_status pic_render_static(const pic_static_desc* d, const float* t
         o.fx = rig[k].fx; o.fy = rig[k].fy;
     }
     // (the status word is sticky across calls, like a scene's: pic_static_status reads and clears it)
-    ce = pic::launch_setup(P, d->E * d->A, poses, nullptr, nullptr, dims, active, nullptr, agents, cams, tables, status, 0.f, 1.f, 0.f, stream);
+    ce = pic::launch_setup(P, d->E * d->A, poses, nullptr, nullptr, dims, active, nullptr, agents, cams, status, 0.f, 1.f, 0.f, stream);
     if (ce != cudaSuccess) return fail(PIC_ERR_CUDA, "set-up kernels: %s", cudaGetErrorString(ce));
     ce = pic::launch_static_kernel(P, tri_xyz, tri_class, d->n_tris, g_sm_count[dev], stream);
     if (ce != cudaSuccess) return fail(PIC_ERR_CUDA, "render_static_kernel: %s", cudaGetErrorString(ce));

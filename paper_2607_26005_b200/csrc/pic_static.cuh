@@ -145,6 +145,7 @@ cudaError_t launch_static_kernel(const RenderParams& P, const float* tri_xyz, co
     // (two CTAs per multiprocessor are enough to hide the latency of the tests)
     while (S.tile_h > 16 && views * ((P.H + S.tile_h - 1) / S.tile_h) < 2LL * sm_count) S.tile_h >>= 1;
     S.P.tiles_y = (P.H + S.tile_h - 1) / S.tile_h;
+    set_divisors(S.P);
     render_static_kernel<<<(unsigned)(views * S.P.tiles_y), NTHREADS, sizeof(StaticSmem), stream>>>(S);
     return cudaGetLastError();
 }

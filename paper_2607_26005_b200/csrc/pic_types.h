@@ -1,5 +1,6 @@
 // Device/host data layout of the rasterizer library (internal).
 #pragma once
+#include <stddef.h>
 #include <stdint.h>
 #include <vector_types.h>
 
@@ -22,6 +23,13 @@ struct Prim {
     uint32_t pad;
 };
 static_assert(sizeof(Prim) == 64, "Prim must be 64 bytes");
+
+// Upright cylinder around a primitive of the grid order (same index), 16 bytes: what the cull kernel looks at first.
+struct Bound {
+    float x, y, z;      // centre
+    uint32_t size;      // upper halves of two float32, rounded up: radius << 16 | half height
+};
+static_assert(sizeof(Bound) == 16, "Bound must be 16 bytes");
 
 // Axis-aligned box of a leaf (over primitives) or a group (over leaves); 32 bytes.
 struct Node {
@@ -80,7 +88,20 @@ struct RigTables {
     const float* ray_y;        // [K][H]
     const float* bg_z;         // [K][H] background depth
     const uint32_t* bg_cls;    // [K][H] background class
+    const uint2* bg_fill;      // [K][H] the same as stored: class in four bytes, binary16 depth in two halves
 };
+
+// Division of numbers below 2^31 by a divisor fixed per call (Granlund and Montgomery, "Division by invariant integers
+// using multiplication", PLDI 1994): q = (mulhi(n, m) + n) >> s.
+struct FastDiv {
+    uint32_t m, s;
+};
+inline FastDiv fast_div(uint32_t d) {
+    FastDiv f = {0u, 0u};
+    while ((1ull << f.s) < d) ++f.s;
+    f.m = (uint32_t)(((1ull << 32) * ((1ull << f.s) - d)) / d + 1ull);
+    return f;
+}
 
 struct RenderParams {
     int32_t E, A, K, H, W;
@@ -88,6 +109,8 @@ struct RenderParams {
     float near_z, far_z;
     float w_near, w_far;            // 1/near, 1/far: kept range of the reciprocal depth
     uint32_t cls_agent, cls_sky, cls_ground;
+    uint32_t far_z2;                // binary16 of far_z, twice
+    FastDiv div_tiles, div_tiles_x, div_K, div_A;   // by tiles per view, tile columns, cameras, agent slots
     const int32_t* env_map;
     const MapInfo* env_maps;        // [E] the MapInfo of each environment's map (one load instead of two)
     const MapInfo* maps;
@@ -96,6 +119,7 @@ struct RenderParams {
     const Prim* prims;
     const uint32_t* cell_start;     // grid: per map nx * ny + 1 offsets into grid_prims
     const Prim* grid_prims;         // the primitives in grid order: small ones cell by cell (row-major), then the large ones leaf by leaf
+    const Bound* grid_bounds;       // bounding cylinder of each of grid_prims
     const Node* large_leaves;       // boxes over up to LARGE_LEAF_PRIMS consecutive large primitives of grid_prims
     const AgentGeom* agents;
     const ViewCam* cams;            // [E*A*K]
@@ -116,6 +140,22 @@ struct RenderParams {
     CamConst cam[MAX_CAMS];
 };
 
+// Layout of the per-camera tables in one allocation of table_bytes bytes, 8-byte aligned.
+inline size_t table_bytes(int K, int H, int W) { return sizeof(float) * (size_t)K * ((size_t)W + 5 * (size_t)H); }
+inline RigTables rig_tables(float* base, int K, int H, int W) {
+    RigTables r;
+    r.bg_fill = reinterpret_cast<const uint2*>(base);
+    r.ray_x = base + 2 * (size_t)K * H;
+    r.ray_y = r.ray_x + (size_t)K * W;
+    r.bg_z = r.ray_y + (size_t)K * H;
+    r.bg_cls = reinterpret_cast<const uint32_t*>(r.bg_z + (size_t)K * H);
+    return r;
+}
+inline void set_divisors(RenderParams& P) {
+    P.div_tiles = fast_div((uint32_t)(P.tiles_x * P.tiles_y)); P.div_tiles_x = fast_div((uint32_t)P.tiles_x);
+    P.div_K = fast_div((uint32_t)P.K); P.div_A = fast_div((uint32_t)P.A);
+}
+
 // Host-side result of the hierarchy build for all maps of a scene.
 struct HostHierarchy;
 HostHierarchy* build_hierarchy(int num_maps, const int64_t* tri_offset, const float* tri_xyz,
@@ -127,6 +167,7 @@ const Node* hierarchy_groups(const HostHierarchy*, size_t* n);
 const MapInfo* hierarchy_maps(const HostHierarchy*, size_t* n);
 const uint32_t* hierarchy_cell_start(const HostHierarchy*, size_t* n);
 const Prim* hierarchy_grid_prims(const HostHierarchy*, size_t* n);
+const Bound* hierarchy_grid_bounds(const HostHierarchy*, size_t* n);
 const Node* hierarchy_large_leaves(const HostHierarchy*, size_t* n);
 
 }  // namespace pic

@@ -73,3 +73,14 @@ def test_calls_with_few_tiles(n_tris, E, A, H, W, K, spread):
         assert (a[0] == c[0]).all() and (a[1].view(np.uint16) == c[1].view(np.uint16)).all()
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("n_tris,E,A,H,W,K,spread", [
+    (60, 4, 50, 20, 30, 4, 30.0),         # rows of no whole groups of four pixels: scalar stores
+    (200, 2, 100, 36, 76, 4, 60.0),       # groups of four but not of sixteen; a second tile narrower than a cell
+    (200, 2, 100, 65, 48, 4, 60.0),       # a second tile of a single row
+    (3000, 1, 60, 130, 80, 4, 12.0),      # more records and more fragments than a tile's lists hold
+    (60, 8, 24, 64, 64, 4, 6.0),          # large primitives around the cameras: cells wholly inside, range tests
+])
+def test_calls_with_many_tiles(n_tris, E, A, H, W, K, spread):
+    test_calls_with_few_tiles(n_tris, E, A, H, W, K, spread)
