@@ -27,17 +27,23 @@ constexpr int CSTRIP = 8;                       // pixel rows of a strip
 constexpr int CSTRIPS = TILE / CSTRIP;
 constexpr int CSTRIP_KEYS = TILE * CSTRIP;
 constexpr int CPOOL = 254;                      // records shared by the four tiles (a tile's survivors always fit: W_SURV < CPOOL)
+#ifndef PIC_COLOUR_SMALL
+#define PIC_COLOUR_SMALL 256
+#endif
+constexpr int COLOUR_SMALL = PIC_COLOUR_SMALL;  // pixels in the conservative box of a primitive that is worked off pixel by pixel (at most 511 in a strip)
 constexpr int CFRAGS = 1023;                    // partially covering fragments of a strip (10-bit links, 0 ends a list)
 constexpr uint32_t STATUS_COLOUR_INCOMPLETE = 2u;   // = PIC_FLAG_COLOUR_INCOMPLETE of the public header
 constexpr uint32_t STATUS_COLOUR_FRAGMENTS = 4u;    // = PIC_FLAG_COLOUR_FRAGMENTS
 static_assert(W_SURV <= CPOOL && CPOOL <= 256, "a tile's survivors fit the pool; a slot fits the key's low byte");
 
+constexpr unsigned long long KEY_RESOLVED = 1ull << 63;     // (a key's high word is the bits of a positive float: bit 63 is free)
+
 __constant__ float FACE_SHADE[6] = {0.60f, 1.00f, 0.70f, 0.85f, 0.40f, 0.92f};   // rear, front, right, left, bottom, top
 
 struct __align__(16) ColourPool {
-    float4 nx[CPOOL], ny[CPOOL], nz[CPOOL];     // edge functions E_i = nx[i] rx + ny[i] ry + nz[i]
+    float4 nx[CPOOL], ny[CPOOL], nz[CPOOL];     // edge functions E_i = nx[i] rx + ny[i] ry + nz[i]; REC_TINY: nx, ny the projected vertices
     float4 w[CPOOL];                            // 1/z plane wx, wy, wz; key low word (index, class)
-    uint32_t box[CPOOL];                        // pixel box (6 bits per coordinate), top-left bits << 24, REC_DEAD
+    uint32_t box[CPOOL];                        // pixel box (6 bits per coordinate), top-left bits << 24, REC_DEAD, REC_TINY
     float shade[CPOOL];                         // box faces: the face's factor; map primitives: 0 (not shaded)
     uint32_t surface[CPOOL];                    // fragments of equal surface merge: a map primitive's class, 256 + agent of a box
 };
@@ -79,6 +85,23 @@ __device__ __forceinline__ uint32_t coverage14(const PixelLines& L, const PrimEq
     return min((uint32_t)(edge_coverage(e1, a1, b1) * 16383.f + 0.5f), COVERAGE_MAX);
 }
 
+// The fragments of the lanes of mask m (a14 != 0) become the entries n_frag + 1, ... of the array and join their pixels'
+// lists; lanes that share a pixel are chained in lane order.
+__device__ __forceinline__ void push_fragments(unsigned long long* frag, uint16_t* head, int n_frag, unsigned m, uint32_t a14, uint32_t pix, uint32_t slot,
+                                               float wc, int lane) {
+    const unsigned below = (1u << lane) - 1u;
+    const unsigned peers = __match_any_sync(0xffffffffu, a14 != 0u ? pix : 0x10000u + lane);
+    if (a14 != 0u) {
+        const unsigned lower = peers & below;
+        const int i = n_frag + 1 + __popc(m & below);
+        const uint32_t next = lower ? (uint32_t)(n_frag + 1 + __popc(m & ((1u << (31 - __clz(lower))) - 1u))) : (uint32_t)head[pix];
+        frag[i] = ((unsigned long long)__float_as_uint(wc) << 32) | (a14 << 18) | (slot << 10) | next;
+    }
+    __syncwarp();
+    if (a14 != 0u && (peers >> lane) == 1u) head[pix] = (uint16_t)(n_frag + 1 + __popc(m & below));
+    __syncwarp();
+}
+
 // The strip's queue of pending pixels (pixel << 8 | slot; it grows down from the top of the fragment array while
 // the lists grow up from its bottom), a lane each: the record's six lines at the pixel, the exact area, the depth;
 // pixels with a positive area join their pixel's list.  The newest items -- those next to the lists' end -- go first,
@@ -115,25 +138,63 @@ __device__ __noinline__ void flush_pending(const unsigned long long* key, unsign
             if (!(make_key(__float_as_uint(wc), 0xffffffffu) > key[key_index((int)(pix & (TILE - 1)), (int)(pix >> 6))])) a14 = 0u;
         }
         n_pend -= take;
-        // (two items of a round may belong to one pixel -- two records with a vertex there -- so the lists are
-        // extended one lane after the other)
         const unsigned m = __ballot_sync(0xffffffffu, a14 != 0u);
-        const int idx = n_frag + 1 + __popc(m & ((1u << lane) - 1u));
-        // lanes whose pixel no other lane of the round shares link their entries at once
-        const bool alone = __popc(__match_any_sync(0xffffffffu, a14 != 0u ? pix : 0x10000u + lane)) == 1;
-        if (a14 != 0u && alone) {
-            frag[idx] = ((unsigned long long)__float_as_uint(wc) << 32) | (a14 << 18) | (slot << 10) | head[pix];
-            head[pix] = (uint16_t)idx;
-        }
-        for (unsigned rest = __ballot_sync(0xffffffffu, a14 != 0u && !alone); rest; rest &= rest - 1) {
-            if (lane == __ffs(rest) - 1) {
-                frag[idx] = ((unsigned long long)__float_as_uint(wc) << 32) | (a14 << 18) | (slot << 10) | head[pix];
-                head[pix] = (uint16_t)idx;
-            }
-            __syncwarp();
-        }
+        push_fragments(frag, head, n_frag, m, a14, pix, slot, wc, lane);
         n_frag += __popc(m);
     }
+}
+
+// The pixels of the small records slot0 + lane that have any here (cnt of them, w per row from column x0 and strip row y0
+// on), a lane each whatever the record: exact area, depth at the pixel centre; pixels with a positive area in front of
+// the nearest fully covering fragment join their pixel's list.
+__device__ __noinline__ void small_fragments(unsigned long long* key, unsigned long long* frag, uint16_t* head, int& n_frag, int n_pend, bool& dropped,
+                                             const ColourPool& pool, uint32_t slot0, int cnt, int w, int x0, int y0, int ys, const float* ray_x,
+                                             const float* ray_y, float w_near, float w_far, int lane) {
+    int incl = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += up;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31), before = incl - cnt;
+    // (i * inv) >> 15 is i / w for i < 512, w <= 64
+    const uint32_t packed = (uint32_t)x0 | ((uint32_t)y0 << 6) | ((uint32_t)w << 9) | ((uint32_t)(cnt ? (32768 + w - 1) / w : 0) << 16);
+#pragma unroll 1
+    for (int p0 = 0; p0 < total; p0 += 32) {
+        const int p = p0 + lane;
+        int own = 0;                                         // the last lane whose pixels begin at or before p
+#pragma unroll
+        for (int st = 16; st; st >>= 1)
+            if (__shfl_sync(0xffffffffu, before, own + st) <= p) own += st;
+        const uint32_t pk = __shfl_sync(0xffffffffu, packed, own);
+        const int idx = p - __shfl_sync(0xffffffffu, before, own);
+        const int dy = (int)(((uint32_t)idx * (pk >> 16)) >> 15), x = (int)(pk & 63u) + idx - dy * (int)((pk >> 9) & 127u), y = (int)((pk >> 6) & 7u) + dy;
+        const uint32_t slot = slot0 + (uint32_t)own;
+        uint32_t a14 = 0u, pix = 0u;
+        float wc = 0.f;
+        if (p < total) {
+            pix = (uint32_t)(y * TILE + x);
+            const float4 X = pool.nx[slot], Y = pool.ny[slot], pw = pool.w[slot];
+            const float ox = (float)x, oy = (float)(ys + y);
+            const float vx[4] = {X.x - ox, X.y - ox, X.z - ox, X.w - ox}, vy[4] = {Y.x - oy, Y.y - oy, Y.z - oy, Y.w - oy};
+            const float area = polygon_coverage(vx, vy);
+            a14 = min((uint32_t)(area * 16383.f + 0.5f), COVERAGE_MAX);
+            wc = fminf(fmaxf(fm(pw.x, ray_x[x], fm(pw.y, ray_y[y], pw.z)), w_far), w_near);
+            unsigned long long* kp = key + key_index(x, y);
+            const unsigned long long old = *kp;
+            // (only fragments in front of the pixel's nearest fully covering fragment so far are kept)
+            if (!(make_key(__float_as_uint(wc), 0xffffffffu) > old)) a14 = 0u;
+            else if (area > 0.99999f) {
+                if (!(old & KEY_RESOLVED)) atomicMax(kp, make_key(__float_as_uint(wc), (__float_as_uint(pw.w) & 0xffffff00u) | slot));
+                a14 = 0u;
+            }
+        }
+        const unsigned m = __ballot_sync(0xffffffffu, a14 != 0u);
+        if (n_frag + n_pend + __popc(m) > CFRAGS) { dropped = true; break; }
+        push_fragments(frag, head, n_frag, m, a14, pix, slot, wc, lane);
+        n_frag += __popc(m);
+    }
+    __syncwarp();
 }
 
 // A 16 x 4 pixel cell of a strip against one record; a lane handles two adjacent pixels.
@@ -259,7 +320,6 @@ __device__ __forceinline__ uint32_t composite_pixel(unsigned long long k, uint32
            ((uint32_t)fminf(fmaxf(B + 0.5f, 0.f), 255.f) << 16);
 }
 
-constexpr unsigned long long KEY_RESOLVED = 1ull << 63;     // (a key's high word is the bits of a positive float: bit 63 is free)
 
 // Rows of a strip of tile `jb` -> colours: the pixels that have a list are composited, lane l taking pixels l, l + 32, ...
 // so that a row crowded with fragments (the horizon) is shared by all lanes; their colour replaces the pixel's key
@@ -468,11 +528,21 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
                 if (drop || !prim_equations(V, flags & 1u, flags, Pn, q)) { s.pool.box[slot] = REC_DEAD; continue; }
                 const uint32_t box = svi.y;
                 const uint32_t bx0 = box & 0xff, by0 = (box >> 8) & 0xff, bx1 = (box >> 16) & 0xff, by1 = box >> 24;
+                // a small primitive wholly within the depth range: its vertices in the tile's pixel coordinates instead of edges
+                const bool small = AA && (bx1 - bx0 + 1u) * (by1 - by0 + 1u) <= (uint32_t)COLOUR_SMALL && record_in_range(V, P);
+                if (small) {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const float iz = __fdividef(1.f, V[k].z);
+                        q.nx[k] = fm(c.focx, mul(V[k].x, iz), c.cx - (float)job.t.x0);
+                        q.ny[k] = fm(c.focy, mul(V[k].y, iz), c.cy - (float)job.t.y0);
+                    }
+                }
                 s.pool.nx[slot] = make_float4(q.nx[0], q.nx[1], q.nx[2], q.nx[3]);
                 s.pool.ny[slot] = make_float4(q.ny[0], q.ny[1], q.ny[2], q.ny[3]);
                 s.pool.nz[slot] = make_float4(q.nz[0], q.nz[1], q.nz[2], q.nz[3]);
                 s.pool.w[slot] = make_float4(q.wx, q.wy, q.wz, __uint_as_float(key_lo));
-                s.pool.box[slot] = bx0 | (by0 << 6) | (bx1 << 12) | (by1 << 18) | (q.tl << 24);
+                s.pool.box[slot] = bx0 | (by0 << 6) | (bx1 << 12) | (by1 << 18) | (q.tl << 24) | (small ? REC_TINY : 0u);
                 s.pool.shade[slot] = shade;
                 s.pool.surface[slot] = surface;
             }
@@ -521,36 +591,18 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
                     hit = !(bw_lane & REC_DEAD) && by1 >= ys && by0 < ys + CSTRIP;
                 }
                 if (AA) {
-                    // records whose pixel box is at most 4 x 4: every pixel of the box (in this strip's window) is queued as
-                    // a (pixel, record) pair and worked off with the other pending pixels, a lane each -- far cheaper
-                    // than walking a 64-pixel cell per record for the handful of pixels a distant primitive touches
+                    // small records: every pixel of the box (in this strip's window) is worked off, a lane each whatever
+                    // the record -- far cheaper than walking a 64-pixel cell per record for the handful of pixels a
+                    // distant primitive touches
                     const int bx0 = bw_lane & 63, bx1 = (bw_lane >> 12) & 63, by0 = (bw_lane >> 6) & 63, by1 = (bw_lane >> 18) & 63;
-                    const bool small = hit && bx1 - bx0 < 4 && by1 - by0 < 4;
+                    const bool small = hit && (bw_lane & REC_TINY);
                     hit = hit && !small;
                     const int x0 = max(bx0, col_lo), x1 = min(bx1, col_hi - 1);
                     const int w = max(x1 - x0 + 1, 0), y0 = max(by0 - ys, row_lo), y1 = min(by1 - ys, row_hi - 1);
                     const int cnt = small ? w * max(y1 - y0 + 1, 0) : 0;
-                    if (__any_sync(0xffffffffu, cnt > 0)) {
-                        int incl = cnt;
-#pragma unroll
-                        for (int d = 1; d < 32; d <<= 1) {
-                            const int up = __shfl_up_sync(0xffffffffu, incl, d);
-                            if (lane >= d) incl += up;
-                        }
-                        const int total = __shfl_sync(0xffffffffu, incl, 31);
-                        if (n_frag + n_pend + total <= CFRAGS) {
-                            const uint32_t slot = (uint32_t)(first + base + lane);
-                            for (int k = 0; k < cnt; ++k) {
-                                const uint32_t pix = (uint32_t)((y0 + k / w) * TILE + x0 + k % w);
-                                frag[CFRAGS - (n_pend + (incl - cnt) + k)] = (pix << 8) | slot;
-                            }
-                            n_pend += total;
-                        } else {
-                            dropped = true;
-                        }
-                        __syncwarp();
-                        if (n_pend >= 96) flush_pending(key, frag, head, n_frag, n_pend, s.pool, ray_x, ray_y, du, dv, P.w_near, P.w_far, lane);
-                    }
+                    if (__any_sync(0xffffffffu, cnt > 0))
+                        small_fragments(key, frag, head, n_frag, n_pend, dropped, s.pool, (uint32_t)(first + base), cnt, w, x0, y0, ys, ray_x, ray_y,
+                                        P.w_near, P.w_far, lane);
                 }
                 for (unsigned hits = __ballot_sync(0xffffffffu, hit); hits; hits &= hits - 1) {
                     const int src = __ffs(hits) - 1;

