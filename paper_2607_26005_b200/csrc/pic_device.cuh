@@ -186,14 +186,14 @@ __device__ __forceinline__ unsigned long long make_key(uint32_t wbits, uint32_t 
 // vertex is too close to the camera plane to project.  Returns false if the primitive cannot
 // touch any pixel centre of the tile (with the default margin m) or lies entirely before near / beyond far.
 // (Triangles pass their third vertex twice.)
-__device__ __forceinline__ bool pixel_box(const Cam& c, const TileCtx& t, const V3 (&V)[4], uint32_t& packed, const float m = 0.00390625f) {
+__device__ __forceinline__ bool pixel_box_int(const Cam& c, const TileCtx& t, const V3 (&V)[4], int& bx0, int& by0, int& bx1, int& by1, const float m = 0.00390625f) {
     constexpr int n = 4;
     float zmin = V[0].z, zmax = V[0].z;
 #pragma unroll
     for (int i = 1; i < n; ++i) { zmin = fminf(zmin, V[i].z); zmax = fmaxf(zmax, V[i].z); }
     // (written without early exits: the lanes of a warp rarely agree, so exits save nothing)
     bool ok = (zmax >= t.near_z * 0.9999f) && (zmin <= t.far_z * 1.0001f);
-    int bx0 = 0, by0 = 0, bx1 = t.tw - 1, by1 = t.th - 1;
+    bx0 = 0; by0 = 0; bx1 = t.tw - 1; by1 = t.th - 1;
     if (zmin >= t.near_z * ZPROJ_FRAC) {
         float sx0 = 3e38f, sx1 = -3e38f, sy0 = 3e38f, sy1 = -3e38f;
 #pragma unroll
@@ -223,6 +223,13 @@ __device__ __forceinline__ bool pixel_box(const Cam& c, const TileCtx& t, const 
         }
         ok = !(ol || orr || ou || od);
     }
+    return ok;
+}
+
+// The same in a word, 8 bits per coordinate.
+__device__ __forceinline__ bool pixel_box(const Cam& c, const TileCtx& t, const V3 (&V)[4], uint32_t& packed, const float m = 0.00390625f) {
+    int bx0, by0, bx1, by1;
+    const bool ok = pixel_box_int(c, t, V, bx0, by0, bx1, by1, m);
     packed = (uint32_t)bx0 | ((uint32_t)by0 << 8) | ((uint32_t)bx1 << 16) | ((uint32_t)by1 << 24);
     return ok;
 }

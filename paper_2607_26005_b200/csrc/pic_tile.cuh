@@ -20,7 +20,7 @@
 #pragma once
 
 constexpr int TREC = 32;                     // records of a tile: a 32-bit mask
-constexpr int TFRAG = 160;                   // fragments of its small primitives
+constexpr int TFRAG = 256;                   // fragments of its small primitives
 constexpr int SMALL_PIXELS = PIC_SMALL_PIXELS;   // pixel centres in the box of a small primitive (at most 32)
 constexpr int CELL_W = 32, CELL_H = 4;       // pixels of a cell
 static_assert((TILE / CELL_W) * (TILE / CELL_H) == 32, "a lane per cell");
@@ -211,8 +211,8 @@ __device__ __forceinline__ void store_background(const RenderParams& P, size_t t
     }
 }
 
-// VEC: rows of a multiple of four pixels, and none of the options (float32 depth image, occlusion counts).
-template <class TL, bool VEC>
+// VEC: rows of a multiple of four pixels and no float32 depth image.  OCC: with occlusion counts.
+template <class TL, bool VEC, bool OCC>
 __global__ void __launch_bounds__(32, PIC_TILE_CTAS) render_tile_kernel(const __grid_constant__ RenderParams P) {
     __shared__ TileWarp s;
     const int lane = threadIdx.x;
@@ -335,7 +335,7 @@ __global__ void __launch_bounds__(32, PIC_TILE_CTAS) render_tile_kernel(const __
     const size_t tile0 = job.view * ((size_t)P.H * P.W) + (size_t)t.y0 * P.W + t.x0;
     const uint32_t* bg_cls = P.rig.bg_cls + (size_t)job.k * P.H + t.y0;
     const float* bg_z = P.rig.bg_z + (size_t)job.k * P.H + t.y0;
-    uint32_t* occ = (!VEC && P.occlusion) ? P.occlusion + job.view * (size_t)P.A * 2u : nullptr;   // visible-pixel counts of this view
+    uint32_t* occ = (OCC && P.occlusion) ? P.occlusion + job.view * (size_t)P.A * 2u : nullptr;   // visible-pixel counts of this view
     // cells that hold anything
     uint32_t busy = __ballot_sync(0xffffffffu, hit != 0u);
     if (n_frag > 0) {
@@ -373,7 +373,7 @@ __global__ void __launch_bounds__(32, PIC_TILE_CTAS) render_tile_kernel(const __
         raster_records_cell(s, m, cell, rx, ry, P.w_near, P.w_far, best);
         const bool row_ok = y < t.th;
         const int n_px = row_ok ? t.tw - x : 0;
-        if (!VEC && occ) {
+        if (OCC && occ) {
 #pragma unroll
             for (int k = 0; k < 4; ++k)
                 if (k >= n_px) best[k] = 0ull;

@@ -92,3 +92,16 @@ def test_occlusion_ragged_multi_tile_images(gu):
     st = _compare(s, occ, act[::3])
     print("occlusion, paper rig 96x54:", st)
     assert st["seen"] > 0
+
+
+@pytest.mark.parametrize("A,H,W,far", [(40, 33, 300, 100.0), (33, 16, 20, 12.0), (12, 17, 64, 100.0)])
+def test_occlusion_bands_and_wide_images(gu, A, H, W, far):
+    # bands of 16 rows with a remainder of one, boxes of more than 255 columns, a pass of 32 agents and a rest, boxes cut by far
+    from scenes import custom_scene, make_rig
+    rng = np.random.default_rng(A)
+    poses = np.concatenate([rng.uniform(-14, 14, size=(1, A, 2)), rng.uniform(-3, 3, size=(1, A, 1))], axis=2).astype(np.float32)
+    s = custom_scene(np.zeros((0, 3, 3), np.float32), np.zeros(0, np.uint8), poses, np.tile(np.array(CAR, np.float32), (1, A, 1)),
+                     make_rig((10.0,), 90.0, 60.0, W, H), H, W, far=far)
+    occ, _ = _gpu_counts(gu, s)
+    st = _compare(s, occ, np.arange(0, A, max(1, A // 8)))
+    assert st["seen"] > 0
