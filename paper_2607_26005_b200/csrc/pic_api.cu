@@ -17,7 +17,7 @@ cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses
                          const float* dims, const uint8_t* active, const uint8_t* agent_cls, AgentGeom* agents_out, ViewCam* cams_out,
                          uint32_t* status, float dt, float wheelbase, float v_max, cudaStream_t stream);
 cudaError_t launch_render(const RenderParams& P, long long n_views, bool brute, int sm_count, cudaStream_t stream);
-cudaError_t launch_colour(const RenderParams& P, long long n_views, bool antialias, cudaStream_t stream);
+cudaError_t launch_colour(const RenderParams& P, long long n_views, bool antialias, int sm_count, cudaStream_t stream);
 size_t survivor_bytes_per_tile();
 }  // namespace pic
 
@@ -85,7 +85,7 @@ struct pic_scene {
     uint8_t* d_agent_cls = nullptr; // [E*A] class of each agent's box
     bool have_agent_cls = false;
     uint32_t* d_status = nullptr;
-    uint8_t* d_palette = nullptr;   // [256][3] RGB of every class, for the colour output
+    uint32_t* d_palette = nullptr;  // [256] RGB of every class (R in the low byte), for the colour output
     // staging for pic_render_host
     float* d_in_poses = nullptr;
     float* d_in_dims = nullptr;
@@ -274,7 +274,7 @@ pic_status pic_scene_create(const pic_scene_desc* d, pic_scene** out) {
     dmalloc((void**)&s->d_active, n_agents);
     dmalloc((void**)&s->d_agent_cls, n_agents);
     dmalloc((void**)&s->d_status, sizeof(uint32_t));
-    dmalloc((void**)&s->d_palette, 768);
+    dmalloc((void**)&s->d_palette, sizeof(uint32_t) * 256);
     upload(s->d_env_map, env_map, sizeof(int32_t) * d->E);
     upload(s->d_maps, maps, sizeof(pic::MapInfo) * nm);
     {
@@ -295,9 +295,9 @@ pic_status pic_scene_create(const pic_scene_desc* d, pic_scene** out) {
     upload(s->d_large_leaves, large_leaves, sizeof(pic::Node) * nll);
     if (ce == cudaSuccess) ce = cudaMemset(s->d_status, 0, sizeof(uint32_t));
     if (ce == cudaSuccess) {          // until pic_set_palette: class c is the grey (c, c, c)
-        uint8_t grey[768];
-        for (int c = 0; c < 256; ++c) grey[3 * c] = grey[3 * c + 1] = grey[3 * c + 2] = (uint8_t)c;
-        ce = cudaMemcpy(s->d_palette, grey, 768, cudaMemcpyHostToDevice);
+        uint32_t grey[256];
+        for (uint32_t c = 0; c < 256; ++c) grey[c] = 0x010101u * c;
+        ce = cudaMemcpy(s->d_palette, grey, sizeof(grey), cudaMemcpyHostToDevice);
     }
     if (ce == cudaSuccess) ce = cudaMemset(s->d_state, 0, sizeof(float) * 4 * n_agents);
     if (ce == cudaSuccess) ce = cudaMemset(s->d_dims, 0, sizeof(float) * 3 * n_agents);
@@ -423,7 +423,7 @@ static pic_status render_from(pic_scene* s, const float* poses, float* state, co
         CUDA_TRY(cudaMemsetAsync(P.occlusion + (size_t)s->view_first * s->A * 2, 0, sizeof(uint32_t) * 2 * (size_t)count * s->A, stream));
     const bool timed = s->timing && s->n_timed < kMaxTimed;
     if (timed) CUDA_TRY(cudaEventRecord(s->ev[2 * s->n_timed], stream));
-    if (out_rgb) CUDA_TRY(pic::launch_colour(P, count, antialias, stream));
+    if (out_rgb) CUDA_TRY(pic::launch_colour(P, count, antialias, s->sm_count, stream));
     else CUDA_TRY(pic::launch_render(P, count, s->brute, s->sm_count, stream));
     if (timed) { CUDA_TRY(cudaEventRecord(s->ev[2 * s->n_timed + 1], stream)); ++s->n_timed; }
     return PIC_OK;
@@ -441,8 +441,10 @@ pic_status pic_set_palette(pic_scene* s, const uint8_t* rgb, void* cuda_stream) 
     DeviceGuard guard(s->device);
     if (!guard.ok) return fail(PIC_ERR_CUDA, "cannot select device %d", s->device);
     cudaStream_t stream = static_cast<cudaStream_t>(cuda_stream);
-    CUDA_TRY(cudaMemcpyAsync(s->d_palette, rgb, 768, cudaMemcpyHostToDevice, stream));
-    CUDA_TRY(cudaStreamSynchronize(stream));          // the host array may be reused by the caller
+    uint32_t packed[256];
+    for (int c = 0; c < 256; ++c) packed[c] = (uint32_t)rgb[3 * c] | ((uint32_t)rgb[3 * c + 1] << 8) | ((uint32_t)rgb[3 * c + 2] << 16);
+    CUDA_TRY(cudaMemcpyAsync(s->d_palette, packed, sizeof(packed), cudaMemcpyHostToDevice, stream));
+    CUDA_TRY(cudaStreamSynchronize(stream));          // (the array above goes out of scope)
     return PIC_OK;
 }
 

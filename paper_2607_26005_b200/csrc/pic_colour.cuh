@@ -38,8 +38,6 @@ static_assert(W_SURV <= CPOOL && CPOOL <= 256, "a tile's survivors fit the pool;
 
 constexpr unsigned long long KEY_RESOLVED = 1ull << 63;     // (a key's high word is the bits of a positive float: bit 63 is free)
 
-__constant__ float FACE_SHADE[6] = {0.60f, 1.00f, 0.70f, 0.85f, 0.40f, 0.92f};   // rear, front, right, left, bottom, top
-
 struct __align__(16) ColourPool {
     float4 nx[CPOOL], ny[CPOOL], nz[CPOOL];     // edge functions E_i = nx[i] rx + ny[i] ry + nz[i]; REC_TINY: nx, ny the projected vertices
     float4 w[CPOOL];                            // 1/z plane wx, wy, wz; key low word (index, class)
@@ -278,8 +276,8 @@ __device__ __forceinline__ void shade_fragment(const ColourPool& pool, const Ren
     const float sh = pool.shade[slot];
     float k = 1.f;
     if (sh > 0.f) k = sh * (1.f - 0.5f * __fdividef(__fdividef(1.f, w) - P.near_z, P.far_z - P.near_z));
-    const uint8_t* pal = P.palette + 3u * cls;
-    r = k * (float)__ldg(pal); g = k * (float)__ldg(pal + 1); b = k * (float)__ldg(pal + 2);
+    const uint32_t pal = __ldg(P.palette + cls);
+    r = k * (float)(pal & 0xffu); g = k * (float)((pal >> 8) & 0xffu); b = k * (float)((pal >> 16) & 0xffu);
 }
 
 // Colour of a pixel with a list of partially covering fragments: front to back, the list's fragments in front of the
@@ -339,57 +337,11 @@ __device__ __forceinline__ void composite_rows(unsigned long long* key, uint16_t
                 uint32_t bgc = P.cls_sky;
                 if (ego_active && gy < P.H) bgc = __ldg(P.rig.bg_cls + (size_t)jb.k * P.H + gy);
                 unsigned long long* kp = key + key_index(x, y);
-                *kp = KEY_RESOLVED | composite_pixel(*kp, hd, frag, pool, P, (float)__ldg(P.palette + 3u * bgc), (float)__ldg(P.palette + 3u * bgc + 1),
-                                                     (float)__ldg(P.palette + 3u * bgc + 2));
+                const uint32_t bg = __ldg(P.palette + bgc);
+                *kp = KEY_RESOLVED | composite_pixel(*kp, hd, frag, pool, P, (float)(bg & 0xffu), (float)((bg >> 8) & 0xffu), (float)((bg >> 16) & 0xffu));
             }
         }
         __syncwarp();
-    }
-}
-
-// (the same with all 16 pixels of a lane unrolled and three 128-bit stores: faster where the kernel's code is small
-// enough anyway -- the plain instantiation)
-__device__ __forceinline__ void resolve_store_wide(unsigned long long* key, const ColourPool& pool, const RenderParams& P, const Job& jb,
-                                                     bool ego_active, int ys, bool vec_ok, int lane) {
-    const int y = lane >> 2, xs = (lane & 3) * 16;
-    const int gy = jb.t.y0 + ys + y;
-    uint32_t bgc = P.cls_sky;
-    if (ego_active && gy < P.H) bgc = __ldg(P.rig.bg_cls + (size_t)jb.k * P.H + gy);
-    const uint32_t bg8 = (uint32_t)__ldg(P.palette + 3u * bgc) | ((uint32_t)__ldg(P.palette + 3u * bgc + 1) << 8) | ((uint32_t)__ldg(P.palette + 3u * bgc + 2) << 16);
-    uint32_t ow[12];
-#pragma unroll
-    for (int i = 0; i < 12; ++i) ow[i] = 0u;
-#pragma unroll
-    for (int j = 0; j < 16; j += 2) {
-        ulonglong2* kp = reinterpret_cast<ulonglong2*>(key + key_index(xs + j, y));
-        const ulonglong2 kk = *kp;
-        *kp = make_ulonglong2(0ull, 0ull);
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const unsigned long long k = h ? kk.y : kk.x;
-            uint32_t c = bg8;
-            if (k & KEY_RESOLVED) c = (uint32_t)k & 0xffffffu;
-            else if (k) {
-                float R, G, B;
-                shade_fragment(pool, P, (uint32_t)k & 0xffu, __uint_as_float((uint32_t)(k >> 32)), R, G, B);
-                c = (uint32_t)fminf(R + 0.5f, 255.f) | ((uint32_t)fminf(G + 0.5f, 255.f) << 8) | ((uint32_t)fminf(B + 0.5f, 255.f) << 16);
-            }
-            const int n = 3 * (j + h);           // byte offset of the pixel in the lane's 48 bytes
-            ow[n >> 2] |= c << (8 * (n & 3));
-            if ((n & 3) > 1) ow[(n >> 2) + 1] |= c >> (8 * (4 - (n & 3)));
-        }
-    }
-    if (ys + y >= jb.t.th || xs >= jb.t.tw) return;
-    uint8_t* dst = P.out_rgb + 3u * ((jb.view * (size_t)P.H + gy) * (size_t)P.W + jb.t.x0 + xs);
-    if (vec_ok && xs + 16 <= jb.t.tw) {
-        uint4* d4 = reinterpret_cast<uint4*>(dst);
-        d4[0] = make_uint4(ow[0], ow[1], ow[2], ow[3]);
-        d4[1] = make_uint4(ow[4], ow[5], ow[6], ow[7]);
-        d4[2] = make_uint4(ow[8], ow[9], ow[10], ow[11]);
-    } else {
-#pragma unroll
-        for (int n = 0; n < 48; ++n)
-            if (n / 3 + xs < jb.t.tw) dst[n] = (uint8_t)(ow[n >> 2] >> (8 * (n & 3)));
     }
 }
 
@@ -399,7 +351,7 @@ __device__ __forceinline__ void resolve_store_colour(unsigned long long* key, co
     const int gy = jb.t.y0 + ys + y;
     uint32_t bgc = P.cls_sky;
     if (ego_active && gy < P.H) bgc = __ldg(P.rig.bg_cls + (size_t)jb.k * P.H + gy);
-    const uint32_t bg8 = (uint32_t)__ldg(P.palette + 3u * bgc) | ((uint32_t)__ldg(P.palette + 3u * bgc + 1) << 8) | ((uint32_t)__ldg(P.palette + 3u * bgc + 2) << 16);
+    const uint32_t bg8 = __ldg(P.palette + bgc);
     const bool row_ok = ys + y < jb.t.th;
     uint8_t* dst = P.out_rgb + 3u * ((jb.view * (size_t)P.H + gy) * (size_t)P.W + jb.t.x0 + xs);
     // four groups of four pixels (12 bytes, three words) each; the loop is not unrolled: one copy of the shading code
@@ -446,8 +398,13 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
     ColourSmem& s = *reinterpret_cast<ColourSmem*>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     launch_dependents();
-    const unsigned id = await_previous(blockIdx.x) * (unsigned)NW + warp;
-    const bool valid = id < P.n_jobs;
+    const unsigned cta = await_previous(blockIdx.x);
+    // antialiased: every tile; else: the tiles that the tile kernel left out, one wave of CTAs walking the list
+    const unsigned n_ids = AA ? P.n_jobs : __ldcg(&P.overflow[0]);
+#pragma unroll 1
+    for (unsigned at = cta * (unsigned)NW; at < n_ids; at += gridDim.x * (unsigned)NW) {
+    const bool valid = at + warp < n_ids;
+    const unsigned id = AA || !valid ? at + warp : __ldcg(&P.overflow[1u + at + warp]);
     const uint2* blk = P.surv + (size_t)id * SURV_STRIDE;
     int ns = -2;
     Job job;
@@ -653,13 +610,14 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
             if (col_next >= TILE) { col_next = 0; row_next = row_hi; }
             }   // (windows)
             __syncwarp();
-            if (AA) resolve_store_colour(key, s.pool, P, jb, s.active[j] != 0, ys, vec_ok, lane);
-            else resolve_store_wide(key, s.pool, P, jb, s.active[j] != 0, ys, vec_ok, lane);
+            resolve_store_colour(key, s.pool, P, jb, s.active[j] != 0, ys, vec_ok, lane);
             __syncwarp();
         }
         done |= now;
         if (done != (1u << NW) - 1u) __syncthreads();        // the pool is reused by the next round
     }
+    if (!AA) __syncthreads();
+    }   // (tiles of the list)
 }
 
 cudaError_t configure_colour_kernel() {
@@ -669,7 +627,7 @@ cudaError_t configure_colour_kernel() {
 }
 
 // Colour images of n_views views: the cull kernel (conservative pixel boxes when antialiasing), then the colour kernel.
-cudaError_t launch_colour_kernel(const RenderParams& P0, long long n_views, bool antialias, cudaStream_t stream) {
+cudaError_t launch_colour_kernel(const RenderParams& P0, long long n_views, bool antialias, int sm_count, cudaStream_t stream) {
     RenderParams P = P0;
     const long long jobs = n_views * P.tiles_x * P.tiles_y;
     if (jobs > 0x7fffffffLL || (long long)P.E * P.A * P.K > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
@@ -680,5 +638,12 @@ cudaError_t launch_colour_kernel(const RenderParams& P0, long long n_views, bool
     const unsigned grid = (unsigned)((jobs + NW - 1) / NW);
     const cudaError_t err = launch_next(antialias ? cull_kernel<NoTally, true> : cull_kernel<NoTally, false>, grid, sizeof(CullSmem), stream, P);
     if (err != cudaSuccess) return err;
-    return launch_next(antialias ? colour_kernel<true> : colour_kernel<false>, grid, sizeof(ColourSmem), stream, P);
+    if (antialias) return launch_next(colour_kernel<true>, grid, sizeof(ColourSmem), stream, P);
+    // plain colours: the tile kernel, then the tiles it left out
+    const cudaError_t terr = launch_next(P.W % 4 == 0 && (reinterpret_cast<uintptr_t>(P.out_rgb) & 3u) == 0 ? render_tile_kernel<NoTally, true, false, true>
+                                                                                                            : render_tile_kernel<NoTally, false, false, true>,
+                                         (unsigned)jobs, 0, stream, P, 32);
+    if (terr != cudaSuccess) return terr;
+    const unsigned wave = 3u * (unsigned)sm_count;
+    return launch_next(colour_kernel<false>, grid < wave ? grid : wave, sizeof(ColourSmem), stream, P);
 }

@@ -155,7 +155,7 @@ cudaError_t configure_render_kernel();            // pic_render.cu
 cudaError_t launch_render_kernel(const RenderParams& P, long long n_views, int sm_count, cudaStream_t stream);
 cudaError_t launch_coverage_kernel(const RenderParams& P, long long n_views, cudaStream_t stream);
 cudaError_t configure_colour_kernel();            // pic_colour.cuh (part of pic_render.cu)
-cudaError_t launch_colour_kernel(const RenderParams& P, long long n_views, bool antialias, cudaStream_t stream);
+cudaError_t launch_colour_kernel(const RenderParams& P, long long n_views, bool antialias, int sm_count, cudaStream_t stream);
 
 size_t max_smem_bytes() { return render_smem_bytes() > sizeof(ExhaustiveSmem) ? render_smem_bytes() : sizeof(ExhaustiveSmem); }
 
@@ -187,8 +187,8 @@ cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses
     return cudaGetLastError();
 }
 
-cudaError_t launch_colour(const RenderParams& P, long long n_views, bool antialias, cudaStream_t stream) {
-    return n_views <= 0 ? cudaSuccess : launch_colour_kernel(P, n_views, antialias, stream);
+cudaError_t launch_colour(const RenderParams& P, long long n_views, bool antialias, int sm_count, cudaStream_t stream) {
+    return n_views <= 0 ? cudaSuccess : launch_colour_kernel(P, n_views, antialias, sm_count, stream);
 }
 
 cudaError_t launch_render(const RenderParams& P, long long n_views, bool brute, int sm_count, cudaStream_t stream) {

@@ -1397,8 +1397,8 @@ cudaError_t launch_next(K kernel, unsigned grid, size_t smem, cudaStream_t strea
 }  // namespace pic
 #include "pic_coverage.cuh"
 namespace pic {
-#include "pic_colour.cuh"
 #include "pic_tile.cuh"
+#include "pic_colour.cuh"
 #include "pic_static.cuh"
 #include "pic_small.cuh"
 

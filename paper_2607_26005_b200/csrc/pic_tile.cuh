@@ -186,6 +186,57 @@ __device__ __forceinline__ void store_class_depth(const RenderParams& P, size_t 
     }
 }
 
+__constant__ float FACE_SHADE[6] = {0.60f, 1.00f, 0.70f, 0.85f, 0.40f, 0.92f};   // rear, front, right, left, bottom, top
+
+// Colour of a key's fragment: its class's, for a box face (primitives from n_map_tris on, two per face) shaded by face
+// and depth.
+__device__ __forceinline__ uint32_t key_colour(const RenderParams& P, unsigned long long key, uint32_t n_map_tris) {
+    const uint32_t pal = __ldg(P.palette + ((uint32_t)key & 0xffu)), index = 0xFFFFFFu - ((uint32_t)key >> 8);
+    if (index < n_map_tris) return pal;
+    const uint32_t face = ((index - n_map_tris) >> 1) % 6u;
+    const float k = FACE_SHADE[face] * (1.f - 0.5f * __fdividef(__fdividef(1.f, __uint_as_float((uint32_t)(key >> 32))) - P.near_z, P.far_z - P.near_z));
+    const float r = k * (float)(pal & 0xffu), g = k * (float)((pal >> 8) & 0xffu), b = k * (float)((pal >> 16) & 0xffu);
+    return (uint32_t)fminf(r + 0.5f, 255.f) | ((uint32_t)fminf(g + 0.5f, 255.f) << 8) | ((uint32_t)fminf(b + 0.5f, 255.f) << 16);
+}
+
+// The four pixels of a lane -> colour image (o: pixel offset).
+template <bool VEC>
+__device__ __forceinline__ void store_rgb(const RenderParams& P, size_t o, const unsigned long long (&best)[4], uint32_t bg, uint32_t n_map_tris, int n_px) {
+    uint32_t c[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) c[k] = best[k] ? key_colour(P, best[k], n_map_tris) : bg;
+    uint8_t* dst = P.out_rgb + 3 * o;
+    if (VEC) {
+        uint32_t* d = reinterpret_cast<uint32_t*>(dst);
+        d[0] = c[0] | (c[1] << 24); d[1] = (c[1] >> 8) | (c[2] << 16); d[2] = (c[2] >> 16) | (c[3] << 8);
+    } else {
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+            if (k < n_px) { dst[3 * k] = (uint8_t)c[k]; dst[3 * k + 1] = (uint8_t)(c[k] >> 8); dst[3 * k + 2] = (uint8_t)(c[k] >> 16); }
+    }
+}
+
+// store_background for colours.
+__device__ __forceinline__ void store_background_rgb(const RenderParams& P, size_t tile0, const TileCtx& t, bool ego_active, const uint32_t* bg_cls, uint32_t busy, int lane) {
+    const bool wide = (P.W & 15) == 0 && (reinterpret_cast<uintptr_t>(P.out_rgb) & 15u) == 0;
+    const int x = wide ? (lane & 3) * 16 : (lane & 15) * 4, dy = wide ? 8 : 2;
+    if (x >= t.tw) return;
+    const uint32_t my_col = busy >> (x / CELL_W), sky = __ldg(P.palette + P.cls_sky);
+    for (uint32_t y = wide ? lane >> 2 : lane >> 4; y < (uint32_t)t.th; y += dy) {
+        if ((my_col >> ((y >> 2) * 2)) & 1u) continue;
+        const uint32_t c = ego_active ? __ldg(P.palette + __ldg(bg_cls + y)) : sky;
+        const uint32_t w0 = c | (c << 24), w1 = (c >> 8) | (c << 16), w2 = (c >> 16) | (c << 8);
+        uint8_t* dst = P.out_rgb + 3 * (tile0 + (size_t)(y * P.W + x));
+        if (wide) {
+            uint4* d = reinterpret_cast<uint4*>(dst);
+            d[0] = make_uint4(w0, w1, w2, w0); d[1] = make_uint4(w1, w2, w0, w1); d[2] = make_uint4(w2, w0, w1, w2);
+        } else {
+            uint32_t* d = reinterpret_cast<uint32_t*>(dst);
+            d[0] = w0; d[1] = w1; d[2] = w2;
+        }
+    }
+}
+
 // Background of the cells not in `busy`: 16 pixels per lane where rows allow it (128-bit class, two 128-bit depth stores), else 4.
 __device__ __forceinline__ void store_background(const RenderParams& P, size_t tile0, const TileCtx& t, bool ego_active, const uint2* bg_fill, uint32_t busy, int lane) {
     const bool wide = (P.W & 15) == 0;                       // (then tiles are whole 16-pixel segments wide)
@@ -211,8 +262,9 @@ __device__ __forceinline__ void store_background(const RenderParams& P, size_t t
     }
 }
 
-// VEC: rows of a multiple of four pixels and no float32 depth image.  OCC: with occlusion counts.
-template <class TL, bool VEC, bool OCC>
+// VEC: rows of a multiple of four pixels and no float32 depth image.  OCC: with occlusion counts.  RGB: colours instead of
+// classes and depths.
+template <class TL, bool VEC, bool OCC, bool RGB = false>
 __global__ void __launch_bounds__(32, PIC_TILE_CTAS) render_tile_kernel(const __grid_constant__ RenderParams P) {
     __shared__ TileWarp s;
     const int lane = threadIdx.x;
@@ -344,7 +396,8 @@ __global__ void __launch_bounds__(32, PIC_TILE_CTAS) render_tile_kernel(const __
         busy |= __reduce_or_sync(0xffffffffu, fc);
     }
     // ---- the background of the other cells
-    if (VEC) store_background(P, tile0, t, ego_active, P.rig.bg_fill + (size_t)job.k * P.H + t.y0, busy, lane);
+    if (VEC && RGB) store_background_rgb(P, tile0, t, ego_active, bg_cls, busy, lane);
+    else if (VEC) store_background(P, tile0, t, ego_active, P.rig.bg_fill + (size_t)job.k * P.H + t.y0, busy, lane);
     else busy = 0xffffffffu;
     // ---- cell after cell
     const int px = (lane & 7) * 4, py = lane >> 3;
@@ -382,8 +435,10 @@ __global__ void __launch_bounds__(32, PIC_TILE_CTAS) render_tile_kernel(const __
         if (n_px > 0) {
             uint32_t bc = P.cls_sky;
             float bz = P.far_z;
-            if (ego_active) { bc = __ldg(bg_cls + y); bz = __ldg(bg_z + y); }
-            store_class_depth<VEC>(P, tile0 + (size_t)(y * P.W + x), best, bc, bz, n_px);
+            if (ego_active) { bc = __ldg(bg_cls + y); if (!RGB) bz = __ldg(bg_z + y); }
+            const size_t o = tile0 + (size_t)(y * P.W + x);
+            if (RGB) store_rgb<VEC>(P, o, best, __ldg(P.palette + bc), n_map_tris, n_px);
+            else store_class_depth<VEC>(P, o, best, bc, bz, n_px);
         }
     }
     flush_counters(P, n);
