@@ -114,9 +114,8 @@ __device__ __noinline__ void flush_pending(const unsigned long long* key, unsign
         uint32_t a14 = 0u;
         float wc = 0.f;
         const uint32_t pix = item >> 8, slot = item & 0xffu;
-        float area = 0.f;
+        float area = 0.f, w = 0.f;
         float e[CLINES], a[CLINES], b[CLINES];
-        float w = 0.f;
 #pragma unroll
         for (int j = 0; j < CLINES; ++j) { e[j] = 1.f; a[j] = 0.f; b[j] = 0.f; }
         if (have) {
@@ -127,8 +126,8 @@ __device__ __noinline__ void flush_pending(const unsigned long long* key, unsign
             for (int j = 0; j < 4; ++j) { e[j] = fm(nx[j], rx, fm(ny[j], ry, nz[j])); a[j] = nx[j] * du; b[j] = ny[j] * dv; }
             w = fm(r3.x, rx, fm(r3.y, ry, r3.z));
             e[4] = w - w_far; e[5] = w_near - w; a[4] = r3.x * du; b[4] = r3.y * dv; a[5] = -a[4]; b[5] = -b[4];
-            area = pixel_coverage<CLINES>(e, a, b);
         }
+        area = have ? pixel_coverage<CLINES>(e, a, b) : 0.f;
         if (have) {
             a14 = min((uint32_t)(area * 16383.f + 0.5f), COVERAGE_MAX);
             wc = fminf(fmaxf(w, w_far), w_near);
@@ -323,26 +322,41 @@ __device__ __forceinline__ uint32_t composite_pixel(unsigned long long k, uint32
 // so that a row crowded with fragments (the horizon) is shared by all lanes; their colour replaces the pixel's key
 // (composite_rows).  At the end every lane converts 16 consecutive pixels of a row, resets what it reads, and stores
 // (resolve_store_colour).
-__device__ __forceinline__ void composite_rows(unsigned long long* key, uint16_t* head, const unsigned long long* frag,
+__device__ __forceinline__ void composite_rows(unsigned long long* key, uint16_t* head, unsigned long long* frag, int n_frag,
                                                const ColourPool& pool, const RenderParams& P, const Job& jb, bool ego_active,
                                                int ys, int row_lo, int row_hi, int lane) {
-    {
+    // the pixels that have a list, packed (few of a strip's pixels have one): at the end of the fragment array, or, when the
+    // lists reach there, not at all
+    uint16_t* list = reinterpret_cast<uint16_t*>(frag + (CFRAGS + 1 - CSTRIP_KEYS / 4));
+    const bool pack = n_frag < CFRAGS + 1 - CSTRIP_KEYS / 4;
+    int count = (row_hi - row_lo) * TILE;
+    if (pack) {
+        count = 0;
 #pragma unroll 1
         for (int i = row_lo * (TILE / 32); i < row_hi * (TILE / 32); ++i) {
-            const int p = i * 32 + lane, x = p & (TILE - 1), y = p >> 6;
-            const uint32_t hd = head[p];
-            if (hd) {
-                head[p] = 0;
-                const int gy = jb.t.y0 + ys + y;
-                uint32_t bgc = P.cls_sky;
-                if (ego_active && gy < P.H) bgc = __ldg(P.rig.bg_cls + (size_t)jb.k * P.H + gy);
-                unsigned long long* kp = key + key_index(x, y);
-                const uint32_t bg = __ldg(P.palette + bgc);
-                *kp = KEY_RESOLVED | composite_pixel(*kp, hd, frag, pool, P, (float)(bg & 0xffu), (float)((bg >> 8) & 0xffu), (float)((bg >> 16) & 0xffu));
-            }
+            const int p = i * 32 + lane;
+            const bool any = head[p] != 0;
+            const unsigned m = __ballot_sync(0xffffffffu, any);
+            if (any) list[count + __popc(m & ((1u << lane) - 1u))] = (uint16_t)p;
+            count += __popc(m);
         }
         __syncwarp();
     }
+#pragma unroll 1
+    for (int i = lane; i < count; i += 32) {
+        const int p = pack ? (int)list[i] : row_lo * TILE + i, x = p & (TILE - 1), y = p >> 6;
+        const uint32_t hd = head[p];
+        if (hd) {
+            head[p] = 0;
+            const int gy = jb.t.y0 + ys + y;
+            uint32_t bgc = P.cls_sky;
+            if (ego_active && gy < P.H) bgc = __ldg(P.rig.bg_cls + (size_t)jb.k * P.H + gy);
+            unsigned long long* kp = key + key_index(x, y);
+            const uint32_t bg = __ldg(P.palette + bgc);
+            *kp = KEY_RESOLVED | composite_pixel(*kp, hd, frag, pool, P, (float)(bg & 0xffu), (float)((bg >> 8) & 0xffu), (float)((bg >> 16) & 0xffu));
+        }
+    }
+    __syncwarp();
 }
 
 __device__ __forceinline__ void resolve_store_colour(unsigned long long* key, const ColourPool& pool, const RenderParams& P, const Job& jb,
@@ -415,7 +429,8 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
         n_map_tris = __ldg(&P.env_maps[job.e].n_tris);
         const bool ego_active = __ldg(&P.agents[(size_t)job.e * P.A + job.a].active) != 0u;
         RayView rv = {s.ray_x[warp], s.ray_y[warp]};
-        load_rays(rv, P, job, lane); load_rays(rv, P, job, lane + 32);
+#pragma unroll 1
+        for (int i = lane; i < TILE; i += 32) load_rays(rv, P, job, i);
         if (lane == 0) {
             load_camera(s.cam[warp], P.cams[job.view], P.cam[job.k], P.W, P.H);
             s.job[warp] = job;
@@ -580,9 +595,26 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
 #pragma unroll
                     for (int e = 0; e < 4; ++e) hh[e] = 0.5f * (fabsf(q.nx[e]) * du + fabsf(q.ny[e]) * dv);
                     hh[4] = hh[5] = 0.5f * (fabsf(q.wx) * du + fabsf(q.wy) * dv);
-                    for (int yy = ly0 & ~3; yy <= ly1; yy += 4)
-                        for (int xx = bx0 & ~15; xx <= bx1; xx += 16)
+                    // a lane per 16 x 4 cell of the strip: does a line keep the record out of all of its pixels?  A line's
+                    // values at the cell's pixel centres lie within +-h of its value at the cell's centre, h widened by
+                    // several times what float32 can lose; a pixel is touched while the value at its centre is above -hh
+                    const int xa = (lane & 3) * 16, ya = ((lane >> 2) & 1) * 4;
+                    bool out = lane >= 8 || xa + 15 < bx0 || xa > bx1 || ya + 3 < ly0 || ya > ly1;
+                    if (AA) {
+                        const float rxc = 0.5f * (ray_x[xa] + ray_x[xa + 15]), ryc = 0.5f * (ray_y[ya] + ray_y[ya + 3]);
+                        const float hx = 8.001f * du + 1e-6f * fabsf(rxc), hy = 2.001f * dv + 1e-6f * fabsf(ryc);   // from the cell's centre to its pixels' far sides
+#pragma unroll
+                        for (int e = 0; e < 5; ++e) {
+                            const float a = e < 4 ? q.nx[e] : q.wx, b = e < 4 ? q.ny[e] : q.wy, z = e < 4 ? q.nz[e] : q.wz;
+                            const float c = fm(a, rxc, fm(b, ryc, z)), h = fm(fabsf(a), hx, fm(fabsf(b), hy, 1e-6f * fabsf(z)));
+                            out = out || (e < 4 ? c + h < 0.f : c + h < P.w_far || c - h > P.w_near);
+                        }
+                    }
+#pragma unroll 1
+                    for (unsigned cells = __ballot_sync(0xffffffffu, !out); cells; cells &= cells - 1) {
+                            const int cell = __ffs(cells) - 1, xx = (cell & 3) * 16, yy = (cell >> 2) * 4;
                             colour_cell<AA>(key, head, frag, n_frag, n_pend, dropped, ray_x, ray_y, q, thr, hh, du, dv, key_lo, slot, P.w_near, P.w_far, xx, yy, row_lo, row_hi, col_lo, col_hi, lane);
+                    }
                     // the queue is worked off when it holds a few rounds' worth (working it off frees room only for the
                     // pixels whose area turns out to be zero, so a nearly full array is no reason to do it earlier)
                     if (AA && n_pend >= 96) {
@@ -605,7 +637,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
                 continue;
             }
             if (AA && dropped && lane == 0) atomicOr(P.status, STATUS_COLOUR_FRAGMENTS);   // (more than 1 023 in front of the opaque surface of one pixel)
-            if (AA) composite_rows(key, head, frag, s.pool, P, jb, s.active[j] != 0, ys, row_lo, row_hi, lane);
+            if (AA) composite_rows(key, head, frag, n_frag, s.pool, P, jb, s.active[j] != 0, ys, row_lo, row_hi, lane);
             col_next += cw;
             if (col_next >= TILE) { col_next = 0; row_next = row_hi; }
             }   // (windows)

@@ -84,3 +84,32 @@ def test_calls_with_few_tiles(n_tris, E, A, H, W, K, spread):
 ])
 def test_calls_with_many_tiles(n_tris, E, A, H, W, K, spread):
     test_calls_with_few_tiles(n_tris, E, A, H, W, K, spread)
+
+
+@pytest.mark.parametrize("side", [15.0, 15.5, 16.0, 40.0])      # pixels: boxes of 16 x 16 and 17 x 17, around the limit of 256, and a large one
+@pytest.mark.parametrize("far", [100.0, 10.3])                  # wholly in the depth range, cut by the far plane
+def test_antialiased_primitives_around_the_size_limit(side, far):
+    import oracle
+    from scenes import default_palette
+    from tests.gpu_util import CudaRun
+    from tests.test_gpu_colour import compare_colour
+    H, W = 70, 100
+    rig = make_rig((0.0,), 90.0, 80.0, W, H, mount=(0.0, 0.0, 1.5))
+    z, fx = 10.0, rig[0, 5]
+    tris = []
+    for k, (u, v, tilt) in enumerate([(-30.3, -20.2, 0.0), (12.6, -18.4, 0.5), (-9.7, 5.1, 1.0), (30.2, 12.4, 0.3)]):   # tilted squares, pixels off the axis
+        h = 0.5 * side * z / fx
+        c, y0, z0 = np.array([z, 0.0, 1.5]), -u * z / fx, -v * z / fx
+        corners = [c + np.array([tilt * a, y0 + a, z0 + b]) for a, b in ((-h, -h), (h, -h), (h, h), (-h, h))]
+        tris += [[corners[0], corners[1], corners[2]], [corners[0], corners[2], corners[3]]]
+    s = custom_scene(np.asarray(tris, np.float32), np.repeat([2, 3, 4, 5], 2).astype(np.uint8), np.zeros((1, 1, 3), np.float32),
+                     np.array([[CAR]], np.float32), rig, H, W, far=far)
+    pal = default_palette()
+    g = CudaRun(s)
+    try:
+        got, flags = g.render_rgb(pal, True)
+    finally:
+        g.close()
+    ref = oracle.render_rgb(s, pal, True)
+    assert flags == 0
+    compare_colour(ref, got)
