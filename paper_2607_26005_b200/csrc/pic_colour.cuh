@@ -668,7 +668,7 @@ cudaError_t launch_colour_kernel(const RenderParams& P0, long long n_views, bool
     P.debug_flags = 0;
     P.counters = nullptr;
     const unsigned grid = (unsigned)((jobs + NW - 1) / NW);
-    const cudaError_t err = launch_next(antialias ? cull_kernel<NoTally, true> : cull_kernel<NoTally, false>, grid, sizeof(CullSmem), stream, P);
+    const cudaError_t err = launch_cull(P, n_views, antialias, sm_count, stream);
     if (err != cudaSuccess) return err;
     if (antialias) return launch_next(colour_kernel<true>, grid, sizeof(ColourSmem), stream, P);
     // plain colours: the tile kernel, then the tiles it left out

@@ -38,15 +38,6 @@
 
 namespace pic {
 
-// Profiling aid, compiled in only with -DPIC_PROFILE (never in the shipped library): bits 4-7 of the
-// debug flags leave work out so that the cost of a phase can be timed by difference.  The images
-// are then incomplete.
-#ifdef PIC_PROFILE
-#define PIC_STOP(P) (((P).debug_flags >> 4) & 15)
-#else
-#define PIC_STOP(P) 0
-#endif
-
 constexpr int NTHREADS = 128;
 constexpr int NW = NTHREADS / 32;
 constexpr int RCAP = 64;          // records (primitives rasterized by a warp) per tile
@@ -436,9 +427,6 @@ __device__ __forceinline__ void store_tile(S& s, const TileCtx& t, const RenderP
                     if ((j & 3) == 0) cw[j >> 2] = c0 | (c1 << 8); else cw[j >> 2] |= (c0 << 16) | (c1 << 24);
                 }
             }
-#ifdef PIC_PROFILE
-            if (PIC_STOP(P) == 6 && !(P.debug_flags & 0x10000)) continue;
-#endif
             *reinterpret_cast<uint4*>(oc + o) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
             if (FULL) {
                 store_256(od + o, dw);
@@ -506,7 +494,6 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool classify = !(P.debug_flags & 1);
     const int rec_cap = (P.debug_flags & 2) ? 2 : RCAP;
-    const int stop = PIC_STOP(P);
     const int k = job.k, a = job.a, e = job.e;
     const size_t view = job.view;
     const TileCtx t = job.t;
@@ -537,7 +524,7 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
         reinterpret_cast<ulonglong2*>(s.key)[i * NT + threadIdx.x] = make_ulonglong2(0ull, 0ull);
     __syncthreads();
 
-    if (ego_active && stop != 1) {
+    if (ego_active) {
         const Cam& c = s.cam;
         const uint32_t n_groups = mi.group_end - mi.group_begin;
         const int n_rounds = max((int)((n_groups + GROUP_BATCH - 1) / GROUP_BATCH), (P.A + BOX_ROUND - 1) / BOX_ROUND);
@@ -579,7 +566,7 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
             __syncthreads();
             // ---- phase 2a (a): one thread per candidate: camera space, pixel box; survivors are compacted
             const int nl = s.n_leaf, nf = s.n_face;
-            const int n_items = (stop == 2) ? 0 : nl * LEAF_PRIMS + nf;
+            const int n_items = nl * LEAF_PRIMS + nf;
             for (int i0 = 0; i0 < n_items; i0 += NT) {
                 const int i = i0 + threadIdx.x;
                 V3 V[4], Pn;
@@ -604,7 +591,7 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
             }
             __syncthreads();
             // ---- phase 2b (c): one thread per survivor: edge functions, 1/z plane, tiny raster or record
-            const int ns = (stop == 3) ? 0 : min(s.n_surv, SCAP);
+            const int ns = min(s.n_surv, SCAP);
             for (int j = threadIdx.x; j < ns; j += NT) {
                 const uint2 sv = s.surv[j];
                 V3 V[4], Pn;
@@ -623,8 +610,7 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
             }
         }
         // ---- phase 3 (b)+(c): one warp per record
-        if (stop == 0 || stop > 5) raster_records<NT / 32>(s, s.rec, s.touched, t, min(s.n_rec, rec_cap), classify, n);
-        if (stop == 5 && threadIdx.x == 0) { s.touched[0] = 0xffffffffu; s.touched[1] = 0xffffffffu; }
+        raster_records<NT / 32>(s, s.rec, s.touched, t, min(s.n_rec, rec_cap), classify, n);
         __syncthreads();
     }
     // ---- phase 4 (d)
@@ -728,6 +714,63 @@ __device__ __forceinline__ void append_survivor(uint2* __restrict__ surv, bool k
     const unsigned m = __ballot_sync(0xffffffffu, keep);
     if (keep) { const int slot = n + __popc(m & ((1u << lane) - 1u)); if (slot < W_SURV) surv[slot] = make_uint2(id, box); }
     n += __popc(m);
+}
+
+// Pixel box of camera-space vertices in a whole image, inclusive; false: no pixel centre (margin m) can be touched.  Where
+// pixel_box gives up because a vertex lies behind or close to the camera, the primitive is cut at the near depth -- nothing
+// nearer is kept -- and what remains is projected, so that a road under the camera reaches only the tiles it is seen in.
+__device__ __forceinline__ bool view_box(const Cam& c, const TileCtx& t, const V3 (&V)[4], int& bx0, int& by0, int& bx1, int& by1, float m) {
+    bool ok = pixel_box_int(c, t, V, bx0, by0, bx1, by1, m);
+    if (ok && fminf(fminf(V[0].z, V[1].z), fminf(V[2].z, V[3].z)) < t.near_z * ZPROJ_FRAC) {
+        const float zc = t.near_z * 0.999f;
+        float sx0 = 3e38f, sx1 = -3e38f, sy0 = 3e38f, sy1 = -3e38f;
+        auto include = [&](float x, float y, float iz) {
+            const float sx = fm(c.focx, mul(x, iz), c.cx), sy = fm(c.focy, mul(y, iz), c.cy);
+            sx0 = fminf(sx0, sx); sx1 = fmaxf(sx1, sx); sy0 = fminf(sy0, sy); sy1 = fmaxf(sy1, sy);
+        };
+        const float izc = __fdividef(1.f, zc);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const V3 a = V[i], b = V[(i + 1) & 3];
+            if (a.z >= zc) include(a.x, a.y, __fdividef(1.f, a.z));
+            if ((a.z < zc) != (b.z < zc)) {
+                const float u = __fdividef(zc - a.z, b.z - a.z);
+                include(fm(u, b.x - a.x, a.x), fm(u, b.y - a.y, a.y), izc);
+            }
+        }
+        const float mm = m + 0.25f;                          // (the cut of an edge of some hundred metres is good to a tenth of a pixel)
+        const float fx0 = fmaxf(ceilf(sx0 - 0.5f - mm), 0.f), fx1 = fminf(floorf(sx1 - 0.5f + mm), (float)(t.tw - 1));
+        const float fy0 = fmaxf(ceilf(sy0 - 0.5f - mm), 0.f), fy1 = fminf(floorf(sy1 - 0.5f + mm), (float)(t.th - 1));
+        ok = fx0 <= fx1 && fy0 <= fy1;
+        bx0 = (int)fx0; by0 = (int)fy0; bx1 = (int)fx1; by1 = (int)fy1;
+    }
+    return ok;
+}
+
+// Bit per tile (row-major, at most 32 per view) reached by a pixel box of the image.
+__device__ __forceinline__ uint32_t box_tiles(const RenderParams& P, int bx0, int by0, int bx1, int by1) {
+    const uint32_t cols = (uint32_t)((2ull << (bx1 / TILE)) - (1ull << (bx0 / TILE)));
+    uint32_t tiles = 0u;
+    for (int ty = by0 / TILE; ty <= by1 / TILE; ++ty) tiles |= cols << (ty * P.tiles_x);
+    return tiles;
+}
+
+// Appends each lane's survivor to the lists of the tiles it reaches, with its box cut to the tile.  Lane l keeps the count of tile l.
+__device__ __forceinline__ void deal_survivors(uint2* __restrict__ surv, const RenderParams& P, uint32_t tiles, uint32_t id, int bx0, int by0, int bx1, int by1,
+                                               int& n, int lane) {
+#pragma unroll 1
+    for (uint32_t any = __reduce_or_sync(0xffffffffu, tiles); any; any &= any - 1) {
+        const int tile = __ffs(any) - 1;
+        const bool in = (tiles >> tile) & 1u;
+        const unsigned m = __ballot_sync(0xffffffffu, in);
+        const int slot = __shfl_sync(0xffffffffu, n, tile) + __popc(m & ((1u << lane) - 1u));
+        if (in && slot < W_SURV) {
+            const int ty = (int)divide((unsigned)tile, P.div_tiles_x), x0 = (tile - ty * P.tiles_x) * TILE, y0 = ty * TILE;
+            const uint32_t box = (uint32_t)max(bx0 - x0, 0) | ((uint32_t)max(by0 - y0, 0) << 8) | ((uint32_t)min(bx1 - x0, TILE - 1) << 16) | ((uint32_t)min(by1 - y0, TILE - 1) << 24);
+            surv[(size_t)tile * SURV_STRIDE + slot] = make_uint2(id, box);
+        }
+        if (lane == tile) n += __popc(m);
+    }
 }
 
 // Camera, frustum planes and footprint of a tile, by one warp.  The footprint is the convex hull of the apex and the
@@ -845,10 +888,13 @@ __device__ __forceinline__ bool bound_visible(const Cam& c, const TileCtx& t, co
 //
 // Bound by the issue of dependent instructions at 24-32 resident warps: the full test costs some 230 instructions and 64
 // bytes a candidate, the bound's some 60 and 16, and four candidates in five die by it.
-template <class TL, bool CONS>
+//
+// MULTI: the same for all tiles of a view at once (job.t is the whole image): the survivors' pixel boxes are dealt out to the
+// lists of the tiles they reach.  A view of several tiles then pays once for its frustum, grid rows, leaves, agents and
+// candidates, instead of once per tile.
+template <class TL, bool CONS, bool MULTI>
 __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ surv, const RenderParams& P, const Job& job,
                                           const MapInfo& mi, int lane, TL& n) {
-    const int stop = PIC_STOP(P);
     // CONS: conservative pixel boxes -- every pixel whose unit square a primitive touches (antialiased output)
     constexpr float BOX_MARGIN = CONS ? 0.50390625f : 0.00390625f;
     const TileCtx& t = job.t;
@@ -863,7 +909,6 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
     Frustum& fr = f.f;
     if (lane == 0) f.n_item = 0;
     frustum_setup(fr, P, job, lane);
-    if (stop == 11) return 0;
     const Cam& c = fr.cam;
     // ---- the grid rows crossed by the widened footprint; the first 32 rows' ranges are requested now, the boxes below
     // are tested while the loads are under way
@@ -911,7 +956,6 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
     __syncwarp();
     int n_item = f.n_item;
     if (n_item > W_ITEM) return -1;
-    if (stop == 12) return 0;
     int n_surv = 0;
     // ---- fill the item list with the candidates of the grid rows (32 rows per pass), test the items, until both are done
     int row = rows.lo, i0 = 0, total = -1;         // total < 0: the ranges of the pass have not been laid out
@@ -967,10 +1011,10 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
             if (i0 >= total) { row += 32; total = -1; more = row <= rows.hi; }
         }
         __syncwarp();
-        if (stop == 13) return 0;
 #pragma unroll 1
         for (int i = lane; i - lane < n_item; i += 32) {
-            uint32_t box = 0, id = 0;
+            uint32_t box = 0, id = 0, tiles = 0;                // tiles: bit per tile of the view that the box reaches
+            int bx0 = 0, by0 = 0, bx1 = -1, by1 = -1;
             bool keep = false;
             if (i < n_item) {
                 id = f.item[i];
@@ -988,15 +1032,19 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
                     for (int q = 0; q < 4; ++q) V[q] = to_camera(c, v[3 * q], v[3 * q + 1], v[3 * q + 2]);
                 }
                 ++n.tested;
-                keep = pixel_box(c, t, V, box, BOX_MARGIN);
+                if (MULTI) {
+                    if (view_box(c, t, V, bx0, by0, bx1, by1, BOX_MARGIN)) tiles = box_tiles(P, bx0, by0, bx1, by1);
+                } else {
+                    keep = pixel_box(c, t, V, box, BOX_MARGIN);
+                }
             }
-            append_survivor(surv, keep, id, box, n_surv, lane);
+            if (MULTI) deal_survivors(surv, P, tiles, id, bx0, by0, bx1, by1, n_surv, lane);
+            else append_survivor(surv, keep, id, box, n_surv, lane);
         }
         __syncwarp();
         n_item = 0;
     } while (more);
-    if (stop == 14) return 0;
-    return n_surv > W_SURV ? -1 : n_surv;
+    return n_surv > W_SURV ? -1 : n_surv;        // (MULTI: of the tile of this lane)
 }
 
 // Survivor `id` in camera space with its plane normal.
@@ -1045,27 +1093,29 @@ struct __align__(16) CullSmem {
 #ifndef PIC_TILE_CTAS
 #define PIC_TILE_CTAS 24
 #endif
-template <class TL, bool CONS>
+// MULTI: a warp per view of several tiles (P.n_jobs counts tiles all the same).
+template <class TL, bool CONS, bool MULTI = false>
 __global__ void __launch_bounds__(NTHREADS, PIC_CULL_CTAS) cull_kernel(const __grid_constant__ RenderParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     CullSmem& s = *reinterpret_cast<CullSmem*>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int stop = PIC_STOP(P);
     const unsigned cta = await_previous(blockIdx.x);
-    const unsigned id = cta * (unsigned)NW + warp;
+    const int tiles = MULTI ? P.tiles_x * P.tiles_y : 1;
+    const unsigned id = (cta * (unsigned)NW + warp) * (unsigned)tiles;
     if (id >= P.n_jobs) return;
     TL n = {};
-    const Job job = decode_job(P, id);
+    Job job = decode_job(P, id);
+    if (MULTI) { job.t.tw = P.W; job.t.th = P.H; }
     const MapInfo mi = P.env_maps[job.e];
     const bool ego_active = P.agents[(size_t)job.e * P.A + job.a].active != 0;
     uint2* blk = P.surv + (size_t)id * SURV_STRIDE;
     int ns = 0;
     if (P.debug_flags & 4) ns = -1;             // test aid: every tile through cooperative_job
-    else if (ego_active && stop != 1 && !(stop >= 8 && stop <= 10)) ns = front_cull<TL, CONS>(s.lists[warp], blk + 2, P, job, mi, lane, n);
+    else if (ego_active) ns = front_cull<TL, CONS, MULTI>(s.lists[warp], blk + 2, P, job, mi, lane, n);
     // (the work counts are summed over the warp's lanes; without counters they are constants)
     const uint32_t c_grp = __reduce_add_sync(0xffffffffu, (uint32_t)tally_value(n.grp)), c_leaf = __reduce_add_sync(0xffffffffu, (uint32_t)tally_value(n.leaf)),
                    c_tested = __reduce_add_sync(0xffffffffu, (uint32_t)tally_value(n.tested));
-    if (lane == 0) *reinterpret_cast<uint4*>(blk) = make_uint4((uint32_t)ns, c_grp, c_leaf, c_tested);
+    if (lane < tiles) *reinterpret_cast<uint4*>(blk + (size_t)lane * SURV_STRIDE) = make_uint4((uint32_t)ns, c_grp, c_leaf, c_tested);
     // (only now: blocks of the next kernel that came in earlier would crowd the multiprocessors that still have room
     // instead of spreading over all of them)
     launch_dependents();
@@ -1139,7 +1189,7 @@ __device__ __forceinline__ void strip_cell(unsigned long long* key, const float*
 // the records that reach it, cell by cell.  Returns the touched 8 x 8 blocks.
 template <int ROWS, int N>
 __device__ __forceinline__ uint32_t raster_strip(StripView& s, const RecordPool<N>& pool, int first, int n_rec, int ys, float w_near,
-                                                      float w_far, int stop, int lane) {
+                                                      float w_far, int lane) {
     uint32_t touched = 0u;                       // bit (row >> 3) * 8 + (column >> 3)
     const int kbase = (lane >> 3) << 6, lsw = (lane & 7) ^ (((lane >> 3) & 1) << 2);   // see strip_cell
     for (int base = 0; base < n_rec; base += 32) {
@@ -1159,7 +1209,7 @@ __device__ __forceinline__ uint32_t raster_strip(StripView& s, const RecordPool<
                 read_record(pool, slot, q, key_lo);
                 q.tl = (bw_lane >> 24) & 15u;
                 // at most TINY_MAX_PIXELS pixels: one column (w == 1), two columns, or one row
-                const int w = bx1 - bx0 + 1, npx = (stop == 7) ? 0 : w * (y1 - y0 + 1);
+                const int w = bx1 - bx0 + 1, npx = w * (y1 - y0 + 1);
                 bool any = false;
 #pragma unroll
                 for (int px = 0; px < TINY_MAX_PIXELS; ++px) {
@@ -1174,7 +1224,6 @@ __device__ __forceinline__ uint32_t raster_strip(StripView& s, const RecordPool<
         }
         __syncwarp();
         unsigned hits = __ballot_sync(0xffffffffu, hit);
-        if (!(stop == 0 || stop == 2 || stop == 3 || stop > 5)) hits = 0u;
         for (; hits; hits &= hits - 1) {
             const int src = __ffs(hits) - 1;
             const uint32_t bw = __shfl_sync(0xffffffffu, bw_lane, src);
@@ -1188,7 +1237,7 @@ __device__ __forceinline__ uint32_t raster_strip(StripView& s, const RecordPool<
             float thr[4];
             edge_thresholds(q.tl, thr);
             const bool range = !(bw & REC_INRANGE);
-            if (stop != 3 && (bx1 - bx0 + 1) * (ly1 - ly0 + 1) >= CLASSIFY_MIN_STRIP * ROWS / 16) {
+            if ((bx1 - bx0 + 1) * (ly1 - ly0 + 1) >= CLASSIFY_MIN_STRIP * ROWS / 16) {
                 // a lane per 16 x 4 pixel cell of the strip classifies it: reject / partly covered / inside
                 const int xa = (lane & 3) * 16, xb = xa + 15, ya = ((lane >> 2) & 3) * 4, yb = ya + 3;
                 bool reject = lane >= ROWS || xb < bx0 || xa > bx1 || yb < ly0 || ya > ly1;
@@ -1215,13 +1264,13 @@ __device__ __forceinline__ uint32_t raster_strip(StripView& s, const RecordPool<
                     const int cell = __ffs(m) - 1;
                     const int xx = (cell & 3) * 16, yy = (cell >> 2) * 4;
                     const uint32_t need_c = __shfl_sync(0xffffffffu, need, cell);
-                    if (stop != 2 && stop != 3) strip_cell(s.key, s.ray_x, s.ray_y, q, thr, key_lo, w_near, w_far, xx, yy, need_c, true, kbase, lsw, lane);
+                    strip_cell(s.key, s.ray_x, s.ray_y, q, thr, key_lo, w_near, w_far, xx, yy, need_c, true, kbase, lsw, lane);
                     touched |= 3u << ((yy >> 3) * 8 + (xx >> 3));
                 }
             } else {
                 for (int yy = ly0 & ~3; yy <= ly1; yy += 4)
                     for (int xx = bx0 & ~15; xx <= bx1; xx += 16)
-                        if (stop != 2 && stop != 3) strip_cell(s.key, s.ray_x, s.ray_y, q, thr, key_lo, w_near, w_far, xx, yy, 0xFu, range, kbase, lsw, lane);
+                        strip_cell(s.key, s.ray_x, s.ray_y, q, thr, key_lo, w_near, w_far, xx, yy, 0xFu, range, kbase, lsw, lane);
                 touched |= (uint32_t)block_mask(bx0, ly0, bx1, ly1);
             }
         }
@@ -1381,10 +1430,23 @@ static cudaError_t run_coverage(const RenderParams& P, long long n_views, cudaSt
     return cudaGetLastError();
 }
 
+// The cull pass of a call.  Views of several tiles are culled a warp per view while that leaves enough warps to hide the
+// latency of each: measured, the two ways meet at about 600 views of 8 tiles (city) and 1 400 of 2 tiles (96 x 54); at 4 096
+// views of 8 tiles the call takes 653 instead of 1 008 us.
+template <class K>
+cudaError_t launch_next(K kernel, unsigned grid, size_t smem, cudaStream_t stream, const RenderParams& P, unsigned threads = NTHREADS);
+static cudaError_t launch_cull(const RenderParams& P, long long n_views, bool conservative, int sm_count, cudaStream_t stream) {
+    const int tiles = P.tiles_x * P.tiles_y;
+    if (!P.counters && !(P.debug_flags & 4) && tiles > 1 && tiles <= 32 && n_views >= (tiles > 2 ? 4 : 10) * (long long)sm_count)
+        return launch_next(conservative ? cull_kernel<NoTally, true, true> : cull_kernel<NoTally, false, true>, (unsigned)((n_views + NW - 1) / NW), sizeof(CullSmem), stream, P);
+    const unsigned grid = (P.n_jobs + NW - 1) / NW;
+    return launch_next(P.counters ? cull_kernel<Tally, false> : conservative ? cull_kernel<NoTally, true> : cull_kernel<NoTally, false>, grid, sizeof(CullSmem), stream, P);
+}
+
 // Launches the next kernel of a call: its blocks may be brought in while the last blocks of the kernel before it still
 // run (it waits for that kernel itself, see await_previous).
 template <class K>
-cudaError_t launch_next(K kernel, unsigned grid, size_t smem, cudaStream_t stream, const RenderParams& P, unsigned threads = NTHREADS) {
+cudaError_t launch_next(K kernel, unsigned grid, size_t smem, cudaStream_t stream, const RenderParams& P, unsigned threads) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid); cfg.blockDim = dim3(threads); cfg.dynamicSmemBytes = smem; cfg.stream = stream;
     cudaLaunchAttribute attr;
@@ -1412,14 +1474,13 @@ cudaError_t launch_render_kernel(const RenderParams& P0, long long n_views, int 
     if (jobs <= 0) return cudaSuccess;
     P.n_jobs = (uint32_t)jobs;
     P.far_z2 = 0x10001u * (uint32_t)__half_as_ushort(__float2half_rn(P.far_z));
-    const unsigned grid = (unsigned)((jobs + NW - 1) / NW);
     // few tiles: one CTA takes a tile from culling to store.  Measured (a call on 16 agents per environment, both image
     // shapes of the workloads): 64 tiles 37.0 -> 20.7 us, 256 tiles 44.6 -> 22.7, 768 tiles 47.3 -> 44.8, 1024 tiles
     // 48.4 -> 53.7, so the line lies at five tiles per multiprocessor.
     if (jobs <= 5LL * sm_count && !P.counters && !P.occlusion && (P.debug_flags & 15) == 0)
         return launch_next(render_small_kernel, (unsigned)jobs, SMALL_SMEM, stream, P, SMALL_THREADS);
     // (a) cull: survivors per tile
-    cudaError_t err = launch_next(P.counters ? cull_kernel<Tally, false> : cull_kernel<NoTally, false>, grid, sizeof(CullSmem), stream, P);
+    cudaError_t err = launch_cull(P, n_views, false, sm_count, stream);
     if (err != cudaSuccess) return err;
     // (b)-(d) set-up, raster, store
     const bool vec = P.W % 4 == 0 && !P.out_depth32;

@@ -149,7 +149,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 2) render_small_kernel(const __
     StripView sv;
     sv.key = s.key + ys * TILE; sv.ray_x = s.ray_x; sv.ray_y = s.ray_y + ys;
     uint32_t touched = 0u;
-    if (ego_active) touched = raster_strip<SMALL_STRIP>(sv, s.pool, 0, s.n_rec, ys, P.w_near, P.w_far, 0, lane);
+    if (ego_active) touched = raster_strip<SMALL_STRIP>(sv, s.pool, 0, s.n_rec, ys, P.w_near, P.w_far, lane);
     __syncwarp();
     TileCtx ts = t;
     ts.y0 = t.y0 + ys; ts.th = min(SMALL_STRIP, t.th - ys);
