@@ -113,3 +113,29 @@ def test_antialiased_primitives_around_the_size_limit(side, far):
     ref = oracle.render_rgb(s, pal, True)
     assert flags == 0
     compare_colour(ref, got)
+
+
+@pytest.mark.parametrize("n_tris,E,A,H,W,K,spread", [
+    (300, 4, 50, 65, 129, 4, 60.0),       # 800 views of 6 tiles, the last row and column of one pixel: culled a warp per view
+    (300, 8, 50, 64, 70, 4, 60.0),        # 1 600 views of 2 tiles
+    (40, 2, 75, 30, 1990, 4, 6.0),        # the most tiles a view can have there (32), large primitives under the cameras
+    (2000, 4, 38, 130, 80, 4, 10.0),      # tiles whose survivor lists overflow
+])
+def test_views_of_several_tiles(n_tris, E, A, H, W, K, spread):
+    test_calls_with_few_tiles(n_tris, E, A, H, W, K, spread)
+
+
+@pytest.mark.parametrize("E,A", [(1, 2), (37, 12), (38, 12)])       # 4 tiles per view: one per CTA up to 1 776 tiles (148 multiprocessors), else four
+def test_antialiased_calls_with_few_and_many_tiles(E, A):
+    from scenes import default_palette
+    from tests.gpu_util import CudaRun
+    s = soup(A, 80, E, A, 70, 100, K=1, spread=40.0)
+    g = CudaRun(s)
+    try:
+        pal = default_palette()
+        whole, flags = g.render_rgb(pal, True)
+        part, _ = g.render_rgb(pal, True, view_first=E * A - 2, view_count=2)        # the same views in a call of few tiles
+        assert flags == 0
+        assert (np.abs(whole[-2:].astype(int) - part[-2:].astype(int)) <= 1).all()
+    finally:
+        g.close()
