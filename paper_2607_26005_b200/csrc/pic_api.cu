@@ -25,6 +25,8 @@ namespace {
 
 constexpr float kDt = 0.1f, kWheelbase = 2.8f, kVMax = 30.0f;
 constexpr int kMaxTimed = 1024;
+constexpr int kMaxHostChunks = 8;              // pic_render_host: most parts in which images are rendered and copied back,
+constexpr size_t kHostChunkBytes = 6u << 20;   //   and about the least size of a part
 
 thread_local char g_err[512] = "";
 
@@ -92,6 +94,8 @@ struct pic_scene {
     uint8_t* d_in_active = nullptr;
     uint8_t* d_out_class = nullptr;
     uint16_t* d_out_depth = nullptr;
+    cudaStream_t copy_stream = nullptr;                 // images go back on it while the next views are rendered
+    cudaEvent_t copy_ev[kMaxHostChunks] = {};
     // options
     bool brute = false;
     float* depth32 = nullptr;
@@ -123,6 +127,9 @@ void free_scene(pic_scene* s) {
     cudaFree(s->d_agents); cudaFree(s->d_cams); cudaFree(s->d_overflow); cudaFree(s->d_surv); cudaFree(s->d_tables); cudaFree(s->d_state); cudaFree(s->d_dims); cudaFree(s->d_active); cudaFree(s->d_agent_cls); cudaFree(s->d_status); cudaFree(s->d_palette);
     cudaFree(s->d_in_poses); cudaFree(s->d_in_dims); cudaFree(s->d_in_active); cudaFree(s->d_out_class);
     cudaFree(s->d_out_depth);
+    if (s->copy_stream) cudaStreamDestroy(s->copy_stream);
+    for (cudaEvent_t e : s->copy_ev)
+        if (e) cudaEventDestroy(e);
     if (s->ev) {
         for (int i = 0; i < 2 * kMaxTimed; ++i) if (s->ev[i]) cudaEventDestroy(s->ev[i]);
         delete[] s->ev;
@@ -396,7 +403,7 @@ pic_status pic_scene_set_option(pic_scene* s, int32_t option, uint64_t value) {
 
 static pic_status render_from(pic_scene* s, const float* poses, float* state, const float* actions, const float* dims,
                               const uint8_t* active, const pic_camera* rig, uint8_t* out_class, uint16_t* out_depth,
-                              cudaStream_t stream, uint8_t* out_rgb = nullptr, bool antialias = false) {
+                              cudaStream_t stream, uint8_t* out_rgb = nullptr, bool antialias = false, int chunks = 1) {
     pic::RenderParams P;
     pic_status st = fill_params(s, rig, out_class, out_depth, P, out_rgb != nullptr);
     if (st != PIC_OK) return st;
@@ -424,7 +431,16 @@ static pic_status render_from(pic_scene* s, const float* poses, float* state, co
     const bool timed = s->timing && s->n_timed < kMaxTimed;
     if (timed) CUDA_TRY(cudaEventRecord(s->ev[2 * s->n_timed], stream));
     if (out_rgb) CUDA_TRY(pic::launch_colour(P, count, antialias, s->sm_count, stream));
-    else CUDA_TRY(pic::launch_render(P, count, s->brute, s->sm_count, stream));
+    else {
+        // (chunks > 1: pic_render_host; an event after each part of the views)
+        for (int c = 0; c < chunks; ++c) {
+            const long long v0 = count * c / chunks, v1 = count * (c + 1) / chunks;
+            if (c > 0) CUDA_TRY(cudaMemsetAsync(P.overflow, 0, sizeof(uint32_t), stream));   // the list of left-out tiles starts empty again
+            P.view_first = s->view_first + v0;
+            CUDA_TRY(pic::launch_render(P, v1 - v0, s->brute, s->sm_count, stream));
+            if (chunks > 1) CUDA_TRY(cudaEventRecord(s->copy_ev[c], stream));
+        }
+    }
     if (timed) { CUDA_TRY(cudaEventRecord(s->ev[2 * s->n_timed + 1], stream)); ++s->n_timed; }
     return PIC_OK;
 }
@@ -470,16 +486,32 @@ pic_status pic_render_host(pic_scene* s, const float* poses, const float* dims, 
         CUDA_TRY(cudaMalloc((void**)&s->d_in_dims, sizeof(float) * 3 * n_agents));
         CUDA_TRY(cudaMalloc((void**)&s->d_in_active, n_agents));
         CUDA_TRY(cudaMalloc((void**)&s->d_out_depth, sizeof(uint16_t) * n_px));
+        if (!s->copy_stream) CUDA_TRY(cudaStreamCreateWithFlags(&s->copy_stream, cudaStreamNonBlocking));
+        for (cudaEvent_t& e : s->copy_ev)
+            if (!e) CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         CUDA_TRY(cudaMalloc((void**)&s->d_out_class, n_px));
     }
     CUDA_TRY(cudaMemcpyAsync(s->d_in_poses, poses, sizeof(float) * 3 * n_agents, cudaMemcpyHostToDevice, stream));
     CUDA_TRY(cudaMemcpyAsync(s->d_in_dims, dims, sizeof(float) * 3 * n_agents, cudaMemcpyHostToDevice, stream));
     if (active) CUDA_TRY(cudaMemcpyAsync(s->d_in_active, active, n_agents, cudaMemcpyHostToDevice, stream));
+    // The images go back in parts while the next views are rendered, so the call takes as long as the copies and the first
+    // part's render; parts of less than some megabytes would cost more in launches than they hide.
+    const long long n_views = (long long)n_agents * s->K;
+    const size_t per_view = (size_t)s->H * s->W, parts = 3 * n_px / kHostChunkBytes;
+    const bool whole = s->view_first == 0 && (s->view_count <= 0 || s->view_count >= n_views) && !s->occlusion && !s->counters;
+    int chunks = whole ? (int)(parts < (size_t)kMaxHostChunks ? parts : (size_t)kMaxHostChunks) : 1;
+    if (chunks < 1 || n_views < chunks) chunks = 1;
     pic_status st = render_from(s, s->d_in_poses, nullptr, nullptr, s->d_in_dims, active ? s->d_in_active : nullptr, rig,
-                                s->d_out_class, s->d_out_depth, stream);
+                                s->d_out_class, s->d_out_depth, stream, nullptr, false, chunks);
     if (st != PIC_OK) return st;
-    CUDA_TRY(cudaMemcpyAsync(out_class, s->d_out_class, n_px, cudaMemcpyDeviceToHost, stream));
-    CUDA_TRY(cudaMemcpyAsync(out_depth, s->d_out_depth, sizeof(uint16_t) * n_px, cudaMemcpyDeviceToHost, stream));
+    for (int c = 0; c < chunks; ++c) {
+        const size_t p0 = (size_t)(n_views * c / chunks) * per_view, p1 = (size_t)(n_views * (c + 1) / chunks) * per_view;
+        const cudaStream_t to = chunks > 1 ? s->copy_stream : stream;
+        if (chunks > 1) CUDA_TRY(cudaStreamWaitEvent(to, s->copy_ev[c], 0));
+        CUDA_TRY(cudaMemcpyAsync(out_class + p0, s->d_out_class + p0, p1 - p0, cudaMemcpyDeviceToHost, to));
+        CUDA_TRY(cudaMemcpyAsync(out_depth + p0, s->d_out_depth + p0, sizeof(uint16_t) * (p1 - p0), cudaMemcpyDeviceToHost, to));
+    }
+    if (chunks > 1) CUDA_TRY(cudaStreamSynchronize(s->copy_stream));
     CUDA_TRY(cudaStreamSynchronize(stream));
     return PIC_OK;
 }

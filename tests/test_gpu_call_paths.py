@@ -139,3 +139,19 @@ def test_antialiased_calls_with_few_and_many_tiles(E, A):
         assert (np.abs(whole[-2:].astype(int) - part[-2:].astype(int)) <= 1).all()
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("E,A,H,W", [(1, 5, 40, 40), (1, 11, 500, 384), (2, 24, 250, 300)])    # one part, two parts of an odd number of views, five parts
+def test_host_images_in_parts(E, A, H, W):
+    from tests.gpu_util import CudaRun
+    s = soup(E * A, 200, E, A, H, W, K=3, spread=30.0)
+    g = CudaRun(s)
+    try:
+        want = g.render(depth32=False)
+        for _ in range(2):
+            cls, dep = np.full((E, A, 3, H, W), 255, np.uint8), np.full((E, A, 3, H, W), -1, np.float16)
+            g.scene.render_host(np.ascontiguousarray(s.poses), np.ascontiguousarray(s.dims), s.rig, cls, dep)
+            assert (cls.reshape(want[0].shape) == want[0]).all()
+            assert (dep.reshape(want[1].shape).view(np.uint16) == want[1].view(np.uint16)).all()
+    finally:
+        g.close()
