@@ -40,7 +40,7 @@ if ROOT not in sys.path:
 CFG = 2                       # scene of the stepping workload
 ALU_LANES_PER_SM = 128        # FP32 lanes per SM
 FALLBACK_HBM_GBS = 6650.0
-KERNELS_PER_CALL = 5          # rig, agent, cull, render, cooperative
+KERNELS_PER_CALL = 4          # set-up, cull, tile, cooperative
 
 
 def _affinity_cores() -> int:
@@ -421,7 +421,7 @@ def run_cuda(args, rank: int, world: int, local_rank: int) -> None:
             # kernel_ms: the library's event pair around the render kernels of a call (cull_kernel, the render
             # kernel, and the cooperative kernel for tiles whose lists overflow), i.e. all the render work of a step;
             # their shares are in profiles/
-            "kernel": "cull_kernel + " + ("render_kernel" if paper else "render_full_kernel") + " (+ cooperative_kernel)",
+            "kernel": "cull_kernel + render_tile_kernel (+ cooperative_kernel)",
             "kernel_ms": k_ms, "kernel_ms_series": _series(kt), "kernel_launches_timed": int(len(kt)),
             "algorithmic_bytes": alg_bytes, "t_hbm_ms": 1e3 * t_hbm, "t_alu_ms": 1e3 * t_alu,
             "alg_lane_ops_per_view": float(n_alg_view), "write_only_fill_gbs": fill_gbs,
@@ -447,7 +447,7 @@ def run_cuda(args, rank: int, world: int, local_rank: int) -> None:
             "clocks": clocks,
             "e2e": {"value": e2e_value, "unit": "agent-steps/s", "h2d_bytes_per_step": 25 * s.E * s.A,
                     "d2h_bytes_per_step": 3 * px, "steps": n_e2e, "entry": "pic_render_host, pinned host buffers"},
-            "gpu_launches": KERNELS_PER_CALL * args.steps,   # rig, agent, cull, render and cooperative kernels per step
+            "gpu_launches": KERNELS_PER_CALL * args.steps,   # set-up, cull, tile and cooperative kernels per step
             "roofline": roof,
             "roofline_static": roof_static,
             "cpu_baseline": {"value": cpu_value, "unit": "agent-steps/s", "cores": min(cores, 64), "kind": "oracle",
