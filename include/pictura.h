@@ -197,7 +197,7 @@ pic_status pic_get_status(pic_scene* scene, uint32_t* flags, void* cuda_stream);
  *                         accept/reject; bit 1: shrink the fused kernel's record pool and the
  *                         cooperative kernel's record list to 2 entries so that the overflow paths
  *                         run; bit 2: send every tile to the cooperative kernel; bit 3: shrink the
- *                         record pool to 40 so that both kernels share the tiles.  All leave the
+ *                         record lists to 6 entries so that both kernels share the tiles.  All leave the
  *                         images unchanged (tests rely on it); other bits are ignored.
  *   PIC_OPT_TIMING        1: bracket the render kernels of every call with CUDA events on its stream
  *                         (up to 1024 launches between two pic_get_kernel_times calls); 0: off.

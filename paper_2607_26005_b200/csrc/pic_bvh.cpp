@@ -19,6 +19,9 @@
 #include <cmath>
 #include <cstdio>
 #include <cstring>
+#include <exception>
+#include <system_error>
+#include <thread>
 #include <vector>
 
 #include "pic_types.h"
@@ -212,13 +215,18 @@ void build_grid(HostHierarchy& h, MapInfo& mi) {
 
 }  // namespace
 
-HostHierarchy* build_hierarchy(int num_maps, const int64_t* tri_offset, const float* tri_xyz,
-                               const uint8_t* tri_class, const float* tri_vis_cos, int agents_per_env, char* err, int err_len) {
+namespace {
+
+// The hierarchy of maps m0 .. m1 - 1, with offsets that count from 0.
+HostHierarchy* build_maps(int m0, int m1, const int64_t* tri_offset, const float* tri_xyz,
+                          const uint8_t* tri_class, const float* tri_vis_cos, int agents_per_env, char* err, int err_len) {
     HostHierarchy* h = new HostHierarchy();
-    h->maps.resize(num_maps);
+    h->maps.resize(m1 - m0);
+    const size_t n_most = (size_t)(tri_offset[m1] - tri_offset[m0]);
+    h->prims.reserve(n_most / 2); h->grid_prims.reserve(n_most / 2); h->grid_bounds.reserve(n_most / 2);
     std::vector<Prim> local;
     std::vector<Item> items;
-    for (int m = 0; m < num_maps; ++m) {
+    for (int m = m0; m < m1; ++m) {
         int64_t t0 = tri_offset[m], t1 = tri_offset[m + 1];
         int64_t n = t1 - t0;
         if (n + 12LL * agents_per_env > (1LL << 24)) {
@@ -287,7 +295,7 @@ HostHierarchy* build_hierarchy(int num_maps, const int64_t* tri_offset, const fl
             return a.code != b.code ? a.code < b.code : a.id < b.id;
         });
         // ---- leaves
-        MapInfo& mi = h->maps[m];
+        MapInfo& mi = h->maps[m - m0];
         std::memset(&mi, 0, sizeof(mi));
         mi.n_tris = (uint32_t)n;
         mi.prim_begin = (uint32_t)h->prims.size();
@@ -338,6 +346,68 @@ HostHierarchy* build_hierarchy(int num_maps, const int64_t* tri_offset, const fl
             return nullptr;
         }
     }
+    return h;
+}
+
+template <class T>
+void append(std::vector<T>& to, const std::vector<T>& from) { to.insert(to.end(), from.begin(), from.end()); }
+
+// Appends the maps of `b` to `h`.
+void append_maps(HostHierarchy& h, HostHierarchy& b) {
+    const uint32_t prim0 = (uint32_t)h.prims.size(), leaf0 = (uint32_t)h.leaves.size(), group0 = (uint32_t)h.groups.size(),
+                   cell0 = (uint32_t)h.cell_start.size(), grid0 = (uint32_t)h.grid_prims.size(), large0 = (uint32_t)h.large_leaves.size();
+    for (MapInfo& mi : b.maps) {
+        mi.prim_begin += prim0; mi.prim_end += prim0; mi.group_begin += group0; mi.group_end += group0;
+        mi.cell_begin += cell0; mi.large_begin += large0; mi.large_end += large0;
+    }
+    for (Node& n : b.leaves) n.first += prim0;
+    for (Node& n : b.groups) n.first += leaf0;
+    for (Node& n : b.large_leaves) n.first += grid0;
+    for (uint32_t& c : b.cell_start) c += grid0;
+    append(h.maps, b.maps); append(h.prims, b.prims); append(h.leaves, b.leaves); append(h.groups, b.groups);
+    append(h.cell_start, b.cell_start); append(h.grid_prims, b.grid_prims); append(h.grid_bounds, b.grid_bounds); append(h.large_leaves, b.large_leaves);
+}
+
+}  // namespace
+
+// Maps are independent: from eight maps of some size on, runs of them are built by up to eight threads and joined in order
+// (the result does not depend on the number of threads).
+HostHierarchy* build_hierarchy(int num_maps, const int64_t* tri_offset, const float* tri_xyz,
+                               const uint8_t* tri_class, const float* tri_vis_cos, int agents_per_env, char* err, int err_len) {
+    const int n_threads = (int)std::min<int64_t>({8, (int64_t)std::max(1u, std::thread::hardware_concurrency()), num_maps / 4, tri_offset[num_maps] / 8192});
+    if (n_threads < 2) return build_maps(0, num_maps, tri_offset, tri_xyz, tri_class, tri_vis_cos, agents_per_env, err, err_len);
+    std::vector<HostHierarchy*> part(n_threads, nullptr);
+    std::vector<std::vector<char>> errs(n_threads, std::vector<char>(256, 0));
+    auto work = [&](int t) {
+        try {
+            part[t] = build_maps((int)((int64_t)num_maps * t / n_threads), (int)((int64_t)num_maps * (t + 1) / n_threads), tri_offset, tri_xyz, tri_class, tri_vis_cos,
+                                 agents_per_env, errs[t].data(), 256);
+        } catch (const std::exception&) {
+            std::snprintf(errs[t].data(), 256, "host allocation failed");
+        }
+    };
+    std::vector<std::thread> threads;
+    for (int t = 1; t < n_threads; ++t) {
+        try { threads.emplace_back(work, t); } catch (const std::system_error&) { work(t); }      // (no thread to be had)
+    }
+    work(0);
+    for (std::thread& t : threads) t.join();
+    HostHierarchy* h = part[0];
+    for (int t = 0; t < n_threads; ++t)
+        if (!part[t]) {
+            std::snprintf(err, err_len, "%s", errs[t].data());
+            for (HostHierarchy* p : part) delete p;
+            return nullptr;
+        }
+    size_t n_prims = 0;
+    for (HostHierarchy* p : part) n_prims += p->prims.size();
+    if (n_prims >= (1ull << 28)) {
+        std::snprintf(err, err_len, "more than 2^28 primitives in one scene");
+        for (HostHierarchy* p : part) delete p;
+        return nullptr;
+    }
+    h->prims.reserve(n_prims); h->grid_prims.reserve(n_prims); h->grid_bounds.reserve(n_prims);
+    for (int t = 1; t < n_threads; ++t) { append_maps(*h, *part[t]); delete part[t]; }
     return h;
 }
 

@@ -27,10 +27,8 @@ constexpr int CSTRIP = 8;                       // pixel rows of a strip
 constexpr int CSTRIPS = TILE / CSTRIP;
 constexpr int CSTRIP_KEYS = TILE * CSTRIP;
 constexpr int CPOOL = 254;                      // records shared by the four tiles (a tile's survivors always fit: W_SURV < CPOOL)
-#ifndef PIC_COLOUR_SMALL
-#define PIC_COLOUR_SMALL 256
-#endif
-constexpr int COLOUR_SMALL = PIC_COLOUR_SMALL;  // pixels in the conservative box of a primitive that is worked off pixel by pixel (at most 511 in a strip)
+constexpr int COLOUR_SMALL = 256;               // pixels in the conservative box of a primitive that is worked off pixel by pixel (at most 511 in a
+                                                // strip; paper chunk / step at 216 x 384: 64 1 120 / 315 us, 128 1 109 / 296, 256 1 112 / 298, 512 1 130 / 306)
 constexpr int CFRAGS = 1023;                    // partially covering fragments of a strip (10-bit links, 0 ends a list)
 constexpr uint32_t STATUS_COLOUR_INCOMPLETE = 2u;   // = PIC_FLAG_COLOUR_INCOMPLETE of the public header
 constexpr uint32_t STATUS_COLOUR_FRAGMENTS = 4u;    // = PIC_FLAG_COLOUR_FRAGMENTS

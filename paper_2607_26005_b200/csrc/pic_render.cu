@@ -76,13 +76,6 @@ __device__ __forceinline__ int key_index(int x, int y) {
     return (y << 6) | (((c ^ (((y & 1) << 2) | (c >> 3))) << 1) | (x & 1));
 }
 
-// 256-bit store (sm_100): a lane's 16 depth values land in one fully written 32-byte sector.
-__device__ __forceinline__ void store_256(void* p, const uint32_t (&w)[8]) {
-    asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(p), "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]),
-                 "r"(w[4]), "r"(w[5]), "r"(w[6]), "r"(w[7])
-                 : "memory");
-}
-
 // Bit mask of the 8x8 blocks touched by a pixel box (inclusive).
 __device__ __forceinline__ unsigned long long block_mask(int bx0, int by0, int bx1, int by1) {
     const int c0 = bx0 >> 3, c1 = bx1 >> 3, r0 = by0 >> 3, r1 = by1 >> 3;
@@ -269,7 +262,7 @@ __device__ __forceinline__ void edge_thresholds(uint32_t tl, float (&thr)[4]) {
 }
 
 // One 16 x 4 cell at (xx, yy): every lane tests its two pixels and updates their keys with plain
-// loads and stores -- the rows of a cell belong to exactly one warp (its strip in the fused kernel,
+// loads and stores -- the rows of a cell belong to exactly one warp (its strip in render_small_kernel,
 // its bands in the cooperative kernel).  `need`: the edges
 // that still have to be tested on this cell (0: the cell is known to be covered and in depth
 // range; the range test rides on the edge tests).  Returns whether any lane produced a fragment.
@@ -377,32 +370,30 @@ __device__ __forceinline__ void raster_records(S& s, const float4* rec, uint32_t
 
 // (d) keys -> class / depth images.  `touched`: the 8x8 blocks that may hold a fragment; with
 // `clear`, the keys that were read are reset to "no fragment" for the next tile.
-// FULL: the caller guarantees full tiles of an image whose rows allow 128-bit stores and no float32
-// depth image, so that only the vector path is compiled in.
-template <bool FULL = false, class S>
+template <class S>
 __device__ __forceinline__ void store_tile(S& s, const TileCtx& t, const RenderParams& P, size_t view, int k, bool ego_active,
                                            unsigned long long touched, bool clear, int tid = threadIdx.x, int nthr = NTHREADS,
                                            uint32_t n_map_tris = 0u) {
     const size_t img = (size_t)P.H * P.W;
-    uint32_t* occ = (!FULL && P.occlusion) ? P.occlusion + view * (size_t)P.A * 2u : nullptr;   // visible-pixel counts of this view
+    uint32_t* occ = P.occlusion ? P.occlusion + view * (size_t)P.A * 2u : nullptr;   // visible-pixel counts of this view
     uint8_t* oc = P.out_class + view * img;
     uint16_t* od = P.out_depth + view * img;
     float* o32 = P.out_depth32 ? P.out_depth32 + view * img : nullptr;
     // (pic_render_static takes outputs of any alignment)
-    const bool vec_ok = FULL || ((P.W % 16 == 0) && o32 == nullptr && ((reinterpret_cast<uintptr_t>(P.out_class) | reinterpret_cast<uintptr_t>(P.out_depth)) & 15u) == 0);
-    const int segs_per_row = FULL ? TILE / 16 : (t.tw + 15) >> 4;
+    const bool vec_ok = (P.W % 16 == 0) && o32 == nullptr && ((reinterpret_cast<uintptr_t>(P.out_class) | reinterpret_cast<uintptr_t>(P.out_depth)) & 15u) == 0;
+    const int segs_per_row = (t.tw + 15) >> 4;
     const int n_seg = t.th * segs_per_row;
     // consecutive threads take consecutive 16-pixel segments of a row, then the next row: a warp's
     // class stores cover 512 contiguous bytes of a 64-pixel-wide image, its depth stores 1 KB
     for (int seg = tid; seg < n_seg; seg += nthr) {
-        const int y = FULL ? seg >> 2 : seg / segs_per_row;
+        const int y = seg / segs_per_row;
         const int xs = (seg - y * segs_per_row) * 16;
         uint32_t bg_cls = P.cls_sky;
         float bg_z = P.far_z;
         if (ego_active) { bg_cls = __ldg(P.rig.bg_cls + (size_t)k * P.H + t.y0 + y); bg_z = __ldg(P.rig.bg_z + (size_t)k * P.H + t.y0 + y); }
         const size_t o = (size_t)(t.y0 + y) * P.W + t.x0 + xs;
         const bool empty = ((touched >> ((y >> 3) * 8 + (xs >> 3))) & 3ull) == 0ull;   // both blocks of the segment
-        if (FULL || (vec_ok && xs + 16 <= t.tw)) {
+        if (vec_ok && xs + 16 <= t.tw) {
             uint32_t cw[4], dw[8];
             if (empty) {
                 const uint32_t c4 = bg_cls * 0x01010101u;
@@ -428,12 +419,8 @@ __device__ __forceinline__ void store_tile(S& s, const TileCtx& t, const RenderP
                 }
             }
             *reinterpret_cast<uint4*>(oc + o) = make_uint4(cw[0], cw[1], cw[2], cw[3]);
-            if (FULL) {
-                store_256(od + o, dw);
-            } else {
-                *reinterpret_cast<uint4*>(od + o) = make_uint4(dw[0], dw[1], dw[2], dw[3]);
-                *reinterpret_cast<uint4*>(od + o + 8) = make_uint4(dw[4], dw[5], dw[6], dw[7]);
-            }
+            *reinterpret_cast<uint4*>(od + o) = make_uint4(dw[0], dw[1], dw[2], dw[3]);
+            *reinterpret_cast<uint4*>(od + o + 8) = make_uint4(dw[4], dw[5], dw[6], dw[7]);
         } else {
             for (int j = 0; j < 16 && xs + j < t.tw; ++j) {
                 const unsigned long long key = empty ? 0ull : s.key[key_index(xs + j, y)];
@@ -488,7 +475,7 @@ __device__ __forceinline__ void load_rays(S& s, const RenderParams& P, const Job
 
 // A whole tile rendered by the CTA in barrier-separated phases with per-round lists: any number of
 // groups, boxes, survivors and records.  It serves the tiles that a render kernel's lists cannot hold.
-template <class TL, bool FULL, int NT>
+template <class TL, int NT>
 __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams& P, unsigned job_id, TL& n) {
     const Job job = decode_job(P, job_id);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -614,7 +601,7 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
         __syncthreads();
     }
     // ---- phase 4 (d)
-    store_tile<FULL>(s, t, P, view, k, ego_active, ((unsigned long long)s.touched[1] << 32) | s.touched[0], false, threadIdx.x, NT, mi.n_tris);
+    store_tile(s, t, P, view, k, ego_active, ((unsigned long long)s.touched[1] << 32) | s.touched[0], false, threadIdx.x, NT, mi.n_tris);
     if (threadIdx.x == 0) { ++n.jobs; ++n.coop; }
 }
 
@@ -1084,18 +1071,10 @@ struct __align__(16) CullSmem {
     FrontLists lists[NW];
 };
 
-#ifndef PIC_CULL_CTAS
-#define PIC_CULL_CTAS 6
-#endif
-#ifndef PIC_SMALL_PIXELS
-#define PIC_SMALL_PIXELS 16
-#endif
-#ifndef PIC_TILE_CTAS
-#define PIC_TILE_CTAS 24
-#endif
+constexpr int CULL_CTAS = 7;       // CTAs per multiprocessor the cull kernel's registers are bounded for (rollout 256x32x4: 5 256, 6 249.9, 7 247.1, 8 246.1 us; city: 661, 658, 656, 660)
 // MULTI: a warp per view of several tiles (P.n_jobs counts tiles all the same).
 template <class TL, bool CONS, bool MULTI = false>
-__global__ void __launch_bounds__(NTHREADS, PIC_CULL_CTAS) cull_kernel(const __grid_constant__ RenderParams P) {
+__global__ void __launch_bounds__(NTHREADS, CULL_CTAS) cull_kernel(const __grid_constant__ RenderParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     CullSmem& s = *reinterpret_cast<CullSmem*>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -1281,7 +1260,7 @@ __device__ __forceinline__ uint32_t raster_strip(StripView& s, const RecordPool<
 
 // The tiles the render kernels left out, a CTA at a time.  (Called from the end of those kernels instead, the same code
 // costs them 2 % -- a call bounds their registers -- which is more than a launch that overlaps their last blocks.)
-template <class TL, bool FULL>
+template <class TL>
 __global__ void __launch_bounds__(NTHREADS, 5) cooperative_kernel(const __grid_constant__ RenderParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TileSmem& cs = *reinterpret_cast<TileSmem*>(smem_raw);
@@ -1289,7 +1268,7 @@ __global__ void __launch_bounds__(NTHREADS, 5) cooperative_kernel(const __grid_c
     TL n = {};
     const unsigned count = __ldcg(&P.overflow[0]);
     for (unsigned i = cta; i < count; i += gridDim.x) {
-        cooperative_job<TL, FULL, NTHREADS>(cs, P, __ldcg(&P.overflow[1u + i]), n);
+        cooperative_job<TL, NTHREADS>(cs, P, __ldcg(&P.overflow[1u + i]), n);
         __syncthreads();
     }
     flush_counters(P, n);
@@ -1300,9 +1279,9 @@ cudaError_t configure_small_kernel();
 cudaError_t configure_render_kernel() {
     cudaError_t err = configure_small_kernel();
     if (err != cudaSuccess) return err;
-    err = cudaFuncSetAttribute(cooperative_kernel<NoTally, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem));
+    err = cudaFuncSetAttribute(cooperative_kernel<NoTally>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem));
     if (err != cudaSuccess) return err;
-    return cudaFuncSetAttribute(cooperative_kernel<Tally, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem));
+    return cudaFuncSetAttribute(cooperative_kernel<Tally>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(TileSmem));
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1492,7 +1471,7 @@ cudaError_t launch_render_kernel(const RenderParams& P0, long long n_views, int 
     // the tiles left out (their number is only known on the device): one wave of CTAs walks the list
     const long long wave = (long long)sm_count * 5;
     const unsigned cgrid = (unsigned)(jobs < wave ? jobs : wave);
-    err = launch_next(P.counters ? cooperative_kernel<Tally, false> : cooperative_kernel<NoTally, false>, cgrid, sizeof(TileSmem), stream, P);
+    err = launch_next(P.counters ? cooperative_kernel<Tally> : cooperative_kernel<NoTally>, cgrid, sizeof(TileSmem), stream, P);
     if (err != cudaSuccess || !P.occlusion) return err;
     return run_coverage(P, n_views, stream);
 }

@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 2) render_small_kernel(const __
         if (fits) fits = s.n_rec <= SMALL_POOL;
         if (!fits) {
             __syncthreads();                         // (the job takes over the CTA's shared memory)
-            cooperative_job<NoTally, false, SMALL_THREADS>(*reinterpret_cast<TileSmem*>(smem_raw), P, id, n);
+            cooperative_job<NoTally, SMALL_THREADS>(*reinterpret_cast<TileSmem*>(smem_raw), P, id, n);
             return;
         }
     }

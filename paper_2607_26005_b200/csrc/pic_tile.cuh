@@ -3,25 +3,26 @@
 //
 // Bound by instruction issue (the images of a step are a seventh of the time at the copy bandwidth), so the split is
 // chosen to execute little per pixel.
-//   set-up    a lane per survivor.  Primitives of at most 4 pixel centres are evaluated at once and leave fragments (pixel,
-//             key); the others leave a record (edge functions, 1/z plane) in shared memory -- on the benchmark workload 16
-//             and 11 per tile.
+//   set-up    a lane per survivor.  The pixels of primitives of at most 16 pixel centres are evaluated at once, a lane each
+//             whatever the primitive, and leave fragments (pixel, key); the other primitives leave a record (edge functions,
+//             1/z plane) -- on the benchmark workload 20 primitives, 33 fragments and 7 records per tile.
 //   classify  a tile is 32 cells of 32 x 4 pixels, one per lane: for every record each lane decides whether its cell is
-//             outside, partly inside or inside, from the float32 edge functions at the cell's corners (fma is monotone in
-//             each argument, so the decision is exact).  The result is two bit masks over the records per lane.
-//   raster    cell after cell, four adjacent pixels per lane: the records of the cell's mask in turn, keeping the
-//             largest key per pixel in registers; then the cell's fragments; then conversion and store.  A pixel's key
-//             never passes through memory, background cells cost little more than their stores, and the warps share
-//             nothing, so no barrier holds one back.
-// Against the kernel it replaced (four tiles per CTA, keys of 16-row strips in shared memory, records looked at per
-// strip): see the figures at launch_render_kernel.
+//             outside, partly inside or inside (14 cells hold anything, 28 pairs of record and cell meet, 20 of them partly).
+//   raster    cell after cell, four adjacent pixels per lane: the cell's fragments meet in shared memory, then the records of
+//             the cell's mask in turn, keeping the largest key per pixel in registers; then conversion and store.  A
+//             pixel's key passes through memory only where a cell has fragments, background cells cost their stores, and
+//             the warps share nothing, so no barrier holds one back.
+// Against the kernel it replaced (four tiles per CTA, keys of 16-row strips in shared memory, records looked at once per
+// strip), a step of 65 536 agents x 4 cameras at 64 x 64: 6.2 k instead of 8.0 k warp instructions per tile, 2 430 instead of
+// 3 103 us per call.  24 warps per multiprocessor (72 registers): 20 take 3 % longer, 28 1 %.
 //
 // A tile with more records or fragments than fit is left to the cooperative kernel.
 #pragma once
 
 constexpr int TREC = 32;                     // records of a tile: a 32-bit mask
 constexpr int TFRAG = 256;                   // fragments of its small primitives
-constexpr int SMALL_PIXELS = PIC_SMALL_PIXELS;   // pixel centres in the box of a small primitive (at most 32)
+constexpr int SMALL_PIXELS = 16;             // pixel centres in the box of a small primitive (4, 8, 24, 32: within 2 %)
+constexpr int TILE_CTAS = 24;                // warps per multiprocessor the registers are bounded for
 constexpr int CELL_W = 32, CELL_H = 4;       // pixels of a cell
 static_assert((TILE / CELL_W) * (TILE / CELL_H) == 32, "a lane per cell");
 
@@ -265,7 +266,7 @@ __device__ __forceinline__ void store_background(const RenderParams& P, size_t t
 // VEC: rows of a multiple of four pixels and no float32 depth image.  OCC: with occlusion counts.  RGB: colours instead of
 // classes and depths.
 template <class TL, bool VEC, bool OCC, bool RGB = false>
-__global__ void __launch_bounds__(32, PIC_TILE_CTAS) render_tile_kernel(const __grid_constant__ RenderParams P) {
+__global__ void __launch_bounds__(32, TILE_CTAS) render_tile_kernel(const __grid_constant__ RenderParams P) {
     __shared__ TileWarp s;
     const int lane = threadIdx.x;
     launch_dependents();
