@@ -1,28 +1,17 @@
 // Production render kernels of the batched egocentric rasterizer (sm_100a).
 //
-// The z-buffer lives in shared memory as one 64-bit key per pixel,
+// The z-buffer holds one 64-bit key per pixel (in registers or shared memory),
 //     key = float_bits(1/z) << 32 | (0xFFFFFF - primitive index) << 8 | class,
 // so "nearest fragment wins, exact ties go to the lower index" is an unsigned max that does not
 // depend on the order in which primitives arrive; 0 means "no fragment" (background).
 //
 // A unit of work is a tile: up to 64 x 64 pixels of one view.
 //
-// cull_kernel.  A warp per tile finds the primitives and box faces that can touch a pixel centre and leaves them as a
-// list in device memory.
+// cull_kernel.  A warp per tile, or per view of several tiles, finds the primitives and box faces that can touch a pixel
+// centre and leaves them as a list per tile in device memory.
 //
-// render_full_kernel (images of full tiles, the workloads) and render_kernel (ragged tiles, options).  A CTA of 4 warps
-// takes 4 consecutive tiles.
-//   set-up  the survivors of the 4 tiles get consecutive ranges of a shared record pool and are set up, a lane per
-//           survivor: 3-4 edge functions + 1/z plane in a 17-word record.
-//   raster  the 16 strips of 16 pixel rows (4 per tile) are tasks that the warps draw from a counter.  A warp owns one
-//           strip of keys (8 KB).  Per strip it looks at the tile's records 32 at a time (a lane each: does the box
-//           reach the strip?), rasterizes primitives of <= 4 pixels from their lane with atomic max, then walks the
-//           other hits together: a lane per pixel pair of a 16 x 4 pixel cell, plain loads and stores; boxes of >= 256
-//           pixels first classify the strip's 16 cells (trivial reject / trivial accept / which edges still need
-//           testing) from the same float32 edge functions.
-//   store   converts keys to class u8 + depth binary16 with 128- and 256-bit stores, resets the keys it read, and
-//           writes 8 x 8 blocks that nothing touched without reading keys.
-//   Tiles whose lists overflow, or whose records do not fit the pool, are appended to a list in device memory.
+// render_tile_kernel (pic_tile.cuh).  A warp per tile: set-up, raster and store with the z-buffer in registers.  Tiles whose
+// lists overflow are appended to a list in device memory.
 //
 // cooperative_kernel.  One wave of CTAs walks that list; a whole CTA renders a tile in
 // barrier-separated phases with per-round lists (any number of groups, boxes, survivors and
@@ -30,8 +19,10 @@
 //
 // render_small_kernel (pic_small.cuh).  Calls with few tiles: a CTA of 8 warps takes one tile from culling to store.
 //
+// coverage_kernel (occlusion counts), colour_kernel (pic_colour.cuh), render_static_kernel (pic_static.cuh).
+//
 // Cameras (one 64-byte record per view) and per-camera ray / background tables are prepared by
-// the agent and rig kernels, so the prologues are a few loads.
+// the set-up kernel, so the prologues are a few loads.
 #include <cstddef>
 
 #include "pic_device.cuh"
@@ -48,9 +39,7 @@ constexpr int BOX_ROUND = 64;     // boxes examined per round
 constexpr int FACECAP = 6 * BOX_ROUND;
 constexpr int SCAP = 128;         // candidates that survive the pixel-box test, per round
 constexpr int TINY_MAX_PIXELS = 4;         // pixel centres in the box of a primitive rasterized by its own thread
-static_assert(TINY_MAX_PIXELS == 4, "the strip back end enumerates the pixels of such a box for at most 4");
 constexpr int CLASSIFY_MIN_PIXELS = 192;   // pixel boxes at least this large classify cells before rasterizing
-constexpr int CLASSIFY_MIN_STRIP = 256;    // the same for the part of a box inside a 16-row strip
 
 struct __align__(16) TileSmem {
     unsigned long long key[TILE * TILE];      // 32 KB, 16-byte chunks XOR-swizzled by row (key_index)
@@ -262,8 +251,7 @@ __device__ __forceinline__ void edge_thresholds(uint32_t tl, float (&thr)[4]) {
 }
 
 // One 16 x 4 cell at (xx, yy): every lane tests its two pixels and updates their keys with plain
-// loads and stores -- the rows of a cell belong to exactly one warp (its strip in render_small_kernel,
-// its bands in the cooperative kernel).  `need`: the edges
+// loads and stores -- the rows of a cell belong to exactly one warp (its bands).  `need`: the edges
 // that still have to be tested on this cell (0: the cell is known to be covered and in depth
 // range; the range test rides on the edge tests).  Returns whether any lane produced a fragment.
 template <class S>
@@ -632,7 +620,6 @@ constexpr int W_SURV = SURV_STRIDE - 2;
 constexpr uint32_t SURV_OVERFLOW = 0xffffffffu;
 constexpr uint32_t SURV_FACE = 0x80000000u;   // survivor id: index into grid_prims, or SURV_FACE | agent << 3 | face
 constexpr uint32_t REC_TINY = 1u << 28, REC_DEAD = 1u << 29;   // flags in the box word of a record
-constexpr uint32_t REC_INRANGE = 1u << 30;   // every covered pixel is within [near, far]: no per-pixel range test
 
 // A tile's frustum and its footprint on the ground plane.
 struct __align__(16) Frustum {
@@ -653,12 +640,6 @@ struct __align__(16) FrontLists {
     int n_item;
 };
 
-// What the raster and store templates need of a warp's strip: rows are counted from the strip's first.
-struct StripView {
-    unsigned long long* key;
-    const float* ray_x;
-    const float* ray_y;
-};
 // Box test against planes held in registers (see box_visible).
 __device__ __forceinline__ bool box_visible_reg(const float4 (&pl)[6], float px, float py, const Node& b) {
     const float ax = sub(b.lo[0], px), bx = sub(b.hi[0], px);
@@ -689,11 +670,6 @@ __device__ __forceinline__ AgentGeom load_agent(const AgentGeom* p) {
     AgentGeom g;
     g.x = a.x; g.y = a.y; g.c = a.z; g.s = a.w; g.hl = b.x; g.hw = b.y; g.h = b.z; g.active = __float_as_uint(b.w);
     return g;
-}
-
-__device__ __forceinline__ bool tiny_box(uint32_t box) {
-    const int bx0 = box & 0xff, by0 = (box >> 8) & 0xff, bx1 = (box >> 16) & 0xff, by1 = box >> 24;
-    return (bx1 - bx0 + 1) * (by1 - by0 + 1) <= TINY_MAX_PIXELS;
 }
 
 // Warp-wide append to the survivor list (a slot past the end is not written; the caller checks the total).
@@ -1100,164 +1076,6 @@ __global__ void __launch_bounds__(NTHREADS, CULL_CTAS) cull_kernel(const __grid_
     launch_dependents();
 }
 
-// A record pool, one array per 16-byte part of a record: 17 words per
-// record instead of the 20 of an array of padded records.
-template <int N>
-struct __align__(16) RecordPool {
-    float4 nx[N], ny[N], nz[N];               // edge functions E_i = nx[i] rx + ny[i] ry + nz[i]
-    float4 w[N];                              // 1/z plane wx, wy, wz; key low word
-    uint32_t box[N];                          // pixel box (6 bits per coordinate), top-left bits, flags
-};
-
-template <int N>
-__device__ __forceinline__ void write_record(RecordPool<N>& pool, int slot, const PrimEq& q, uint32_t key_lo, uint32_t box, uint32_t extra) {
-    const uint32_t bx0 = box & 0xff, by0 = (box >> 8) & 0xff, bx1 = (box >> 16) & 0xff, by1 = box >> 24;
-    pool.nx[slot] = make_float4(q.nx[0], q.nx[1], q.nx[2], q.nx[3]);
-    pool.ny[slot] = make_float4(q.ny[0], q.ny[1], q.ny[2], q.ny[3]);
-    pool.nz[slot] = make_float4(q.nz[0], q.nz[1], q.nz[2], q.nz[3]);
-    pool.w[slot] = make_float4(q.wx, q.wy, q.wz, __uint_as_float(key_lo));
-    pool.box[slot] = bx0 | (by0 << 6) | (bx1 << 12) | (by1 << 18) | (q.tl << 24) | extra;
-}
-
-template <int N>
-__device__ __forceinline__ void read_record(const RecordPool<N>& pool, int slot, PrimEq& q, uint32_t& key_lo) {
-    const float4 r0 = pool.nx[slot], r1 = pool.ny[slot], r2 = pool.nz[slot], r3 = pool.w[slot];
-    q.nx[0] = r0.x; q.nx[1] = r0.y; q.nx[2] = r0.z; q.nx[3] = r0.w;
-    q.ny[0] = r1.x; q.ny[1] = r1.y; q.ny[2] = r1.z; q.ny[3] = r1.w;
-    q.nz[0] = r2.x; q.nz[1] = r2.y; q.nz[2] = r2.z; q.nz[3] = r2.w;
-    q.wx = r3.x; q.wy = r3.y; q.wz = r3.z;
-    key_lo = __float_as_uint(r3.w);
-}
-
-// The 16 x 4 cell of strip_cell's comment, for the full-tile kernel: `kbase` and `lsw` are the
-// lane's share of the key address (row lane >> 3, chunk lane & 7, swizzle), `range` says whether
-// the depth range still has to be tested (warp-uniform), keys are written with one predicated
-// 64-bit store per pixel; the caller marks the touched blocks.
-__device__ __forceinline__ void strip_cell(unsigned long long* key, const float* ray_x, const float* ray_y, const PrimEq& q,
-                                           const float (&thr)[4], uint32_t key_lo, float w_near, float w_far, int xx, int yy,
-                                           uint32_t need, bool range, int kbase, int lsw, int lane) {
-    const float2 rx = *reinterpret_cast<const float2*>(ray_x + xx + (lane & 7) * 2);
-    const float ry = ray_y[yy + (lane >> 3)];
-    const float wt = fm(q.wy, ry, q.wz);
-    const float w0 = fm(q.wx, rx.x, wt), w1 = fm(q.wx, rx.y, wt);
-    bool in0 = true, in1 = true;
-    if (need) {
-#pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            if ((need >> e) & 1u) {          // warp-uniform: edges known to be positive on the whole cell are skipped
-                const float te = fm(q.ny[e], ry, q.nz[e]);
-                const float e0 = fm(q.nx[e], rx.x, te), e1 = fm(q.nx[e], rx.y, te);
-                in0 = in0 && (e0 > thr[e]);
-                in1 = in1 && (e1 > thr[e]);
-            }
-        }
-        if (range) {
-            in0 = in0 && (w0 >= w_far) && (w0 <= w_near);
-            in1 = in1 && (w1 >= w_far) && (w1 <= w_near);
-        }
-    }
-    const int cb = xx >> 4;
-    unsigned long long* kp = key + (kbase + (yy << 6) + (cb << 4) + ((lsw ^ cb) << 1));
-    const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(kp);
-    const unsigned long long k0 = make_key(__float_as_uint(w0), key_lo), k1 = make_key(__float_as_uint(w1), key_lo);
-    if (in0 && k0 > kk.x) kp[0] = k0;
-    if (in1 && k1 > kk.y) kp[1] = k1;
-}
-
-// One strip (rows ys .. of the tile) by one warp: the tile's fragments that fall into it, then
-// the records that reach it, cell by cell.  Returns the touched 8 x 8 blocks.
-template <int ROWS, int N>
-__device__ __forceinline__ uint32_t raster_strip(StripView& s, const RecordPool<N>& pool, int first, int n_rec, int ys, float w_near,
-                                                      float w_far, int lane) {
-    uint32_t touched = 0u;                       // bit (row >> 3) * 8 + (column >> 3)
-    const int kbase = (lane >> 3) << 6, lsw = (lane & 7) ^ (((lane >> 3) & 1) << 2);   // see strip_cell
-    for (int base = 0; base < n_rec; base += 32) {
-        uint32_t bw_lane = 0u;
-        bool hit = false;
-        if (base + lane < n_rec) {
-            const int slot = first + base + lane;
-            bw_lane = pool.box[slot];
-            const int by0 = (bw_lane >> 6) & 63, by1 = (bw_lane >> 18) & 63;
-            hit = !(bw_lane & REC_DEAD) && by1 >= ys && by0 < ys + ROWS;
-            if (hit && (bw_lane & REC_TINY)) {           // a few pixels: rasterized by this lane (atomic max)
-                hit = false;
-                const int bx0 = bw_lane & 63, bx1 = (bw_lane >> 12) & 63;
-                const int y0 = max(by0, ys) - ys, y1 = min(by1, ys + ROWS - 1) - ys;
-                PrimEq q;
-                uint32_t key_lo;
-                read_record(pool, slot, q, key_lo);
-                q.tl = (bw_lane >> 24) & 15u;
-                // at most TINY_MAX_PIXELS pixels: one column (w == 1), two columns, or one row
-                const int w = bx1 - bx0 + 1, npx = w * (y1 - y0 + 1);
-                bool any = false;
-#pragma unroll
-                for (int px = 0; px < TINY_MAX_PIXELS; ++px) {
-                    if (px < npx) {
-                        const int x = bx0 + (w == 1 ? 0 : w == 2 ? (px & 1) : px), y = y0 + (w == 1 ? px : w == 2 ? (px >> 1) : 0);
-                        const uint32_t wb = fragment(q, s.ray_x[x], s.ray_y[y], w_near, w_far);
-                        if (wb) { put_fragment(s, x, y, wb, key_lo); any = true; }
-                    }
-                }
-                if (any) touched |= (uint32_t)block_mask(bx0, y0, bx1, y1);
-            }
-        }
-        __syncwarp();
-        unsigned hits = __ballot_sync(0xffffffffu, hit);
-        for (; hits; hits &= hits - 1) {
-            const int src = __ffs(hits) - 1;
-            const uint32_t bw = __shfl_sync(0xffffffffu, bw_lane, src);
-            const int by0 = (bw >> 6) & 63, by1 = (bw >> 18) & 63;
-            const int bx0 = bw & 63, bx1 = (bw >> 12) & 63;
-            const int ly0 = max(by0, ys) - ys, ly1 = min(by1, ys + ROWS - 1) - ys;
-            PrimEq q;
-            uint32_t key_lo;
-            read_record(pool, first + base + src, q, key_lo);
-            q.tl = (bw >> 24) & 15u;
-            float thr[4];
-            edge_thresholds(q.tl, thr);
-            const bool range = !(bw & REC_INRANGE);
-            if ((bx1 - bx0 + 1) * (ly1 - ly0 + 1) >= CLASSIFY_MIN_STRIP * ROWS / 16) {
-                // a lane per 16 x 4 pixel cell of the strip classifies it: reject / partly covered / inside
-                const int xa = (lane & 3) * 16, xb = xa + 15, ya = ((lane >> 2) & 3) * 4, yb = ya + 3;
-                bool reject = lane >= ROWS || xb < bx0 || xa > bx1 || yb < ly0 || ya > ly1;
-                uint32_t need = 0u;
-                if (!reject) {
-                    const float rxa = s.ray_x[xa], rxb = s.ray_x[xb], rya = s.ray_y[ya], ryb = s.ray_y[yb];   // rxa < rxb, rya < ryb
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        // fma is monotone in each argument, so the cell's extreme values are at its corners
-                        const float ta = fm(q.ny[e], rya, q.nz[e]), tb = fm(q.ny[e], ryb, q.nz[e]);
-                        const float emax = fm(q.nx[e], q.nx[e] >= 0.f ? rxb : rxa, fmaxf(ta, tb));
-                        const float emin = fm(q.nx[e], q.nx[e] >= 0.f ? rxa : rxb, fminf(ta, tb));
-                        reject = reject || (emax < 0.f);
-                        if (!(emin > 0.f)) need |= 1u << e;
-                    }
-                    const float wa = fm(q.wy, rya, q.wz), wb = fm(q.wy, ryb, q.wz);
-                    const float wmax = fm(q.wx, q.wx >= 0.f ? rxb : rxa, fmaxf(wa, wb));
-                    const float wmin = fm(q.wx, q.wx >= 0.f ? rxa : rxb, fminf(wa, wb));
-                    reject = reject || (wmax < w_far) || (wmin > w_near);
-                    // the depth range test rides on the edge tests: if it is still needed, so is one edge
-                    if (need == 0u && !((wmin >= w_far) && (wmax <= w_near))) need = 1u;
-                }
-                for (unsigned m = __ballot_sync(0xffffffffu, !reject); m; m &= m - 1) {
-                    const int cell = __ffs(m) - 1;
-                    const int xx = (cell & 3) * 16, yy = (cell >> 2) * 4;
-                    const uint32_t need_c = __shfl_sync(0xffffffffu, need, cell);
-                    strip_cell(s.key, s.ray_x, s.ray_y, q, thr, key_lo, w_near, w_far, xx, yy, need_c, true, kbase, lsw, lane);
-                    touched |= 3u << ((yy >> 3) * 8 + (xx >> 3));
-                }
-            } else {
-                for (int yy = ly0 & ~3; yy <= ly1; yy += 4)
-                    for (int xx = bx0 & ~15; xx <= bx1; xx += 16)
-                        strip_cell(s.key, s.ray_x, s.ray_y, q, thr, key_lo, w_near, w_far, xx, yy, 0xFu, range, kbase, lsw, lane);
-                touched |= (uint32_t)block_mask(bx0, ly0, bx1, ly1);
-            }
-        }
-        __syncwarp();
-    }
-    return __reduce_or_sync(0xffffffffu, touched);
-}
-
 // The tiles the render kernels left out, a CTA at a time.  (Called from the end of those kernels instead, the same code
 // costs them 2 % -- a call bounds their registers -- which is more than a launch that overlaps their last blocks.)
 template <class TL>
@@ -1453,11 +1271,9 @@ cudaError_t launch_render_kernel(const RenderParams& P0, long long n_views, int 
     if (jobs <= 0) return cudaSuccess;
     P.n_jobs = (uint32_t)jobs;
     P.far_z2 = 0x10001u * (uint32_t)__half_as_ushort(__float2half_rn(P.far_z));
-    // few tiles: one CTA takes a tile from culling to store.  Measured (a call on 16 agents per environment, both image
-    // shapes of the workloads): 64 tiles 37.0 -> 20.7 us, 256 tiles 44.6 -> 22.7, 768 tiles 47.3 -> 44.8, 1024 tiles
-    // 48.4 -> 53.7, so the line lies at five tiles per multiprocessor.
+    // few tiles: one CTA takes a tile from culling to store.  Measured (a call on 16 agents per environment, both image shapes of the workloads): 64 tiles 37 -> 17 us, 256 tiles 45 -> 14.5, 512 tiles 45 -> 23.
     if (jobs <= 5LL * sm_count && !P.counters && !P.occlusion && (P.debug_flags & 15) == 0)
-        return launch_next(render_small_kernel, (unsigned)jobs, SMALL_SMEM, stream, P, SMALL_THREADS);
+        return launch_next(P.W % 4 == 0 && !P.out_depth32 ? render_small_kernel<true> : render_small_kernel<false>, (unsigned)jobs, SMALL_SMEM, stream, P, SMALL_THREADS);
     // (a) cull: survivors per tile
     cudaError_t err = launch_cull(P, n_views, false, sm_count, stream);
     if (err != cudaSuccess) return err;

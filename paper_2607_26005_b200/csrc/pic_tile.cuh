@@ -88,6 +88,56 @@ __device__ __forceinline__ void keep_nearer(unsigned long long& best, bool in, f
     best = make_key(up ? __float_as_uint(w) : bh, up ? lo : bl);
 }
 
+// Cell << 7 | pixel of the cell (row << 5 | column).
+__device__ __forceinline__ uint32_t cell_pixel(int x, int y) { return (uint32_t)((((y >> 2) << 1) | (x >> 5)) << 7 | (y & 3) << 5 | (x & 31)); }
+
+// The pixels of the warp's small primitives -- lane l's is small[l], w x h pixels from (bx0, by0), if `is_small` -- a lane
+// each whatever the primitive; `push` gets every lane's result (covered?, 1/z, low key word, pixel).
+template <class Push>
+__device__ __forceinline__ void small_pixels(const TileRecords<32>& small, const float* ray_x, const float* ray_y, bool is_small, int bx0, int by0, int w, int h,
+                                             float w_near, float w_far, int lane, Push push) {
+    const int cnt = is_small ? w * h : 0;
+    int incl = cnt;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int up = __shfl_up_sync(0xffffffffu, incl, d);
+        if (lane >= d) incl += up;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31), before = incl - cnt;
+    // x, y of the box and 1024 / w rounded up: (i * inv) >> 10 is i / w for i < 32
+    const uint32_t packed = (uint32_t)bx0 | ((uint32_t)by0 << 6) | ((uint32_t)w << 12) | ((uint32_t)((1024 + w - 1) / w) << 18);
+    __syncwarp();
+#pragma unroll 1
+    for (int p0 = 0; p0 < total; p0 += 32) {
+        const int p = p0 + lane;
+        int own = 0;                                         // the lane whose range holds p: the last with before <= p (and pixels)
+#pragma unroll
+        for (int st = 16; st; st >>= 1) {
+            const int b = __shfl_sync(0xffffffffu, before, own + st);
+            if (b <= p) own += st;
+        }
+        const uint32_t pk = __shfl_sync(0xffffffffu, packed, own);
+        const int idx = p - __shfl_sync(0xffffffffu, before, own);
+        const int dy = (idx * (int)(pk >> 18)) >> 10, x = (int)(pk & 63u) + idx - dy * (int)((pk >> 12) & 63u), y = (int)((pk >> 6) & 63u) + dy;
+        bool in = p < total;
+        float wv = 0.f;
+        uint32_t lo = 0u;
+        if (in) {
+            const float rx = ray_x[x], ry = ray_y[y];
+            const float4 pw = small.w[own];
+            wv = fm(pw.x, rx, fm(pw.y, ry, pw.z));
+            lo = __float_as_uint(pw.w);
+            in = (wv >= w_far) & (wv <= w_near);
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const float4 q4 = small.edge[e][own];
+                in = in & (fm(q4.x, rx, fm(q4.y, ry, q4.z)) > q4.w);
+            }
+        }
+        push(in, wv, lo, x, y);
+    }
+}
+
 // Cells (bit 2 row + column) reached by a pixel box.
 __device__ __forceinline__ uint32_t box_cells(uint32_t box) {
     const int bx0 = box & 0xff, by0 = (box >> 8) & 0xff, bx1 = (box >> 16) & 0xff, by1 = box >> 24;
@@ -100,15 +150,16 @@ __device__ __forceinline__ uint32_t box_cells(uint32_t box) {
 // tested there pixel by pixel.  An edge function's values on the cell's pixel centres lie within +-h of its value at the
 // cell's centre; h is widened by 1e-6 of the terms' sizes, several times what the float32 evaluations can lose, so
 // "outside" and "inside" hold for every pixel as it would be evaluated itself.
-template <class TL>
-__device__ __forceinline__ uint32_t classify_records(TileWarp& s, int n_rec, bool exact, float w_near, float w_far, int lane, TL& n) {
+// (first, step: the records looked at.)
+template <class S, class TL>
+__device__ __forceinline__ uint32_t classify_records(S& s, int n_rec, bool exact, float w_near, float w_far, int lane, TL& n, int first = 0, int step = 1) {
     const int xa = (lane & 1) * CELL_W, ya = (lane >> 1) * CELL_H;
     const float rxa = s.ray_x[xa], rxb = s.ray_x[xa + CELL_W - 1], rya = s.ray_y[ya], ryb = s.ray_y[ya + CELL_H - 1];
     const float rxc = 0.5f * (rxa + rxb), ryc = 0.5f * (rya + ryb);
     const float hx = 0.5f * (rxb - rxa) + 1e-6f * fmaxf(fabsf(rxa), fabsf(rxb)), hy = 0.5f * (ryb - rya) + 1e-6f * fmaxf(fabsf(rya), fabsf(ryb));
     uint32_t hit = 0u;
 #pragma unroll 1
-    for (int r = 0; r < n_rec; ++r) {
+    for (int r = first; r < n_rec; r += step) {
         bool out = !((s.cells[r] >> lane) & 1u);
         uint32_t need = 0u;
 #pragma unroll
@@ -131,7 +182,8 @@ __device__ __forceinline__ uint32_t classify_records(TileWarp& s, int n_rec, boo
 }
 
 // The records of mask m against the lane's four pixels of cell `cell`.
-__device__ __forceinline__ void raster_records_cell(const TileWarp& s, uint32_t m, int cell, const float4 rx, float ry, float w_near,
+template <class S>
+__device__ __forceinline__ void raster_records_cell(const S& s, uint32_t m, int cell, const float4 rx, float ry, float w_near,
                                                     float w_far, unsigned long long (&best)[4]) {
 #pragma unroll 1
     for (; m; m &= m - 1) {
@@ -318,52 +370,15 @@ __global__ void __launch_bounds__(32, TILE_CTAS) render_tile_kernel(const __grid
             }
             n_rec += __popc(mb);
             // ---- the pixels of the small primitives, a lane each whatever the primitive
-            const int cnt = small ? w * h : 0;
-            int incl = cnt;
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const int up = __shfl_up_sync(0xffffffffu, incl, d);
-                if (lane >= d) incl += up;
-            }
-            const int total = __shfl_sync(0xffffffffu, incl, 31), before = incl - cnt;
-            // x, y of the box and 1024 / w rounded up: (i * inv) >> 10 is i / w for i < 32
-            const uint32_t packed = (uint32_t)bx0 | ((uint32_t)by0 << 6) | ((uint32_t)w << 12) | ((uint32_t)((1024 + w - 1) / w) << 18);
-            __syncwarp();
-#pragma unroll 1
-            for (int p0 = 0; p0 < total; p0 += 32) {
-                const int p = p0 + lane;
-                int own = 0;                                 // the lane whose range holds p: the last with before <= p (and pixels)
-#pragma unroll
-                for (int st = 16; st; st >>= 1) {
-                    const int b = __shfl_sync(0xffffffffu, before, own + st);
-                    if (b <= p) own += st;
-                }
-                const uint32_t pk = __shfl_sync(0xffffffffu, packed, own);
-                const int idx = p - __shfl_sync(0xffffffffu, before, own);
-                const int dy = (idx * (int)(pk >> 18)) >> 10, x = (int)(pk & 63u) + idx - dy * (int)((pk >> 12) & 63u), y = (int)((pk >> 6) & 63u) + dy;
-                bool in = p < total;
-                float wv = 0.f;
-                uint32_t lo = 0u;
-                if (in) {
-                    const float rx = s.ray_x[x], ry = s.ray_y[y];
-                    const float4 pw = s.small.w[own];
-                    wv = fm(pw.x, rx, fm(pw.y, ry, pw.z));
-                    lo = __float_as_uint(pw.w);
-                    in = (wv >= P.w_far) & (wv <= P.w_near);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float4 q4 = s.small.edge[e][own];
-                        in = in & (fm(q4.x, rx, fm(q4.y, ry, q4.z)) > q4.w);
-                    }
-                }
+            small_pixels(s.small, s.ray_x, s.ray_y, small, bx0, by0, w, h, P.w_near, P.w_far, lane, [&](bool in, float wv, uint32_t lo, int x, int y) {
                 const unsigned mf = __ballot_sync(0xffffffffu, in);
                 const int slot = n_frag + __popc(mf & below);
                 if (in && slot < TFRAG) {
                     s.frag_key[slot] = make_key(__float_as_uint(wv), lo);
-                    s.frag_px[slot] = (uint16_t)(((((y >> 2) << 1) | (x >> 5)) << 7) | ((y & 3) << 5) | (x & 31));
+                    s.frag_px[slot] = (uint16_t)cell_pixel(x, y);
                 }
                 n_frag += __popc(mf);
-            }
+            });
             __syncwarp();
         }
         fits = fits && n_rec <= rec_cap && n_frag <= TFRAG;
