@@ -1271,8 +1271,9 @@ cudaError_t launch_render_kernel(const RenderParams& P0, long long n_views, int 
     if (jobs <= 0) return cudaSuccess;
     P.n_jobs = (uint32_t)jobs;
     P.far_z2 = 0x10001u * (uint32_t)__half_as_ushort(__float2half_rn(P.far_z));
-    // few tiles: one CTA takes a tile from culling to store.  Measured (a call on 16 agents per environment, both image shapes of the workloads): 64 tiles 37 -> 17 us, 256 tiles 45 -> 14.5, 512 tiles 45 -> 23.
-    if (jobs <= 5LL * sm_count && !P.counters && !P.occlusion && (P.debug_flags & 15) == 0)
+    // few tiles: one CTA takes a tile from culling to store.  Measured (a call on 16 agents per environment, both image shapes of the workloads): 64 tiles 37 -> 17 us, 256 tiles 45 -> 14.5, 512 tiles 45 -> 23,
+    // and against cull + tile kernel 768 tiles 41.7 -> 31.1, 1 024 tiles 43.5 -> 37.3, 1 280 tiles 44.0 -> 44.9.
+    if (jobs <= 8LL * sm_count && !P.counters && !P.occlusion && (P.debug_flags & 15) == 0)
         return launch_next(P.W % 4 == 0 && !P.out_depth32 ? render_small_kernel<true> : render_small_kernel<false>, (unsigned)jobs, SMALL_SMEM, stream, P, SMALL_THREADS);
     // (a) cull: survivors per tile
     cudaError_t err = launch_cull(P, n_views, false, sm_count, stream);

@@ -52,8 +52,8 @@ def test_static_pieces_lists_and_alignment(n_tris, E, A, H, W, offset):
 @pytest.mark.parametrize("n_tris,E,A,H,W,K,spread", [
     (40, 1, 1, 8, 16, 1, 25.0),           # one tile of one strip
     (300, 1, 3, 17, 33, 2, 25.0),         # ragged in both directions
-    (300, 5, 37, 64, 64, 4, 200.0),       # 740 tiles: the most that take one CTA each (on 148 multiprocessors) ...
-    (300, 57, 13, 64, 64, 1, 200.0),      # ... and one more
+    (300, 8, 37, 64, 64, 4, 200.0),       # 1 184 tiles: the most that take one CTA each (on 148 multiprocessors) ...
+    (300, 79, 15, 64, 64, 1, 200.0),      # ... and one more
     (3000, 1, 2, 130, 70, 2, 12.0),       # more survivors than the record pool holds
     (20, 1, 120, 64, 64, 1, 25.0),        # more visible box faces than their list holds, all around the cameras
     (4000, 1, 4, 64, 64, 2, 90.0),        # a map of small cells: more grid rows in view than one pass takes
@@ -76,11 +76,11 @@ def test_calls_with_few_tiles(n_tris, E, A, H, W, K, spread):
 
 
 @pytest.mark.parametrize("n_tris,E,A,H,W,K,spread", [
-    (60, 4, 50, 20, 30, 4, 30.0),         # rows of no whole groups of four pixels: scalar stores
+    (60, 6, 50, 20, 30, 4, 30.0),         # rows of no whole groups of four pixels: scalar stores
     (200, 2, 100, 36, 76, 4, 60.0),       # groups of four but not of sixteen; a second tile narrower than a cell
     (200, 2, 100, 65, 48, 4, 60.0),       # a second tile of a single row
-    (3000, 1, 60, 130, 80, 4, 12.0),      # more records and more fragments than a tile's lists hold
-    (60, 8, 24, 64, 64, 4, 6.0),          # large primitives around the cameras: cells wholly inside, range tests
+    (3000, 1, 60, 130, 80, 4, 12.0),      # (1 440 tiles) more records and more fragments than a tile's lists hold
+    (60, 13, 24, 64, 64, 4, 6.0),         # large primitives around the cameras: cells wholly inside, range tests
 ])
 def test_calls_with_many_tiles(n_tris, E, A, H, W, K, spread):
     test_calls_with_few_tiles(n_tris, E, A, H, W, K, spread)
