@@ -26,6 +26,7 @@
 #include <cstddef>
 
 #include "pic_device.cuh"
+#include "pic_rows.h"
 
 namespace pic {
 
@@ -770,7 +771,7 @@ __device__ __forceinline__ void frustum_setup(Frustum& f, const RenderParams& P,
 
 // The grid rows crossed by the footprint, widened by the map's margin.
 struct GridRows {
-    int lo, hi;             // (hi < lo if the footprint misses the grid)
+    int lo, hi;             // (within the grid; hi < lo if the footprint misses it)
     float gx0, gy0;         // the grid's corner, ego-relative
 };
 __device__ __forceinline__ GridRows grid_rows(const Frustum& f, const MapInfo& mi) {
@@ -780,7 +781,7 @@ __device__ __forceinline__ GridRows grid_rows(const Frustum& f, const MapInfo& m
 #pragma unroll
     for (int k = 1; k < 5; ++k) { ylo = fminf(ylo, f.pt[k][1]); yhi = fmaxf(yhi, f.pt[k][1]); }
     const float fr0 = floorf((ylo - mi.margin - g.gy0) * mi.inv_cell), fr1 = floorf((yhi + mi.margin - g.gy0) * mi.inv_cell);
-    g.lo = (int)fmaxf(fr0, 0.f); g.hi = (int)fminf(fr1, (float)mi.ny - 1.f);
+    clamp_rows(fr0, fr1, mi.ny, g.lo, g.hi);
     return g;
 }
 

@@ -82,7 +82,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 2) render_small_kernel(const __
             }
         }
         int n_large = 0, n_face = 0;
-        for (int r0 = rows.lo;; r0 += 32) {
+        for (int r0 = rows.lo;; r0 += ROW_PASS) {
             if (warp == 0) {
                 uint32_t first, cnt;
                 row_range(s.f, P, mi, rows, r0 + lane, first, cnt);
@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 2) render_small_kernel(const __
                 }
             }
             __syncthreads();
-            if (r0 + 32 > rows.hi) break;
+            if (!rows_after(r0, rows.hi)) break;
         }
         if (fits) fits = s.n_rec <= TREC;
         if (!fits) {

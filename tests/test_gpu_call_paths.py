@@ -155,3 +155,27 @@ def test_host_images_in_parts(E, A, H, W):
             assert (dep.reshape(want[1].shape).view(np.uint16) == want[1].view(np.uint16)).all()
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("E,A,H,W,K", [
+    (4, 3, 40, 64, 2),                    # few tiles
+    (64, 12, 40, 64, 2),                  # a warp per tile
+    (64, 14, 130, 96, 2),                 # culled a warp per view
+])
+def test_poses_far_outside_the_map(E, A, H, W, K):
+    """Finite poses more than 2^31 grid cells from the map, in every direction: nothing but other agents at the same place is in view."""
+    from tests.gpu_util import CudaRun
+    from tests.util import assert_same_as_exhaustive
+    s = soup(E + A, 200, E, A, H, W, K=K, spread=40.0)
+    poses = s.poses.copy()
+    far = np.array([1e9, 1e11, 1e12, 1e30, 3e38], np.float32)
+    for i in range(E * A // 2):
+        poses.reshape(-1, 3)[2 * i, i % 2] = far[i % 5] * (1 if (i // 2) % 2 else -1)
+    g = CudaRun(s)
+    try:
+        V = E * A * K
+        n = min(V, 300)
+        a = g.render(poses=poses)
+        assert_same_as_exhaustive(a, g.render(poses=poses, brute=True, view_first=V - n, view_count=n), slice(V - n, V))
+    finally:
+        g.close()
