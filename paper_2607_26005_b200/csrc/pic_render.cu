@@ -638,7 +638,6 @@ struct __align__(16) FrontLists {
     uint32_t item[W_ITEM];                    // survivor ids to be tested
     uint32_t row_first[32];                   // grid rows of a pass: first entry of the row's range in cell_prims
     uint32_t row_off[33];                     //   and the number of candidates before the row (the total at [32])
-    int n_item;
 };
 
 // Box test against planes held in registers (see box_visible).
@@ -871,9 +870,10 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
     if (lane < P.A) ag0 = load_agent(env_agents + lane);
     if (lane + 32 < P.A) ag1 = load_agent(env_agents + lane + 32);
     Frustum& fr = f.f;
-    if (lane == 0) f.n_item = 0;
     frustum_setup(fr, P, job, lane);
     const Cam& c = fr.cam;
+    const unsigned below = (1u << lane) - 1u;
+    int n_item = 0;                                // (entries are appended in order of lane, so that a call's lists are the same every time)
     // ---- the grid rows crossed by the widened footprint; the first 32 rows' ranges are requested now, the boxes below
     // are tested while the loads are under way
     const GridRows rows = grid_rows(fr, mi);
@@ -887,14 +887,20 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
         for (int p = 0; p < 6; ++p) pl[p] = *reinterpret_cast<const float4*>(fr.plane[p]);
         for (uint32_t l0 = mi.large_begin; l0 < mi.large_end; l0 += 32) {
             const uint32_t l = l0 + lane;
-            if (l >= mi.large_end) continue;
-            const Node ln = (l0 == mi.large_begin) ? ln0 : load_node(P.large_leaves + l);
-            ++n.leaf;
-            if (box_visible_reg(pl, c.px, c.py, ln)) {
-                const int slot = atomicAdd(&f.n_item, (int)ln.count);
+            bool vis = false;
+            Node ln = ln0;
+            if (l < mi.large_end) {
+                if (l0 != mi.large_begin) ln = load_node(P.large_leaves + l);
+                ++n.leaf;
+                vis = box_visible_reg(pl, c.px, c.py, ln);
+            }
+            const unsigned m = __ballot_sync(0xffffffffu, vis);
+            if (vis) {
+                const int slot = n_item + LARGE_LEAF_PRIMS * __popc(m & below);     // (only a map's last leaf may be shorter)
                 for (uint32_t k = 0; k < ln.count; ++k)
                     if (slot + (int)k < W_ITEM) f.item[slot + k] = ln.first + k;
             }
+            n_item += (int)__reduce_add_sync(0xffffffffu, vis ? ln.count : 0u);
         }
     }
     // ---- other agents' boxes, two per lane at a time
@@ -910,15 +916,17 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
             const int b = b0 + lane + 32 * u;
             uint32_t faces = 0u;
             if (b < P.A && b != job.a && g.active) faces = box_faces(fr, c, t, g);
-            if (faces) {
-                int slot = atomicAdd(&f.n_item, __popc(faces));
+            if (__any_sync(0xffffffffu, faces != 0u)) {
+                // (a sum over the lanes below of numbers up to 6, bit by bit)
+                const int cnt = __popc(faces);
+                const unsigned m1 = __ballot_sync(0xffffffffu, cnt & 1), m2 = __ballot_sync(0xffffffffu, cnt & 2), m4 = __ballot_sync(0xffffffffu, cnt & 4);
+                int slot = n_item + __popc(m1 & below) + 2 * __popc(m2 & below) + 4 * __popc(m4 & below);
                 for (; faces; faces &= faces - 1, ++slot)
                     if (slot < W_ITEM) f.item[slot] = SURV_FACE | ((uint32_t)b << 3) | (uint32_t)(__ffs(faces) - 1);
+                n_item += __popc(m1) + 2 * __popc(m2) + 4 * __popc(m4);
             }
         }
     }
-    __syncwarp();
-    int n_item = f.n_item;
     if (n_item > W_ITEM) return -1;
     int n_surv = 0;
     // ---- fill the item list with the candidates of the grid rows (32 rows per pass), test the items, until both are done
@@ -967,7 +975,7 @@ __device__ __forceinline__ int front_cull(FrontLists& f, uint2* __restrict__ sur
                     const bool have = i0 + 32 * u + lane < total;
                     const bool keep = have && bound_visible(c, t, b[u], BOX_MARGIN);
                     const unsigned m = __ballot_sync(0xffffffffu, keep);
-                    if (keep) f.item[n_item + __popc(m & ((1u << lane) - 1u))] = id[u];
+                    if (keep) f.item[n_item + __popc(m & below)] = id[u];
                     n_item += __popc(m);
                 }
                 i0 += 64;

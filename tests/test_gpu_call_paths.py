@@ -179,3 +179,26 @@ def test_poses_far_outside_the_map(E, A, H, W, K):
         assert_same_as_exhaustive(a, g.render(poses=poses, brute=True, view_first=V - n, view_count=n), slice(V - n, V))
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("E,A,H,W", [(40, 12, 64, 64), (60, 12, 70, 130)])       # culled a warp per tile, a warp per view
+def test_antialiased_depth_ties_are_the_same_every_time(E, A, H, W):
+    """Large triangles of many classes in one plane: equal depths everywhere, so the image shows the order of the lists."""
+    from scenes import default_palette
+    from tests.gpu_util import CudaRun
+    rng = np.random.default_rng(W)
+    n = 150
+    yz = rng.uniform(-30.0, 30.0, size=(n, 1, 2)) + rng.uniform(-12.0, 12.0, size=(n, 3, 2))
+    tris = np.concatenate([np.full((n, 3, 1), 20.0), yz], axis=2).astype(np.float32)
+    poses = np.zeros((E, A, 3), np.float32)
+    poses[..., 0] = rng.uniform(-10.0, 5.0, (E, A)); poses[..., 1] = rng.uniform(-20.0, 20.0, (E, A))
+    dims = np.tile(np.array(CAR, np.float32), (E, A, 1))
+    s = custom_scene(tris, rng.integers(2, 9, n).astype(np.uint8), poses, dims, make_rig((0.0,), 90.0, 70.0, W, H), H, W, env_map_id=np.zeros(E, np.int32))
+    g = CudaRun(s)
+    try:
+        first, _ = g.render_rgb(default_palette(), True)
+        for _ in range(4):
+            again, _ = g.render_rgb(default_palette(), True)
+            assert (first == again).all()
+    finally:
+        g.close()
