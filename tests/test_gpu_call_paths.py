@@ -202,3 +202,59 @@ def test_antialiased_depth_ties_are_the_same_every_time(E, A, H, W):
             assert (first == again).all()
     finally:
         g.close()
+
+
+def crowd(A, H, W, K, hfov, vfov, spacing, size, walls=0):
+    """A agents on a lattice in one environment, each seeing up to all the others; `walls`: so many large primitives around them."""
+    rng = np.random.default_rng(A + walls)
+    n = int(np.ceil(np.sqrt(A)))
+    xy = np.stack(np.meshgrid(np.arange(n), np.arange(n)), axis=-1).reshape(-1, 2)[:A] * spacing + rng.uniform(-0.3, 0.3, (A, 2))
+    xy -= xy.mean(0)
+    poses = np.concatenate([xy, rng.uniform(-3.1, 3.1, (A, 1))], axis=1)[None].astype(np.float32)
+    tris = []
+    r, a = 35.0, 0.0
+    for _ in range(walls):                                 # upright 9 m walls on rings 2 m apart: too large for the cells of a map of this many
+        c, d = np.array([r * np.cos(a), r * np.sin(a), 0.0]), np.array([-4.5 * np.sin(a), 4.5 * np.cos(a), 0.0])
+        p = [c - d, c + d, c + d + [0, 0, 2.0], c - d + [0, 0, 2.0]]
+        tris += [[p[0], p[1], p[2]], [p[0], p[2], p[3]]]
+        a += 10.0 / r
+        if a > 2 * np.pi - 10.0 / r:
+            r, a = r + 2.0, 0.0
+    s = custom_scene(np.asarray(tris, np.float32).reshape(-1, 3, 3), np.repeat(rng.integers(2, 9, walls), 2).astype(np.uint8), poses,
+                     np.tile(np.array(size, np.float32), (1, A, 1)), make_rig(tuple(np.arange(K) * 360.0 / K), hfov, vfov, W, H), H, W)
+    # how many agents and walls each view has within its horizontal field
+    at = np.concatenate([poses[0, :, :2]] + [np.asarray(t)[:, :2].mean(0)[None] for t in tris[::2]])
+    rel = at[None] - poses[0, :, None, :2]
+    ang = (np.arctan2(rel[..., 1], rel[..., 0])[:, None] - poses[0, :, None, None, 2] - s.rig[None, :, None, 3] + np.pi) % (2 * np.pi) - np.pi
+    return s, (np.abs(ang) < np.radians(hfov / 2)).sum(-1).reshape(-1)
+
+
+@pytest.mark.parametrize("A,H,W,K,hfov,vfov,spacing,size,walls,modes", [
+    (320, 64, 64, 1, 120.0, 120.0, 7.5, (2.0, 1.0, 1.2), 0, (False,)),            # a tile per view: some 600 box faces in sight
+    (300, 72, 512, 2, 110.0, 30.0, 5.0, (2.5, 1.2, 1.5), 0, (False, True)),       # culled a warp per view
+    (100, 64, 1024, 6, 120.0, 40.0, 2.0, (0.6, 0.6, 1.0), 1100, (False, True)),   # large primitives, with the faces
+])
+def test_views_with_more_items_than_the_cull_list(A, H, W, K, hfov, vfov, spacing, size, walls, modes):
+    import oracle
+    from scenes import default_palette
+    from tests.gpu_util import CudaRun
+    from tests.test_gpu_colour import compare_colour
+    from tests.util import assert_same_as_exhaustive
+    s, seen = crowd(A, H, W, K, hfov, vfov, spacing, size, walls)
+    busiest = np.sort(np.argsort(seen)[-3:])
+    pal = default_palette()
+    g = CudaRun(s)
+    try:
+        for aa in modes:
+            got, flags = g.render_rgb(pal, aa)
+            assert flags == 0, f"antialias {aa}: status {flags}"
+            # (a mismatch has to lie on a flagged pixel, so the share of those bounds the share of mismatches)
+            compare_colour(oracle.render_rgb(s, pal, aa, busiest), got[busiest], max_mismatch_frac=2e-2, max_flag_frac=2e-2)
+            for v in busiest:                              # the same views culled a warp per tile
+                alone, _ = g.render_rgb(pal, aa, view_first=int(v), view_count=1)
+                assert (alone[v] == got[v]).all()
+        a = g.render()
+        n = min(len(seen), 100)
+        assert_same_as_exhaustive(a, g.render(brute=True, view_first=0, view_count=n), slice(0, n))
+    finally:
+        g.close()
