@@ -681,32 +681,47 @@ __device__ __forceinline__ void append_survivor(uint2* __restrict__ surv, bool k
 }
 
 // Pixel box of camera-space vertices in a whole image, inclusive; false: no pixel centre (margin m) can be touched.  Where
-// pixel_box gives up because a vertex lies behind or close to the camera, the primitive is cut at the near depth -- nothing
-// nearer is kept -- and what remains is projected, so that a road under the camera reaches only the tiles it is seen in.
+// pixel_box gives up because a vertex lies behind or close to the camera, the primitive is cut a little before the near depth --
+// nothing nearer is kept -- and what remains is projected, so that a road under the camera reaches only the tiles it is seen in.
+//
+// The box has to hold every pixel that the edge functions and the 1/z plane, as they are evaluated, let through.  Against the exact
+// polygon, with L the largest vertex distance, h the plane's distance from the camera, and focal length f in pixels:
+//   1/z is off by 5e-7 L / h of itself: within the 1 % before the near depth while L / h <= 1e4;
+//   an edge function carries some 5 roundings of |V| |edge|, which moves its line by shift = 3e-7 f L / h pixels, and the corner
+//     of two lines by a few times that (8: down to an angle of a quarter; a thinner tip is narrower than the shift);
+//   the cut of an edge is off by 8 roundings of the edge's length, f |edge| / near times that in pixels (twice that is allowed, L
+//     being taken as a sum of three components and an edge as 2 L).
+// A plane too close to the camera for this (an edge-on one) keeps the whole image as its box.
 __device__ __forceinline__ bool view_box(const Cam& c, const TileCtx& t, const V3 (&V)[4], int& bx0, int& by0, int& bx1, int& by1, float m) {
     bool ok = pixel_box_int(c, t, V, bx0, by0, bx1, by1, m);
     if (ok && fminf(fminf(V[0].z, V[1].z), fminf(V[2].z, V[3].z)) < t.near_z * ZPROJ_FRAC) {
-        const float zc = t.near_z * 0.999f;
-        float sx0 = 3e38f, sx1 = -3e38f, sy0 = 3e38f, sy1 = -3e38f;
-        auto include = [&](float x, float y, float iz) {
-            const float sx = fm(c.focx, mul(x, iz), c.cx), sy = fm(c.focy, mul(y, iz), c.cy);
-            sx0 = fminf(sx0, sx); sx1 = fmaxf(sx1, sx); sy0 = fminf(sy0, sy); sy1 = fmaxf(sy1, sy);
-        };
-        const float izc = __fdividef(1.f, zc);
+        float reach = 0.f;
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const V3 a = V[i], b = V[(i + 1) & 3];
-            if (a.z >= zc) include(a.x, a.y, __fdividef(1.f, a.z));
-            if ((a.z < zc) != (b.z < zc)) {
-                const float u = __fdividef(zc - a.z, b.z - a.z);
-                include(fm(u, b.x - a.x, a.x), fm(u, b.y - a.y, a.y), izc);
+        for (int i = 0; i < 4; ++i) reach = fmaxf(reach, fabsf(V[i].x) + fabsf(V[i].y) + fabsf(V[i].z));
+        const V3 n = plane_normal(V, true);                  // (of a triangle too: its third vertex is there twice)
+        const float ratio = __fdividef(reach * sqrtf(vdot(n, n)), fabsf(vdot(n, V[0])));      // L / h
+        const float zc = t.near_z * 0.99f, izc = __fdividef(1.f, zc), f = fmaxf(c.focx, c.focy), shift = 3e-7f * f * ratio;
+        if (ratio <= 1e4f && shift <= 0.5f) {
+            const float mm = m + 0.25f + 8.f * shift + 2e-6f * f * reach * izc;               // (an edge is at most 2 L)
+            float sx0 = 3e38f, sx1 = -3e38f, sy0 = 3e38f, sy1 = -3e38f;
+            auto include = [&](float x, float y, float iz) {
+                const float sx = fm(c.focx, mul(x, iz), c.cx), sy = fm(c.focy, mul(y, iz), c.cy);
+                sx0 = fminf(sx0, sx); sx1 = fmaxf(sx1, sx); sy0 = fminf(sy0, sy); sy1 = fmaxf(sy1, sy);
+            };
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const V3 a = V[i], b = V[(i + 1) & 3];
+                if (a.z >= zc) include(a.x, a.y, __fdividef(1.f, a.z));
+                if ((a.z < zc) != (b.z < zc)) {
+                    const float u = __fdividef(zc - a.z, b.z - a.z);
+                    include(fm(u, b.x - a.x, a.x), fm(u, b.y - a.y, a.y), izc);
+                }
             }
+            const float fx0 = fmaxf(ceilf(sx0 - 0.5f - mm), 0.f), fx1 = fminf(floorf(sx1 - 0.5f + mm), (float)(t.tw - 1));
+            const float fy0 = fmaxf(ceilf(sy0 - 0.5f - mm), 0.f), fy1 = fminf(floorf(sy1 - 0.5f + mm), (float)(t.th - 1));
+            ok = fx0 <= fx1 && fy0 <= fy1;
+            bx0 = (int)fx0; by0 = (int)fy0; bx1 = (int)fx1; by1 = (int)fy1;
         }
-        const float mm = m + 0.25f;                          // (the cut of an edge of some hundred metres is good to a tenth of a pixel)
-        const float fx0 = fmaxf(ceilf(sx0 - 0.5f - mm), 0.f), fx1 = fminf(floorf(sx1 - 0.5f + mm), (float)(t.tw - 1));
-        const float fy0 = fmaxf(ceilf(sy0 - 0.5f - mm), 0.f), fy1 = fminf(floorf(sy1 - 0.5f + mm), (float)(t.th - 1));
-        ok = fx0 <= fx1 && fy0 <= fy1;
-        bx0 = (int)fx0; by0 = (int)fy0; bx1 = (int)fx1; by1 = (int)fy1;
     }
     return ok;
 }

@@ -258,3 +258,38 @@ def test_views_with_more_items_than_the_cull_list(A, H, W, K, hfov, vfov, spacin
         assert_same_as_exhaustive(a, g.render(brute=True, view_first=0, view_count=n), slice(0, n))
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("length,near,hfov,H,W,pitch", [
+    (300.0, 0.1, 46.0, 100, 384, 0.0),
+    (1000.0, 0.1, 90.0, 100, 192, 0.0),
+    (1000.0, 0.02, 46.0, 100, 384, 12.0),
+    (3000.0, 0.1, 46.0, 100, 384, -20.0),
+])
+def test_long_primitives_cut_at_the_near_plane(length, near, hfov, H, W, pitch):
+    """Triangles of hundreds of metres that pass the cameras at centimetres: where float32 puts their edges depends on focal length,
+    length and distance, and views culled as a whole must not lose a pixel of them."""
+    from scenes import default_palette
+    from tests.gpu_util import CudaRun
+    from tests.util import assert_same_as_exhaustive
+    rng = np.random.default_rng(int(length))
+    E, A, n = 40, 16, 40
+    unit = lambda v: v / np.linalg.norm(v)
+    tris = []
+    for _ in range(n):
+        along, side = unit(rng.normal(size=3) * [1, 1, 0.15]), unit(rng.normal(size=3) * [1, 1, 0.3])
+        o = np.array([rng.uniform(-3, 3), rng.uniform(-3, 3), 1.5 + rng.uniform(-0.6, 0.6)])
+        a, b = o + along * length * rng.uniform(0.3, 1.0), o - along * length * rng.uniform(0.3, 1.0)
+        tris.append([a, b, b + side * rng.uniform(0.2, 3.0)])
+    poses = rng.uniform(-3.0, 3.0, (E, A, 3)).astype(np.float32)
+    dims = np.full((E, A, 3), 0.01, np.float32)
+    rig = make_rig((0.0,), hfov, hfov * H / W, W, H, mount=(0.0, 0.0, 1.5), pitch_deg=pitch)
+    s = custom_scene(np.asarray(tris, np.float32), rng.integers(2, 9, n).astype(np.uint8), poses, dims, rig, H, W, near, 200.0, env_map_id=np.zeros(E, np.int32))
+    g = CudaRun(s)
+    try:
+        assert_same_as_exhaustive(g.render(), g.render(brute=True))
+        whole, flags = g.render_rgb(default_palette(), True)
+        part, flags_part = g.render_rgb(default_palette(), True, view_first=0, view_count=50)       # culled a warp per tile
+        assert flags == flags_part == 0 and (np.abs(whole[:50].astype(int) - part[:50].astype(int)) <= 1).all()
+    finally:
+        g.close()
