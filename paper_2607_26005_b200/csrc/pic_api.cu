@@ -504,14 +504,20 @@ pic_status pic_render_host(pic_scene* s, const float* poses, const float* dims, 
     pic_status st = render_from(s, s->d_in_poses, nullptr, nullptr, s->d_in_dims, active ? s->d_in_active : nullptr, rig,
                                 s->d_out_class, s->d_out_depth, stream, nullptr, false, chunks);
     if (st != PIC_OK) return st;
-    for (int c = 0; c < chunks; ++c) {
+    cudaError_t ce = cudaSuccess;
+    for (int c = 0; c < chunks && ce == cudaSuccess; ++c) {
         const size_t p0 = (size_t)(n_views * c / chunks) * per_view, p1 = (size_t)(n_views * (c + 1) / chunks) * per_view;
         const cudaStream_t to = chunks > 1 ? s->copy_stream : stream;
-        if (chunks > 1) CUDA_TRY(cudaStreamWaitEvent(to, s->copy_ev[c], 0));
-        CUDA_TRY(cudaMemcpyAsync(out_class + p0, s->d_out_class + p0, p1 - p0, cudaMemcpyDeviceToHost, to));
-        CUDA_TRY(cudaMemcpyAsync(out_depth + p0, s->d_out_depth + p0, sizeof(uint16_t) * (p1 - p0), cudaMemcpyDeviceToHost, to));
+        if (chunks > 1) ce = cudaStreamWaitEvent(to, s->copy_ev[c], 0);
+        if (ce == cudaSuccess) ce = cudaMemcpyAsync(out_class + p0, s->d_out_class + p0, p1 - p0, cudaMemcpyDeviceToHost, to);
+        if (ce == cudaSuccess) ce = cudaMemcpyAsync(out_depth + p0, s->d_out_depth + p0, sizeof(uint16_t) * (p1 - p0), cudaMemcpyDeviceToHost, to);
     }
-    if (chunks > 1) CUDA_TRY(cudaStreamSynchronize(s->copy_stream));
+    // (also after an error: no copy into the caller's memory may go on on a stream that the caller cannot wait for)
+    if (chunks > 1) {
+        const cudaError_t waited = cudaStreamSynchronize(s->copy_stream);
+        if (ce == cudaSuccess) ce = waited;
+    }
+    if (ce != cudaSuccess) return fail(PIC_ERR_CUDA, "copying the images to the host: %s", cudaGetErrorString(ce));
     CUDA_TRY(cudaStreamSynchronize(stream));
     return PIC_OK;
 }
