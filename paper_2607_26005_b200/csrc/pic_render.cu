@@ -298,7 +298,6 @@ __device__ __forceinline__ void raster_records(S& s, const float4* rec, uint32_t
     for (int p = 0; p < n_rec; ++p) {
         const float4* r = &rec[p * (REC / 4)];
         const uint32_t bw = __float_as_uint(r[4].x);
-        if (bw >> 28) continue;                  // rasterized by its own thread, or degenerate
         const int bx0 = bw & 63, by0 = (bw >> 6) & 63, bx1 = (bw >> 12) & 63, by1 = (bw >> 18) & 63;
         // first band of this warp at or after the box's first band
         const int band0 = by0 >> 2, band1 = by1 >> 2;
@@ -357,11 +356,10 @@ __device__ __forceinline__ void raster_records(S& s, const float4* rec, uint32_t
     if (lane == 0 && touched) mark_touched(touched_out, touched);
 }
 
-// (d) keys -> class / depth images.  `touched`: the 8x8 blocks that may hold a fragment; with
-// `clear`, the keys that were read are reset to "no fragment" for the next tile.
+// (d) keys -> class / depth images.  `touched`: the 8x8 blocks that may hold a fragment.
 template <class S>
 __device__ __forceinline__ void store_tile(S& s, const TileCtx& t, const RenderParams& P, size_t view, int k, bool ego_active,
-                                           unsigned long long touched, bool clear, int tid = threadIdx.x, int nthr = NTHREADS,
+                                           unsigned long long touched, int tid = threadIdx.x, int nthr = NTHREADS,
                                            uint32_t n_map_tris = 0u) {
     const size_t img = (size_t)P.H * P.W;
     uint32_t* occ = P.occlusion ? P.occlusion + view * (size_t)P.A * 2u : nullptr;   // visible-pixel counts of this view
@@ -395,9 +393,7 @@ __device__ __forceinline__ void store_tile(S& s, const TileCtx& t, const RenderP
             } else {
 #pragma unroll
                 for (int j = 0; j < 16; j += 2) {
-                    ulonglong2* kp = reinterpret_cast<ulonglong2*>(&s.key[key_index(xs + j, y)]);
-                    const ulonglong2 kk = *kp;
-                    if (clear) *kp = make_ulonglong2(0ull, 0ull);
+                    const ulonglong2 kk = *reinterpret_cast<const ulonglong2*>(&s.key[key_index(xs + j, y)]);
                     if (occ) { count_visible(occ, kk.x, n_map_tris); count_visible(occ, kk.y, n_map_tris); }
                     const float z0 = kk.x ? fast_rcp(__uint_as_float((uint32_t)(kk.x >> 32))) : bg_z;
                     const float z1 = kk.y ? fast_rcp(__uint_as_float((uint32_t)(kk.y >> 32))) : bg_z;
@@ -413,7 +409,6 @@ __device__ __forceinline__ void store_tile(S& s, const TileCtx& t, const RenderP
         } else {
             for (int j = 0; j < 16 && xs + j < t.tw; ++j) {
                 const unsigned long long key = empty ? 0ull : s.key[key_index(xs + j, y)];
-                if (clear && !empty) s.key[key_index(xs + j, y)] = 0ull;
                 if (occ) count_visible(occ, key, n_map_tris);
                 const float z = key ? fast_rcp(__uint_as_float((uint32_t)(key >> 32))) : bg_z;
                 oc[o + j] = (uint8_t)(key ? (uint32_t)(key & 0xff) : bg_cls);
@@ -590,7 +585,7 @@ __device__ __forceinline__ void cooperative_job(TileSmem& s, const RenderParams&
         __syncthreads();
     }
     // ---- phase 4 (d)
-    store_tile(s, t, P, view, k, ego_active, ((unsigned long long)s.touched[1] << 32) | s.touched[0], false, threadIdx.x, NT, mi.n_tris);
+    store_tile(s, t, P, view, k, ego_active, ((unsigned long long)s.touched[1] << 32) | s.touched[0], threadIdx.x, NT, mi.n_tris);
     if (threadIdx.x == 0) { ++n.jobs; ++n.coop; }
 }
 

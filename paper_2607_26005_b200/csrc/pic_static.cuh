@@ -129,7 +129,7 @@ __global__ void __launch_bounds__(NTHREADS, 4) render_static_kernel(const __grid
             ns = 0;
         }
     }
-    store_tile(s, t, P, job.view, job.k, ego_active, ((unsigned long long)s.touched[1] << 32) | s.touched[0], false);
+    store_tile(s, t, P, job.view, job.k, ego_active, ((unsigned long long)s.touched[1] << 32) | s.touched[0]);
 }
 
 cudaError_t configure_static_kernel() {
