@@ -74,6 +74,35 @@ class CudaRun:
         self.scene.close()
 
 
+def check_in_a_large_call(scene, images, palette=None, colours=None):
+    """The scene repeated over so many environments that its call takes the kernels for many tiles, and views of several tiles
+    are culled as a whole: `images` (class, f16, f32 depth of a call of few tiles; None: not compared) and `colours` ({antialias:
+    RGB}) have to come out again in every copy."""
+    import torch
+    from tests.util import repeated
+    V, tiles = scene.E * scene.A * scene.K, -(-scene.H // 64) * -(-scene.W // 64)
+    sm = torch.cuda.get_device_properties(0).multi_processor_count
+    views = max(8 * sm // tiles + 1, 10 * sm if tiles > 1 else 0)
+    big = CudaRun(repeated(scene, -(-views // V)))
+    try:
+        same = lambda got, want: (got.reshape((-1,) + want.shape) == want).all()
+        for depth32 in (True, False) if images is not None else ():
+            cls, d16, d32 = big.render(depth32=depth32)
+            assert same(cls, images[0]) and same(d16.view(np.uint16), images[1].view(np.uint16)) and (d32 is None or same(d32, images[2])), \
+                "a call of many tiles gives other images than one of few"
+        for aa, want in (colours or {}).items():
+            got, flags = big.render_rgb(palette, aa)
+            off = np.abs(got.reshape((-1,) + want.shape).astype(np.int16) - want).max(axis=(0, -1))
+            assert flags == 0 and (aa or off.max() == 0), f"antialias {aa}: a call of many tiles is {off.max()} levels off, status {flags}"
+            if off.max() > 1:
+                # the same coverages, but composited in another order where depths are equal: only where the oracle says so
+                import oracle
+                flagged = (oracle.render_rgb(scene, palette, aa).flag & 47) != 0
+                assert not (off[~flagged] > 1).any(), f"antialiased: a call of many tiles is {off[~flagged].max()} levels off at an unflagged pixel"
+    finally:
+        big.close()
+
+
 def check_against_oracle(scene, view_ids=None, gpu: CudaRun = None, **kw):
     """Render `view_ids` with the oracle and all views with the CUDA path; apply the acceptance rule."""
     import oracle
@@ -86,6 +115,7 @@ def check_against_oracle(scene, view_ids=None, gpu: CudaRun = None, **kw):
         # without the float32 depth image the kernels take their vector-store paths: same images
         cls_v, d16_v, _ = gpu.render(depth32=False)
         assert (cls_v == cls).all() and (d16_v.view(np.uint16) == d16.view(np.uint16)).all()
+        check_in_a_large_call(scene, (cls, d16, d32))
         if view_ids is None:
             view_ids = np.arange(scene.E * scene.A * scene.K)
         view_ids = np.asarray(view_ids, dtype=np.int64)

@@ -22,9 +22,9 @@ def gu():
 
 
 def _sample_and_check(gu, s, n_oracle, n_brute, seed, env0_views=None):
-    """Full-size run in the launch configuration the benchmark times (no float32 depth image: the full-tile
-    kernels), compared with the oracle on `n_oracle` seeded views plus every view of environment 0; the same
-    views once more with the float32 depth image (the general kernels) at the literal 1e-4 depth tolerance; and a
+    """Full-size run in the launch configuration the benchmark times (no float32 depth image: vector stores),
+    compared with the oracle on `n_oracle` seeded views plus every view of environment 0; the same
+    views once more with the float32 depth image (scalar stores) at the literal 1e-4 depth tolerance; and a
     window of `n_brute` views against the exhaustive kernel."""
     import oracle
     g = gu.CudaRun(s)

@@ -25,8 +25,7 @@ def test_fuzz_scenes_match_oracle_and_exhaustive_kernel():
             cls, d16, d32 = g.render()
             b = g.render(brute=True)
             assert_same_as_exhaustive((cls, d16, d32), b)
-            # without the float32 depth image the kernels take their vector-store paths and, for
-            # images made of full tiles, their full-tile instantiations: the same images
+            # without the float32 depth image the kernels take their vector-store paths: the same images
             cls_v, d16_v, _ = g.render(depth32=False)
             assert (cls_v == cls).all() and (d16_v.view(np.uint16) == d16.view(np.uint16)).all()
             ref = oracle.render(s)
@@ -38,3 +37,23 @@ def test_fuzz_scenes_match_oracle_and_exhaustive_kernel():
         finally:
             g.close()
     assert flagged < 0.02 * pixels
+
+
+def test_fuzz_scenes_in_calls_of_many_tiles():
+    """The same scenes repeated over enough environments for the kernels that work tile by tile, and for views culled as a
+    whole (which meet pitched cameras and triangles through the camera plane here): class, depth and colour images."""
+    from scenes import default_palette
+    from tests.gpu_util import CudaRun, check_in_a_large_call
+    pal = default_palette()
+    for i, seed in enumerate(SEEDS):
+        s = random_scene(seed, full_tiles=(i % 3 == 2))
+        g = CudaRun(s)
+        try:
+            images = g.render()
+            colours = {aa: g.render_rgb(pal, aa)[0] for aa in (False, True)}
+        finally:
+            g.close()
+        try:
+            check_in_a_large_call(s, images, pal, colours)
+        except AssertionError as ex:
+            raise AssertionError(f"seed {seed}: {ex}") from ex

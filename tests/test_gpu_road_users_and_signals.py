@@ -1,6 +1,6 @@
 """Road users with their own class and triangles with a limited angular range (traffic-light disks as fans),
-through the C ABI against the oracle: every kernel that sets a primitive up -- the full-tile kernels, the general
-kernels, the cooperative kernel alone, the exhaustive kernel -- must drop a triangle outside its range alike and
+through the C ABI against the oracle: every kernel that sets a primitive up -- the few-tile kernel, the tile
+kernel, the cooperative kernel alone, the exhaustive kernel -- must drop a triangle outside its range alike and
 write each agent's own class."""
 import numpy as np
 import pytest
@@ -81,7 +81,7 @@ def test_platoons_with_pedestrians_cyclists_and_signals(gu):
 
 
 def test_disk_at_its_limit_and_ragged_tiles(gu):
-    # one disk straight ahead, the ego turning from 0 to 60 degrees off its normal in steps; 70 x 100 images (general kernels)
+    # one disk straight ahead, the ego turning from 0 to 60 degrees off its normal in steps; 70 x 100 images (ragged tiles)
     rig = make_rig((0.0,), 80.0, 60.0, 100, 70, mount=(0.0, 0.0, 1.0))
     tris = disk_triangles((9.0, 0.0, 1.2), (-1.0, 0.0, 0.0), 0.7, n=16)
     angs = np.radians(np.arange(0.0, 61.0, 5.0))

@@ -1,6 +1,8 @@
 """Shared helpers of the test-suite: hand-made scenes and the acceptance rule."""
 from __future__ import annotations
 
+import dataclasses
+
 import numpy as np
 
 from scenes import custom_scene, make_rig, NOMINAL_DIMS, MOUNT
@@ -71,11 +73,18 @@ def assert_same_as_exhaustive(prod, brute, sl=slice(None)):
     assert (np.abs(a - b) <= 5e-7 * b).all(), "depths differ between the production and the exhaustive kernel"
 
 
+def repeated(scene, n: int):
+    """The scene's environments n times over, on the same maps."""
+    rep = lambda a: None if a is None else np.concatenate([a] * n)
+    return dataclasses.replace(scene, E=scene.E * n, env_map_id=rep(scene.env_map_id), poses=rep(scene.poses), dims=rep(scene.dims),
+                               active=rep(scene.active), speed=rep(scene.speed), agent_classes=rep(scene.agent_classes))
+
+
 def random_scene(seed: int, full_tiles: bool = False):
     """A seeded random scene for fuzzing: triangle soups far from the origin with planar quad pairs
     and a degenerate triangle, random rigs (mounts, yaw, pitch up to 0.5 rad, unequal focal lengths),
-    random image sizes incl. ragged ones (`full_tiles`: multiples of 64 only, the sizes that take the
-    kernels' full-tile instantiations), random near/far, inactive agents."""
+    random image sizes incl. ragged ones (`full_tiles`: multiples of 64 only, whose tiles are all whole),
+    random near/far, inactive agents."""
     car = (4.5, 1.9, 1.5)
     rng = np.random.default_rng(seed)
     H = int(rng.choice([16, 36, 54, 64, 70, 128])); W = int(rng.choice([16, 48, 64, 96, 100, 160]))
