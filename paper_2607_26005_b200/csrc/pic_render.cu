@@ -1274,14 +1274,21 @@ static cudaError_t run_coverage(const RenderParams& P, long long n_views, cudaSt
     return cudaGetLastError();
 }
 
-// The cull pass of a call.  Views of several tiles are culled a warp per view while that leaves enough warps to hide the
-// latency of each: measured, the two ways meet at about 600 views of 8 tiles (city) and 1 400 of 2 tiles (96 x 54); at 4 096
-// views of 8 tiles the call takes 653 instead of 1 008 us.
+// The cull pass of a call.  Views of several tiles (as many as a warp has lanes) are culled a warp per view while that leaves
+// enough warps to hide the latency of each; a view then does the work of its tiles at once, so the line is a number of tiles.
+// Measured, time culled per tile / per view at so many views per multiprocessor (class and depth, maps of 5 640 / 1 950 triangles):
+//    2 tiles   8: 0.98 / 0.94   10: 1.00 / 0.98   12: 1.00 / 1.01   16: 1.06 / 1.08
+//    4 tiles   5: 1.00 / 0.91    6: 0.97 / 0.96    8: 1.07 / 1.09   12: 1.08 / 1.12
+//    8 tiles   3: 0.95 / 0.91    4: 1.00 / 1.05    6: 1.07 / 1.14   10: 1.10 / 1.21
+//   16 tiles   1: 0.92 / 0.96    2: 1.01 / 1.09    4: 1.12 / 1.19   10: 1.21 / 1.30
+//   32 tiles   1: 0.99 / 1.05    2: 1.05 / 1.17    4: 1.15 / 1.28    8: 1.33 / 1.39
+// (antialiased colour: the same lines, 0.96 to 1.08).
+constexpr int VIEW_CULL_TILES = 28;        // tiles per multiprocessor from which views are culled as a whole
 template <class K>
 cudaError_t launch_next(K kernel, unsigned grid, size_t smem, cudaStream_t stream, const RenderParams& P, unsigned threads = NTHREADS);
 static cudaError_t launch_cull(const RenderParams& P, long long n_views, bool conservative, int sm_count, cudaStream_t stream) {
     const int tiles = P.tiles_x * P.tiles_y;
-    if (!P.counters && !(P.debug_flags & 4) && tiles > 1 && tiles <= 32 && n_views >= (tiles > 2 ? 4 : 10) * (long long)sm_count)
+    if (!P.counters && !(P.debug_flags & 4) && tiles > 1 && tiles <= 32 && n_views * tiles >= VIEW_CULL_TILES * (long long)sm_count)
         return launch_next(conservative ? cull_kernel<NoTally, true, true> : cull_kernel<NoTally, false, true>, (unsigned)((n_views + NW - 1) / NW), sizeof(CullSmem), stream, P);
     const unsigned grid = (P.n_jobs + NW - 1) / NW;
     return launch_next(P.counters ? cull_kernel<Tally, false> : conservative ? cull_kernel<NoTally, true> : cull_kernel<NoTally, false>, grid, sizeof(CullSmem), stream, P);

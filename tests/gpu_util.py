@@ -82,7 +82,7 @@ def check_in_a_large_call(scene, images, palette=None, colours=None):
     from tests.util import repeated
     V, tiles = scene.E * scene.A * scene.K, -(-scene.H // 64) * -(-scene.W // 64)
     sm = torch.cuda.get_device_properties(0).multi_processor_count
-    views = max(8 * sm // tiles + 1, 10 * sm if tiles > 1 else 0)
+    views = (28 * sm if tiles > 1 else 8 * sm) // tiles + 1
     big = CudaRun(repeated(scene, -(-views // V)))
     try:
         same = lambda got, want: (got.reshape((-1,) + want.shape) == want).all()

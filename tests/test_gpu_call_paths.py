@@ -118,8 +118,11 @@ def test_antialiased_primitives_around_the_size_limit(side, far):
 @pytest.mark.parametrize("n_tris,E,A,H,W,K,spread", [
     (300, 4, 50, 65, 129, 4, 60.0),       # 800 views of 6 tiles, the last row and column of one pixel: culled a warp per view
     (300, 8, 50, 64, 70, 4, 60.0),        # 1 600 views of 2 tiles
+    (300, 37, 14, 64, 70, 4, 60.0),       # 2 072 of them: the fewest that are culled as a whole (on 148 multiprocessors)
+    (100, 5, 26, 250, 500, 1, 40.0),      # 130 views of 32 tiles: as many tiles
     (40, 2, 75, 30, 1990, 4, 6.0),        # the most tiles a view can have there (32), large primitives under the cameras
-    (2000, 4, 38, 130, 80, 4, 10.0),      # tiles whose survivor lists overflow
+    (2000, 4, 38, 130, 80, 4, 10.0),      # tiles whose survivor lists overflow ...
+    (2000, 5, 38, 130, 80, 4, 10.0),      # ... in views culled as a whole
 ])
 def test_views_of_several_tiles(n_tris, E, A, H, W, K, spread):
     test_calls_with_few_tiles(n_tris, E, A, H, W, K, spread)
@@ -273,7 +276,7 @@ def test_long_primitives_cut_at_the_near_plane(length, near, hfov, H, W, pitch):
     from tests.gpu_util import CudaRun
     from tests.util import assert_same_as_exhaustive
     rng = np.random.default_rng(int(length))
-    E, A, n = 40, 16, 40
+    E, A, n = 44, 16, 40
     unit = lambda v: v / np.linalg.norm(v)
     tris = []
     for _ in range(n):
