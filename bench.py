@@ -453,7 +453,7 @@ def run_cuda(args, rank: int, world: int, local_rank: int) -> None:
             "cpu_baseline": {"value": cpu_value, "unit": "agent-steps/s", "cores": min(cores, 64), "kind": "oracle",
                              "sample": f"{len(or_views)} seeded views of this workload in {t_or:.1f} s"},
             "colour": None if colour is None else {
-                "entry": "pic_render_rgb (u8 RGB, 3 B per pixel) on the same chunk; cull_kernel + colour_kernel between the library's events",
+                "entry": "pic_render_rgb (u8 RGB, 3 B per pixel) on the same chunk; cull_kernel and render_tile_kernel (plain) or colour_kernel (antialiased) between the library's events",
                 **{("antialiased" if aa else "plain"): {
                     "kernel_ms_median": float(np.median(k)), "kernel_ms_min": float(np.min(k)), "calls": int(len(k)),
                     "agent_steps_per_s": n_active / (float(np.median(k)) * 1e-3), "images_per_s": n_active * s.K / (float(np.median(k)) * 1e-3),

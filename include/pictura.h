@@ -173,10 +173,11 @@ pic_status pic_get_status(pic_scene* scene, uint32_t* flags, void* cuda_stream);
  *   PIC_OPT_DEPTH32       value = dev f32* [E,A,K,H,W] (as uintptr) or 0: also write the float32
  *                         depth the binary16 image was rounded from.
  *   PIC_OPT_COUNTERS      value = dev u64* [16] (as uintptr) or 0: accumulate work counters (tiles,
- *                         group tests, leaf tests, primitives tested, set up, rasterized by their
- *                         thread, records, record-list overflows, records classified per cell (once
- *                         per 16-row strip they reach), cells visited, tiles rendered by the
- *                         cooperative kernel).
+ *                         grid-row or group tests, leaf tests, primitives tested, set up, of which
+ *                         small ones worked off pixel by pixel, records, record-list overflows of the
+ *                         cooperative kernel, records classified per cell, cells visited, tiles
+ *                         rendered by the cooperative kernel).  Calls of few tiles take the kernels
+ *                         for many tiles then.
  *   PIC_OPT_VIEW_FIRST,   render only views [first, first + count) (flat index (e*A + a)*K + k);
  *   PIC_OPT_VIEW_COUNT    count 0 = through the last view.  Other views' pixels are left untouched.
  *   PIC_OPT_OCCLUSION     value = dev u32* [E,A,K,A,2] (as uintptr) or 0: per view and per OTHER agent b of the
@@ -186,18 +187,19 @@ pic_status pic_get_status(pic_scene* scene, uint32_t* flags, void* cuda_stream);
  *                         user's occlusion percentage as the renderer sees it (Sec. 5.2, counterfactual
  *                         probes; the paper gives no formula, this is the reading taken).  Entries of the
  *                         ego itself and of inactive agents are 0; the entries of the rendered views are
- *                         overwritten, indexed by absolute view.  Costs an extra pass over the agents' boxes
- *                         and selects the general kernels.
+ *                         overwritten, indexed by absolute view.  Costs an extra pass over the agents' boxes;
+ *                         calls of few tiles take the kernels for many tiles.
  *   PIC_OPT_OUT_RELATIVE  1: out_class / out_depth (and the PIC_OPT_DEPTH32 image) hold only the rendered
  *                         views, the first rendered view at offset 0 -- so a batch can be streamed in
  *                         passes through buffers of count*H*W pixels (the paper's renderer likewise
  *                         streams a batch in passes bounded by free memory, App. "Renderer memory
  *                         usage"); 0: the images are indexed by absolute view.
  *   PIC_OPT_DEBUG_FLAGS   bit 0: rasterize large primitives without the per-cell trivial
- *                         accept/reject; bit 1: shrink the fused kernel's record pool and the
- *                         cooperative kernel's record list to 2 entries so that the overflow paths
+ *                         accept/reject; bit 1: shrink the tile kernel's and the
+ *                         cooperative kernel's record lists to 2 entries so that the overflow paths
  *                         run; bit 2: send every tile to the cooperative kernel; bit 3: shrink the
- *                         record lists to 6 entries so that both kernels share the tiles.  All leave the
+ *                         tile kernel's list to 6 entries so that both kernels share the tiles.  Any of
+ *                         them also keeps calls of few tiles from the kernel for those.  All leave the
  *                         images unchanged (tests rely on it); other bits are ignored.
  *   PIC_OPT_TIMING        1: bracket the render kernels of every call with CUDA events on its stream
  *                         (up to 1024 launches between two pic_get_kernel_times calls); 0: off.
@@ -271,17 +273,18 @@ pic_status pic_step_rgb(pic_scene* scene, const float* actions, const pic_camera
  * a tool that must keep working when the device is nearly full.  pic_scene_create allocates (map
  * copy, hierarchy, per-agent and per-view buffers), so those callers cannot use the scene API.
  *
- * What it does: the same image definition as pic_render, computed by a variant of the exhaustive
- * kernel that reads the caller's triangles directly (one map shared by all environments, every
- * triangle against every pixel -- meant for small batches and small maps).  Per-agent geometry,
+ * What it does: the same image definition as pic_render, computed by a kernel that reads the
+ * caller's triangles directly (one map shared by all environments, every triangle tested against
+ * every tile, those that reach it rasterized -- meant for small batches and small maps).  Per-agent geometry,
  * per-view cameras, per-camera tables and the status word live in one fixed device array that is
  * part of the library image (about 490 KB on every device that loads the library, until exit).
  * The call itself uses no cudaMalloc/cudaFree and no allocating library routine.
  *
  * Limits (PIC_ERR_CAPACITY beyond them): E*A <= PIC_STATIC_MAX_AGENTS, E*A*K <= PIC_STATIC_MAX_VIEWS,
- * H, W <= PIC_STATIC_MAX_SIDE, n_tris <= PIC_STATIC_MAX_TRIS, K <= 16, and, because every primitive
- * is tested against every pixel of every view by one launch that cannot be interrupted,
- * (n_tris + 6*A) * E*A*K*H*W <= PIC_STATIC_MAX_WORK (a few tenths of a second on a B200).
+ * H, W <= PIC_STATIC_MAX_SIDE, n_tris <= PIC_STATIC_MAX_TRIS, K <= 16, and, because one launch that
+ * cannot be interrupted does all the work and every primitive may cover every pixel,
+ * (n_tris + 6*A) * E*A*K*H*W <= PIC_STATIC_MAX_WORK (such a request takes a few tenths of a second at
+ * worst, ordinary ones far less).
  *
  *   tri_xyz    dev f32 [n_tris,3,3], tri_class dev u8 [n_tris]   (may be NULL when n_tris == 0)
  *   poses, dims, active, rig, out_class, out_depth: as in pic_render (outputs need no alignment)

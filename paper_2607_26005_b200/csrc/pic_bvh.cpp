@@ -4,8 +4,8 @@
 // (two consecutive triangles of one class sharing an edge: road, marking and wall quads), then
 // sorted along a Morton curve and cut into leaves of up to LEAF_PRIMS primitives; leaves are
 // grouped by GROUP_LEAVES.  Primitives much longer than the average get leaves of their own, so
-// that one long road quad does not inflate the box of its neighbouring lane markings.  The renderer tests group boxes, then
-// leaf boxes, then primitives against each view frustum.
+// that one long road quad does not inflate the box of its neighbouring lane markings.  The cooperative kernel tests group
+// boxes, then leaf boxes, then primitives against a tile's frustum.
 //
 // The cull kernel uses a second, flatter structure over the same primitives: a uniform grid on
 // the ground plane.  A primitive whose box (xy) has a half-diagonal of at most half a cell is

@@ -16,7 +16,7 @@
 //                 is full.
 //
 // Structure: the cull kernel's survivor lists (made with conservative pixel boxes when antialiasing) are set up
-// into a record pool shared by the CTA's four tiles, in rounds like render_full_kernel; 8-row strips are tasks.
+// into a record pool shared by the CTA's four tiles, as many tiles at a time as fit it; 8-row strips are tasks.
 // A strip keeps, per pixel, the nearest FULLY covering fragment as a 64-bit key (unsigned max, as in the other
 // kernels, with the record's slot in the low byte) and a linked list of the partially covering fragments in
 // front of it (1/z, coverage in 14 bits, slot); the strip's warp owns both, so no atomics are needed.  The
@@ -546,8 +546,8 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
             // or, when the fragment array overflows (a dense soup of edges), half as many, again and again down to one
             // row -- the window is rasterized anew, the rows before it keep their composited colours (parked in their
             // keys, which no fragment can replace).  Before the first such retry the strip is rasterized once with an
-            // empty window: that leaves every pixel's nearest fully covering fragment in its key, so the retries keep
-            // only the fragments in front of it (in a soup, few).  A single row that still overflows (many coplanar
+            // empty window: that leaves every pixel's nearest full cover by a large record in its key (small records
+            // take no part in it), so the retries keep only the fragments in front of it (in a soup, few).  A single row that still overflows (many coplanar
             // primitives cut by the near plane along it) is taken half as many columns at a time, down to one pixel.
             int win = CSTRIP, cw = TILE, row_next = 0, col_next = 0;
             bool prepass = false, prepass_done = false;

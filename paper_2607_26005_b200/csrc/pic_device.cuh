@@ -131,7 +131,7 @@ __device__ __forceinline__ V3 plane_normal_world(const Cam& c, const float (&v)[
 // Returns false for degenerate / edge-on primitives (D == 0), which cover nothing.
 __device__ __forceinline__ bool prim_equations(const V3 (&V)[4], bool quad, uint32_t flags, const V3 P, PrimEq& q) {
     const float D = vdot(P, V[0]);
-    if (!(D != 0.f)) return false;               // also drops NaN
+    if (D == 0.f) return false;                  // (a NaN covers nothing either: it fails every comparison of a fragment)
     const float s = D < 0.f ? -1.f : 1.f;
     uint32_t tl = 0;
 #pragma unroll

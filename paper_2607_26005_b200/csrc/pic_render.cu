@@ -1087,7 +1087,7 @@ struct __align__(16) CullSmem {
     FrontLists lists[NW];
 };
 
-constexpr int CULL_CTAS = 7;       // CTAs per multiprocessor the cull kernel's registers are bounded for (rollout 256x32x4: 5 256, 6 249.9, 7 247.1, 8 246.1 us; city: 661, 658, 656, 660)
+constexpr int CULL_CTAS = 7;       // CTAs per multiprocessor the cull kernel's registers are bounded for (8 192 agents, a tile per view: 5 256.8, 6 248.7, 7 243.4, 8 245.1 us; views of 8 tiles: 662.5, 659.4, 656.5, 660.5)
 // MULTI: a warp per view of several tiles (P.n_jobs counts tiles all the same).
 template <class TL, bool CONS, bool MULTI = false>
 __global__ void __launch_bounds__(NTHREADS, CULL_CTAS) cull_kernel(const __grid_constant__ RenderParams P) {

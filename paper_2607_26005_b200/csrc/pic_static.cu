@@ -79,8 +79,8 @@ extern "C" pic_status pic_render_static(const pic_static_desc* d, const float* t
         return fail(PIC_ERR_CAPACITY, "pic_render_static renders images up to %d x %d, got %d x %d", kMaxSide, kMaxSide, d->H, d->W);
     if (d->n_tris > PIC_STATIC_MAX_TRIS) return fail(PIC_ERR_CAPACITY, "pic_render_static reads at most %d triangles, got %d", PIC_STATIC_MAX_TRIS, d->n_tris);
     {
-        // every primitive is tested against every pixel of every view: bound the product, so that a
-        // request at all the limits at once cannot occupy the GPU for hours
+        // any primitive may cover every pixel of every view: bound the product, so that a request at all
+        // the limits at once cannot occupy the GPU for hours
         const double work = ((double)d->n_tris + 6.0 * d->A) * (double)d->E * d->A * d->K * (double)d->H * d->W;
         if (work > (double)PIC_STATIC_MAX_WORK)
             return fail(PIC_ERR_CAPACITY, "pic_render_static: (n_tris + 6A) * E*A*K*H*W = %.3g primitive-pixel tests, at most %.3g", work,

@@ -6,7 +6,7 @@
 
 namespace pic {
 
-constexpr int TILE = 64;        // a view is rendered in tiles of up to TILE x TILE pixels (one CTA each)
+constexpr int TILE = 64;        // a view is rendered in tiles of up to TILE x TILE pixels
 constexpr int MAX_CAMS = 16;    // cameras per rig
 constexpr int LEAF_PRIMS = 8;   // primitives per leaf (8 threads per leaf in the cull pass)
 constexpr int LONG_LEAF_PRIMS = 8;   // long primitives get leaves of their own so the others' boxes stay tight
@@ -56,7 +56,7 @@ struct MapInfo {
 };
 static_assert(sizeof(MapInfo) == 64, "MapInfo must be 64 bytes");
 
-// Per-agent geometry written once per render by the agent kernel; 32 bytes.
+// Per-agent geometry written once per render by the set-up kernel; 32 bytes.
 struct AgentGeom {
     float x, y;       // box centre on the ground plane
     float c, s;       // cos, sin of the heading
@@ -70,7 +70,7 @@ struct CamConst {
     float fx, fy;
 };
 
-// Per-view camera written by the agent kernel: ego position, mount and rotation rows; 64 bytes.
+// Per-view camera written by the set-up kernel: ego position, mount and rotation rows; 64 bytes.
 struct ViewCam {
     float px, py;              // ego position
     float mwx, mwy, mwz;       // mount in world axes
