@@ -404,12 +404,14 @@ __global__ void __launch_bounds__(32, TILE_CTAS) render_tile_kernel(const __grid
     const uint32_t* bg_cls = P.rig.bg_cls + (size_t)job.k * P.H + t.y0;
     const float* bg_z = P.rig.bg_z + (size_t)job.k * P.H + t.y0;
     uint32_t* occ = (OCC && P.occlusion) ? P.occlusion + job.view * (size_t)P.A * 2u : nullptr;   // visible-pixel counts of this view
-    // cells that hold anything
-    uint32_t busy = __ballot_sync(0xffffffffu, hit != 0u);
+    // cells that hold anything, and those with fragments: only they look for them (64 views of 128 x 256 per environment of a large map,
+    // many tiles with more than 32 fragments: 655 us with every busy cell going through the list, 630 with this mask)
+    uint32_t busy = __ballot_sync(0xffffffffu, hit != 0u), frag_cells = 0u;
     if (n_frag > 0) {
-        uint32_t fc = lane < n_frag ? 1u << (my_frag >> 7) : 0u;
-        for (int f = 32 + lane; f < n_frag; f += 32) fc |= 1u << (s.frag_px[f] >> 7);
-        busy |= __reduce_or_sync(0xffffffffu, fc);
+        frag_cells = lane < n_frag ? 1u << (my_frag >> 7) : 0u;
+        for (int f = 32 + lane; f < n_frag; f += 32) frag_cells |= 1u << (s.frag_px[f] >> 7);
+        frag_cells = __reduce_or_sync(0xffffffffu, frag_cells);
+        busy |= frag_cells;
     }
     // ---- the background of the other cells
     if (VEC && RGB) store_background_rgb(P, tile0, t, ego_active, bg_cls, busy, lane);
@@ -423,7 +425,7 @@ __global__ void __launch_bounds__(32, TILE_CTAS) render_tile_kernel(const __grid
         const int x = (cell & 1) * CELL_W + px, y = (cell >> 1) * CELL_H + py;
         const uint32_t m = __shfl_sync(0xffffffffu, hit, cell);
         unsigned long long best[4] = {0ull, 0ull, 0ull, 0ull};
-        if (n_frag > 0 && __any_sync(0xffffffffu, (int)(my_frag >> 7) == cell || n_frag > 32)) {   // the cell's fragments meet in shared memory
+        if ((frag_cells >> cell) & 1u) {                     // the cell's fragments meet in shared memory
             if ((int)(my_frag >> 7) == cell) atomicMax(&s.cell_key[my_frag & 127u], my_key);
             for (int f = 32 + lane; f < n_frag; f += 32) {
                 const uint32_t fp = s.frag_px[f];
