@@ -12,6 +12,7 @@ struct RigParams {
     int32_t K, W, H;
     float far_z;
     uint32_t cls_sky, cls_ground;
+    const uint32_t* palette;      // NULL: no colours are rendered
     CamConst cam[MAX_CAMS];
 };
 
@@ -96,7 +97,7 @@ __device__ __forceinline__ void rig_setup(const RigParams& R, int k, const RigTa
     float* ray_y = const_cast<float*>(T.ray_y);
     float* bg_z = const_cast<float*>(T.bg_z);
     uint32_t* bg_cls = const_cast<uint32_t*>(T.bg_cls);
-    uint2* bg_fill = const_cast<uint2*>(T.bg_fill);
+    uint32_t* bg_rgb = const_cast<uint32_t*>(T.bg_rgb);
     const CamConst c = R.cam[k];
     const float cx = 0.5f * (float)R.W, cy = 0.5f * (float)R.H;
     for (int u = threadIdx.x; u < R.W; u += blockDim.x)
@@ -108,8 +109,7 @@ __device__ __forceinline__ void rig_setup(const RigParams& R, int k, const RigTa
         background(c.cphi, c.sphi, c.mz, ry, R.far_z, R.cls_sky, R.cls_ground, cls, z);
         bg_z[(size_t)k * R.H + v] = z;
         bg_cls[(size_t)k * R.H + v] = cls;
-        const __half2 h = __floats2half2_rn(z, z);
-        bg_fill[(size_t)k * R.H + v] = make_uint2(cls * 0x01010101u, *reinterpret_cast<const uint32_t*>(&h));
+        if (R.palette) bg_rgb[(size_t)k * R.H + v] = R.palette[cls];
     }
 }
 
@@ -170,6 +170,7 @@ cudaError_t configure_kernels() {
 static RigParams rig_params(const RenderParams& P) {
     RigParams R;
     R.K = P.K; R.W = P.W; R.H = P.H; R.far_z = P.far_z; R.cls_sky = P.cls_sky; R.cls_ground = P.cls_ground;
+    R.palette = P.out_rgb ? P.palette : nullptr;
     for (int k = 0; k < MAX_CAMS; ++k) R.cam[k] = P.cam[k];
     return R;
 }

@@ -448,13 +448,16 @@ __device__ __forceinline__ Job decode_job(const RenderParams& P, unsigned id, in
 // Ray coordinates of tile column / row i (threads 0..63 of a pass call this with i = 0..63).
 // Columns / rows past the image edge (ragged tiles) continue the same formula, so the tables
 // stay monotone for the cell classification.
+__device__ __forceinline__ float ray_column(const RenderParams& P, const Job& j, int i) {
+    return (j.t.x0 + i < P.W) ? __ldg(P.rig.ray_x + (size_t)j.k * P.W + j.t.x0 + i) : __fdiv_rn(sub(add((float)(j.t.x0 + i), 0.5f), 0.5f * (float)P.W), P.cam[j.k].fx);
+}
+__device__ __forceinline__ float ray_row(const RenderParams& P, const Job& j, int i) {
+    return (j.t.y0 + i < P.H) ? __ldg(P.rig.ray_y + (size_t)j.k * P.H + j.t.y0 + i) : __fdiv_rn(sub(add((float)(j.t.y0 + i), 0.5f), 0.5f * (float)P.H), P.cam[j.k].fy);
+}
 template <class S>
 __device__ __forceinline__ void load_rays(S& s, const RenderParams& P, const Job& j, int i) {
-    const CamConst& ck = P.cam[j.k];
-    s.ray_x[i] = (j.t.x0 + i < P.W) ? __ldg(P.rig.ray_x + (size_t)j.k * P.W + j.t.x0 + i)
-                                    : __fdiv_rn(sub(add((float)(j.t.x0 + i), 0.5f), 0.5f * (float)P.W), ck.fx);
-    s.ray_y[i] = (j.t.y0 + i < P.H) ? __ldg(P.rig.ray_y + (size_t)j.k * P.H + j.t.y0 + i)
-                                    : __fdiv_rn(sub(add((float)(j.t.y0 + i), 0.5f), 0.5f * (float)P.H), ck.fy);
+    s.ray_x[i] = ray_column(P, j, i);
+    s.ray_y[i] = ray_row(P, j, i);
 }
 
 // A whole tile rendered by the CTA in barrier-separated phases with per-round lists: any number of
@@ -1324,7 +1327,6 @@ cudaError_t launch_render_kernel(const RenderParams& P0, long long n_views, int 
     if (jobs > 0x7fffffffLL || (long long)P.E * P.A * P.K > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
     if (jobs <= 0) return cudaSuccess;
     P.n_jobs = (uint32_t)jobs;
-    P.far_z2 = 0x10001u * (uint32_t)__half_as_ushort(__float2half_rn(P.far_z));
     // few tiles: one CTA takes a tile from culling to store.  Measured (a call on 16 agents per environment, both image shapes of the workloads): 64 tiles 37 -> 17 us, 256 tiles 45 -> 14.5, 512 tiles 45 -> 23,
     // and against cull + tile kernel 768 tiles 41.7 -> 31.1, 1 024 tiles 43.5 -> 37.3, 1 280 tiles 44.0 -> 44.9.
     if (jobs <= 8LL * sm_count && !P.counters && !P.occlusion && (P.debug_flags & 15) == 0)

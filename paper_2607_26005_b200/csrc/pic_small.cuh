@@ -18,12 +18,13 @@ constexpr int SMALL_LARGE = 64, SMALL_FACES = 384;              // visible large
 
 struct __align__(16) SmallSmem {
     unsigned long long key[32][CELL_W * CELL_H];   // keys of the small primitives' fragments, cell by cell
-    TileRecords<TREC> rec;
-    TileRecords<32> small[SMALL_WARPS];            // a warp's small primitives, by lane
-    float ray_x[TILE], ray_y[TILE];
-    uint32_t cells[TREC], hit[32];                 // cells a record's box reaches; records that reach a cell
+    TileRecord rec[TREC];
+    TileRecord small[SMALL_WARPS][32];             // a warp's small primitives, by lane
+    f32x2 ray_xx[TILE];                            // see TileWarp
+    float ray_y[TILE];
+    uint32_t cells[TREC];                          // cells a record's box reaches
+    CellRecords recs[32];                          // records that reach a cell
     uint32_t frag_cells;                           // cells with fragments
-    uint8_t need[TREC][32];                        // see TileWarp
     Frustum f;
     uint32_t row_first[32], row_off[33];       // candidate ranges of the grid rows of a pass (see FrontLists)
     uint32_t lleaf[SMALL_LARGE], face[SMALL_FACES];
@@ -47,9 +48,12 @@ __global__ void __launch_bounds__(SMALL_THREADS, 2) render_small_kernel(const __
         frustum_setup(s.f, P, job, lane);
     } else if (warp == 1) {
         if (lane == 0) { s.n_rec = 0; s.n_leaf = 0; s.n_face = 0; s.frag_cells = 0u; }
-        s.hit[lane] = 0u;
+        s.recs[lane] = {0u, 0u, 0u};
     } else if (warp < 4) {
-        load_rays(s, P, job, threadIdx.x - 64);
+        const int i = (int)threadIdx.x - 64;
+        const float rx = ray_column(P, job, i);
+        s.ray_xx[i] = pack2(rx, rx);
+        s.ray_y[i] = ray_row(P, job, i);
     }
     {
         ulonglong2* k2 = reinterpret_cast<ulonglong2*>(s.key);
@@ -138,10 +142,10 @@ __global__ void __launch_bounds__(SMALL_THREADS, 2) render_small_kernel(const __
                 if (lane == 0 && m) base = atomicAdd(&s.n_rec, __popc(m));
                 base = __shfl_sync(0xffffffffu, base, 0);
                 const int slot = base + __popc(m & ((1u << lane) - 1u));
-                if (big && slot < TREC) { s.rec.write(slot, q, key_lo); s.cells[slot] = box_cells(box); }
+                if (big && slot < TREC) { s.rec[slot].write(q, key_lo); s.cells[slot] = box_cells(box); }
                 if (__any_sync(0xffffffffu, small)) {
-                    if (small) s.small[warp].write(lane, q, key_lo);
-                    small_pixels(s.small[warp], s.ray_x, s.ray_y, small, bx0, by0, w, h, P.w_near, P.w_far, lane, [&](bool in, float wv, uint32_t lo, int x, int y) {
+                    if (small) s.small[warp][lane].write(q, key_lo);
+                    small_pixels(s.small[warp], s.ray_xx, s.ray_y, small, bx0, by0, w, h, P.w_near, P.w_far, lane, [&](bool in, float wv, uint32_t lo, int x, int y) {
                         if (!in) return;
                         const uint32_t at = cell_pixel(x, y);
                         atomicMax(&s.key[at >> 7][at & 127u], make_key(__float_as_uint(wv), lo));
@@ -164,8 +168,12 @@ __global__ void __launch_bounds__(SMALL_THREADS, 2) render_small_kernel(const __
     const int n_rec = ego_active ? s.n_rec : 0;
     if (n_rec > 0) {
         NoTally n;
-        const uint32_t hit = classify_records(s, n_rec, true, P.w_near, P.w_far, lane, n, warp, SMALL_WARPS);
-        if (hit) atomicOr(&s.hit[lane], hit);
+        const CellRecords mine = classify_records(s, n_rec, true, P.w_near, P.w_far, lane, n, warp, SMALL_WARPS);
+        if (mine.hit) {
+            atomicOr(&s.recs[lane].hit, mine.hit);
+            atomicOr(&s.recs[lane].edges, mine.edges);
+            if (mine.range) atomicOr(&s.recs[lane].range, mine.range);
+        }
     }
     __syncthreads();
     // ---- cells w, w + 8, ... by warp w: four adjacent pixels per lane
@@ -175,20 +183,24 @@ __global__ void __launch_bounds__(SMALL_THREADS, 2) render_small_kernel(const __
 #pragma unroll 1
     for (int cell = warp; cell < 32; cell += SMALL_WARPS) {
         const int x = (cell & 1) * CELL_W + px, y = (cell >> 1) * CELL_H + py;
-        unsigned long long best[4] = {0ull, 0ull, 0ull, 0ull};
+        const int n_px = y < t.th ? t.tw - x : 0;
+        uint32_t bc = P.cls_sky;
+        float bz = P.far_z;
+        if (ego_active && n_px > 0) { bc = __ldg(P.rig.bg_cls + (size_t)job.k * P.H + t.y0 + y); bz = __ldg(P.rig.bg_z + (size_t)job.k * P.H + t.y0 + y); }
+        float bw[4] = {0.f, 0.f, 0.f, 0.f};
+        uint32_t bl[4] = {bc, bc, bc, bc};
         if ((frag_cells >> cell) & 1u) {
             const ulonglong2* ck = reinterpret_cast<const ulonglong2*>(s.key[cell]) + 2 * lane;
             const ulonglong2 a = ck[0], b = ck[1];
-            best[0] = a.x; best[1] = a.y; best[2] = b.x; best[3] = b.y;
+            const unsigned long long key[4] = {a.x, a.y, b.x, b.y};
+#pragma unroll
+            for (int k = 0; k < 4; ++k)
+                if (key[k]) { bw[k] = __uint_as_float((uint32_t)(key[k] >> 32)); bl[k] = (uint32_t)key[k]; }
         }
-        const float4 rx = *reinterpret_cast<const float4*>(s.ray_x + x);
-        raster_records_cell(s, s.hit[cell], cell, rx, s.ray_y[y], P.w_near, P.w_far, best);
-        const int n_px = y < t.th ? t.tw - x : 0;
+        raster_cell_records<false, true>(s, s.recs[cell], x, s.ray_y[y], P.w_near, P.w_far, bw, bl);
         if (n_px > 0) {
-            uint32_t bc = P.cls_sky;
-            float bz = P.far_z;
-            if (ego_active) { bc = __ldg(P.rig.bg_cls + (size_t)job.k * P.H + t.y0 + y); bz = __ldg(P.rig.bg_z + (size_t)job.k * P.H + t.y0 + y); }
-            store_class_depth<VEC>(P, tile0 + (size_t)(y * P.W + x), best, bc, bz, n_px);
+            const size_t o = tile0 + (size_t)(y * P.W + x);
+            store_class_depth<VEC>(P.out_class + o, P.out_depth + o, !VEC && P.out_depth32 ? P.out_depth32 + o : nullptr, bw, bl, bz, n_px);
         }
     }
 }

@@ -88,7 +88,7 @@ struct RigTables {
     const float* ray_y;        // [K][H]
     const float* bg_z;         // [K][H] background depth
     const uint32_t* bg_cls;    // [K][H] background class
-    const uint2* bg_fill;      // [K][H] the same as stored: class in four bytes, binary16 depth in two halves
+    const uint32_t* bg_rgb;    // [K][H] background colour (calls that render colours)
 };
 
 // Division of numbers below 2^31 by a divisor fixed per call (Granlund and Montgomery, "Division by invariant integers
@@ -109,7 +109,6 @@ struct RenderParams {
     float near_z, far_z;
     float w_near, w_far;            // 1/near, 1/far: kept range of the reciprocal depth
     uint32_t cls_agent, cls_sky, cls_ground;
-    uint32_t far_z2;                // binary16 of far_z, twice
     FastDiv div_tiles, div_tiles_x, div_K, div_A;   // by tiles per view, tile columns, cameras, agent slots
     const int32_t* env_map;
     const MapInfo* env_maps;        // [E] the MapInfo of each environment's map (one load instead of two)
@@ -141,15 +140,15 @@ struct RenderParams {
     CamConst cam[MAX_CAMS];
 };
 
-// Layout of the per-camera tables in one allocation of table_bytes bytes, 8-byte aligned.
-inline size_t table_bytes(int K, int H, int W) { return sizeof(float) * (size_t)K * ((size_t)W + 5 * (size_t)H); }
+// Layout of the per-camera tables in one allocation of table_bytes bytes.
+inline size_t table_bytes(int K, int H, int W) { return sizeof(float) * (size_t)K * ((size_t)W + 4 * (size_t)H); }
 inline RigTables rig_tables(float* base, int K, int H, int W) {
     RigTables r;
-    r.bg_fill = reinterpret_cast<const uint2*>(base);
-    r.ray_x = base + 2 * (size_t)K * H;
+    r.ray_x = base;
     r.ray_y = r.ray_x + (size_t)K * W;
     r.bg_z = r.ray_y + (size_t)K * H;
     r.bg_cls = reinterpret_cast<const uint32_t*>(r.bg_z + (size_t)K * H);
+    r.bg_rgb = r.bg_cls + (size_t)K * H;
     return r;
 }
 inline void set_divisors(RenderParams& P) {

@@ -296,3 +296,42 @@ def test_long_primitives_cut_at_the_near_plane(length, near, hfov, H, W, pitch):
         assert flags == flags_part == 0 and (np.abs(whole[:50].astype(int) - part[:50].astype(int)) <= 1).all()
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("copies,step,n_side,dots,dot", [
+    (1, 0.375, 3, 8, 0.25),      # primitives of a few pixels: fragments only
+    (2, 1.5, 3, 8, 0.25),        # fragments and records at the same depth, each primitive twice
+    (3, 2.5, 3, 8, 0.25),        # 27 records
+    (8, 4.0, 2, 8, 0.25),        # 32 records, the most a tile holds, and 40 survivors: set up in two passes
+    (9, 4.0, 2, 8, 0.25),        # one more than it holds
+    (7, 4.0, 2, 10, 0.75),       # 28 records and 90 fragments, which fit the memory they share ...
+    (7, 4.0, 2, 16, 0.75),       # ... and 144, which do not
+    (1, 0.75, 1, 26, 0.75),      # 243 fragments and hardly a record
+])
+def test_equal_depths_and_pixel_centres_on_edges(copies, step, n_side, dots, dot):
+    """Walls of squares that share their edges, facing the camera at whole distances, so that depths are exactly equal and edges run
+    through pixel centres: the lower index wins, and a shared edge belongs to one side."""
+    from tests.gpu_util import CudaRun
+    from tests.util import assert_same_as_exhaustive
+    rng = np.random.default_rng(copies + dots)
+    squares = [(8.0, y, z, step) for y in range(n_side) for z in range(n_side)] * copies + [(8.0, 0.25 * i, 0.25, dot) for i in range(dots)]
+    tris = []
+    for i in rng.permutation(len(squares)):
+        x, iy, iz, d = squares[i]
+        y0, z0 = (iy - n_side / 2) * d, 1.5 + (iz - n_side / 2) * d
+        p = [(x, y0, z0), (x, y0 + d, z0), (x, y0 + d, z0 + d), (x, y0, z0 + d)]
+        tris += [[p[0], p[1], p[2]], [p[0], p[2], p[3]]]
+    E, A, K = 80, 16, 1
+    poses = np.zeros((E, A, 3), np.float32)
+    poses[..., 0] = rng.choice([-8.0, 0.0, 4.0], (E, A))
+    poses[..., 1] = rng.integers(-8, 9, (E, A)) * 0.125
+    s = custom_scene(np.asarray(tris, np.float32), rng.integers(2, 200, len(squares)).repeat(2).astype(np.uint8), poses, np.full((E, A, 3), 0.01, np.float32),
+                     make_rig((0.0,), 90.0, 90.0, 64, 64, mount=(0.0, 0.0, 1.5)), 64, 64, env_map_id=np.zeros(E, np.int32))
+    g = CudaRun(s)
+    try:
+        want = g.render(brute=True)
+        assert_same_as_exhaustive(g.render(), want)
+        few = g.render(view_first=0, view_count=100)
+        assert (few[0][:100] == want[0][:100]).all()
+    finally:
+        g.close()
