@@ -12,8 +12,8 @@ __device__ __forceinline__ float edge_coverage(float e0, float a, float b) {
     if (e0 >= h) return 1.f;
     if (e0 <= -h) return 0.f;
     const float hi = fmaxf(A, B), lo = fminf(A, B), g = 0.5f * (hi - lo);
-    if (fabsf(e0) <= g) return 0.5f + __fdividef(e0, hi);
-    const float d = h - fabsf(e0), corner = __fdividef(d * d, 2.f * A * B);     // the corner triangle cut off
+    if (fabsf(e0) <= g) return 0.5f + fast_div(e0, hi);
+    const float d = h - fabsf(e0), corner = fast_div(d * d, 2.f * A * B);     // the corner triangle cut off
     return e0 < 0.f ? corner : 1.f - corner;
 }
 
@@ -30,10 +30,10 @@ __device__ __forceinline__ float polygon_coverage(const float (&x)[4], const flo
         const int j = (i + 1) & 3;
         const float x0 = x[i], y0 = y[i], x1 = x[j], y1 = y[j];
         const float ya = __saturatef(y0), yb = __saturatef(y1);
-        const float m = y1 != y0 ? __fdividef(x1 - x0, y1 - y0) : 0.f;
+        const float m = fabsf(y1 - y0) > 1e-30f ? fast_div(x1 - x0, y1 - y0) : 0.f;
         const float xa = fm(ya - y0, m, x0), xb = fm(yb - y1, m, x1), d = xb - xa;
         const float ca = __saturatef(xa), cb = __saturatef(xb), mean = 0.5f * (ca + cb);
-        const float r = __fdividef(1.f, d);
+        const float r = fast_rcp(d);
         const float part = fm((cb - ca) * r, mean, (fmaxf(xb, 1.f) - fmaxf(xa, 1.f)) * r);
         sum = fm(yb - ya, fabsf(d) < 1e-7f ? mean : part, sum);
     }
@@ -69,7 +69,7 @@ __device__ __forceinline__ float pixel_coverage(const float (&e)[NL], const floa
 #pragma unroll 1
     for (int j = 0; j < N; ++j) {
         const float n2 = fm(A[0], A[0], mul(B[0], B[0]));
-        const float k = -__fdividef(C[0], n2), p0x = k * A[0], p0y = k * B[0];     // the line's point nearest the centre
+        const float k = -fast_div(C[0], n2), p0x = k * A[0], p0y = k * B[0];     // the line's point nearest the centre
         float t0 = -3e38f, t1 = 3e38f;
 #pragma unroll
         for (int p = 1; p < N; ++p) {
@@ -77,7 +77,7 @@ __device__ __forceinline__ float pixel_coverage(const float (&e)[NL], const floa
             const bool same_side = p >= N - j && fm(A[p], A[0], mul(B[p], B[0])) > 0.f;
             const float nudge = 1e-5f * (fabsf(A[p]) + fabsf(B[p]));
             const float al = fm(A[p], p0x, fm(B[p], p0y, C[p])) + (same_side ? -nudge : nudge);
-            const float t = -__fdividef(al, be);
+            const float t = -fast_div(al, be);
             // (written with selects: the lanes of a warp rarely agree on the sign of be)
             t0 = be > 0.f ? fmaxf(t0, t) : t0;
             t1 = be < 0.f ? fminf(t1, t) : t1;

@@ -48,6 +48,17 @@ struct PrimEq {
     uint32_t tl;                 // bit i: exact zeros of edge i belong to the primitive
 };
 
+// 1 / x to an ulp or so, one instruction.  (__fdividef takes some five more, for the subnormal divisors it serves and this does not:
+// they count as 0.)  Used where a last digit does not matter or the divisor is a depth, a depth range or a difference of pixels.
+// With the ray tables that go on beyond the image (no division in the render kernels): 8 192 agents 220 -> 217 us, 65 536 agents 2 251 ->
+// 2 217, 14 880 views of 96 x 54 129.6 -> 126.7, their colours 157.6 -> 153.5.
+__device__ __forceinline__ float fast_rcp(float x) {
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ float fast_div(float a, float b) { return __fmul_rn(a, fast_rcp(b)); }
+
 struct V3 { float x, y, z; };
 
 __device__ __forceinline__ unsigned divide(unsigned n, const FastDiv& f) { return (__umulhi(n, f.m) + n) >> f.s; }
@@ -198,7 +209,7 @@ __device__ __forceinline__ bool pixel_box_int(const Cam& c, const TileCtx& t, co
         float sx0 = 3e38f, sx1 = -3e38f, sy0 = 3e38f, sy1 = -3e38f;
 #pragma unroll
         for (int i = 0; i < n; ++i) {
-            float iz = __fdividef(1.0f, V[i].z);
+            float iz = fast_rcp(V[i].z);
             float sx = fm(c.focx, mul(V[i].x, iz), c.cx), sy = fm(c.focy, mul(V[i].y, iz), c.cy);
             sx0 = fminf(sx0, sx); sx1 = fmaxf(sx1, sx); sy0 = fminf(sy0, sy); sy1 = fmaxf(sy1, sy);
         }
@@ -303,12 +314,6 @@ __device__ __forceinline__ void background(float cphi, float sphi, float mz, flo
     const float wr = fm(-ry, cphi, sphi);          // world-z component of the ray
     cls = cls_sky; z = far_z;
     if (wr < 0.f && mz > 0.f) { cls = cls_ground; z = fminf(far_z, __fdiv_rn(mz, -wr)); }
-}
-
-__device__ __forceinline__ float fast_rcp(float x) {
-    float r;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-    return r;
 }
 
 }  // namespace pic

@@ -38,8 +38,8 @@ __device__ __forceinline__ void exhaustive_tile(ExhaustiveSmem& s, const RenderP
     for (int i = threadIdx.x; i < TILE * TILE; i += EXH_THREADS) s.key[i] = 0ull;
     if (threadIdx.x < TILE) {
         const int i = threadIdx.x;
-        s.ray_x[i] = (t.x0 + i < P.W) ? P.rig.ray_x[(size_t)k * P.W + t.x0 + i] : 0.f;
-        s.ray_y[i] = (t.y0 + i < P.H) ? P.rig.ray_y[(size_t)k * P.H + t.y0 + i] : 0.f;
+        s.ray_x[i] = (t.x0 + i < P.W) ? P.rig.ray_x[(size_t)k * ray_stride(P.W) + t.x0 + i] : 0.f;
+        s.ray_y[i] = (t.y0 + i < P.H) ? P.rig.ray_y[(size_t)k * ray_stride(P.H) + t.y0 + i] : 0.f;
     }
     __syncthreads();
     const Cam& c = s.cam;

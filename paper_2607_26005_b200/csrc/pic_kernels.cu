@@ -100,11 +100,13 @@ __device__ __forceinline__ void rig_setup(const RigParams& R, int k, const RigTa
     uint32_t* bg_rgb = const_cast<uint32_t*>(T.bg_rgb);
     const CamConst c = R.cam[k];
     const float cx = 0.5f * (float)R.W, cy = 0.5f * (float)R.H;
-    for (int u = threadIdx.x; u < R.W; u += blockDim.x)
-        ray_x[(size_t)k * R.W + u] = __fdiv_rn(sub(add((float)u, 0.5f), cx), c.fx);
-    for (int v = threadIdx.x; v < R.H; v += blockDim.x) {
+    const int nx = ray_stride(R.W), ny = ray_stride(R.H);
+    for (int u = threadIdx.x; u < nx; u += blockDim.x)
+        ray_x[(size_t)k * nx + u] = __fdiv_rn(sub(add((float)u, 0.5f), cx), c.fx);
+    for (int v = threadIdx.x; v < ny; v += blockDim.x) {
         const float ry = __fdiv_rn(sub(add((float)v, 0.5f), cy), c.fy);
-        ray_y[(size_t)k * R.H + v] = ry;
+        ray_y[(size_t)k * ny + v] = ry;
+        if (v >= R.H) continue;
         uint32_t cls; float z;
         background(c.cphi, c.sphi, c.mz, ry, R.far_z, R.cls_sky, R.cls_ground, cls, z);
         bg_z[(size_t)k * R.H + v] = z;

@@ -445,15 +445,9 @@ __device__ __forceinline__ Job decode_job(const RenderParams& P, unsigned id, in
     return j;
 }
 
-// Ray coordinates of tile column / row i (threads 0..63 of a pass call this with i = 0..63).
-// Columns / rows past the image edge (ragged tiles) continue the same formula, so the tables
-// stay monotone for the cell classification.
-__device__ __forceinline__ float ray_column(const RenderParams& P, const Job& j, int i) {
-    return (j.t.x0 + i < P.W) ? __ldg(P.rig.ray_x + (size_t)j.k * P.W + j.t.x0 + i) : __fdiv_rn(sub(add((float)(j.t.x0 + i), 0.5f), 0.5f * (float)P.W), P.cam[j.k].fx);
-}
-__device__ __forceinline__ float ray_row(const RenderParams& P, const Job& j, int i) {
-    return (j.t.y0 + i < P.H) ? __ldg(P.rig.ray_y + (size_t)j.k * P.H + j.t.y0 + i) : __fdiv_rn(sub(add((float)(j.t.y0 + i), 0.5f), 0.5f * (float)P.H), P.cam[j.k].fy);
-}
+// Ray coordinates of tile column / row i, 0..63.
+__device__ __forceinline__ float ray_column(const RenderParams& P, const Job& j, int i) { return __ldg(P.rig.ray_x + (size_t)j.k * ray_stride(P.W) + j.t.x0 + i); }
+__device__ __forceinline__ float ray_row(const RenderParams& P, const Job& j, int i) { return __ldg(P.rig.ray_y + (size_t)j.k * ray_stride(P.H) + j.t.y0 + i); }
 template <class S>
 __device__ __forceinline__ void load_rays(S& s, const RenderParams& P, const Job& j, int i) {
     s.ray_x[i] = ray_column(P, j, i);
@@ -697,8 +691,8 @@ __device__ __forceinline__ bool view_box(const Cam& c, const TileCtx& t, const V
 #pragma unroll
         for (int i = 0; i < 4; ++i) reach = fmaxf(reach, fabsf(V[i].x) + fabsf(V[i].y) + fabsf(V[i].z));
         const V3 n = plane_normal(V, true);                  // (of a triangle too: its third vertex is there twice)
-        const float ratio = __fdividef(reach * sqrtf(vdot(n, n)), fabsf(vdot(n, V[0])));      // L / h
-        const float zc = t.near_z * 0.99f, izc = __fdividef(1.f, zc), f = fmaxf(c.focx, c.focy), shift = 3e-7f * f * ratio;
+        const float ratio = fast_div(reach * sqrtf(vdot(n, n)), fabsf(vdot(n, V[0])));      // L / h
+        const float zc = t.near_z * 0.99f, izc = fast_rcp(zc), f = fmaxf(c.focx, c.focy), shift = 3e-7f * f * ratio;
         if (ratio <= 1e4f && shift <= 0.5f) {
             const float mm = m + 0.25f + 8.f * shift + 2e-6f * f * reach * izc;               // (an edge is at most 2 L)
             float sx0 = 3e38f, sx1 = -3e38f, sy0 = 3e38f, sy1 = -3e38f;
@@ -709,9 +703,9 @@ __device__ __forceinline__ bool view_box(const Cam& c, const TileCtx& t, const V
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 const V3 a = V[i], b = V[(i + 1) & 3];
-                if (a.z >= zc) include(a.x, a.y, __fdividef(1.f, a.z));
+                if (a.z >= zc) include(a.x, a.y, fast_rcp(a.z));
                 if ((a.z < zc) != (b.z < zc)) {
-                    const float u = __fdividef(zc - a.z, b.z - a.z);
+                    const float u = fast_div(zc - a.z, b.z - a.z);
                     include(fm(u, b.x - a.x, a.x), fm(u, b.y - a.y, a.y), izc);
                 }
             }
@@ -839,7 +833,7 @@ __device__ __forceinline__ bool bound_visible(const Cam& c, const TileCtx& t, co
     const float z0 = q.z - rz, z1 = q.z + rz;
     bool ok = z1 >= t.near_z * 0.9999f && z0 <= t.far_z * 1.0001f;
     if (z0 >= t.near_z * ZPROJ_FRAC) {                                         // (else a vertex may not project: pixel_box looks closer)
-        const float i0 = __fdividef(1.f, z0), i1 = __fdividef(1.f, z1);
+        const float i0 = fast_rcp(z0), i1 = fast_rcp(z1);
         const float xa = q.x - r, xb = q.x + r, ya = q.y - ry, yb = q.y + ry;
         const float mm = m + 0.015625f;                                        // 1/64 pixel for the rounding above
         const float sx0 = fm(c.focx, xa * (xa < 0.f ? i0 : i1), c.cx), sx1 = fm(c.focx, xb * (xb < 0.f ? i1 : i0), c.cx);
@@ -1185,8 +1179,8 @@ __global__ void __launch_bounds__(32) coverage_kernel(const __grid_constant__ Re
     if (!env_agents[job.a].active) return;
     frustum_setup(s.f, P, job, lane);
     const Cam& c = s.f.cam;
-    const float* ray_x = P.rig.ray_x + (size_t)job.k * P.W;
-    const float* ray_y = P.rig.ray_y + (size_t)job.k * P.H + t.y0;
+    const float* ray_x = P.rig.ray_x + (size_t)job.k * ray_stride(P.W);
+    const float* ray_y = P.rig.ray_y + (size_t)job.k * ray_stride(P.H) + t.y0;
     uint32_t* occ = P.occlusion + job.view * (size_t)P.A * 2u;
     for (int b0 = 0; b0 < P.A; b0 += 32) {
         uint32_t draw = 0u;

@@ -304,7 +304,7 @@ __device__ __forceinline__ uint32_t key_colour(const RenderParams& P, float w, u
     const uint32_t pal = __ldg(P.palette + (lo & 0xffu)), index = 0xFFFFFFu - (lo >> 8);
     if (index < n_map_tris) return pal;
     const uint32_t face = ((index - n_map_tris) >> 1) % 6u;
-    const float k = FACE_SHADE[face] * (1.f - 0.5f * __fdividef(__fdividef(1.f, w) - P.near_z, P.far_z - P.near_z));
+    const float k = FACE_SHADE[face] * (1.f - 0.5f * fast_div(fast_rcp(w) - P.near_z, P.far_z - P.near_z));
     const float r = k * (float)(pal & 0xffu), g = k * (float)((pal >> 8) & 0xffu), b = k * (float)((pal >> 16) & 0xffu);
     return (uint32_t)fminf(r + 0.5f, 255.f) | ((uint32_t)fminf(g + 0.5f, 255.f) << 8) | ((uint32_t)fminf(b + 0.5f, 255.f) << 16);
 }

@@ -84,8 +84,8 @@ static_assert(sizeof(ViewCam) == 64, "ViewCam must be 64 bytes");
 // Per-camera tables shared by all views of a call: ray coordinates of pixel columns / rows and the
 // background (analytic ground plane / sky) of every row.
 struct RigTables {
-    const float* ray_x;        // [K][W]
-    const float* ray_y;        // [K][H]
+    const float* ray_x;        // [K][ray_stride(W)], [K][ray_stride(H)]: beyond the image the same formula goes on, so that a tile that
+    const float* ray_y;        //   reaches over the edge reads a monotone table
     const float* bg_z;         // [K][H] background depth
     const uint32_t* bg_cls;    // [K][H] background class
     const uint32_t* bg_rgb;    // [K][H] background colour (calls that render colours)
@@ -140,13 +140,19 @@ struct RenderParams {
     CamConst cam[MAX_CAMS];
 };
 
+// Entries of a ray table for n columns or rows: a tile that begins inside the image ends inside the table.
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline int ray_stride(int n) { return (n + 2 * TILE - 1) / TILE * TILE; }
+
 // Layout of the per-camera tables in one allocation of table_bytes bytes.
-inline size_t table_bytes(int K, int H, int W) { return sizeof(float) * (size_t)K * ((size_t)W + 4 * (size_t)H); }
+inline size_t table_bytes(int K, int H, int W) { return sizeof(float) * (size_t)K * ((size_t)ray_stride(W) + (size_t)ray_stride(H) + 3 * (size_t)H); }
 inline RigTables rig_tables(float* base, int K, int H, int W) {
     RigTables r;
     r.ray_x = base;
-    r.ray_y = r.ray_x + (size_t)K * W;
-    r.bg_z = r.ray_y + (size_t)K * H;
+    r.ray_y = r.ray_x + (size_t)K * ray_stride(W);
+    r.bg_z = r.ray_y + (size_t)K * ray_stride(H);
     r.bg_cls = reinterpret_cast<const uint32_t*>(r.bg_z + (size_t)K * H);
     r.bg_rgb = r.bg_cls + (size_t)K * H;
     return r;
