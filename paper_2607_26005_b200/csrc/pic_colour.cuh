@@ -20,7 +20,13 @@
 // A strip keeps, per pixel, the nearest FULLY covering fragment as a 64-bit key (unsigned max, as in the other
 // kernels, with the record's slot in the low byte) and a linked list of the partially covering fragments in
 // front of it (1/z, coverage in 14 bits, slot); the strip's warp owns both, so no atomics are needed.  The
-// resolve walks each pixel's list in depth order, merges, composites and stores 16 pixels (48 bytes) per lane.
+// resolve walks each pixel's list in depth order, merges, composites and stores four pixels (12 bytes) per lane, side by side.
+//
+// Bound by instruction issue and fetch: at 61 KB of code a fifth of the issue slots waited for instructions, at 48 KB few do, so what
+// is not hot is rolled or out of line.  14 880 views of 96 x 54 (16 384 tiles with anything in them) 1 005 -> 776 us, 192 views of
+// 384 x 216 252 -> 217, by: cells that a record covers wholly updating their keys and no more (three in seven); strips that nothing
+// reaches storing their background (two thirds); one rolled copy of the shading with the colours in the pool; stores side by side;
+// divisions of one reciprocal.  Four CTAs per multiprocessor with strips of four rows: 15 % more work for 2 % more speed.
 #pragma once
 
 constexpr int CSTRIP = 8;                       // pixel rows of a strip
@@ -41,6 +47,7 @@ struct __align__(16) ColourPool {
     float4 w[CPOOL];                            // 1/z plane wx, wy, wz; key low word (index, class)
     uint32_t box[CPOOL];                        // pixel box (6 bits per coordinate), top-left bits << 24, REC_DEAD, REC_TINY
     float shade[CPOOL];                         // box faces: the face's factor; map primitives: 0 (not shaded)
+    uint32_t rgb[CPOOL];                        // the class's colour
     uint32_t surface[CPOOL];                    // fragments of equal surface merge: a map primitive's class, 256 + agent of a box
 };
 
@@ -56,7 +63,7 @@ struct __align__(16) ColourSmem {
     int n_surv[NW];
     int next_task;
 };
-static_assert(sizeof(ColourSmem) <= 74 * 1024, "three CTAs per SM");
+static_assert(sizeof(ColourSmem) <= 75 * 1024, "three CTAs per SM");
 
 struct RayView { float* ray_x; float* ray_y; };
 
@@ -192,6 +199,17 @@ __device__ __noinline__ void small_fragments(unsigned long long* key, unsigned l
     __syncwarp();
 }
 
+// A 16 x 4 pixel cell of a strip that a record covers wholly.
+__device__ __forceinline__ void cover_cell(unsigned long long* key, const float* ray_x, const float* ray_y, const PrimEq& q, uint32_t key_lo, int xx, int yy, int lane) {
+    const int x = xx + (lane & 7) * 2, y = yy + (lane >> 3);
+    const float2 rx = *reinterpret_cast<const float2*>(ray_x + x);
+    const float wt = fm(q.wy, ray_y[y], q.wz);
+    ulonglong2* kp = reinterpret_cast<ulonglong2*>(key + key_index(x, y));
+    const ulonglong2 kk = *kp;
+    const unsigned long long k0 = make_key(__float_as_uint(fm(q.wx, rx.x, wt)), key_lo), k1 = make_key(__float_as_uint(fm(q.wx, rx.y, wt)), key_lo);
+    if (k0 > kk.x || k1 > kk.y) *kp = make_ulonglong2(k0 > kk.x ? k0 : kk.x, k1 > kk.y ? k1 : kk.y);
+}
+
 // A 16 x 4 pixel cell of a strip against one record; a lane handles two adjacent pixels.
 template <bool AA>
 __device__ __forceinline__ void colour_cell(unsigned long long* key, uint16_t* head, unsigned long long* frag, int& n_frag, int& n_pend, bool& dropped,
@@ -269,11 +287,10 @@ __device__ __forceinline__ void colour_cell(unsigned long long* key, uint16_t* h
 
 // Colour of a fragment of the record in `slot` at reciprocal depth w.
 __device__ __forceinline__ void shade_fragment(const ColourPool& pool, const RenderParams& P, uint32_t slot, float w, float& r, float& g, float& b) {
-    const uint32_t cls = __float_as_uint(pool.w[slot].w) & 0xffu;
     const float sh = pool.shade[slot];
     float k = 1.f;
-    if (sh > 0.f) k = sh * (1.f - 0.5f * __fdividef(__fdividef(1.f, w) - P.near_z, P.far_z - P.near_z));
-    const uint32_t pal = __ldg(P.palette + cls);
+    if (sh > 0.f) k = sh * (1.f - 0.5f * fast_div(fast_rcp(w) - P.near_z, P.far_z - P.near_z));
+    const uint32_t pal = pool.rgb[slot];
     r = k * (float)(pal & 0xffu); g = k * (float)((pal >> 8) & 0xffu); b = k * (float)((pal >> 16) & 0xffu);
 }
 
@@ -347,59 +364,69 @@ __device__ __forceinline__ void composite_rows(unsigned long long* key, uint16_t
         if (hd) {
             head[p] = 0;
             const int gy = jb.t.y0 + ys + y;
-            uint32_t bgc = P.cls_sky;
-            if (ego_active && gy < P.H) bgc = __ldg(P.rig.bg_cls + (size_t)jb.k * P.H + gy);
             unsigned long long* kp = key + key_index(x, y);
-            const uint32_t bg = __ldg(P.palette + bgc);
+            const uint32_t bg = __ldg(ego_active && gy < P.H ? P.rig.bg_rgb + (size_t)jb.k * P.H + gy : P.palette + P.cls_sky);
             *kp = KEY_RESOLVED | composite_pixel(*kp, hd, frag, pool, P, (float)(bg & 0xffu), (float)((bg >> 8) & 0xffu), (float)((bg >> 16) & 0xffu));
         }
     }
     __syncwarp();
 }
 
+// Four pixels (n_px of them exist) packed in three words -> dst.  vec: whole groups may be stored as words.
+__device__ __forceinline__ void store_four_colours(uint8_t* dst, uint32_t w0, uint32_t w1, uint32_t w2, bool vec, int n_px) {
+    if (vec && n_px >= 4) {
+        uint32_t* d = reinterpret_cast<uint32_t*>(dst);
+        d[0] = w0; d[1] = w1; d[2] = w2;
+    } else {
+#pragma unroll 1
+        for (int n = 0; n < 3 * min(n_px, 4); ++n) dst[n] = (uint8_t)((n < 4 ? w0 : n < 8 ? w1 : w2) >> (8 * (n & 3)));
+    }
+}
+
+// A strip's colours, two rows at a time, four pixels (12 bytes, three words) per lane: lanes side by side store side by side.  The
+// loops are not unrolled: one copy of the shading code.
 __device__ __forceinline__ void resolve_store_colour(unsigned long long* key, const ColourPool& pool, const RenderParams& P, const Job& jb,
                                                      bool ego_active, int ys, bool vec_ok, int lane) {
-    const int y = lane >> 2, xs = (lane & 3) * 16;
-    const int gy = jb.t.y0 + ys + y;
-    uint32_t bgc = P.cls_sky;
-    if (ego_active && gy < P.H) bgc = __ldg(P.rig.bg_cls + (size_t)jb.k * P.H + gy);
-    const uint32_t bg8 = __ldg(P.palette + bgc);
-    const bool row_ok = ys + y < jb.t.th;
-    uint8_t* dst = P.out_rgb + 3u * ((jb.view * (size_t)P.H + gy) * (size_t)P.W + jb.t.x0 + xs);
-    // four groups of four pixels (12 bytes, three words) each; the loop is not unrolled: one copy of the shading code
+    const int x = (lane & 15) * 4;
 #pragma unroll 1
-    for (int g = 0; g < 4; ++g) {
-        uint32_t ow[3] = {0u, 0u, 0u};
-#pragma unroll
-        for (int h2 = 0; h2 < 2; ++h2) {
-            ulonglong2* kp = reinterpret_cast<ulonglong2*>(key + key_index(xs + 4 * g + 2 * h2, y));
-            const ulonglong2 kk = *kp;
-            *kp = make_ulonglong2(0ull, 0ull);
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const unsigned long long k = h ? kk.y : kk.x;
-                uint32_t c = bg8;
-                if (k & KEY_RESOLVED) c = (uint32_t)k & 0xffffffu;
-                else if (k) {
-                    float R, G, B;
-                    shade_fragment(pool, P, (uint32_t)k & 0xffu, __uint_as_float((uint32_t)(k >> 32)), R, G, B);
-                    c = (uint32_t)fminf(R + 0.5f, 255.f) | ((uint32_t)fminf(G + 0.5f, 255.f) << 8) | ((uint32_t)fminf(B + 0.5f, 255.f) << 16);
-                }
-                const int n = 3 * (2 * h2 + h);      // byte offset of the pixel in the group's 12 bytes
-                ow[n >> 2] |= c << (8 * (n & 3));
-                if ((n & 3) > 1) ow[(n >> 2) + 1] |= c >> (8 * (4 - (n & 3)));
+    for (int y = lane >> 4; y < CSTRIP; y += 2) {
+        const int gy = jb.t.y0 + ys + y;
+        const uint32_t bg = __ldg(ego_active && gy < P.H ? P.rig.bg_rgb + (size_t)jb.k * P.H + gy : P.palette + P.cls_sky);
+        uint32_t w0 = 0u, w1 = 0u, w2 = 0u;
+#pragma unroll 1
+        for (int i = 0; i < 4; ++i) {
+            unsigned long long* kp = key + key_index(x + i, y);
+            const unsigned long long k = *kp;
+            *kp = 0ull;
+            uint32_t c = bg;
+            if (k & KEY_RESOLVED) c = (uint32_t)k & 0xffffffu;
+            else if (k) {
+                float R, G, B;
+                shade_fragment(pool, P, (uint32_t)k & 0xffu, __uint_as_float((uint32_t)(k >> 32)), R, G, B);
+                c = (uint32_t)fminf(R + 0.5f, 255.f) | ((uint32_t)fminf(G + 0.5f, 255.f) << 8) | ((uint32_t)fminf(B + 0.5f, 255.f) << 16);
             }
+            w0 = __funnelshift_r(w0, w1, 24); w1 = __funnelshift_r(w1, w2, 24); w2 = (w2 >> 24) | (c << 8);
         }
-        const int x = xs + 4 * g;
-        if (row_ok && x < jb.t.tw) {
-            if (vec_ok && x + 4 <= jb.t.tw) {
-                uint32_t* d32 = reinterpret_cast<uint32_t*>(dst + 12 * g);
-                d32[0] = ow[0]; d32[1] = ow[1]; d32[2] = ow[2];
-            } else {
-#pragma unroll
-                for (int n = 0; n < 12; ++n)
-                    if (n / 3 + x < jb.t.tw) dst[12 * g + n] = (uint8_t)(ow[n >> 2] >> (8 * (n & 3)));
-            }
+        if (ys + y < jb.t.th && x < jb.t.tw) store_four_colours(P.out_rgb + 3u * ((jb.view * (size_t)P.H + gy) * (size_t)P.W + jb.t.x0 + x), w0, w1, w2, vec_ok, jb.t.tw - x);
+    }
+}
+
+// A strip that no primitive reaches.
+__device__ __forceinline__ void store_strip_background(const RenderParams& P, const Job& jb, bool ego_active, int ys, int lane) {
+    const bool wide = (P.W & 15) == 0 && (reinterpret_cast<uintptr_t>(P.out_rgb) & 15u) == 0;
+    const bool vec_ok = (P.W & 3) == 0 && (reinterpret_cast<uintptr_t>(P.out_rgb) & 3u) == 0;
+    const int x = wide ? (lane & 3) * 16 : (lane & 15) * 4;
+#pragma unroll 1
+    for (int y = wide ? lane >> 2 : lane >> 4; ys + y < jb.t.th && y < CSTRIP && x < jb.t.tw; y += wide ? 8 : 2) {
+        const int gy = jb.t.y0 + ys + y;
+        const uint32_t c = __ldg(ego_active ? P.rig.bg_rgb + (size_t)jb.k * P.H + gy : P.palette + P.cls_sky);
+        const uint32_t w0 = c | (c << 24), w1 = (c >> 8) | (c << 16), w2 = (c >> 16) | (c << 8);
+        uint8_t* dst = P.out_rgb + 3u * ((jb.view * (size_t)P.H + gy) * (size_t)P.W + jb.t.x0 + x);
+        if (wide) {
+            uint4* d = reinterpret_cast<uint4*>(dst);
+            d[0] = make_uint4(w0, w1, w2, w0); d[1] = make_uint4(w1, w2, w0, w1); d[2] = make_uint4(w2, w0, w1, w2);
+        } else {
+            store_four_colours(dst, w0, w1, w2, vec_ok, jb.t.tw - x);
         }
     }
 }
@@ -453,7 +480,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
     for (int i = 0; i < CSTRIP_KEYS / 8 / 32; ++i)
         reinterpret_cast<uint4*>(s.head[warp])[i * 32 + lane] = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
-    const bool vec_ok = (P.W % 16 == 0) && ((reinterpret_cast<uintptr_t>(P.out_rgb) & 15u) == 0);
+    const bool vec_ok = (P.W & 3) == 0 && (reinterpret_cast<uintptr_t>(P.out_rgb) & 3u) == 0;
     uint32_t done = 0u;
 #pragma unroll
     for (int j = 0; j < NW; ++j)
@@ -507,7 +534,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
                 if (small) {
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        const float iz = __fdividef(1.f, V[k].z);
+                        const float iz = fast_rcp(V[k].z);
                         q.nx[k] = fm(c.focx, mul(V[k].x, iz), c.cx - (float)job.t.x0);
                         q.ny[k] = fm(c.focy, mul(V[k].y, iz), c.cy - (float)job.t.y0);
                     }
@@ -518,6 +545,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
                 s.pool.w[slot] = make_float4(q.wx, q.wy, q.wz, __uint_as_float(key_lo));
                 s.pool.box[slot] = bx0 | (by0 << 6) | (bx1 << 12) | (by1 << 18) | (q.tl << 24) | (small ? REC_TINY : 0u);
                 s.pool.shade[slot] = shade;
+                s.pool.rgb[slot] = __ldg(P.palette + (key_lo & 0xffu));
                 s.pool.surface[slot] = surface;
             }
         }
@@ -541,7 +569,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
             const int first = (int)((bases >> (8 * j)) & 0xffu);
             const float* ray_x = s.ray_x[j];
             const float* ray_y = s.ray_y[j] + ys;
-            const float du = __fdividef(1.f, s.cam[j].focx), dv = __fdividef(1.f, s.cam[j].focy);
+            const float du = fast_rcp(s.cam[j].focx), dv = fast_rcp(s.cam[j].focy);
             // The lists of partially covering fragments are kept for a window of the strip's rows at a time: all eight,
             // or, when the fragment array overflows (a dense soup of edges), half as many, again and again down to one
             // row -- the window is rasterized anew, the rows before it keep their composited colours (parked in their
@@ -550,7 +578,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
             // take no part in it), so the retries keep only the fragments in front of it (in a soup, few).  A single row that still overflows (many coplanar
             // primitives cut by the near plane along it) is taken half as many columns at a time, down to one pixel.
             int win = CSTRIP, cw = TILE, row_next = 0, col_next = 0;
-            bool prepass = false, prepass_done = false;
+            bool prepass = false, prepass_done = false, touched = false;
             while (row_next < CSTRIP) {
             const int row_lo = prepass ? 0 : row_next, row_hi = prepass ? 0 : min(row_next + win, CSTRIP);
             const int col_lo = col_next, col_hi = col_next + cw;
@@ -564,6 +592,8 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
                     const int by0 = (bw_lane >> 6) & 63, by1 = (bw_lane >> 18) & 63;
                     hit = !(bw_lane & REC_DEAD) && by1 >= ys && by0 < ys + CSTRIP;
                 }
+                if (!__any_sync(0xffffffffu, hit)) continue;
+                touched = true;
                 if (AA) {
                     // small records: every pixel of the box (in this strip's window) is worked off, a lane each whatever
                     // the record -- far cheaper than walking a 64-pixel cell per record for the handful of pixels a
@@ -601,7 +631,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
                     // values at the cell's pixel centres lie within +-h of its value at the cell's centre, h widened by
                     // several times what float32 can lose; a pixel is touched while the value at its centre is above -hh
                     const int xa = (lane & 3) * 16, ya = ((lane >> 2) & 1) * 4;
-                    bool out = lane >= 8 || xa + 15 < bx0 || xa > bx1 || ya + 3 < ly0 || ya > ly1;
+                    bool out = lane >= 8 || xa + 15 < bx0 || xa > bx1 || ya + 3 < ly0 || ya > ly1, inside = AA && !out;
                     if (AA) {
                         const float rxc = 0.5f * (ray_x[xa] + ray_x[xa + 15]), ryc = 0.5f * (ray_y[ya] + ray_y[ya + 3]);
                         const float hx = 8.001f * du + 1e-6f * fabsf(rxc), hy = 2.001f * dv + 1e-6f * fabsf(ryc);   // from the cell's centre to its pixels' far sides
@@ -610,12 +640,23 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
                             const float a = e < 4 ? q.nx[e] : q.wx, b = e < 4 ? q.ny[e] : q.wy, z = e < 4 ? q.nz[e] : q.wz;
                             const float c = fm(a, rxc, fm(b, ryc, z)), h = fm(fabsf(a), hx, fm(fabsf(b), hy, 1e-6f * fabsf(z)));
                             out = out || (e < 4 ? c + h < 0.f : c + h < P.w_far || c - h > P.w_near);
+                            inside = inside && (e < 4 ? c - h >= 0.f : c - h >= P.w_far && c + h <= P.w_near);
+                        }
+                    }
+                    unsigned cells = __ballot_sync(0xffffffffu, !out);
+                    if (AA) {
+                        const unsigned full = __ballot_sync(0xffffffffu, inside);
+                        cells &= ~full;
+#pragma unroll 1
+                        for (unsigned m = full; m; m &= m - 1) {
+                            const int cell = __ffs(m) - 1;
+                            cover_cell(key, ray_x, ray_y, q, key_lo, (cell & 3) * 16, (cell >> 2) * 4, lane);
                         }
                     }
 #pragma unroll 1
-                    for (unsigned cells = __ballot_sync(0xffffffffu, !out); cells; cells &= cells - 1) {
-                            const int cell = __ffs(cells) - 1, xx = (cell & 3) * 16, yy = (cell >> 2) * 4;
-                            colour_cell<AA>(key, head, frag, n_frag, n_pend, dropped, ray_x, ray_y, q, thr, hh, du, dv, key_lo, slot, P.w_near, P.w_far, xx, yy, row_lo, row_hi, col_lo, col_hi, lane);
+                    for (; cells; cells &= cells - 1) {
+                        const int cell = __ffs(cells) - 1, xx = (cell & 3) * 16, yy = (cell >> 2) * 4;
+                        colour_cell<AA>(key, head, frag, n_frag, n_pend, dropped, ray_x, ray_y, q, thr, hh, du, dv, key_lo, slot, P.w_near, P.w_far, xx, yy, row_lo, row_hi, col_lo, col_hi, lane);
                     }
                     // the queue is worked off when it holds a few rounds' worth (working it off frees room only for the
                     // pixels whose area turns out to be zero, so a nearly full array is no reason to do it earlier)
@@ -626,6 +667,7 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
                 }
                 __syncwarp();
             }
+            if (!touched) break;
             if (AA) flush_pending(key, frag, head, n_frag, n_pend, s.pool, ray_x, ray_y, du, dv, P.w_near, P.w_far, lane);
             __syncwarp();
             if (AA && prepass) { prepass = false; prepass_done = true; continue; }
@@ -644,7 +686,8 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
             if (col_next >= TILE) { col_next = 0; row_next = row_hi; }
             }   // (windows)
             __syncwarp();
-            resolve_store_colour(key, s.pool, P, jb, s.active[j] != 0, ys, vec_ok, lane);
+            if (touched) resolve_store_colour(key, s.pool, P, jb, s.active[j] != 0, ys, vec_ok, lane);
+            else store_strip_background(P, jb, s.active[j] != 0, ys, lane);
             __syncwarp();
         }
         done |= now;
