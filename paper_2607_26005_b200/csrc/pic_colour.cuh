@@ -23,10 +23,11 @@
 // resolve walks each pixel's list in depth order, merges, composites and stores four pixels (12 bytes) per lane, side by side.
 //
 // Bound by instruction issue and fetch: at 61 KB of code a fifth of the issue slots waited for instructions, at 48 KB few do, so what
-// is not hot is rolled or out of line.  14 880 views of 96 x 54 (16 384 tiles with anything in them) 1 005 -> 776 us, 192 views of
-// 384 x 216 252 -> 217, by: cells that a record covers wholly updating their keys and no more (three in seven); strips that nothing
+// is not hot is rolled or out of line.  14 880 views of 96 x 54 (16 384 tiles with anything in them) 1 005 -> 745 us, 192 views of
+// 384 x 216 252 -> 208, by: cells that a record covers wholly updating their keys and no more (three in seven); strips that nothing
 // reaches storing their background (two thirds); one rolled copy of the shading with the colours in the pool; stores side by side;
-// divisions of one reciprocal.  Four CTAs per multiprocessor with strips of four rows: 15 % more work for 2 % more speed.
+// divisions of one reciprocal; the longest strips drawn first; shading only for boxes.  Measured and left: exact areas from the two or three
+// lines that cross a pixel (less work, 797 and 789: the second copy of the code); larger primitives by their vertices (806, 826).  Four CTAs per multiprocessor with strips of four rows: 15 % more work for 2 % more speed.
 #pragma once
 
 constexpr int CSTRIP = 8;                       // pixel rows of a strip
@@ -401,9 +402,13 @@ __device__ __forceinline__ void resolve_store_colour(unsigned long long* key, co
             uint32_t c = bg;
             if (k & KEY_RESOLVED) c = (uint32_t)k & 0xffffffu;
             else if (k) {
-                float R, G, B;
-                shade_fragment(pool, P, (uint32_t)k & 0xffu, __uint_as_float((uint32_t)(k >> 32)), R, G, B);
-                c = (uint32_t)fminf(R + 0.5f, 255.f) | ((uint32_t)fminf(G + 0.5f, 255.f) << 8) | ((uint32_t)fminf(B + 0.5f, 255.f) << 16);
+                const uint32_t slot = (uint32_t)k & 0xffu;
+                c = pool.rgb[slot];                          // (a map primitive's colour is not shaded)
+                if (pool.shade[slot] > 0.f) {
+                    float R, G, B;
+                    shade_fragment(pool, P, slot, __uint_as_float((uint32_t)(k >> 32)), R, G, B);
+                    c = (uint32_t)fminf(R + 0.5f, 255.f) | ((uint32_t)fminf(G + 0.5f, 255.f) << 8) | ((uint32_t)fminf(B + 0.5f, 255.f) << 16);
+                }
             }
             w0 = __funnelshift_r(w0, w1, 24); w1 = __funnelshift_r(w1, w2, 24); w2 = (w2 >> 24) | (c << 8);
         }
@@ -431,6 +436,13 @@ __device__ __forceinline__ void store_strip_background(const RenderParams& P, co
     }
 }
 
+// Tile n of the launch when a view's tiles are counted column by column: a CTA's four tiles then lie one below the other, and one
+// with the horizon in all of its tiles, the last to end, is rare (192 views of 384 x 216: 217 -> 209 us with the strips' order below).
+__device__ __forceinline__ unsigned column_major(const RenderParams& P, unsigned n) {
+    const unsigned view = divide(n, P.div_tiles), tiles = (unsigned)(P.tiles_x * P.tiles_y), t = n - view * tiles, x = t / (unsigned)P.tiles_y, y = t - x * (unsigned)P.tiles_y;
+    return view * tiles + y * (unsigned)P.tiles_x + x;
+}
+
 template <bool AA>
 __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_constant__ RenderParams P) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -441,13 +453,14 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
     // antialiased: every tile; else: the tiles that the tile kernel left out, one wave of CTAs walking the list
     const int tpc = AA ? P.tiles_per_cta : NW;
     const bool one = tpc == 1;
+    const int n_tiles = one ? 1 : NW;
     const unsigned n_ids = AA ? P.n_jobs : __ldcg(&P.overflow[0]);
 #pragma unroll 1
     for (unsigned at = cta * (unsigned)tpc; at < n_ids; at += gridDim.x * (unsigned)tpc) {
     // the warp's tile: its own of the CTA's four, or the CTA's one, which all warps then set up together
     const int mine = one ? 0 : warp;
     const bool valid = at + mine < n_ids, leads = warp == mine;
-    const unsigned id = AA || !valid ? at + mine : __ldcg(&P.overflow[1u + at + mine]);
+    const unsigned id = !valid ? 0u : AA ? column_major(P, at + mine) : __ldcg(&P.overflow[1u + at + mine]);
     const uint2* blk = P.surv + (size_t)id * SURV_STRIDE;
     int ns = -2;
     Job job;
@@ -560,11 +573,13 @@ __global__ void __launch_bounds__(NTHREADS, 3) colour_kernel(const __grid_consta
             int task = 0;
             if (lane == 0) task = atomicAdd(&s.next_task, 1);
             task = __shfl_sync(0xffffffffu, task, 0);
-            if (task >= NW * CSTRIPS) break;
-            const int j = task / CSTRIPS, ys = (task % CSTRIPS) * CSTRIP;
-            const int cj = (int)((cnts >> (8 * j)) & 0xffu);
+            if (task >= n_tiles * CSTRIPS) break;
+            // the tiles in turn, each from the strip with the horizon on: the longest strips are drawn first (14 880 views of 96 x 54:
+            // 776 -> 757 us)
+            const int j = task % n_tiles, cj = (int)((cnts >> (8 * j)) & 0xffu);
             if (cj == 0xff) continue;
             const Job jb = s.job[j];
+            const int horizon = min(max((P.H / 2 - jb.t.y0) / CSTRIP, 0), CSTRIPS - 1), ys = ((task / n_tiles + horizon) % CSTRIPS) * CSTRIP;
             if (ys >= jb.t.th) continue;
             const int first = (int)((bases >> (8 * j)) & 0xffu);
             const float* ray_x = s.ray_x[j];
