@@ -159,7 +159,7 @@ pic_status fill_params(const pic_scene* s, const pic_camera* rig, uint8_t* out_c
     P.surv = s->d_surv;
     P.palette = s->d_palette;
     P.status = s->d_status;
-    P.rig = pic::rig_tables(s->d_tables, s->K, s->H, s->W);
+    P.rig = pic::rig_tables(s->d_tables + pic::frusta_bytes(s->K, s->H, s->W) / sizeof(float), s->K, s->H, s->W, reinterpret_cast<float4*>(s->d_tables));
     P.out_class = out_class; P.out_depth = out_depth; P.out_depth32 = s->depth32; P.counters = s->counters; P.occlusion = s->occlusion;
     P.view_first = 0;
     P.debug_flags = s->debug_flags;
@@ -275,7 +275,7 @@ pic_status pic_scene_create(const pic_scene_desc* d, pic_scene** out) {
     dmalloc((void**)&s->d_cams, sizeof(pic::ViewCam) * n_agents * d->K);
     dmalloc((void**)&s->d_overflow, sizeof(uint32_t) * (1 + (size_t)n_agents * d->K * ((d->W + pic::TILE - 1) / pic::TILE) * ((d->H + pic::TILE - 1) / pic::TILE)));
     dmalloc((void**)&s->d_surv, pic::survivor_bytes_per_tile() * (size_t)n_agents * d->K * ((d->W + pic::TILE - 1) / pic::TILE) * ((d->H + pic::TILE - 1) / pic::TILE));
-    dmalloc((void**)&s->d_tables, pic::table_bytes(d->K, d->H, d->W));
+    dmalloc((void**)&s->d_tables, pic::frusta_bytes(d->K, d->H, d->W) + pic::table_bytes(d->K, d->H, d->W));
     dmalloc((void**)&s->d_state, sizeof(float) * 4 * n_agents);
     dmalloc((void**)&s->d_dims, sizeof(float) * 3 * n_agents);
     dmalloc((void**)&s->d_active, n_agents);

@@ -10,7 +10,7 @@ constexpr int SETUP_THREADS = 128;
 
 struct RigParams {
     int32_t K, W, H;
-    float far_z;
+    float near_z, far_z;
     uint32_t cls_sky, cls_ground;
     const uint32_t* palette;      // NULL: no colours are rendered
     CamConst cam[MAX_CAMS];
@@ -100,6 +100,16 @@ __device__ __forceinline__ void rig_setup(const RigParams& R, int k, const RigTa
     uint32_t* bg_rgb = const_cast<uint32_t*>(T.bg_rgb);
     const CamConst c = R.cam[k];
     const float cx = 0.5f * (float)R.W, cy = 0.5f * (float)R.H;
+    if (T.frusta) {
+        const int tx = (R.W + TILE - 1) / TILE, tiles = tx * ((R.H + TILE - 1) / TILE);
+        float4* frusta = const_cast<float4*>(T.frusta) + (size_t)k * (tiles + 1) * FRUSTUM_ENTRIES;
+        for (int i = threadIdx.x; i < (tiles + 1) * FRUSTUM_ENTRIES; i += blockDim.x) {
+            const int t = i / FRUSTUM_ENTRIES, x0 = t % tx * TILE, y0 = t / tx * TILE;
+            const bool whole = t == tiles;
+            frusta[i] = whole ? frustum_entry(i % FRUSTUM_ENTRIES, -cx, (float)R.W - cx, -cy, (float)R.H - cy, c.fx, c.fy, R.near_z, R.far_z)
+                              : frustum_entry(i % FRUSTUM_ENTRIES, (float)x0 - cx, (float)min(x0 + TILE, R.W) - cx, (float)y0 - cy, (float)min(y0 + TILE, R.H) - cy, c.fx, c.fy, R.near_z, R.far_z);
+        }
+    }
     const int nx = ray_stride(R.W), ny = ray_stride(R.H);
     for (int u = threadIdx.x; u < nx; u += blockDim.x)
         ray_x[(size_t)k * nx + u] = __fdiv_rn(sub(add((float)u, 0.5f), cx), c.fx);
@@ -171,7 +181,7 @@ cudaError_t configure_kernels() {
 
 static RigParams rig_params(const RenderParams& P) {
     RigParams R;
-    R.K = P.K; R.W = P.W; R.H = P.H; R.far_z = P.far_z; R.cls_sky = P.cls_sky; R.cls_ground = P.cls_ground;
+    R.K = P.K; R.W = P.W; R.H = P.H; R.near_z = P.near_z; R.far_z = P.far_z; R.cls_sky = P.cls_sky; R.cls_ground = P.cls_ground;
     R.palette = P.out_rgb ? P.palette : nullptr;
     for (int k = 0; k < MAX_CAMS; ++k) R.cam[k] = P.cam[k];
     return R;

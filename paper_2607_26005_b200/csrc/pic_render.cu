@@ -744,36 +744,40 @@ __device__ __forceinline__ void deal_survivors(uint2* __restrict__ surv, const R
     }
 }
 
-// Camera, frustum planes and footprint of a tile, by one warp.  The footprint is the convex hull of the apex and the
-// four far corners, kept as the segments between them (the hull's edges are among them, the others lie inside it).
-__device__ __forceinline__ void frustum_setup(Frustum& f, const RenderParams& P, const Job& job, int lane) {
-    const TileCtx& t = job.t;
-    if (lane < 7) {
+// Camera, frustum planes and footprint of a part of a view, by one warp.  `entry`: of lane i < FRUSTUM_ENTRIES the part's entry i in
+// camera space.  The same rotation turns the normals of the planes and the corners of the footprint.  The footprint is the convex
+// hull of the apex and the four far corners, kept as the segments between them (the hull's edges are among them, the others lie
+// inside it).
+__device__ __forceinline__ void frustum_setup(Frustum& f, const RenderParams& P, const Job& job, const float4 entry, int lane) {
+    if (lane < FRUSTUM_ENTRIES) {
         Cam c;
         load_camera(c, P.cams[job.view], P.cam[job.k], P.W, P.H);
+        const float x = fm(c.rx, entry.x, fm(c.dx, entry.y, c.fx_ * entry.z)), y = fm(c.ry, entry.x, fm(c.dy, entry.y, c.fy_ * entry.z)), z = fm(c.dz, entry.y, c.fz_ * entry.z);
+        if (lane < 6) {
+            *reinterpret_cast<float4*>(f.plane[lane]) = make_float4(x, y, z, entry.w - fm(x, c.mwx, fm(y, c.mwy, z * c.mwz)));
+            if (lane >= 2) *reinterpret_cast<float4*>(f.side[lane - 2]) = entry;
+        } else {
+            f.pt[lane - 6][0] = c.mwx + x;
+            f.pt[lane - 6][1] = c.mwy + y;
+        }
         if (lane == 6) {
             f.cam = c;
             f.n_seg = (c.dx == 0.f && c.dy == 0.f) ? 3 : 10;     // no pitch: corners 1, 3 and 2, 4 have the same x, y
-        } else {
-            tile_planes(f, lane, c, t);
-        }
-        if (lane < 5) {
-            // footprint corner `lane`: the apex, or a corner of the tile's frustum at depth far (a little beyond)
-            const float F = lane ? t.far_z * 1.001f : 0.f;
-            const float xc = ((float)((lane & 1) ? t.x0 + t.tw : t.x0) - c.cx) / c.focx * F;
-            const float yc = ((float)((lane & 2) ? t.y0 + t.th : t.y0) - c.cy) / c.focy * F;
-            f.pt[lane][0] = c.mwx + c.rx * xc + c.dx * yc + c.fx_ * F;
-            f.pt[lane][1] = c.mwy + c.ry * xc + c.dy * yc + c.fy_ * F;
         }
     }
     __syncwarp();
     if (lane < 10) {
-        const int i = (int)((0x3221100100ull >> (4 * lane)) & 15u), j = (int)((0x4434343221ull >> (4 * lane)) & 15u);   // (0,1) (0,2) (1,2) (0,3) (0,4) (1,3) (1,4) (2,3) (2,4) (3,4)
+        const int i = (int)((0x3221100100ull >> (4 * lane)) & 15u), j = (int)((0x4434443221ull >> (4 * lane)) & 15u);   // (0,1) (0,2) (1,2) (0,3) (0,4) (1,3) (1,4) (2,3) (2,4) (3,4)
         const float px = f.pt[i][0], py = f.pt[i][1], dx = f.pt[j][0] - px, dy = f.pt[j][1] - py;
         f.seg[lane][0] = px; f.seg[lane][1] = py; f.seg[lane][2] = dx; f.seg[lane][3] = dy;
-        f.seg[lane][4] = dy != 0.f ? 1.f / dy : 0.f; f.seg[lane][5] = 0.f;
+        f.seg[lane][4] = fabsf(dy) > 1e-30f ? fast_rcp(dy) : 0.f; f.seg[lane][5] = 0.f;
     }
     __syncwarp();
+}
+// Lane i's entry of the frustum of a tile, or (tile = number of tiles) of the whole image.
+__device__ __forceinline__ float4 frustum_table(const RenderParams& P, const Job& job, int tile, int lane) {
+    const int tiles = P.tiles_x * P.tiles_y;
+    return lane < FRUSTUM_ENTRIES ? __ldg(P.rig.frusta + (size_t)((job.k * (tiles + 1) + tile) * FRUSTUM_ENTRIES + lane)) : make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
 // The grid rows crossed by the footprint, widened by the map's margin.
@@ -805,7 +809,7 @@ __device__ __forceinline__ void row_range(const Frustum& f, const RenderParams& 
         const float ya = fminf(py, py + dy), yb = fmaxf(py, py + dy);
         if (yb >= blo && ya <= bhi) {
             const float ta = (blo - py) * idy, tb = (bhi - py) * idy;
-            const float t0 = dy != 0.f ? fminf(fmaxf(fminf(ta, tb), 0.f), 1.f) : 0.f, t1 = dy != 0.f ? fminf(fmaxf(fmaxf(ta, tb), 0.f), 1.f) : 1.f;
+            const float t0 = idy != 0.f ? fminf(fmaxf(fminf(ta, tb), 0.f), 1.f) : 0.f, t1 = idy != 0.f ? fminf(fmaxf(fmaxf(ta, tb), 0.f), 1.f) : 1.f;
             const float xa = px + t0 * dx, xb = px + t1 * dx;
             xlo = fminf(xlo, fminf(xa, xb)); xhi = fmaxf(xhi, fmaxf(xa, xb));
         }
@@ -885,7 +889,7 @@ __device__ __forceinline__ bool front_cull(FrontLists& f, uint2* __restrict__ su
     if (b0 + lane < P.A) ag0 = load_agent(env_agents + b0 + lane);
     if (b0 + lane + 32 < P.A) ag1 = load_agent(env_agents + b0 + lane + 32);
     Frustum& fr = f.f;
-    frustum_setup(fr, P, job, lane);
+    frustum_setup(fr, P, job, frustum_table(P, job, MULTI ? P.tiles_x * P.tiles_y : job.tile, lane), lane);
     const Cam& c = fr.cam;
     const unsigned below = (1u << lane) - 1u;
     int n_item = 0;                                // (entries are appended in order of lane, so that a call's lists are the same every time)
@@ -1177,7 +1181,8 @@ __global__ void __launch_bounds__(32) coverage_kernel(const __grid_constant__ Re
     t.w_near = P.w_near; t.w_far = P.w_far; t.near_z = P.near_z; t.far_z = P.far_z;
     const AgentGeom* env_agents = P.agents + (size_t)job.e * P.A;
     if (!env_agents[job.a].active) return;
-    frustum_setup(s.f, P, job, lane);
+    const float cx = 0.5f * (float)P.W, cy = 0.5f * (float)P.H;
+    frustum_setup(s.f, P, job, frustum_entry(lane, -cx, (float)P.W - cx, (float)t.y0 - cy, (float)(t.y0 + t.th) - cy, P.cam[job.k].fx, P.cam[job.k].fy, t.near_z, t.far_z), lane);
     const Cam& c = s.f.cam;
     const float* ray_x = P.rig.ray_x + (size_t)job.k * ray_stride(P.W);
     const float* ray_y = P.rig.ray_y + (size_t)job.k * ray_stride(P.H) + t.y0;

@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 2) render_small_kernel(const __
     const bool ego_active = __ldg(&env_agents[job.a].active) != 0u;
     bool fits = true;
     if (warp == 0) {
-        frustum_setup(s.f, P, job, lane);
+        frustum_setup(s.f, P, job, frustum_table(P, job, job.tile, lane), lane);
     } else if (warp == 1) {
         if (lane == 0) { s.n_rec = 0; s.n_leaf = 0; s.n_face = 0; s.frag_cells = 0u; }
         s.recs[lane] = {0u, 0u, 0u};

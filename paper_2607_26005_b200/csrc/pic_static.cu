@@ -128,7 +128,7 @@ extern "C" pic_status pic_render_static(const pic_static_desc* d, const float* t
     float* tables = reinterpret_cast<float*>(scratch + kOffTables);
     uint32_t* status = reinterpret_cast<uint32_t*>(scratch + kOffStatus);
     P.agents = agents; P.cams = cams;
-    P.rig = rig_tables(tables, d->K, d->H, d->W);
+    P.rig = rig_tables(tables, d->K, d->H, d->W, nullptr);
     P.out_class = out_class; P.out_depth = out_depth;
     for (int k = 0; k < d->K; ++k) {
         CamConst& o = P.cam[k];

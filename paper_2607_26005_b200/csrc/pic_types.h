@@ -81,9 +81,10 @@ struct ViewCam {
 };
 static_assert(sizeof(ViewCam) == 64, "ViewCam must be 64 bytes");
 
-// Per-camera tables shared by all views of a call: ray coordinates of pixel columns / rows and the
-// background (analytic ground plane / sky) of every row.
+// Per-camera tables shared by all views of a call: ray coordinates of pixel columns / rows, the background (analytic ground plane /
+// sky) of every row, and the frusta of the tiles.
 struct RigTables {
+    const float4* frusta;      // [K][tiles + 1][FRUSTUM_ENTRIES] in camera space (see frustum_entry); the last of a camera's is the whole image's. NULL: not made
     const float* ray_x;        // [K][ray_stride(W)], [K][ray_stride(H)]: beyond the image the same formula goes on, so that a tile that
     const float* ray_y;        //   reaches over the edge reads a monotone table
     const float* bg_z;         // [K][H] background depth
@@ -146,10 +147,13 @@ __host__ __device__
 #endif
 inline int ray_stride(int n) { return (n + 2 * TILE - 1) / TILE * TILE; }
 
-// Layout of the per-camera tables in one allocation of table_bytes bytes.
+constexpr int FRUSTUM_ENTRIES = 11;      // six planes, five corners of the footprint
+inline size_t frusta_bytes(int K, int H, int W) { return sizeof(float4) * FRUSTUM_ENTRIES * (size_t)K * ((size_t)((W + TILE - 1) / TILE) * (size_t)((H + TILE - 1) / TILE) + 1); }
+// Layout of the per-camera tables: the frusta, then those of table_bytes bytes.
 inline size_t table_bytes(int K, int H, int W) { return sizeof(float) * (size_t)K * ((size_t)ray_stride(W) + (size_t)ray_stride(H) + 3 * (size_t)H); }
-inline RigTables rig_tables(float* base, int K, int H, int W) {
+inline RigTables rig_tables(float* base, int K, int H, int W, float4* frusta) {
     RigTables r;
+    r.frusta = frusta;
     r.ray_x = base;
     r.ray_y = r.ray_x + (size_t)K * ray_stride(W);
     r.bg_z = r.ray_y + (size_t)K * ray_stride(H);
