@@ -231,11 +231,10 @@ __device__ __forceinline__ bool pixel_box_int(const Cam& c, const TileCtx& t, co
         }
         // pixel centres u + 0.5 in [sx0, sx1], widened by m = 1/256 pixel against rounding (m = 1/2 + 1/256: every pixel
         // whose unit square the primitive touches)
-        float fx0 = ceilf(sx0 - 0.5f - m) - (float)t.x0, fx1 = floorf(sx1 - 0.5f + m) - (float)t.x0;
-        float fy0 = ceilf(sy0 - 0.5f - m) - (float)t.y0, fy1 = floorf(sy1 - 0.5f + m) - (float)t.y0;
-        ok = ok && (fx0 <= fx1) && (fy0 <= fy1) && (fx1 >= 0.f) && (fy1 >= 0.f) && (fx0 <= (float)(t.tw - 1)) && (fy0 <= (float)(t.th - 1));
-        bx0 = (int)fmaxf(fx0, 0.f); by0 = (int)fmaxf(fy0, 0.f);
-        bx1 = (int)fminf(fx1, (float)(t.tw - 1)); by1 = (int)fminf(fy1, (float)(t.th - 1));
+        const float fx0 = fmaxf(ceilf(sx0 - 0.5f - m) - (float)t.x0, 0.f), fx1 = fminf(floorf(sx1 - 0.5f + m) - (float)t.x0, (float)(t.tw - 1));
+        const float fy0 = fmaxf(ceilf(sy0 - 0.5f - m) - (float)t.y0, 0.f), fy1 = fminf(floorf(sy1 - 0.5f + m) - (float)t.y0, (float)(t.th - 1));
+        ok = ok && fx0 <= fx1 && fy0 <= fy1;
+        bx0 = (int)fx0; by0 = (int)fy0; bx1 = (int)fx1; by1 = (int)fy1;
     } else if (ok) {
         // frustum side planes through the camera centre, valid for any sign of z
         float l = (float)t.x0 - c.cx, r = (float)(t.x0 + t.tw) - c.cx, u = (float)t.y0 - c.cy, d = (float)(t.y0 + t.th) - c.cy;

@@ -629,8 +629,7 @@ static_assert(offsetof(Frustum, plane) % 16 == 0 && offsetof(Frustum, side) % 16
 struct __align__(16) FrontLists {
     Frustum f;
     uint32_t item[W_ITEM];                    // survivor ids to be tested
-    uint32_t row_first[32];                   // grid rows of a pass: first entry of the row's range in cell_prims
-    uint32_t row_off[33];                     //   and the number of candidates before the row (the total at [32])
+    uint32_t row_base[32];                    // grid rows of a pass that have candidates: first entry of the row's range in grid_prims less the candidates before it
 };
 
 // Box test against planes held in registers (see box_visible).
@@ -946,7 +945,8 @@ __device__ __forceinline__ bool front_cull(FrontLists& f, uint2* __restrict__ su
     if (!ROUNDS && !boxes_done) return false;
     l_done = l0 - mi.large_begin;
     // ---- fill the item list with the candidates of the grid rows (32 rows per pass), test the items, until both are done
-    int row = rows.lo, i0 = 0, total = -1;         // total < 0: the ranges of the pass have not been laid out
+    int row = rows.lo, i0 = 0, total = -1, rows_seen = 0;    // total < 0: the ranges of the pass have not been laid out; rows_seen: begun before candidate i0
+    uint32_t row_at = 0u;                          // number of candidates before the lane's row (beyond all if it has none)
     bool more = boxes_done && row <= rows.hi;
     if (more && row + lane <= rows.hi) ++n.grp;
 #pragma unroll 1
@@ -965,11 +965,12 @@ __device__ __forceinline__ bool front_cull(FrontLists& f, uint2* __restrict__ su
                 }
                 total = (int)__shfl_sync(0xffffffffu, incl, 31);
                 __syncwarp();
-                f.row_first[lane] = first;
-                f.row_off[lane] = incl - cnt;
-                if (lane == 31) f.row_off[32] = incl;
+                const unsigned any = __ballot_sync(0xffffffffu, cnt > 0u);
+                row_at = cnt > 0u ? incl - cnt : 0x7fffffffu;
+                if (cnt > 0u) f.row_base[__popc(any & below)] = first - row_at;
                 __syncwarp();
                 i0 = 0;
+                rows_seen = 0;
             }
             if (i0 < total) {
                 float4 b[2];
@@ -978,12 +979,12 @@ __device__ __forceinline__ bool front_cull(FrontLists& f, uint2* __restrict__ su
                 for (int u = 0; u < 2; ++u) {
                     const int i = i0 + 32 * u + lane;
                     b[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    // (the rows that begin at one of these 32 candidates, a bit each: a candidate's row is the number of rows begun so far)
+                    const uint32_t at = row_at - (uint32_t)(i0 + 32 * u), starts = __reduce_or_sync(0xffffffffu, at < 32u ? 1u << at : 0u);
+                    const int r = rows_seen + __popc(starts & (below | (1u << lane))) - 1;
+                    rows_seen += __popc(starts);
                     if (i < total) {
-                        int r = 0;
-#pragma unroll
-                        for (int st = 16; st; st >>= 1)
-                            if (f.row_off[r + st] <= (uint32_t)i) r += st;
-                        id[u] = f.row_first[r] + ((uint32_t)i - f.row_off[r]);
+                        id[u] = f.row_base[r] + (uint32_t)i;
                         b[u] = __ldg(reinterpret_cast<const float4*>(P.grid_bounds) + id[u]);
                     }
                 }
