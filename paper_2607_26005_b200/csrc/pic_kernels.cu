@@ -100,16 +100,6 @@ __device__ __forceinline__ void rig_setup(const RigParams& R, int k, const RigTa
     uint32_t* bg_rgb = const_cast<uint32_t*>(T.bg_rgb);
     const CamConst c = R.cam[k];
     const float cx = 0.5f * (float)R.W, cy = 0.5f * (float)R.H;
-    if (T.frusta) {
-        const int tx = (R.W + TILE - 1) / TILE, tiles = tx * ((R.H + TILE - 1) / TILE);
-        float4* frusta = const_cast<float4*>(T.frusta) + (size_t)k * (tiles + 1) * FRUSTUM_ENTRIES;
-        for (int i = threadIdx.x; i < (tiles + 1) * FRUSTUM_ENTRIES; i += blockDim.x) {
-            const int t = i / FRUSTUM_ENTRIES, x0 = t % tx * TILE, y0 = t / tx * TILE;
-            const bool whole = t == tiles;
-            frusta[i] = whole ? frustum_entry(i % FRUSTUM_ENTRIES, -cx, (float)R.W - cx, -cy, (float)R.H - cy, c.fx, c.fy, R.near_z, R.far_z)
-                              : frustum_entry(i % FRUSTUM_ENTRIES, (float)x0 - cx, (float)min(x0 + TILE, R.W) - cx, (float)y0 - cy, (float)min(y0 + TILE, R.H) - cy, c.fx, c.fy, R.near_z, R.far_z);
-        }
-    }
     const int nx = ray_stride(R.W), ny = ray_stride(R.H);
     for (int u = threadIdx.x; u < nx; u += blockDim.x)
         ray_x[(size_t)k * nx + u] = __fdiv_rn(sub(add((float)u, 0.5f), cx), c.fx);
@@ -125,15 +115,32 @@ __device__ __forceinline__ void rig_setup(const RigParams& R, int k, const RigTa
     }
 }
 
-// One launch prepares a call: the first K blocks write a camera's tables each, the others set up an agent per thread.
+// The frusta of camera k's tiles and of its whole image.
+__device__ __forceinline__ void frusta_setup(const RigParams& R, int k, const RigTables& T) {
+    const CamConst c = R.cam[k];
+    const float cx = 0.5f * (float)R.W, cy = 0.5f * (float)R.H;
+    const int tx = (R.W + TILE - 1) / TILE, tiles = tx * ((R.H + TILE - 1) / TILE);
+    float4* frusta = const_cast<float4*>(T.frusta) + (size_t)k * (tiles + 1) * FRUSTUM_ENTRIES;
+    for (int i = threadIdx.x; i < (tiles + 1) * FRUSTUM_ENTRIES; i += blockDim.x) {
+        const int t = i / FRUSTUM_ENTRIES, x0 = t % tx * TILE, y0 = t / tx * TILE;
+        const bool whole = t == tiles;
+        frusta[i] = frustum_entry(i % FRUSTUM_ENTRIES, whole ? -cx : (float)x0 - cx, (float)(whole ? R.W : min(x0 + TILE, R.W)) - cx, whole ? -cy : (float)y0 - cy,
+                                  (float)(whole ? R.H : min(y0 + TILE, R.H)) - cy, c.fx, c.fy, R.near_z, R.far_z);
+    }
+}
+
+// One launch prepares a call: the first K blocks write a camera's tables each, the next K its frusta if wanted, the others set up an
+// agent per thread.
 __global__ void __launch_bounds__(SETUP_THREADS) setup_kernel(const __grid_constant__ AgentArgs G, const __grid_constant__ RigParams R,
                                                               const __grid_constant__ RigTables T, uint32_t* overflow) {
     launch_dependents();
     if (overflow && blockIdx.x == 0 && threadIdx.x == 0) overflow[0] = 0u;   // the render kernels' list of left-out tiles starts empty (absent for callers that do not use them)
     if ((int)blockIdx.x < R.K) {
         rig_setup(R, (int)blockIdx.x, T);
+    } else if (T.frusta && (int)blockIdx.x < 2 * R.K) {
+        frusta_setup(R, (int)blockIdx.x - R.K, T);
     } else {
-        const int i = ((int)blockIdx.x - R.K) * SETUP_THREADS + (int)threadIdx.x;
+        const int i = ((int)blockIdx.x - (T.frusta ? 2 : 1) * R.K) * SETUP_THREADS + (int)threadIdx.x;
         if (i < G.n) agent_setup(G, R, i);
     }
 }
@@ -196,7 +203,7 @@ cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses
     G.n = n_agents; G.poses = poses; G.state = state; G.actions = actions; G.dims = dims; G.active = active;
     G.agent_cls = agent_cls; G.default_cls = P.cls_agent; G.out = agents_out; G.cams = cams_out; G.status = status;
     G.dt = dt; G.wheelbase = wheelbase; G.v_max = v_max;
-    setup_kernel<<<P.K + (n_agents + SETUP_THREADS - 1) / SETUP_THREADS, SETUP_THREADS, 0, stream>>>(G, R, P.rig, P.overflow);
+    setup_kernel<<<(P.rig.frusta ? 2 : 1) * P.K + (n_agents + SETUP_THREADS - 1) / SETUP_THREADS, SETUP_THREADS, 0, stream>>>(G, R, P.rig, P.overflow);
     return cudaGetLastError();
 }
 
