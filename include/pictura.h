@@ -277,7 +277,7 @@ pic_status pic_step_rgb(pic_scene* scene, const float* actions, const pic_camera
  * caller's triangles directly (one map shared by all environments, every triangle tested against
  * every tile, those that reach it rasterized -- meant for small batches and small maps).  Per-agent geometry,
  * per-view cameras, per-camera tables and the status word live in one fixed device array that is
- * part of the library image (about 490 KB on every device that loads the library, until exit).
+ * part of the library image (about 470 KB on every device that loads the library, until exit).
  * The call itself uses no cudaMalloc/cudaFree and no allocating library routine.
  *
  * Limits (PIC_ERR_CAPACITY beyond them): E*A <= PIC_STATIC_MAX_AGENTS, E*A*K <= PIC_STATIC_MAX_VIEWS,

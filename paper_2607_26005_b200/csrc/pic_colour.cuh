@@ -735,9 +735,8 @@ cudaError_t launch_colour_kernel(const RenderParams& P0, long long n_views, bool
     if (err != cudaSuccess) return err;
     if (antialias) return launch_next(colour_kernel<true>, grid, sizeof(ColourSmem), stream, P);
     // plain colours: the tile kernel, then the tiles it left out
-    const cudaError_t terr = launch_next(P.W % 4 == 0 && (reinterpret_cast<uintptr_t>(P.out_rgb) & 3u) == 0 ? render_tile_kernel<NoTally, true, false, true>
-                                                                                                            : render_tile_kernel<NoTally, false, false, true>,
-                                         (unsigned)jobs, 0, stream, P, 32);
+    const cudaError_t terr = P.W % 4 == 0 && (reinterpret_cast<uintptr_t>(P.out_rgb) & 3u) == 0 ? launch_tiles<true, false, true>(P, n_views, sm_count, stream)
+                                                                                               : launch_tiles<false, false, true>(P, n_views, sm_count, stream);
     if (terr != cudaSuccess) return terr;
     const unsigned wave = 3u * (unsigned)sm_count;
     return launch_next(colour_kernel<false>, grid < wave ? grid : wave, sizeof(ColourSmem), stream, P);

@@ -445,6 +445,14 @@ __device__ __forceinline__ Job decode_job(const RenderParams& P, unsigned id, in
     return j;
 }
 
+// The job CTA i of a launch takes where the tiles with the horizon of all views come first, then the rows below, the sky last, so that
+// the last CTAs to come in are not the ones that take longest.
+__device__ __forceinline__ unsigned horizon_first(const RenderParams& P, unsigned i) {
+    const unsigned tiles = (unsigned)(P.tiles_x * P.tiles_y), pos = divide(i, P.div_views), view = i - pos * divide(P.n_jobs, P.div_tiles);
+    const unsigned t = pos + (unsigned)(P.H / (2 * TILE) * P.tiles_x);
+    return view * tiles + (t < tiles ? t : t - tiles);
+}
+
 // Ray coordinates of tile column / row i, 0..63.
 __device__ __forceinline__ float ray_column(const RenderParams& P, const Job& j, int i) { return __ldg(P.rig.ray_x + (size_t)j.k * ray_stride(P.W) + j.t.x0 + i); }
 __device__ __forceinline__ float ray_row(const RenderParams& P, const Job& j, int i) { return __ldg(P.rig.ray_y + (size_t)j.k * ray_stride(P.H) + j.t.y0 + i); }
@@ -1158,7 +1166,7 @@ cudaError_t configure_render_kernel() {
 // spheres, a lane each; the visible ones' faces are set up four agents at a time, eight lanes per agent of which six have a
 // face; then the agents are counted one after the other, a lane per pixel of the box around the agent's faces.  Bound by
 // instruction issue.  (A warp per tile that set up and drew one face of one agent after the other took 299 us for 4 096 views
-// of 100 x 70 pixels and 64 agents.)  The arithmetic that decides a pixel is the production kernels' (pic_device.cuh).
+// of 100 x 70 pixels and 64 agents; one pixel per lane at a time instead of four 81 us where it now takes 64.)  The arithmetic that decides a pixel is the production kernels' (pic_device.cuh).
 // ---------------------------------------------------------------------------------------------
 struct __align__(16) CoverWarp {
     float4 edge[4][32], w[32];                // faces of the batch by lane: edge functions with their thresholds, 1/z plane
@@ -1166,11 +1174,12 @@ struct __align__(16) CoverWarp {
     uint32_t agent[32];                       // visible agents of a pass: agent << 8 | faces to draw
 };
 
-__global__ void __launch_bounds__(32) coverage_kernel(const __grid_constant__ RenderParams P, int bands, int band_rows) {
+__global__ void __launch_bounds__(32) coverage_kernel(const __grid_constant__ RenderParams P, unsigned n_views, int bands, int band_rows) {
     __shared__ CoverWarp s;
     const int lane = threadIdx.x;
-    const unsigned id = blockIdx.x;
-    const unsigned vrel = id / (unsigned)bands, v = (unsigned)P.view_first + vrel, va = divide(v, P.div_K);
+    // (the band with the horizon of all views first: all agents in view are in it, and the last warps to come in have little to do)
+    const unsigned pos = blockIdx.x / n_views, vrel = blockIdx.x - pos * n_views, band = (pos + (unsigned)(P.H / 2 / band_rows)) % (unsigned)bands;
+    const unsigned v = (unsigned)P.view_first + vrel, va = divide(v, P.div_K);
     Job job;
     job.view = v;
     job.k = (int)(v - va * (unsigned)P.K);
@@ -1178,7 +1187,7 @@ __global__ void __launch_bounds__(32) coverage_kernel(const __grid_constant__ Re
     job.a = (int)(va - (unsigned)job.e * (unsigned)P.A);
     job.tile = 0;
     TileCtx& t = job.t;
-    t.x0 = 0; t.tw = P.W; t.y0 = (int)(id - vrel * (unsigned)bands) * band_rows; t.th = min(band_rows, P.H - t.y0);
+    t.x0 = 0; t.tw = P.W; t.y0 = (int)band * band_rows; t.th = min(band_rows, P.H - t.y0);
     t.w_near = P.w_near; t.w_far = P.w_far; t.near_z = P.near_z; t.far_z = P.far_z;
     const AgentGeom* env_agents = P.agents + (size_t)job.e * P.A;
     if (!env_agents[job.a].active) return;
@@ -1240,25 +1249,36 @@ __global__ void __launch_bounds__(32) coverage_kernel(const __grid_constant__ Re
                 int y = lane / w, x = lane - y * w;
                 uint32_t cnt = 0u;
                 for (; __any_sync(0xffffffffu, y < h); ) {
-                    bool in = false;
-                    if (y < h) {
-                        const float rx = __ldg(ray_x + x0 + x), ry = __ldg(ray_y + y0 + y);
-                        for (unsigned fm_ = faces; fm_; fm_ &= fm_ - 1) {
-                            const int f = 8 * i + __ffs(fm_) - 1;
-                            const float4 pw = s.w[f];
-                            const float wv = fm(pw.x, rx, fm(pw.y, ry, pw.z));
-                            bool cov = (wv >= t.w_far) & (wv <= t.w_near);
+                    // four pixels per lane at a time: a face is read once for them, and one's latency hides behind the others
+                    float rx[4], ry[4];
+                    bool have[4], in[4];
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const float4 q = s.edge[e][f];
-                                cov = cov & (fm(q.x, rx, fm(q.y, ry, q.z)) > q.w);
-                            }
-                            in = in | cov;
+                    for (int k = 0; k < 4; ++k) {
+                        have[k] = y < h;
+                        in[k] = false;
+                        rx[k] = have[k] ? __ldg(ray_x + x0 + x) : 0.f;
+                        ry[k] = have[k] ? __ldg(ray_y + y0 + y) : 0.f;
+                        x += dx; y += dy;
+                        if (x >= w) { x -= w; ++y; }
+                    }
+#pragma unroll 1
+                    for (unsigned fm_ = faces; fm_; fm_ &= fm_ - 1) {
+                        const int f = 8 * i + __ffs(fm_) - 1;
+                        const float4 pw = s.w[f], e0 = s.edge[0][f], e1 = s.edge[1][f], e2 = s.edge[2][f], e3 = s.edge[3][f];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            const float wv = fm(pw.x, rx[k], fm(pw.y, ry[k], pw.z));
+                            bool cov = wv >= t.w_far;
+                            cov = cov & (wv <= t.w_near);
+                            cov = cov & (fm(e0.x, rx[k], fm(e0.y, ry[k], e0.z)) > e0.w);
+                            cov = cov & (fm(e1.x, rx[k], fm(e1.y, ry[k], e1.z)) > e1.w);
+                            cov = cov & (fm(e2.x, rx[k], fm(e2.y, ry[k], e2.z)) > e2.w);
+                            cov = cov & (fm(e3.x, rx[k], fm(e3.y, ry[k], e3.z)) > e3.w);
+                            in[k] = in[k] | cov;
                         }
                     }
-                    cnt += in ? 1u : 0u;
-                    x += dx; y += dy;
-                    if (x >= w) { x -= w; ++y; }
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) cnt += have[k] & in[k] ? 1u : 0u;
                 }
                 cnt = __reduce_add_sync(0xffffffffu, cnt);
                 if (lane == 0 && cnt) atomicAdd(occ + 2 * (s.agent[j0 + i] >> 8) + 1, cnt);
@@ -1273,7 +1293,7 @@ __global__ void __launch_bounds__(32) coverage_kernel(const __grid_constant__ Re
 static cudaError_t run_coverage(const RenderParams& P, long long n_views, cudaStream_t stream) {
     const int band_rows = 16, bands = (P.H + band_rows - 1) / band_rows;
     if (n_views * bands > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    coverage_kernel<<<(unsigned)(n_views * bands), 32, 0, stream>>>(P, bands, band_rows);
+    coverage_kernel<<<(unsigned)(n_views * bands), 32, 0, stream>>>(P, (unsigned)n_views, bands, band_rows);
     return cudaGetLastError();
 }
 
@@ -1297,6 +1317,16 @@ static cudaError_t launch_cull(const RenderParams& P, long long n_views, bool co
     return launch_next(P.counters ? cull_kernel<Tally, false> : conservative ? cull_kernel<NoTally, true> : cull_kernel<NoTally, false>, grid, sizeof(CullSmem), stream, P);
 }
 
+// The order of the tile kernel's tiles.  A small launch ends with whatever its last CTAs meet, a large one rather keeps neighbouring
+// tiles together, whose stores share lines.  Horizon first / in order, so many tiles per multiprocessor:
+//   views of 8 tiles    55: 70.8 / 73.6 us   111: 94.8 / 101.4   221: 161.5 / 165.4   443: 311.0 / 293.6
+//   views of 2 tiles    52: 46.9 / 49.4      104: 74.1 / 73.4    201: 126.4 / 125.2   402: 223.9 / 215.9 (colours 104: 85.2 / 88.2, 402: 246.8 / 247.7)
+//   occlusion counts, views of 4 tiles   55: 121.7 / 136.2   111: 191 / 208   221: 327.8 / 338.1
+// (A kernel of its own for each: what the order takes at the start cost the other 1 % in registers.)
+constexpr int HORIZON_FIRST_TILES = 160;   // tiles per multiprocessor up to which the horizon comes first
+template <bool VEC, bool OCC, bool RGB>
+static cudaError_t launch_tiles(const RenderParams& P0, long long n_views, int sm_count, cudaStream_t stream);
+
 // Launches the next kernel of a call: its blocks may be brought in while the last blocks of the kernel before it still
 // run (it waits for that kernel itself, see await_previous).
 template <class K>
@@ -1314,6 +1344,13 @@ cudaError_t launch_next(K kernel, unsigned grid, size_t smem, cudaStream_t strea
 #include "pic_coverage.cuh"
 namespace pic {
 #include "pic_tile.cuh"
+template <bool VEC, bool OCC, bool RGB>
+static cudaError_t launch_tiles(const RenderParams& P0, long long n_views, int sm_count, cudaStream_t stream) {
+    RenderParams P = P0;
+    P.div_views = fast_div((uint32_t)n_views);
+    const bool first = P.tiles_x * P.tiles_y > 1 && (long long)P.n_jobs <= (long long)HORIZON_FIRST_TILES * sm_count;
+    return launch_next(first ? render_tile_kernel<NoTally, VEC, OCC, RGB, true> : render_tile_kernel<NoTally, VEC, OCC, RGB, false>, P.n_jobs, 0, stream, P, 32);
+}
 #include "pic_colour.cuh"
 #include "pic_static.cuh"
 #include "pic_small.cuh"
@@ -1336,10 +1373,9 @@ cudaError_t launch_render_kernel(const RenderParams& P0, long long n_views, int 
     if (err != cudaSuccess) return err;
     // (b)-(d) set-up, raster, store
     const bool vec = P.W % 4 == 0 && !P.out_depth32;
-    err = launch_next(P.counters                    ? render_tile_kernel<Tally, false, true>
-                      : P.occlusion                 ? (vec ? render_tile_kernel<NoTally, true, true> : render_tile_kernel<NoTally, false, true>)
-                                                    : (vec ? render_tile_kernel<NoTally, true, false> : render_tile_kernel<NoTally, false, false>),
-                      (unsigned)jobs, 0, stream, P, 32);
+    err = P.counters    ? launch_next(render_tile_kernel<Tally, false, true>, P.n_jobs, 0, stream, P, 32)
+          : P.occlusion ? (vec ? launch_tiles<true, true, false>(P, n_views, sm_count, stream) : launch_tiles<false, true, false>(P, n_views, sm_count, stream))
+                        : (vec ? launch_tiles<true, false, false>(P, n_views, sm_count, stream) : launch_tiles<false, false, false>(P, n_views, sm_count, stream));
     if (err != cudaSuccess) return err;
     // the tiles left out (their number is only known on the device): one wave of CTAs walks the list
     const long long wave = (long long)sm_count * 5;

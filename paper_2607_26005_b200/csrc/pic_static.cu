@@ -44,7 +44,7 @@ constexpr size_t kOffTables = kOffCams + sizeof(ViewCam) * kMaxViews;
 constexpr size_t kOffStatus = kOffTables + sizeof(float) * MAX_CAMS * (3 * kMaxSide + 2 * (kMaxSide + TILE));
 constexpr size_t kScratchBytes = kOffStatus + 256;
 
-// The only device memory this entry point ever uses besides the caller's buffers (about 490 KB,
+// The only device memory this entry point ever uses besides the caller's buffers (about 470 KB,
 // held by every device that loads the library until the process exits).
 static __device__ __align__(256) unsigned char g_static_scratch[kScratchBytes];
 

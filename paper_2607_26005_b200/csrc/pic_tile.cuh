@@ -388,13 +388,13 @@ __device__ __forceinline__ void sort_records(TileWarp& s, int n_rec, int lane) {
 }
 
 // VEC: rows of a multiple of four pixels and no float32 depth image.  OCC: with occlusion counts.  RGB: colours instead of
-// classes and depths.
-template <class TL, bool VEC, bool OCC, bool RGB = false>
+// classes and depths.  HORIZON_FIRST: the order of the tiles (see launch_tiles).
+template <class TL, bool VEC, bool OCC, bool RGB = false, bool HORIZON_FIRST = false>
 __global__ void __launch_bounds__(32, TILE_CTAS) render_tile_kernel(const __grid_constant__ RenderParams P) {
     __shared__ TileWarp s;
     const int lane = threadIdx.x;
     launch_dependents();
-    const unsigned id = await_previous(blockIdx.x);
+    const unsigned cta = await_previous(blockIdx.x), id = HORIZON_FIRST ? horizon_first(P, cta) : cta;
     const uint2* blk = P.surv + (size_t)id * SURV_STRIDE;
     const uint4 head = __ldcg(reinterpret_cast<const uint4*>(blk));
     const uint2 sv0 = __ldcg(blk + 2 + lane);                // (requested with the head; of a shorter list the rest is not looked at)

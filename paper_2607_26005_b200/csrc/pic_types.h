@@ -111,6 +111,7 @@ struct RenderParams {
     float w_near, w_far;            // 1/near, 1/far: kept range of the reciprocal depth
     uint32_t cls_agent, cls_sky, cls_ground;
     FastDiv div_tiles, div_tiles_x, div_K, div_A;   // by tiles per view, tile columns, cameras, agent slots
+    FastDiv div_views;              // by the views of this launch (tile kernel with the horizon first)
     const int32_t* env_map;
     const MapInfo* env_maps;        // [E] the MapInfo of each environment's map (one load instead of two)
     const MapInfo* maps;

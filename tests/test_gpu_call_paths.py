@@ -335,3 +335,35 @@ def test_equal_depths_and_pixel_centres_on_edges(copies, step, n_side, dots, dot
         assert (few[0][:100] == want[0][:100]).all()
     finally:
         g.close()
+
+
+@pytest.mark.parametrize("H,W,mode", [(70, 100, "class"), (70, 100, "occlusion"), (40, 90, "rgb"), (130, 66, "class")])
+def test_tiles_with_the_horizon_first_up_to_a_number_of_tiles(H, W, mode):
+    """Calls at both sides of the line up to which the tiles with the horizon come first give the same images and counts."""
+    import torch
+    import paper_2607_26005_b200 as pic
+    from scenes import default_palette
+    from tests.gpu_util import CudaRun
+    tiles, A, K = -(-H // 64) * -(-W // 64), 16, 4
+    line = 160 * torch.cuda.get_device_properties(0).multi_processor_count // tiles      # the most views that take this order
+    E = line // (A * K) + 1
+    s = soup(H + W, 150, E, A, H, W, K=K, spread=40.0)
+    g = CudaRun(s)
+    try:
+        out = []
+        for n in (line, 0):                                # 0: all
+            if mode == "rgb":
+                out.append(g.render_rgb(default_palette(), False, view_count=n)[0][:line])
+                continue
+            counts = torch.zeros((E, A, K, A, 2), dtype=torch.int32, device=g.dev)
+            g.scene.set_option(pic.OPT_OCCLUSION, counts if mode == "occlusion" else 0)
+            cls, d16, _ = g.render(depth32=False, view_count=n)
+            out.append(np.concatenate([cls[:line].reshape(-1), d16[:line].view(np.uint8).reshape(-1), counts.cpu().numpy().reshape(E * A * K, -1)[:line].view(np.uint8).reshape(-1)]))
+        assert (out[0] == out[1]).all()
+        if mode != "rgb":
+            g.scene.set_option(pic.OPT_OCCLUSION, 0)
+            n = 40
+            from tests.util import assert_same_as_exhaustive
+            assert_same_as_exhaustive(g.render(view_count=line), g.render(brute=True, view_first=line - n, view_count=n), slice(line - n, line))
+    finally:
+        g.close()
