@@ -118,12 +118,18 @@ def _rig_ptr(rig):
         rig = np.ascontiguousarray(rig, dtype=np.float32)
     if rig.size % 7:
         raise ValueError("a rig has 7 values per camera")
-    return rig.__array_interface__["data"][0], rig
+    try:
+        return C.addressof(C.c_char.from_buffer(rig)), rig          # (a quarter of what numpy's own ways to the address take)
+    except (TypeError, ValueError):                                 # a read-only or empty array
+        return rig.__array_interface__["data"][0], rig
 
 
 def _dev_ptr(t, dtype, numel: Optional[int] = None) -> int:
     if t is None:
         return 0
+    # (one line for the tensors that are right; what is wrong with the others is said below)
+    if type(t) is _torch().Tensor and t.is_cuda and t.dtype is dtype and t.is_contiguous() and (numel is None or t.numel() == numel):
+        return t.data_ptr()
     if not isinstance(t, _torch().Tensor) or not t.is_cuda:
         raise TypeError("expected a CUDA torch tensor")
     if t.dtype != dtype or not t.is_contiguous():
@@ -137,7 +143,7 @@ def _stream_ptr(stream) -> int:
     if stream is None:
         torch = _torch()
         # (the handle alone: torch.cuda.current_stream() builds a Stream object, a microsecond of a small call)
-        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice() if torch.cuda.is_initialized() else torch.cuda.current_device())
     return stream.cuda_stream
 
 
