@@ -727,9 +727,10 @@ cudaError_t launch_colour_kernel(const RenderParams& P0, long long n_views, bool
     P.n_jobs = (uint32_t)jobs;
     P.debug_flags = 0;
     P.counters = nullptr;
-    // few tiles: one per CTA, set up and rasterized by its four warps together.  Measured, antialiased: 64 tiles 200 -> 106 us,
-    // 576 tiles 148 -> 86, 2 048 tiles 218 -> 216, 4 096 tiles 302 -> 346, so the line lies at twelve tiles per multiprocessor.
-    P.tiles_per_cta = antialias && jobs <= 12LL * sm_count ? 1 : NW;
+    // few tiles: one per CTA, set up and rasterized by its four warps together.  Measured, antialiased, four a CTA / one: 64 tiles 200 /
+    // 106 us; views of 96 x 54, 13 tiles per multiprocessor 125 / 110, 20: 127 / 127; views of 384 x 216, 16: 160 / 174, 31: 206 / 240; so the
+    // line lies at fourteen.
+    P.tiles_per_cta = antialias && jobs <= 14LL * sm_count ? 1 : NW;
     const unsigned grid = (unsigned)((jobs + P.tiles_per_cta - 1) / P.tiles_per_cta);
     const cudaError_t err = launch_cull(P, n_views, antialias, sm_count, stream);
     if (err != cudaSuccess) return err;

@@ -199,8 +199,7 @@ __global__ void __launch_bounds__(SMALL_THREADS, 2) render_small_kernel(const __
         }
         raster_cell_records<false, true>(s, s.recs[cell], x, s.ray_y[y], P.w_near, P.w_far, bw, bl);
         if (n_px > 0) {
-            const size_t o = tile0 + (size_t)(y * P.W + x);
-            store_class_depth<VEC>(P.out_class + o, P.out_depth + o, !VEC && P.out_depth32 ? P.out_depth32 + o : nullptr, bw, bl, bz, n_px);
+            store_class_depth<VEC>(P, tile0 + (size_t)(y * P.W + x), bw, bl, bz, n_px);
         }
     }
 }

@@ -275,7 +275,7 @@ __device__ __forceinline__ void raster_cell_records(const S& s, const CellRecord
 // The four pixels of a lane -> class and depth images (bl: the background's class where bw is 0).  VEC: the four pixels exist,
 // 4-pixel groups are aligned, no float32 depth image.
 template <bool VEC>
-__device__ __forceinline__ void store_class_depth(uint8_t* oc, uint16_t* od, float* o32, const float (&bw)[4], const uint32_t (&bl)[4], float bg_z, int n_px) {
+__device__ __forceinline__ void store_class_depth(const RenderParams& P, size_t o, const float (&bw)[4], const uint32_t (&bl)[4], float bg_z, int n_px) {
     float z[4];
 #pragma unroll
     for (int k = 0; k < 4; ++k) z[k] = bw[k] > 0.f ? fast_rcp(bw[k]) : bg_z;     // (a fragment's 1/z is positive)
@@ -283,15 +283,15 @@ __device__ __forceinline__ void store_class_depth(uint8_t* oc, uint16_t* od, flo
     const uint32_t d0 = *reinterpret_cast<const uint32_t*>(&h0), d1 = *reinterpret_cast<const uint32_t*>(&h1);
     const uint32_t cw = __byte_perm(__byte_perm(bl[0], bl[1], 0x0040), __byte_perm(bl[2], bl[3], 0x0040), 0x5410);
     if (VEC) {
-        *reinterpret_cast<uint32_t*>(oc) = cw;
-        *reinterpret_cast<uint2*>(od) = make_uint2(d0, d1);
+        *reinterpret_cast<uint32_t*>(P.out_class + o) = cw;
+        *reinterpret_cast<uint2*>(P.out_depth + o) = make_uint2(d0, d1);
     } else {
 #pragma unroll
         for (int k = 0; k < 4; ++k)
             if (k < n_px) {
-                oc[k] = (uint8_t)(cw >> (8 * k));
-                od[k] = (uint16_t)((k < 2 ? d0 : d1) >> (16 * (k & 1)));
-                if (o32) o32[k] = z[k];
+                P.out_class[o + k] = (uint8_t)(cw >> (8 * k));
+                P.out_depth[o + k] = (uint16_t)((k < 2 ? d0 : d1) >> (16 * (k & 1)));
+                if (P.out_depth32) P.out_depth32[o + k] = z[k];
             }
     }
 }
@@ -501,7 +501,7 @@ __global__ void __launch_bounds__(32, TILE_CTAS) render_tile_kernel(const __grid
     // ---- the background of the other cells
     if (VEC && RGB) store_background_rgb(P, tile0, t, s.bg, busy, lane);
     else if (VEC) store_background(P, tile0, t, s.bg, busy, lane);
-    else busy = 0xffffffffu;
+    else busy = (t.th > TILE - CELL_H ? 0xffffffffu : (1u << (2 * ((t.th + CELL_H - 1) / CELL_H))) - 1u) & (t.tw > CELL_W ? 0xffffffffu : 0x55555555u);   // the image's cells
     // ---- cell after cell
     const int px = (lane & 7) * 4, py = lane >> 3;
     const size_t lane0 = tile0 + (size_t)(py * P.W + px);
@@ -544,7 +544,7 @@ __global__ void __launch_bounds__(32, TILE_CTAS) render_tile_kernel(const __grid
         if (n_px > 0) {
             const size_t o = lane0 + (size_t)((cell >> 1) * 4 * P.W + (cell & 1) * CELL_W);
             if (RGB) store_rgb<VEC>(P, o, bw, bl, n_map_tris, n_px);
-            else store_class_depth<VEC>(P.out_class + o, P.out_depth + o, !VEC && P.out_depth32 ? P.out_depth32 + o : nullptr, bw, bl, bg.x, n_px);
+            else store_class_depth<VEC>(P, o, bw, bl, bg.x, n_px);
         }
     }
     flush_counters(P, n);

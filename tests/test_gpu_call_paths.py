@@ -128,7 +128,7 @@ def test_views_of_several_tiles(n_tris, E, A, H, W, K, spread):
     test_calls_with_few_tiles(n_tris, E, A, H, W, K, spread)
 
 
-@pytest.mark.parametrize("E,A", [(1, 2), (37, 12), (38, 12)])       # 4 tiles per view: one per CTA up to 1 776 tiles (148 multiprocessors), else four
+@pytest.mark.parametrize("E,A", [(1, 2), (37, 12), (38, 12), (37, 14), (38, 14)])       # 4 tiles per view: one per CTA up to 2 072 tiles (148 multiprocessors), else four
 def test_antialiased_calls_with_few_and_many_tiles(E, A):
     from scenes import default_palette
     from tests.gpu_util import CudaRun
