@@ -1166,7 +1166,7 @@ cudaError_t configure_render_kernel() {
 // spheres, a lane each; the visible ones' faces are set up four agents at a time, eight lanes per agent of which six have a
 // face; then the agents are counted one after the other, a lane per pixel of the box around the agent's faces.  Bound by
 // instruction issue.  (A warp per tile that set up and drew one face of one agent after the other took 299 us for 4 096 views
-// of 100 x 70 pixels and 64 agents; one pixel per lane at a time instead of four 81 us where it now takes 64.)  The arithmetic that decides a pixel is the production kernels' (pic_device.cuh).
+// of 100 x 70 pixels and 64 agents; one pixel per lane at a time instead of four, and the bands in order, 81 us where it now takes 66.)  The arithmetic that decides a pixel is the production kernels' (pic_device.cuh).
 // ---------------------------------------------------------------------------------------------
 struct __align__(16) CoverWarp {
     float4 edge[4][32], w[32];                // faces of the batch by lane: edge functions with their thresholds, 1/z plane
