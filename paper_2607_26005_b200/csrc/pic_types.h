@@ -150,6 +150,25 @@ inline int ray_stride(int n) { return (n + 2 * TILE - 1) / TILE * TILE; }
 
 constexpr int FRUSTUM_ENTRIES = 11;      // six planes, five corners of the footprint
 inline size_t frusta_bytes(int K, int H, int W) { return sizeof(float4) * FRUSTUM_ENTRIES * (size_t)K * ((size_t)((W + TILE - 1) / TILE) * (size_t)((H + TILE - 1) / TILE) + 1); }
+
+// What thread t of block b of the set-up kernel does: the first K blocks write a camera's ray and background tables each, the next
+// K * parts an entry of a camera's frusta per thread, the others an agent per thread.  (parts 0: no frusta.)  Entry i belongs to
+// frustum i / FRUSTUM_ENTRIES of the camera; what lies beyond the entries or the agents is left out by the kernel.
+constexpr int SETUP_THREADS = 128;
+enum SetupRole { SETUP_TABLES, SETUP_FRUSTA, SETUP_AGENTS };
+struct SetupItem { SetupRole role; int camera, index; };
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline SetupItem setup_item(int K, int parts, int b, int t) {
+    if (b < K) return {SETUP_TABLES, b, t};
+    const int f = b - K, a = f - K * parts;
+    if (a >= 0) return {SETUP_AGENTS, 0, a * SETUP_THREADS + t};
+    return {SETUP_FRUSTA, f / parts, f % parts * SETUP_THREADS + t};
+}
+inline int frusta_parts(int tiles) { return (int)(((long long)(tiles + 1) * FRUSTUM_ENTRIES + SETUP_THREADS - 1) / SETUP_THREADS); }
+inline int setup_blocks(int K, int parts, int n_agents) { return K * (1 + parts) + (n_agents + SETUP_THREADS - 1) / SETUP_THREADS; }
+
 // Layout of the per-camera tables: the frusta, then those of table_bytes bytes.
 inline size_t table_bytes(int K, int H, int W) { return sizeof(float) * (size_t)K * ((size_t)ray_stride(W) + (size_t)ray_stride(H) + 3 * (size_t)H); }
 inline RigTables rig_tables(float* base, int K, int H, int W, float4* frusta) {

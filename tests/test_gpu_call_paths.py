@@ -128,6 +128,28 @@ def test_views_of_several_tiles(n_tris, E, A, H, W, K, spread):
     test_calls_with_few_tiles(n_tris, E, A, H, W, K, spread)
 
 
+@pytest.mark.parametrize("E,A,H,W", [
+    (1, 2, 128, 320),                     # 10 tiles: their frusta and the image's are 121 entries, one block of the set-up kernel
+    (1, 2, 64, 700),                      # 11 tiles: 132, two blocks
+    (1, 3, 700, 1300),                    # 231 tiles: 20 blocks; 1 386 tiles in all, culled a warp per tile
+    (1, 2, 700, 1300),                    # ... 924 of them: a CTA per tile
+])
+def test_images_of_many_tiles(E, A, H, W):
+    import oracle
+    from scenes import default_palette
+    from tests.test_gpu_colour import compare_colour
+    from tests.gpu_util import CudaRun
+    test_calls_with_few_tiles(120, E, A, H, W, 2, 40.0)
+    s = soup(120 + A, 120, E, A, H, W, K=2, spread=40.0)
+    g = CudaRun(s)
+    try:
+        got, flags = g.render_rgb(default_palette(), False)
+        assert flags == 0
+        compare_colour(oracle.render_rgb(s, default_palette(), False, [1, 2 * E * A - 1]), got[[1, 2 * E * A - 1]])
+    finally:
+        g.close()
+
+
 @pytest.mark.parametrize("E,A", [(1, 2), (37, 12), (38, 12), (37, 14), (38, 14)])       # 4 tiles per view: one per CTA up to 2 072 tiles (148 multiprocessors), else four
 def test_antialiased_calls_with_few_and_many_tiles(E, A):
     from scenes import default_palette
