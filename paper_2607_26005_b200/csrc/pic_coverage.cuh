@@ -12,8 +12,8 @@ __device__ __forceinline__ float edge_coverage(float e0, float a, float b) {
     if (e0 >= h) return 1.f;
     if (e0 <= -h) return 0.f;
     const float hi = fmaxf(A, B), lo = fminf(A, B), g = 0.5f * (hi - lo);
-    if (fabsf(e0) <= g) return 0.5f + fast_div(e0, hi);
-    const float d = h - fabsf(e0), corner = fast_div(d * d, 2.f * A * B);     // the corner triangle cut off
+    if (fabsf(e0) <= g) return 0.5f + fast_div(e0, fmaxf(hi, SMALLEST_NORMAL));
+    const float d = h - fabsf(e0), corner = fast_div(d * d, fmaxf(2.f * A * B, SMALLEST_NORMAL));     // the corner triangle cut off
     return e0 < 0.f ? corner : 1.f - corner;
 }
 
@@ -51,6 +51,8 @@ __device__ __forceinline__ float polygon_coverage(const float (&x)[4], const flo
 // constraint m is moved by 1e-5 pixel, inwards when it cuts such a line of higher index and outwards otherwise,
 // so exactly one of the two keeps the piece whatever the rounding.  (Two coinciding lines that face each
 // other bound a sliver; both keep their piece and the two contributions cancel.)
+// A line that the pixel lies clear of bounds nothing, and is told by its value and gradient: of a plane square to the view but for the
+// rounding of an angle the two depth lines have gradients near 1e-19 and lie further away than the squares and products below can say.
 constexpr int CLINES = 6;
 template <int NL>
 __device__ __forceinline__ float pixel_coverage(const float (&e)[NL], const float (&a)[NL], const float (&b)[NL]) {
@@ -79,12 +81,13 @@ __device__ __forceinline__ float pixel_coverage(const float (&e)[NL], const floa
             const float al = fm(A[p], p0x, fm(B[p], p0y, C[p])) + (same_side ? -nudge : nudge);
             const float t = -fast_div(al, be);
             // (written with selects: the lanes of a warp rarely agree on the sign of be)
-            t0 = be > 0.f ? fmaxf(t0, t) : t0;
-            t1 = be < 0.f ? fminf(t1, t) : t1;
-            t1 = (be == 0.f && al < 0.f) ? -3e38f : t1;                                  // parallel and outside
+            t0 = be >= SMALLEST_NORMAL ? fmaxf(t0, t) : t0;
+            t1 = be <= -SMALLEST_NORMAL ? fminf(t1, t) : t1;
+            t1 = (fabsf(be) < SMALLEST_NORMAL && al < 0.f) ? -3e38f : t1;                // parallel and outside
         }
-        // (a constant, n2 == 0 -- a triangle's fourth edge, an unused slot -- bounds nothing)
-        twice = (n2 > 0.f && t1 > t0) ? fm(C[0], t1 - t0, twice) : twice;
+        // (a constant -- a triangle's fourth edge, an unused slot -- bounds nothing either)
+        const bool near_pixel = fabsf(C[0]) <= 0.501f * (fabsf(A[0]) + fabsf(B[0])) && n2 >= SMALLEST_NORMAL;
+        twice = (near_pixel && t1 > t0) ? fm(C[0], t1 - t0, twice) : twice;
         const float ra = A[0], rb = B[0], rc = C[0];
 #pragma unroll
         for (int p = 0; p + 1 < N; ++p) { A[p] = A[p + 1]; B[p] = B[p + 1]; C[p] = C[p + 1]; }

@@ -48,10 +48,13 @@ struct PrimEq {
     uint32_t tl;                 // bit i: exact zeros of edge i belong to the primitive
 };
 
-// 1 / x to an ulp or so, one instruction.  (__fdividef takes some five more, for the subnormal divisors it serves and this does not:
-// they count as 0.)  Used where a last digit does not matter or the divisor is a depth, a depth range or a difference of pixels.
+// 1 / x to an ulp or so, one instruction.  (__fdividef takes some five more, for the subnormal divisors it serves; here they count as 0,
+// so 1 / x is infinite and 0 / x no number.)  Used where a last digit does not matter and the divisor is a normal number: a depth, a
+// depth range, a focal length, a difference that has been compared with 0 from afar; gradients, whose products need not be, are held up
+// at SMALLEST_NORMAL.
 // With the ray tables that go on beyond the image (no division in the render kernels): 8 192 agents 220 -> 217 us, 65 536 agents 2 251 ->
 // 2 217, 14 880 views of 96 x 54 129.6 -> 126.7, their colours 157.6 -> 153.5.
+constexpr float SMALLEST_NORMAL = 1.17549435e-38f;
 __device__ __forceinline__ float fast_rcp(float x) {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));

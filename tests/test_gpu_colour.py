@@ -80,6 +80,21 @@ def test_hand_made_scenes(gu):
     check_colour(gu, single_env(np.zeros((0, 3, 3)), [], [ego(), (12.5, 0.0, 0.0, 4.5, 1.9, 1.0)], rig=make_rig((0.0,), 90.0, 90.0, mount=(2.25, 0.0, 4.0))))
 
 
+@pytest.mark.parametrize("far", [100.0, 20.05])      # (a line at the depth range's end counts for a pixel's area although it lies nowhere near it)
+@pytest.mark.parametrize("yaw", [3e-17, 1e-16, 4e-16, 1e-12, 1e-8])
+def test_walls_square_to_the_view_but_for_a_rounding(gu, yaw, far):
+    # large upright walls 20 m ahead whose depth hardly changes over a pixel: the planes' gradients are what a heading wrapped around leaves of a
+    # zero, and their squares may be no normal float32; the corners' areas are wide of 0 and 1
+    rig = make_rig((0.0,), 2 * np.degrees(np.arctan(32 / 200)), 2 * np.degrees(np.arctan(32 / 200)), 64, 64, mount=(0.0, 0.0, 1.5))
+    tris, classes = [], []
+    for i, (u, v) in enumerate([(3.3, 4.4), (34.6, 3.2), (2.3, 35.7), (33.85, 34.15)]):          # a wall's first column and row
+        y0, y1, z0, z1 = ((32 - c) / 10.0 for c in (u, u + 25.25, v, v + 24.4))
+        z0, z1 = z0 + 1.5, z1 + 1.5
+        tris += [[(20.0, y0, z0), (20.0, y1, z0), (20.0, y1, z1)], [(20.0, y0, z0), (20.0, y1, z1), (20.0, y0, z1)]]
+        classes += [2 + i] * 2
+    check_colour(gu, single_env(tris, classes, [ego(yaw=yaw)], rig=rig, far=far), modes=(True,))
+
+
 def test_config0_all_views(gu):
     st = check_colour(gu, make_config(0))
     print("cfg0 colour:", st)
