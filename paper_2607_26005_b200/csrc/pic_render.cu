@@ -1317,14 +1317,6 @@ static cudaError_t launch_cull(const RenderParams& P, long long n_views, bool co
     return launch_next(P.counters ? cull_kernel<Tally, false> : conservative ? cull_kernel<NoTally, true> : cull_kernel<NoTally, false>, grid, sizeof(CullSmem), stream, P);
 }
 
-// The order of the tile kernel's tiles.  A small launch ends with whatever its last CTAs meet, a large one rather keeps neighbouring
-// tiles together, whose stores share lines.  Horizon first / in order, so many tiles per multiprocessor:
-//   views of 8 tiles    55: 70.8 / 73.6 us   111: 94.8 / 101.4   221: 161.5 / 165.4   443: 311.0 / 293.6
-//   views of 2 tiles    52: 46.9 / 49.4      104: 74.1 / 73.4    201: 126.4 / 125.2   402: 223.9 / 215.9 (colours 104: 85.2 / 88.2, 402: 246.8 / 247.7)
-//   occlusion counts, views of 4 tiles   55: 121.7 / 136.2   111: 191 / 208   221: 327.8 / 338.1
-// Images whose rows are no groups of four pixels stay in order: neighbouring tiles share 32-byte sectors (1 260 agents x 3 cameras at
-// 159 x 90: 229 us in order, 248 not), but with occlusion counts, which take longer (891 views of 245 x 137: 188 in order, 177 not).  (A kernel of its own for each: what the order takes at the start cost the other 1 % in registers.)
-constexpr int HORIZON_FIRST_TILES = 160;   // tiles per multiprocessor up to which the horizon comes first
 template <bool VEC, bool OCC, bool RGB>
 static cudaError_t launch_tiles(const RenderParams& P0, long long n_views, int sm_count, cudaStream_t stream);
 
@@ -1349,7 +1341,10 @@ template <bool VEC, bool OCC, bool RGB>
 static cudaError_t launch_tiles(const RenderParams& P0, long long n_views, int sm_count, cudaStream_t stream) {
     RenderParams P = P0;
     P.div_views = fast_div((uint32_t)n_views);
-    const bool first = (VEC || OCC) && P.tiles_x * P.tiles_y > 1 && (long long)P.n_jobs <= (long long)HORIZON_FIRST_TILES * sm_count;
+    // (Images whose rows are no groups of four pixels stay in order: neighbouring tiles share 32-byte sectors (1 260 agents x 3 cameras at
+    // 159 x 90: 229 us in order, 248 not), but with occlusion counts, which take longer (891 views of 245 x 137: 188 in order, 177 not).
+    // A kernel of its own for each order: what the order takes at the start cost the other 1 % in registers.)
+    const bool first = (VEC || OCC) && draws_horizon_first(P.H, P.W, P.n_jobs, sm_count);
     return launch_next(first ? render_tile_kernel<NoTally, VEC, OCC, RGB, VEC || OCC> : render_tile_kernel<NoTally, VEC, OCC, RGB, false>, P.n_jobs, 0, stream, P, 32);
 }
 #include "pic_colour.cuh"

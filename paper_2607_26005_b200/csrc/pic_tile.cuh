@@ -388,7 +388,7 @@ __device__ __forceinline__ void sort_records(TileWarp& s, int n_rec, int lane) {
 }
 
 // VEC: rows of a multiple of four pixels and no float32 depth image.  OCC: with occlusion counts.  RGB: colours instead of
-// classes and depths.  HORIZON_FIRST: the order of the tiles (see launch_tiles).
+// classes and depths.  HORIZON_FIRST: the order of the tiles (see draws_horizon_first).
 template <class TL, bool VEC, bool OCC, bool RGB = false, bool HORIZON_FIRST = false>
 __global__ void __launch_bounds__(32, TILE_CTAS) render_tile_kernel(const __grid_constant__ RenderParams P) {
     __shared__ TileWarp s;

@@ -169,6 +169,21 @@ inline SetupItem setup_item(int K, int parts, int b, int t) {
 inline int frusta_parts(int tiles) { return (int)(((long long)(tiles + 1) * FRUSTUM_ENTRIES + SETUP_THREADS - 1) / SETUP_THREADS); }
 inline int setup_blocks(int K, int parts, int n_agents) { return K * (1 + parts) + (n_agents + SETUP_THREADS - 1) / SETUP_THREADS; }
 
+// Does the tile kernel draw the tiles with the horizon of all views first, then the rows below, the sky last?  A small launch ends with
+// whatever its last CTAs meet; a large one, or one whose tiles are all alike, rather keeps neighbouring tiles together, whose stores share
+// lines.  So there has to be an order to make -- more than one row of tiles, or a narrower last column, which then comes last -- and few enough
+// tiles.  Horizon first / in order, us, agents in platoons, so many tiles per multiprocessor (class and depth; colours; occlusion counts):
+//   54 x 96 (2, one narrower)     61: 86 / 92;  95 / 103; 139 / 147    150: 153 / 157; 176 / 183; 254 / 259    259: 237 / 247; 276 / 288; 396 / 405
+//   64 x 128 (2 alike)            61: 102 / 100; 118 / 116; 170 / 166   150: 180 / 178; 212 / 210; 303 / 301    259: 287 / 285; 342 / 338; 485 / 482
+//   128 x 128 (4)                 59: 82 / 92;  99 / 114; 136 / 148    149: 148 / 157; 186 / 195; 248 / 264    259: 231 / 243; 299 / 307; 387 / 406
+//   128 x 256 (8)                 62: 81 / 87; 101 / 106; 142 / 149    152: 128 / 138; 171 / 175; 216 / 226    263: 201 / 209; 269 / 269; 336 / 348
+//   216 x 384 (24)                62: 71 / 74;  92 / 93;  110 / 108    150: 107 / 112; 133 / 144; 149 / 159    259: 160 / 159; 201 / 202; 218 / 220
+// (At 350 tiles: 0.97 to 1.03 of the time in order.)  One line for all lies at 160; between there and 250 tiles the order in rows gives up to 6 % away.
+constexpr int HORIZON_FIRST_TILES = 160;   // tiles per multiprocessor
+inline bool draws_horizon_first(int H, int W, long long tiles, int sm_count) {
+    return (H > TILE || (W > TILE && W % TILE != 0)) && tiles <= (long long)HORIZON_FIRST_TILES * sm_count;
+}
+
 // Layout of the per-camera tables: the frusta, then those of table_bytes bytes.
 inline size_t table_bytes(int K, int H, int W) { return sizeof(float) * (size_t)K * ((size_t)ray_stride(W) + (size_t)ray_stride(H) + 3 * (size_t)H); }
 inline RigTables rig_tables(float* base, int K, int H, int W, float4* frusta) {
