@@ -64,7 +64,6 @@ __device__ __forceinline__ float fast_div(float a, float b) { return __fmul_rn(a
 
 struct V3 { float x, y, z; };
 
-__device__ __forceinline__ unsigned divide(unsigned n, const FastDiv& f) { return (__umulhi(n, f.m) + n) >> f.s; }
 
 __device__ __forceinline__ float fm(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ float mul(float a, float b) { return __fmul_rn(a, b); }

@@ -103,6 +103,12 @@ inline FastDiv fast_div(uint32_t d) {
     f.m = (uint32_t)(((1ull << 32) * ((1ull << f.s) - d)) / d + 1ull);
     return f;
 }
+#ifdef __CUDACC__
+__host__ __device__ __forceinline__
+#else
+inline
+#endif
+unsigned divide(unsigned n, const FastDiv& f) { return ((unsigned)(((unsigned long long)n * f.m) >> 32) + n) >> f.s; }
 
 struct RenderParams {
     int32_t E, A, K, H, W;
@@ -157,17 +163,20 @@ inline size_t frusta_bytes(int K, int H, int W) { return sizeof(float4) * FRUSTU
 constexpr int SETUP_THREADS = 128;
 enum SetupRole { SETUP_TABLES, SETUP_FRUSTA, SETUP_AGENTS };
 struct SetupItem { SetupRole role; int camera, index; };
+struct SetupGrid { int K, parts; FastDiv div_parts; };
+inline SetupGrid setup_grid(int K, int parts) { return {K, parts, fast_div((uint32_t)(parts ? parts : 1))}; }
 #ifdef __CUDACC__
 __host__ __device__
 #endif
-inline SetupItem setup_item(int K, int parts, int b, int t) {
-    if (b < K) return {SETUP_TABLES, b, t};
-    const int f = b - K, a = f - K * parts;
+inline SetupItem setup_item(const SetupGrid& G, int b, int t) {
+    if (b < G.K) return {SETUP_TABLES, b, t};
+    const int f = b - G.K, a = f - G.K * G.parts;
     if (a >= 0) return {SETUP_AGENTS, 0, a * SETUP_THREADS + t};
-    return {SETUP_FRUSTA, f / parts, f % parts * SETUP_THREADS + t};
+    const int camera = (int)divide((unsigned)f, G.div_parts);
+    return {SETUP_FRUSTA, camera, (f - camera * G.parts) * SETUP_THREADS + t};
 }
 inline int frusta_parts(int tiles) { return (int)(((long long)(tiles + 1) * FRUSTUM_ENTRIES + SETUP_THREADS - 1) / SETUP_THREADS); }
-inline int setup_blocks(int K, int parts, int n_agents) { return K * (1 + parts) + (n_agents + SETUP_THREADS - 1) / SETUP_THREADS; }
+inline int setup_blocks(const SetupGrid& G, int n_agents) { return G.K * (1 + G.parts) + (n_agents + SETUP_THREADS - 1) / SETUP_THREADS; }
 
 // Does the tile kernel draw the tiles with the horizon of all views first, then the rows below, the sky last?  A small launch ends with
 // whatever its last CTAs meet; a large one, or one whose tiles are all alike, rather keeps neighbouring tiles together, whose stores share

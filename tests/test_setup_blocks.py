@@ -20,13 +20,14 @@ int main() {
             for (int n : agents)
                 for (int wanted = 0; wanted < 2; ++wanted) {
                     const int tiles = ((hw[0] + TILE - 1) / TILE) * ((hw[1] + TILE - 1) / TILE), per = (tiles + 1) * FRUSTUM_ENTRIES;
-                    const int parts = wanted ? frusta_parts(tiles) : 0, blocks = setup_blocks(K, parts, n);
+                    const SetupGrid grid = setup_grid(K, wanted ? frusta_parts(tiles) : 0);
+                    const int blocks = setup_blocks(grid, n);
                     std::vector<int> table(K, 0), entry((size_t)K * per, 0), agent(n, 0);
                     if (sizeof(float) * 4 * entry.size() != frusta_bytes(K, hw[0], hw[1])) return std::printf("%d entries do not fill the table\n", (int)entry.size()), 1;
                     int idle = 0;
                     for (int b = 0; b < blocks; ++b)
                         for (int t = 0; t < SETUP_THREADS; ++t) {
-                            const SetupItem it = setup_item(K, parts, b, t);
+                            const SetupItem it = setup_item(grid, b, t);
                             if (it.camera < 0 || it.camera >= K || it.index < 0) return std::printf("block %d thread %d: camera %d item %d\n", b, t, it.camera, it.index), 1;
                             if (it.role == SETUP_TABLES) { if (t == 0) ++table[it.camera]; }
                             else if (it.role == SETUP_FRUSTA) { if (it.index < per) ++entry[(size_t)it.camera * per + it.index]; else ++idle; }
