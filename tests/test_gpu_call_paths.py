@@ -359,33 +359,102 @@ def test_equal_depths_and_pixel_centres_on_edges(copies, step, n_side, dots, dot
         g.close()
 
 
-@pytest.mark.parametrize("H,W,mode", [(70, 100, "class"), (70, 100, "occlusion"), (40, 90, "rgb"), (130, 66, "class")])
+# (rows of groups of four pixels take this order, and with occlusion counts all)
+@pytest.mark.parametrize("H,W,mode", [(70, 100, "class"), (70, 100, "occlusion"), (40, 90, "occlusion"), (40, 92, "rgb"), (130, 68, "class"), (130, 68, "rgb")])
 def test_tiles_with_the_horizon_first_up_to_a_number_of_tiles(H, W, mode):
-    """Calls at both sides of the line up to which the tiles with the horizon come first give the same images and counts."""
+    """Calls at both sides of the line up to which the tiles with the horizon come first give the same images and counts, from the first view
+    or a later one on, into the batch's images or the views' own, and the same as the exhaustive kernel or the oracle."""
+    import torch
+    import oracle
+    import paper_2607_26005_b200 as pic
+    from scenes import default_palette
+    from tests.gpu_util import CudaRun
+    from tests.test_gpu_colour import compare_colour
+    from tests.util import f16_ulp_distance
+    tiles, A, K, skip = -(-H // 64) * -(-W // 64), 16, 4, 37
+    line = 160 * torch.cuda.get_device_properties(0).multi_processor_count // tiles      # the most views that take this order
+    E = (line + skip) // (A * K) + 1
+    V = E * A * K
+    s = soup(H + W, 150, E, A, H, W, K=K, spread=40.0)
+    g = CudaRun(s)
+
+    def run(first, n, relative):
+        """The images (and counts) of `n` views from `first` on (0: all), one array per view."""
+        views = slice(first, first + n) if n else slice(0, V)
+        g.scene.set_option(pic.OPT_OUT_RELATIVE, 1 if relative else 0)
+        try:
+            if mode == "rgb":
+                return [g.render_rgb(default_palette(), False, view_first=first, view_count=n)[0][slice(0, n) if relative else views]]
+            counts = torch.zeros((E, A, K, A, 2), dtype=torch.int32, device=g.dev)
+            g.scene.set_option(pic.OPT_OCCLUSION, counts if mode == "occlusion" else 0)
+            cls, d16, _ = g.render(depth32=False, view_first=first, view_count=n)
+            return [a[slice(0, n) if relative else views] for a in (cls, d16.view(np.uint16))] + [counts.cpu().numpy().reshape(V, A, 2)[views]]
+        finally:
+            g.scene.set_option(pic.OPT_OUT_RELATIVE, 0)
+            g.scene.set_option(pic.OPT_OCCLUSION, 0)
+
+    try:
+        whole = run(0, 0, False)                           # more tiles than the line: in order
+        for first, n, relative in ((0, line, False), (skip, line, False), (skip, line, True), (skip, line - 1, False)):
+            for got, want in zip(run(first, n, relative), whole):
+                assert (got == want[first:first + n]).all(), (first, n, relative)
+        last = run(skip, line, False)
+        if mode == "rgb":
+            ids = np.array([skip, skip + line // 2, skip + line - 1])
+            compare_colour(oracle.render_rgb(s, default_palette(), False, ids), last[0][ids - skip])
+        else:
+            n = 40
+            cls, d16, _ = g.render(brute=True, depth32=False, view_first=skip + line - n, view_count=n)
+            assert (last[0][-n:] == cls[skip + line - n:skip + line]).all()
+            assert (f16_ulp_distance(last[1][-n:], d16[skip + line - n:skip + line]) <= 1).all()
+    finally:
+        g.close()
+
+
+@pytest.mark.parametrize("copies,step,n_side,dots,dot", [
+    (8, 4.0, 2, 8, 0.25),        # 32 records, the most a tile holds
+    (9, 4.0, 2, 8, 0.25),        # one more than it holds
+    (7, 4.0, 2, 10, 0.75),       # 28 records and 90 fragments, which fit the memory they share ...
+    (7, 4.0, 2, 16, 0.75),       # ... and 144, which do not
+    (1, 0.75, 1, 26, 0.75),      # 243 fragments and hardly a record
+])
+def test_limits_of_a_tiles_lists_in_colour_and_with_counts(copies, step, n_side, dots, dot):
+    """The squares above as plain colours, which are the class image's, and with other agents among them and occlusion counts, which are the same
+    when every tile is left to the cooperative kernel."""
     import torch
     import paper_2607_26005_b200 as pic
     from scenes import default_palette
     from tests.gpu_util import CudaRun
-    tiles, A, K = -(-H // 64) * -(-W // 64), 16, 4
-    line = 160 * torch.cuda.get_device_properties(0).multi_processor_count // tiles      # the most views that take this order
-    E = line // (A * K) + 1
-    s = soup(H + W, 150, E, A, H, W, K=K, spread=40.0)
-    g = CudaRun(s)
-    try:
-        out = []
-        for n in (line, 0):                                # 0: all
-            if mode == "rgb":
-                out.append(g.render_rgb(default_palette(), False, view_count=n)[0][:line])
-                continue
-            counts = torch.zeros((E, A, K, A, 2), dtype=torch.int32, device=g.dev)
-            g.scene.set_option(pic.OPT_OCCLUSION, counts if mode == "occlusion" else 0)
-            cls, d16, _ = g.render(depth32=False, view_count=n)
-            out.append(np.concatenate([cls[:line].reshape(-1), d16[:line].view(np.uint8).reshape(-1), counts.cpu().numpy().reshape(E * A * K, -1)[:line].view(np.uint8).reshape(-1)]))
-        assert (out[0] == out[1]).all()
-        if mode != "rgb":
-            g.scene.set_option(pic.OPT_OCCLUSION, 0)
-            n = 40
-            from tests.util import assert_same_as_exhaustive
-            assert_same_as_exhaustive(g.render(view_count=line), g.render(brute=True, view_first=line - n, view_count=n), slice(line - n, line))
-    finally:
-        g.close()
+    rng = np.random.default_rng(copies + dots)
+    squares = [(8.0, y, z, step) for y in range(n_side) for z in range(n_side)] * copies + [(8.0, 0.25 * i, 0.25, dot) for i in range(dots)]
+    tris = []
+    for x, iy, iz, d in squares:
+        y0, z0 = (iy - n_side / 2) * d, 1.5 + (iz - n_side / 2) * d
+        p = [(x, y0, z0), (x, y0 + d, z0), (x, y0 + d, z0 + d), (x, y0, z0 + d)]
+        tris += [[p[0], p[1], p[2]], [p[0], p[2], p[3]]]
+    classes = rng.integers(2, 200, len(squares)).repeat(2).astype(np.uint8)
+    E, A, K = 80, 16, 1
+    poses = np.zeros((E, A, 3), np.float32)
+    poses[..., 0] = rng.choice([-8.0, 0.0, 4.0], (E, A))
+    poses[..., 1] = rng.integers(-8, 9, (E, A)) * 0.125
+    rig = make_rig((0.0,), 90.0, 90.0, 64, 64, mount=(0.0, 0.0, 1.5))
+    for size in ((0.01, 0.01, 0.01), (0.3, 0.3, 1.2)):       # the cameras look over the boxes
+        s = custom_scene(np.asarray(tris, np.float32), classes, poses, np.tile(np.array(size, np.float32), (E, A, 1)), rig, 64, 64, env_map_id=np.zeros(E, np.int32))
+        g = CudaRun(s)
+        try:
+            cls, d16, _ = g.render(depth32=False)
+            palette = np.asarray(default_palette())
+            rgb, flags = g.render_rgb(palette, False)
+            of_map = cls != s.agent_class                    # (boxes are shaded)
+            assert flags == 0 and of_map.mean() > 0.5 and (rgb[of_map] == palette[cls[of_map]]).all()
+            results = []
+            for debug in (0, 4):                             # 4: the cooperative kernel alone
+                counts = torch.zeros((E, A, K, A, 2), dtype=torch.int32, device=g.dev)
+                g.scene.set_option(pic.OPT_OCCLUSION, counts)
+                c, d, _ = g.render(depth32=False, debug_flags=debug)
+                g.scene.set_option(pic.OPT_OCCLUSION, 0)
+                assert (c == cls).all() and (d.view(np.uint16) == d16.view(np.uint16)).all()
+                results.append(counts.cpu().numpy())
+            assert (results[0] == results[1]).all() and (size[0] < 0.1 or results[0][..., 0].any())
+        finally:
+            g.close()

@@ -95,6 +95,26 @@ def test_walls_square_to_the_view_but_for_a_rounding(gu, yaw, far):
     check_colour(gu, single_env(tris, classes, [ego(yaw=yaw)], rig=rig, far=far), modes=(True,))
 
 
+@pytest.mark.parametrize("H,W", [(54, 96), (40, 92), (130, 101)])      # rows of groups of sixteen pixels, of four, of none
+@pytest.mark.parametrize("offset", [1, 4, 8])
+def test_colour_images_at_any_address(gu, H, W, offset):
+    import torch
+    from tests.test_gpu_call_paths import soup
+    s = soup(H + W, 120, 2, 6, H, W, spread=30.0)
+    g = gu.CudaRun(s)
+    try:
+        for aa in (False, True):
+            want, status = g.render_rgb(PAL, aa)
+            buf = torch.full((want.size + offset + 16,), 7, dtype=torch.uint8, device=g.dev)
+            out = buf[offset:offset + want.size]
+            g.scene.render_rgb(g.poses, g.dims, s.rig, active=g.active, out_rgb=out, antialias=aa)
+            got = buf.cpu().numpy()
+            assert status == 0 and g.scene.status() == 0
+            assert (got[offset:offset + want.size] == want.reshape(-1)).all() and (got[:offset] == 7).all() and (got[offset + want.size:] == 7).all()
+    finally:
+        g.close()
+
+
 def test_config0_all_views(gu):
     st = check_colour(gu, make_config(0))
     print("cfg0 colour:", st)
