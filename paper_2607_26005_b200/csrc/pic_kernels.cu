@@ -92,28 +92,25 @@ __device__ __forceinline__ void agent_setup(const AgentArgs& G, const RigParams&
     }
 }
 
-// Per-camera tables: ray coordinates of every pixel column / row and the background of every row.
-__device__ __forceinline__ void rig_setup(const RigParams& R, int k, const RigTables& T) {
-    float* ray_x = const_cast<float*>(T.ray_x);
-    float* ray_y = const_cast<float*>(T.ray_y);
-    float* bg_z = const_cast<float*>(T.bg_z);
-    uint32_t* bg_cls = const_cast<uint32_t*>(T.bg_cls);
-    uint32_t* bg_rgb = const_cast<uint32_t*>(T.bg_rgb);
+// Entry i of camera k's tables: the ray coordinate of a pixel column, or that of a pixel row and the row's background.
+__device__ __forceinline__ void rig_setup(const RigParams& R, int k, int i, const RigTables& T) {
     const CamConst c = R.cam[k];
-    const float cx = 0.5f * (float)R.W, cy = 0.5f * (float)R.H;
-    const int nx = ray_stride(R.W), ny = ray_stride(R.H);
-    for (int u = threadIdx.x; u < nx; u += blockDim.x)
-        ray_x[(size_t)k * nx + u] = __fdiv_rn(sub(add((float)u, 0.5f), cx), c.fx);
-    for (int v = threadIdx.x; v < ny; v += blockDim.x) {
-        const float ry = __fdiv_rn(sub(add((float)v, 0.5f), cy), c.fy);
-        ray_y[(size_t)k * ny + v] = ry;
-        if (v >= R.H) continue;
-        uint32_t cls; float z;
-        background(c.cphi, c.sphi, c.mz, ry, R.far_z, R.cls_sky, R.cls_ground, cls, z);
-        bg_z[(size_t)k * R.H + v] = z;
-        bg_cls[(size_t)k * R.H + v] = cls;
-        if (R.palette) bg_rgb[(size_t)k * R.H + v] = R.palette[cls];
+    const int nx = ray_stride(R.W), ny = ray_stride(R.H), v = i - nx;
+    if (v >= ny) return;
+    const bool column = v < 0;
+    const float ray = __fdiv_rn(sub(add((float)(column ? i : v), 0.5f), 0.5f * (float)(column ? R.W : R.H)), column ? c.fx : c.fy);
+    if (column) {
+        const_cast<float*>(T.ray_x)[(size_t)k * nx + i] = ray;
+        return;
     }
+    const_cast<float*>(T.ray_y)[(size_t)k * ny + v] = ray;
+    if (v >= R.H) return;
+    uint32_t cls; float z;
+    background(c.cphi, c.sphi, c.mz, ray, R.far_z, R.cls_sky, R.cls_ground, cls, z);
+    const size_t at = (size_t)k * R.H + v;
+    const_cast<float*>(T.bg_z)[at] = z;
+    const_cast<uint32_t*>(T.bg_cls)[at] = cls;
+    if (R.palette) const_cast<uint32_t*>(T.bg_rgb)[at] = R.palette[cls];
 }
 
 // Entry i of the frusta of camera k's tiles and of its whole image.
@@ -129,16 +126,17 @@ __device__ __forceinline__ void frusta_setup(const RigParams& R, int k, int i, c
                       (float)(whole ? R.H : min(y0 + TILE, R.H)) - cy, c.fx, c.fy, R.near_z, R.far_z);
 }
 
-// One launch prepares a call (who does what: setup_item).  The frusta are made an entry per thread: a block per camera that goes
-// through them is the longest chain of a call of a few views of many tiles.  One view of an empty map, class and depth, such a block / an entry
-// per thread: 720 x 1 280 18.6 / 11.2 us, 1 080 x 1 920 34.9 / 12.4, 2 160 x 3 840 111 / 21.1, 4 096 x 4 096 216 / 28.8.  The divisions that
-// find an entry are by numbers fixed per call: with the machine's own, a call of one view of one tile takes 10.8 us instead of 10.3.
+// One launch prepares a call (who does what: setup_item).  Bound by the length of a thread's chain: an entry of the tables or the frusta per
+// thread, since a block per camera that goes through them is the longest chain of a call of a few views of many pixels, and the divisions that find
+// an entry by numbers fixed per call.  One view, class and depth, a block per camera for both / for the tables / an entry per thread: an empty
+// map at 2 160 x 3 840 111 / 21.2 / 18.5 us, a town at 2 160 x 3 840 124 / 35.1 / 31.6 (colours 132 / 43.2 / 39.2), one tile with eight agents
+// 8.75 / 9.11 / 8.70 on the GPU alone.
 __global__ void __launch_bounds__(SETUP_THREADS) setup_kernel(const __grid_constant__ AgentArgs G, const __grid_constant__ RigParams R,
                                                               const __grid_constant__ RigTables T, uint32_t* overflow) {
     launch_dependents();
     if (overflow && blockIdx.x == 0 && threadIdx.x == 0) overflow[0] = 0u;   // the render kernels' list of left-out tiles starts empty (absent for callers that do not use them)
     const SetupItem it = setup_item(R.grid, (int)blockIdx.x, (int)threadIdx.x);
-    if (it.role == SETUP_TABLES) rig_setup(R, it.camera, T);
+    if (it.role == SETUP_TABLES) rig_setup(R, it.camera, it.index, T);
     else if (it.role == SETUP_FRUSTA) frusta_setup(R, it.camera, it.index, T);
     else if (it.index < G.n) agent_setup(G, R, it.index);
 }
@@ -203,7 +201,7 @@ cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses
     G.n = n_agents; G.poses = poses; G.state = state; G.actions = actions; G.dims = dims; G.active = active;
     G.agent_cls = agent_cls; G.default_cls = P.cls_agent; G.out = agents_out; G.cams = cams_out; G.status = status;
     G.dt = dt; G.wheelbase = wheelbase; G.v_max = v_max;
-    R.grid = setup_grid(P.K, P.rig.frusta ? frusta_parts(R.tiles) : 0);
+    R.grid = setup_grid(P.K, P.H, P.W, P.rig.frusta ? R.tiles : 0);
     setup_kernel<<<setup_blocks(R.grid, n_agents), SETUP_THREADS, 0, stream>>>(G, R, P.rig, P.overflow);
     return cudaGetLastError();
 }

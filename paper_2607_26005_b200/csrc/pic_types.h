@@ -157,26 +157,37 @@ inline int ray_stride(int n) { return (n + 2 * TILE - 1) / TILE * TILE; }
 constexpr int FRUSTUM_ENTRIES = 11;      // six planes, five corners of the footprint
 inline size_t frusta_bytes(int K, int H, int W) { return sizeof(float4) * FRUSTUM_ENTRIES * (size_t)K * ((size_t)((W + TILE - 1) / TILE) * (size_t)((H + TILE - 1) / TILE) + 1); }
 
-// What thread t of block b of the set-up kernel does: the first K blocks write a camera's ray and background tables each, the next
-// K * parts an entry of a camera's frusta per thread, the others an agent per thread.  (parts 0: no frusta.)  Entry i belongs to
+// What thread t of block b of the set-up kernel does: the first blocks write an entry of a camera's ray and background tables per thread
+// (its columns, then its rows), the next an entry of a camera's frusta, the others set up an agent.  Entry i of the frusta belongs to
 // frustum i / FRUSTUM_ENTRIES of the camera; what lies beyond the entries or the agents is left out by the kernel.
 constexpr int SETUP_THREADS = 128;
 enum SetupRole { SETUP_TABLES, SETUP_FRUSTA, SETUP_AGENTS };
 struct SetupItem { SetupRole role; int camera, index; };
-struct SetupGrid { int K, parts; FastDiv div_parts; };
-inline SetupGrid setup_grid(int K, int parts) { return {K, parts, fast_div((uint32_t)(parts ? parts : 1))}; }
+struct SetupGrid { int tables, frusta, table_blocks, frusta_blocks; FastDiv div_tables, div_frusta; };     // blocks per camera, of all cameras
+inline int setup_parts(long long entries) { return (int)((entries + SETUP_THREADS - 1) / SETUP_THREADS); }
+// tiles: of a view, or 0 if no frusta are wanted
+inline SetupGrid setup_grid(int K, int H, int W, int tiles) {
+    SetupGrid G;
+    G.tables = setup_parts((long long)ray_stride(W) + ray_stride(H));
+    G.frusta = tiles ? setup_parts((tiles + 1LL) * FRUSTUM_ENTRIES) : 0;
+    G.table_blocks = K * G.tables; G.frusta_blocks = K * G.frusta;
+    G.div_tables = fast_div((uint32_t)G.tables); G.div_frusta = fast_div((uint32_t)(G.frusta ? G.frusta : 1));
+    return G;
+}
 #ifdef __CUDACC__
 __host__ __device__
 #endif
 inline SetupItem setup_item(const SetupGrid& G, int b, int t) {
-    if (b < G.K) return {SETUP_TABLES, b, t};
-    const int f = b - G.K, a = f - G.K * G.parts;
+    if (b < G.table_blocks) {
+        const int camera = (int)divide((unsigned)b, G.div_tables);
+        return {SETUP_TABLES, camera, (b - camera * G.tables) * SETUP_THREADS + t};
+    }
+    const int f = b - G.table_blocks, a = f - G.frusta_blocks;
     if (a >= 0) return {SETUP_AGENTS, 0, a * SETUP_THREADS + t};
-    const int camera = (int)divide((unsigned)f, G.div_parts);
-    return {SETUP_FRUSTA, camera, (f - camera * G.parts) * SETUP_THREADS + t};
+    const int camera = (int)divide((unsigned)f, G.div_frusta);
+    return {SETUP_FRUSTA, camera, (f - camera * G.frusta) * SETUP_THREADS + t};
 }
-inline int frusta_parts(int tiles) { return (int)(((long long)(tiles + 1) * FRUSTUM_ENTRIES + SETUP_THREADS - 1) / SETUP_THREADS); }
-inline int setup_blocks(const SetupGrid& G, int n_agents) { return G.K * (1 + G.parts) + (n_agents + SETUP_THREADS - 1) / SETUP_THREADS; }
+inline int setup_blocks(const SetupGrid& G, int n_agents) { return G.table_blocks + G.frusta_blocks + setup_parts(n_agents); }
 
 // Does the tile kernel draw the tiles with the horizon of all views first, then the rows below, the sky last?  A small launch ends with
 // whatever its last CTAs meet; a large one, or one whose tiles are all alike, rather keeps neighbouring tiles together, whose stores share

@@ -1,5 +1,5 @@
-"""The set-up kernel's division of its work, on the host: every entry of every camera's frusta and every agent belongs to one thread,
-and no thread has more than one, so that large images do not lengthen the chain of a call."""
+"""The set-up kernel's division of its work, on the host: every entry of every camera's tables and frusta and every agent belongs to one
+thread, and no thread has more than one, so that large images do not lengthen the chain of a call."""
 import os
 import shutil
 import subprocess
@@ -20,23 +20,24 @@ int main() {
             for (int n : agents)
                 for (int wanted = 0; wanted < 2; ++wanted) {
                     const int tiles = ((hw[0] + TILE - 1) / TILE) * ((hw[1] + TILE - 1) / TILE), per = (tiles + 1) * FRUSTUM_ENTRIES;
-                    const SetupGrid grid = setup_grid(K, wanted ? frusta_parts(tiles) : 0);
+                    const SetupGrid grid = setup_grid(K, hw[0], hw[1], wanted ? tiles : 0);
+                    const int rays = ray_stride(hw[0]) + ray_stride(hw[1]);
                     const int blocks = setup_blocks(grid, n);
-                    std::vector<int> table(K, 0), entry((size_t)K * per, 0), agent(n, 0);
+                    std::vector<int> table((size_t)K * rays, 0), entry((size_t)K * per, 0), agent(n, 0);
                     if (sizeof(float) * 4 * entry.size() != frusta_bytes(K, hw[0], hw[1])) return std::printf("%d entries do not fill the table\n", (int)entry.size()), 1;
                     int idle = 0;
                     for (int b = 0; b < blocks; ++b)
                         for (int t = 0; t < SETUP_THREADS; ++t) {
                             const SetupItem it = setup_item(grid, b, t);
                             if (it.camera < 0 || it.camera >= K || it.index < 0) return std::printf("block %d thread %d: camera %d item %d\n", b, t, it.camera, it.index), 1;
-                            if (it.role == SETUP_TABLES) { if (t == 0) ++table[it.camera]; }
+                            if (it.role == SETUP_TABLES) { if (it.index < rays) ++table[(size_t)it.camera * rays + it.index]; else ++idle; }
                             else if (it.role == SETUP_FRUSTA) { if (it.index < per) ++entry[(size_t)it.camera * per + it.index]; else ++idle; }
                             else if (it.index < n) ++agent[it.index];
                         }
-                    for (int c : table) if (c != 1) return std::printf("a camera's tables are made %d times\n", c), 1;
+                    for (int c : table) if (c != 1) return std::printf("an entry of the tables is made %d times\n", c), 1;
                     for (int c : entry) if (c != wanted) return std::printf("%d tiles: an entry is made %d times\n", tiles, c), 1;
                     for (int c : agent) if (c != 1) return std::printf("an agent is set up %d times\n", c), 1;
-                    if (idle >= K * SETUP_THREADS) return std::printf("%d tiles: %d threads without an entry\n", tiles, idle), 1;
+                    if (idle >= 2 * K * SETUP_THREADS) return std::printf("%d tiles: %d threads without an entry\n", tiles, idle), 1;
                 }
     return 0;
 }
