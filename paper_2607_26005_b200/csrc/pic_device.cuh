@@ -124,18 +124,24 @@ __device__ __forceinline__ void load_camera(Cam& c, const ViewCam& v, const CamC
 // Entry i of the frustum of a part of an image, in camera space: columns l to r and rows u to d of it, from the principal point.
 //   0..5   planes n.q + w >= 0 with unit normals: near, far (both with some slack), left, right, top, bottom
 //   6..10  corners of the frustum (w unused): the apex, and those at depth far (a little beyond)
-__device__ __forceinline__ float4 frustum_entry(int i, float l, float r, float u, float d, float fx, float fy, float near_z, float far_z) {
+__device__ __forceinline__ float4 frustum_plane(int i, float l, float r, float u, float d, float fx, float fy, float near_z, float far_z) {
     if (i == 0) return make_float4(0.f, 0.f, 1.f, -near_z * 0.999f);
     if (i == 1) return make_float4(0.f, 0.f, -1.f, far_z * 1.001f);
-    if (i < 6) {
-        const float x = i == 2 ? fx : i == 3 ? -fx : 0.f, y = i == 4 ? fy : i == 5 ? -fy : 0.f, z = i == 2 ? -l : i == 3 ? r : i == 4 ? -u : d;
-        const float inv = rsqrtf(x * x + y * y + z * z);
-        return make_float4(x * inv, y * inv, z * inv, 0.f);
-    }
+    const float x = i == 2 ? fx : i == 3 ? -fx : 0.f, y = i == 4 ? fy : i == 5 ? -fy : 0.f, z = i == 2 ? -l : i == 3 ? r : i == 4 ? -u : d;
+    const float inv = rsqrtf(x * x + y * y + z * z);
+    return make_float4(x * inv, y * inv, z * inv, 0.f);
+}
+__device__ __forceinline__ float4 frustum_entry(int i, float l, float r, float u, float d, float fx, float fy, float near_z, float far_z) {
+    if (i < 6) return frustum_plane(i, l, r, u, d, fx, fy, near_z, far_z);
     if (i == 6) return make_float4(0.f, 0.f, 0.f, 0.f);
     const float F = far_z * 1.001f;
     return make_float4(((i & 1) ? r : l) / fx * F, ((i == 8 || i == 9) ? d : u) / fy * F, F, 0.f);
 }
+// A vector of camera space in world axes (ego-relative), and plane i of a frustum, n.q + w >= 0 there.
+__device__ __forceinline__ V3 rotate_to_world(const Cam& c, const float4 e) {
+    return {fm(c.rx, e.x, fm(c.dx, e.y, c.fx_ * e.z)), fm(c.ry, e.x, fm(c.dy, e.y, c.fy_ * e.z)), fm(c.dz, e.y, c.fz_ * e.z)};
+}
+__device__ __forceinline__ float4 world_plane(const Cam& c, const V3& n, float w) { return make_float4(n.x, n.y, n.z, w - fm(n.x, c.mwx, fm(n.y, c.mwy, n.z * c.mwz))); }
 
 // Plane normal of a primitive from its camera-space vertices (used for box faces, whose corners are
 // a few metres apart).

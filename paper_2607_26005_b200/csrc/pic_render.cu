@@ -56,6 +56,8 @@ struct __align__(16) TileSmem {
     uint32_t touched[2];                      // 8x8 blocks that may hold a fragment (rows 0-3, rows 4-7)
 };
 
+static_assert(offsetof(TileSmem, plane) % 16 == 0 && offsetof(TileSmem, side) % 16 == 0, "planes are written with 128-bit stores");
+
 // Keys are stored so that both access patterns spread over all banks.  A 16-byte chunk holds pixels
 // (2c, 2c+1) of row y; its low three index bits are XORed with (y & 1) << 2 | (c >> 3).  Raster: a
 // 16 x 4 cell is read a row (8 chunks of one 16-pixel column block) per quarter warp.  Store: 32
@@ -123,29 +125,12 @@ __device__ __forceinline__ int raster_in_thread(S& s, uint32_t* touched, const T
     return frags;
 }
 
-// Plane p of the tile frustum, n.(q - m_w) >= 0 with q = X - P_ego (unit normals, offset -n.m_w
-// plus near / far), and for p >= 2 the same side plane in camera space.
+// Plane p of the tile's frustum, ego-relative, and for p >= 2 the same side plane in camera space (see frustum_entry).
 template <class S>
 __device__ __forceinline__ void tile_planes(S& s, int p, const Cam& c, const TileCtx& t) {
-    const float l = (float)t.x0 - c.cx, r = (float)(t.x0 + t.tw) - c.cx, u = (float)t.y0 - c.cy, d = (float)(t.y0 + t.th) - c.cy;
-    float nx, ny, nz, off = 0.f, sx = 0.f, sy = 0.f, sz = 0.f;
-    const float Rx = c.rx, Ry = c.ry, Dx = c.dx, Dy = c.dy, Dz = c.dz, Fx = c.fx_, Fy = c.fy_, Fz = c.fz_;
-    switch (p) {
-        case 0: nx = Fx; ny = Fy; nz = Fz; off = -t.near_z * 0.999f; break;                                       // z >= near
-        case 1: nx = -Fx; ny = -Fy; nz = -Fz; off = t.far_z * 1.001f; break;                                      // z <= far
-        case 2: nx = c.focx * Rx - l * Fx; ny = c.focx * Ry - l * Fy; nz = -l * Fz; sx = c.focx; sz = -l; break;  // x f >= z l
-        case 3: nx = r * Fx - c.focx * Rx; ny = r * Fy - c.focx * Ry; nz = r * Fz; sx = -c.focx; sz = r; break;   // x f <= z r
-        case 4: nx = c.focy * Dx - u * Fx; ny = c.focy * Dy - u * Fy; nz = c.focy * Dz - u * Fz; sy = c.focy; sz = -u; break;
-        default: nx = d * Fx - c.focy * Dx; ny = d * Fy - c.focy * Dy; nz = d * Fz - c.focy * Dz; sy = -c.focy; sz = d; break;
-    }
-    const float inv = rsqrtf(nx * nx + ny * ny + nz * nz);
-    nx *= inv; ny *= inv; nz *= inv;
-    s.plane[p][0] = nx; s.plane[p][1] = ny; s.plane[p][2] = nz;
-    s.plane[p][3] = off - (nx * c.mwx + ny * c.mwy + nz * c.mwz);
-    if (p >= 2) {
-        const float is = rsqrtf(sx * sx + sy * sy + sz * sz);
-        s.side[p - 2][0] = sx * is; s.side[p - 2][1] = sy * is; s.side[p - 2][2] = sz * is; s.side[p - 2][3] = 0.f;
-    }
+    const float4 e = frustum_plane(p, (float)t.x0 - c.cx, (float)(t.x0 + t.tw) - c.cx, (float)t.y0 - c.cy, (float)(t.y0 + t.th) - c.cy, c.focx, c.focy, t.near_z, t.far_z);
+    *reinterpret_cast<float4*>(s.plane[p]) = world_plane(c, rotate_to_world(c, e), e.w);
+    if (p >= 2) *reinterpret_cast<float4*>(s.side[p - 2]) = e;
 }
 
 // Which faces of another agent's box can reach the tile: 0 if its bounding sphere misses the
@@ -759,13 +744,13 @@ __device__ __forceinline__ void frustum_setup(Frustum& f, const RenderParams& P,
     if (lane < FRUSTUM_ENTRIES) {
         Cam c;
         load_camera(c, P.cams[job.view], P.cam[job.k], P.W, P.H);
-        const float x = fm(c.rx, entry.x, fm(c.dx, entry.y, c.fx_ * entry.z)), y = fm(c.ry, entry.x, fm(c.dy, entry.y, c.fy_ * entry.z)), z = fm(c.dz, entry.y, c.fz_ * entry.z);
+        const V3 v = rotate_to_world(c, entry);
         if (lane < 6) {
-            *reinterpret_cast<float4*>(f.plane[lane]) = make_float4(x, y, z, entry.w - fm(x, c.mwx, fm(y, c.mwy, z * c.mwz)));
+            *reinterpret_cast<float4*>(f.plane[lane]) = world_plane(c, v, entry.w);
             if (lane >= 2) *reinterpret_cast<float4*>(f.side[lane - 2]) = entry;
         } else {
-            f.pt[lane - 6][0] = c.mwx + x;
-            f.pt[lane - 6][1] = c.mwy + y;
+            f.pt[lane - 6][0] = c.mwx + v.x;
+            f.pt[lane - 6][1] = c.mwy + v.y;
         }
         if (lane == 6) {
             f.cam = c;
