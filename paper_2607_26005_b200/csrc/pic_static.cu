@@ -41,7 +41,7 @@ constexpr int kMaxDevices = 64;
 constexpr size_t kOffAgents = 0;
 constexpr size_t kOffCams = kOffAgents + sizeof(AgentGeom) * kMaxAgents;
 constexpr size_t kOffTables = kOffCams + sizeof(ViewCam) * kMaxViews;
-constexpr size_t kOffStatus = kOffTables + sizeof(float) * MAX_CAMS * (3 * kMaxSide + 2 * (kMaxSide + TILE));
+constexpr size_t kOffStatus = kOffTables + table_bytes(MAX_CAMS, kMaxSide, kMaxSide);
 constexpr size_t kScratchBytes = kOffStatus + 256;
 
 // The only device memory this entry point ever uses besides the caller's buffers (about 470 KB,

@@ -148,11 +148,12 @@ struct RenderParams {
     CamConst cam[MAX_CAMS];
 };
 
-// Entries of a ray table for n columns or rows: a tile that begins inside the image ends inside the table.
+// Entries of a ray table for n columns or rows: TILE of them may be read from any that belongs to the image on.  (The tiles of most kernels
+// begin at multiples of TILE, those of pic_render_static at multiples of 16 rows, and all read TILE entries.)
 #ifdef __CUDACC__
 __host__ __device__
 #endif
-inline int ray_stride(int n) { return (n + 2 * TILE - 1) / TILE * TILE; }
+constexpr int ray_stride(int n) { return (n + 2 * TILE - 1) / TILE * TILE; }
 
 constexpr int FRUSTUM_ENTRIES = 11;      // six planes, five corners of the footprint
 inline size_t frusta_bytes(int K, int H, int W) { return sizeof(float4) * FRUSTUM_ENTRIES * (size_t)K * ((size_t)((W + TILE - 1) / TILE) * (size_t)((H + TILE - 1) / TILE) + 1); }
@@ -205,7 +206,7 @@ inline bool draws_horizon_first(int H, int W, long long tiles, int sm_count) {
 }
 
 // Layout of the per-camera tables: the frusta, then those of table_bytes bytes.
-inline size_t table_bytes(int K, int H, int W) { return sizeof(float) * (size_t)K * ((size_t)ray_stride(W) + (size_t)ray_stride(H) + 3 * (size_t)H); }
+constexpr size_t table_bytes(int K, int H, int W) { return sizeof(float) * (size_t)K * ((size_t)ray_stride(W) + (size_t)ray_stride(H) + 3 * (size_t)H); }
 inline RigTables rig_tables(float* base, int K, int H, int W, float4* frusta) {
     RigTables r;
     r.frusta = frusta;

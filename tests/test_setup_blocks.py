@@ -52,3 +52,27 @@ def test_every_item_of_the_set_up_belongs_to_one_thread(tmp_path):
                     str(src), "-o", str(exe)], check=True)
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=120)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+RAYS = r"""
+#include <cstdio>
+#include "pic_types.h"
+int main() {
+    size_t most = 0;
+    for (int n = 1; n <= 2048; ++n) {
+        for (int from = 0; from < n; from += 16)             // a tile or a piece of one
+            if (from + pic::TILE > pic::ray_stride(n)) return std::printf("%d: entries %d to %d of %d\n", n, from, from + pic::TILE, pic::ray_stride(n)), 1;
+        if (n <= 512 && pic::table_bytes(16, n, n) > most) most = pic::table_bytes(16, n, n);
+    }
+    return most > pic::table_bytes(16, 512, 512);            // what pic_render_static reserves holds every smaller image's tables
+}
+"""
+
+
+@pytest.mark.skipif(shutil.which("g++") is None or not os.path.exists(os.path.join(CUDA, "vector_types.h")), reason="needs g++ and the CUDA headers")
+def test_what_a_tile_reads_of_the_ray_tables_is_there(tmp_path):
+    src, exe = tmp_path / "rays.cpp", tmp_path / "rays"
+    src.write_text(RAYS)
+    subprocess.run(["g++", "-std=c++17", "-I", CUDA, "-I", os.path.join(ROOT, "paper_2607_26005_b200", "csrc"), str(src), "-o", str(exe)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=60)
+    assert r.returncode == 0, r.stdout + r.stderr
