@@ -19,7 +19,8 @@
 // into a record pool shared by the CTA's four tiles, as many tiles at a time as fit it; 8-row strips are tasks.
 // A strip keeps, per pixel, the nearest FULLY covering fragment as a 64-bit key (unsigned max, as in the other
 // kernels, with the record's slot in the low byte) and a linked list of the partially covering fragments in
-// front of it (1/z, coverage in 14 bits, slot); the strip's warp owns both, so no atomics are needed.  The
+// front of it (1/z, coverage in 14 bits, slot); the strip's warp owns both, so atomics are needed only where two of its
+// lanes may meet at a pixel (keys of small primitives).  The
 // resolve walks each pixel's list in depth order, merges, composites and stores four pixels (12 bytes) per lane, side by side.
 //
 // Bound by instruction issue and fetch: at 61 KB of code a fifth of the issue slots waited for instructions, at 48 KB few do, so what

@@ -788,7 +788,10 @@ __device__ __forceinline__ GridRows grid_rows(const Frustum& f, const MapInfo& m
     return g;
 }
 
-// The range of grid_prims under the part of grid row `row` that the widened footprint crosses.
+// The range of grid_prims under the part of grid row `row` that the widened footprint crosses.  (Rounding: the difference, 1 / dy to an ulp and
+// the product put t off by less than 4 x 2^-24 of itself, which moves a crossing by less than 3e-7 of its distance from the segment's
+// beginning.  From the apex that is 3e-7 of how far away what is looked for is, where the outermost pixel centres lie half a pixel, 0.5 / f of that
+// distance, inside the footprint's sides; a segment between far corners lies 0.1 % beyond the far depth.)
 __device__ __forceinline__ void row_range(const Frustum& f, const RenderParams& P, const MapInfo& mi, const GridRows& g, int row, uint32_t& first, uint32_t& cnt) {
     first = 0u; cnt = 0u;
     if (row > g.hi) return;
@@ -1149,7 +1152,7 @@ cudaError_t configure_render_kernel() {
 // the pixels at which that agent's box, drawn alone, leaves a kept fragment.  Only coverage counts, so there is no
 // z-buffer and no need for tiles: a warp takes a band of 16 rows of a view.  The agents are culled as
 // spheres, a lane each; the visible ones' faces are set up four agents at a time, eight lanes per agent of which six have a
-// face; then the agents are counted one after the other, a lane per pixel of the box around the agent's faces.  Bound by
+// face; then the agents are counted one after the other, four pixels per lane at a time of the box around the agent's faces.  Bound by
 // instruction issue.  (A warp per tile that set up and drew one face of one agent after the other took 299 us for 4 096 views
 // of 100 x 70 pixels and 64 agents; one pixel per lane at a time instead of four, and the bands in order, 81 us where it now takes 66.)  The arithmetic that decides a pixel is the production kernels' (pic_device.cuh).
 // ---------------------------------------------------------------------------------------------
@@ -1274,7 +1277,7 @@ __global__ void __launch_bounds__(32) coverage_kernel(const __grid_constant__ Re
 }
 
 // One warp per band of 16 rows: with more, the longest ones -- an agent that fills the image -- are left running alone
-// (4 096 views of 100 x 70 pixels, 64 agents: whole views 224 us, 32 rows 128 us, 16 rows in CTAs of one warp 81 us).
+// (4 096 views of 100 x 70 pixels, 64 agents, with one pixel per lane: whole views 224 us, 32 rows 128 us, 16 rows in CTAs of one warp 81 us).
 static cudaError_t run_coverage(const RenderParams& P, long long n_views, cudaStream_t stream) {
     const int band_rows = 16, bands = (P.H + band_rows - 1) / band_rows;
     if (n_views * bands > 0x7fffffffLL) return cudaErrorInvalidConfiguration;

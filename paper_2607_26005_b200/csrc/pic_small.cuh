@@ -26,7 +26,7 @@ struct __align__(16) SmallSmem {
     CellRecords recs[32];                          // records that reach a cell
     uint32_t frag_cells;                           // cells with fragments
     Frustum f;
-    uint32_t row_first[32], row_off[33];       // candidate ranges of the grid rows of a pass (see FrontLists)
+    uint32_t row_first[32], row_off[33];           // grid rows of a pass: first entry of the row's range in grid_prims, and the candidates before the row (all at [32])
     uint32_t lleaf[SMALL_LARGE], face[SMALL_FACES];
     int n_rec, n_leaf, n_face;
 };

@@ -1,8 +1,8 @@
 // Render kernel over the cull kernel's survivor lists (included by pic_render.cu, inside namespace pic): set-up, raster
 // and store of one tile by one warp, with the z-buffer in registers.
 //
-// Bound by instruction issue (the images of a step are a seventh of the time at the copy bandwidth), so the split is
-// chosen to execute little per pixel.
+// Bound by instruction issue (the images of a step of 65 536 agents are nearly a quarter of its time at the copy bandwidth), so the split
+// is chosen to execute little per pixel.
 //   set-up    a lane per survivor.  The pixels of primitives of at most 16 pixel centres are evaluated at once, a lane each
 //             whatever the primitive, and leave fragments (pixel, key); the other primitives leave a record (edge functions,
 //             1/z plane) -- on the benchmark workload 20 primitives, 33 fragments and 7 records per tile.
@@ -33,7 +33,7 @@
 constexpr int TREC = 32;                     // records of a tile: a 32-bit mask
 constexpr int TFRAG = 256;                   // fragments of its small primitives
 constexpr int TPOOL = 3328;                  // bytes for both: 32 records and 96 fragments, 256 fragments and 16 records
-constexpr int SMALL_PIXELS = 16;             // pixel centres in the box of a small primitive (4, 8, 24, 32: within 2 %)
+constexpr int SMALL_PIXELS = 16;             // pixel centres in the box of a small primitive (4, 8, 24, 32: within 2 %, measured with 24 warps and one edge per instruction)
 constexpr int TILE_CTAS = 28;                // warps per multiprocessor
 constexpr int CELL_W = 32, CELL_H = 4;       // pixels of a cell
 static_assert((TILE / CELL_W) * (TILE / CELL_H) == 32, "a lane per cell");
