@@ -23,7 +23,7 @@
 // lanes may meet at a pixel (keys of small primitives).  The
 // resolve walks each pixel's list in depth order, merges, composites and stores four pixels (12 bytes) per lane, side by side.
 //
-// Bound by instruction issue and fetch: at 61 KB of code a fifth of the issue slots waited for instructions, at 48 KB few do, so what
+// Bound by instruction issue and fetch: at 61 KB of code a fifth of the issue slots waited for instructions, at 49 KB few do, so what
 // is not hot is rolled or out of line.  14 880 views of 96 x 54 (16 384 tiles with anything in them) 1 005 -> 745 us, 192 views of
 // 384 x 216 252 -> 208, by: cells that a record covers wholly updating their keys and no more (three in seven); strips that nothing
 // reaches storing their background (two thirds); one rolled copy of the shading with the colours in the pool; stores side by side;

@@ -186,8 +186,8 @@ static RigParams rig_params(const RenderParams& P) {
     RigParams R;
     R.K = P.K; R.W = P.W; R.H = P.H; R.near_z = P.near_z; R.far_z = P.far_z; R.cls_sky = P.cls_sky; R.cls_ground = P.cls_ground;
     R.palette = P.out_rgb ? P.palette : nullptr;
-    R.tiles_x = (P.W + TILE - 1) / TILE; R.tiles = R.tiles_x * ((P.H + TILE - 1) / TILE);
-    R.div_tiles_x = fast_div((uint32_t)R.tiles_x);
+    R.tiles_x = P.tiles_x; R.tiles = P.tiles_x * P.tiles_y;
+    R.div_tiles_x = P.div_tiles_x;
     for (int k = 0; k < MAX_CAMS; ++k) R.cam[k] = P.cam[k];
     return R;
 }
@@ -201,7 +201,7 @@ cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses
     G.n = n_agents; G.poses = poses; G.state = state; G.actions = actions; G.dims = dims; G.active = active;
     G.agent_cls = agent_cls; G.default_cls = P.cls_agent; G.out = agents_out; G.cams = cams_out; G.status = status;
     G.dt = dt; G.wheelbase = wheelbase; G.v_max = v_max;
-    R.grid = setup_grid(P.K, P.H, P.W, P.rig.frusta ? R.tiles : 0);
+    R.grid = setup_grid(P.K, P.div_K, P.H, P.W, P.rig.frusta ? R.tiles : 0);
     setup_kernel<<<setup_blocks(R.grid, n_agents), SETUP_THREADS, 0, stream>>>(G, R, P.rig, P.overflow);
     return cudaGetLastError();
 }

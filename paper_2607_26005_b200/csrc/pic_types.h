@@ -164,29 +164,21 @@ inline size_t frusta_bytes(int K, int H, int W) { return sizeof(float4) * FRUSTU
 constexpr int SETUP_THREADS = 128;
 enum SetupRole { SETUP_TABLES, SETUP_FRUSTA, SETUP_AGENTS };
 struct SetupItem { SetupRole role; int camera, index; };
-struct SetupGrid { int tables, frusta, table_blocks, frusta_blocks; FastDiv div_tables, div_frusta; };     // blocks per camera, of all cameras
+struct SetupGrid { int K, table_blocks, frusta_blocks; FastDiv div_K; };       // (the cameras take turns, block by block)
 inline int setup_parts(long long entries) { return (int)((entries + SETUP_THREADS - 1) / SETUP_THREADS); }
 // tiles: of a view, or 0 if no frusta are wanted
-inline SetupGrid setup_grid(int K, int H, int W, int tiles) {
-    SetupGrid G;
-    G.tables = setup_parts((long long)ray_stride(W) + ray_stride(H));
-    G.frusta = tiles ? setup_parts((tiles + 1LL) * FRUSTUM_ENTRIES) : 0;
-    G.table_blocks = K * G.tables; G.frusta_blocks = K * G.frusta;
-    G.div_tables = fast_div((uint32_t)G.tables); G.div_frusta = fast_div((uint32_t)(G.frusta ? G.frusta : 1));
-    return G;
+inline SetupGrid setup_grid(int K, FastDiv div_K, int H, int W, int tiles) {
+    return {K, K * setup_parts((long long)ray_stride(W) + ray_stride(H)), tiles ? K * setup_parts((tiles + 1LL) * FRUSTUM_ENTRIES) : 0, div_K};
 }
 #ifdef __CUDACC__
 __host__ __device__
 #endif
 inline SetupItem setup_item(const SetupGrid& G, int b, int t) {
-    if (b < G.table_blocks) {
-        const int camera = (int)divide((unsigned)b, G.div_tables);
-        return {SETUP_TABLES, camera, (b - camera * G.tables) * SETUP_THREADS + t};
-    }
-    const int f = b - G.table_blocks, a = f - G.frusta_blocks;
-    if (a >= 0) return {SETUP_AGENTS, 0, a * SETUP_THREADS + t};
-    const int camera = (int)divide((unsigned)f, G.div_frusta);
-    return {SETUP_FRUSTA, camera, (f - camera * G.frusta) * SETUP_THREADS + t};
+    const bool table = b < G.table_blocks;
+    const int f = table ? b : b - G.table_blocks, a = f - G.frusta_blocks;
+    if (!table && a >= 0) return {SETUP_AGENTS, 0, a * SETUP_THREADS + t};
+    const int part = (int)divide((unsigned)f, G.div_K);
+    return {table ? SETUP_TABLES : SETUP_FRUSTA, f - part * G.K, part * SETUP_THREADS + t};
 }
 inline int setup_blocks(const SetupGrid& G, int n_agents) { return G.table_blocks + G.frusta_blocks + setup_parts(n_agents); }
 
