@@ -108,7 +108,13 @@ __host__ __device__ __forceinline__
 #else
 inline
 #endif
-unsigned divide(unsigned n, const FastDiv& f) { return ((unsigned)(((unsigned long long)n * f.m) >> 32) + n) >> f.s; }
+unsigned divide(unsigned n, const FastDiv& f) {
+#ifdef __CUDA_ARCH__
+    return (__umulhi(n, f.m) + n) >> f.s;      // (written as below the tile kernel takes 0.7 % longer)
+#else
+    return ((unsigned)(((unsigned long long)n * f.m) >> 32) + n) >> f.s;
+#endif
+}
 
 struct RenderParams {
     int32_t E, A, K, H, W;
