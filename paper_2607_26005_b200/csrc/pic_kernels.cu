@@ -201,8 +201,8 @@ cudaError_t launch_setup(const RenderParams& P, int n_agents, const float* poses
     G.n = n_agents; G.poses = poses; G.state = state; G.actions = actions; G.dims = dims; G.active = active;
     G.agent_cls = agent_cls; G.default_cls = P.cls_agent; G.out = agents_out; G.cams = cams_out; G.status = status;
     G.dt = dt; G.wheelbase = wheelbase; G.v_max = v_max;
-    R.grid = setup_grid(P.K, P.div_K, P.H, P.W, P.rig.frusta ? R.tiles : 0);
-    setup_kernel<<<setup_blocks(R.grid, n_agents), SETUP_THREADS, 0, stream>>>(G, R, P.rig, P.overflow);
+    R.grid = setup_grid(P.K, P.div_K, P.H, P.W, P.rig.frusta ? R.tiles : 0, n_agents);
+    setup_kernel<<<setup_blocks(R.grid), SETUP_THREADS, 0, stream>>>(G, R, P.rig, P.overflow);
     return cudaGetLastError();
 }
 

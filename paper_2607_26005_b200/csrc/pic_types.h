@@ -164,29 +164,30 @@ constexpr int ray_stride(int n) { return (n + 2 * TILE - 1) / TILE * TILE; }
 constexpr int FRUSTUM_ENTRIES = 11;      // six planes, five corners of the footprint
 inline size_t frusta_bytes(int K, int H, int W) { return sizeof(float4) * FRUSTUM_ENTRIES * (size_t)K * ((size_t)((W + TILE - 1) / TILE) * (size_t)((H + TILE - 1) / TILE) + 1); }
 
-// What thread t of block b of the set-up kernel does: the first blocks write an entry of a camera's ray and background tables per thread
-// (its columns, then its rows), the next an entry of a camera's frusta, the others set up an agent.  Entry i of the frusta belongs to
-// frustum i / FRUSTUM_ENTRIES of the camera; what lies beyond the entries or the agents is left out by the kernel.
+// What thread t of block b of the set-up kernel does: the first blocks set up an agent per thread (the longest chain: 0.1 us of a small call),
+// the next write an entry of a camera's ray and background tables (its columns, then its rows), the others an entry of a camera's frusta.  Entry i of
+// the frusta belongs to frustum i / FRUSTUM_ENTRIES of the camera; what lies beyond the entries or the agents is left out by the kernel.
 constexpr int SETUP_THREADS = 128;
 enum SetupRole { SETUP_TABLES, SETUP_FRUSTA, SETUP_AGENTS };
 struct SetupItem { SetupRole role; int camera, index; };
-struct SetupGrid { int K, table_blocks, frusta_blocks; FastDiv div_K; };       // (the cameras take turns, block by block)
+struct SetupGrid { int K, agent_blocks, table_blocks, frusta_blocks; FastDiv div_K; };       // (the cameras take turns, block by block)
 inline int setup_parts(long long entries) { return (int)((entries + SETUP_THREADS - 1) / SETUP_THREADS); }
-// tiles: of a view, or 0 if no frusta are wanted
-inline SetupGrid setup_grid(int K, FastDiv div_K, int H, int W, int tiles) {
-    return {K, K * setup_parts((long long)ray_stride(W) + ray_stride(H)), tiles ? K * setup_parts((tiles + 1LL) * FRUSTUM_ENTRIES) : 0, div_K};
+// tiles: of a view, or 0 if no frusta are wanted; n: agents
+inline SetupGrid setup_grid(int K, FastDiv div_K, int H, int W, int tiles, int n) {
+    return {K, setup_parts(n), K * setup_parts((long long)ray_stride(W) + ray_stride(H)), tiles ? K * setup_parts((tiles + 1LL) * FRUSTUM_ENTRIES) : 0, div_K};
 }
 #ifdef __CUDACC__
 __host__ __device__
 #endif
 inline SetupItem setup_item(const SetupGrid& G, int b, int t) {
-    const bool table = b < G.table_blocks;
-    const int f = table ? b : b - G.table_blocks, a = f - G.frusta_blocks;
-    if (!table && a >= 0) return {SETUP_AGENTS, 0, a * SETUP_THREADS + t};
+    if (b < G.agent_blocks) return {SETUP_AGENTS, 0, b * SETUP_THREADS + t};
+    const int c = b - G.agent_blocks;
+    const bool table = c < G.table_blocks;
+    const int f = table ? c : c - G.table_blocks;
     const int part = (int)divide((unsigned)f, G.div_K);
     return {table ? SETUP_TABLES : SETUP_FRUSTA, f - part * G.K, part * SETUP_THREADS + t};
 }
-inline int setup_blocks(const SetupGrid& G, int n_agents) { return G.table_blocks + G.frusta_blocks + setup_parts(n_agents); }
+inline int setup_blocks(const SetupGrid& G) { return G.agent_blocks + G.table_blocks + G.frusta_blocks; }
 
 // Does the tile kernel draw the tiles with the horizon of all views first, then the rows below, the sky last?  A small launch ends with
 // whatever its last CTAs meet; a large one, or one whose tiles are all alike, rather keeps neighbouring tiles together, whose stores share

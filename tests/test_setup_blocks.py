@@ -20,9 +20,9 @@ int main() {
             for (int n : agents)
                 for (int wanted = 0; wanted < 2; ++wanted) {
                     const int tiles = ((hw[0] + TILE - 1) / TILE) * ((hw[1] + TILE - 1) / TILE), per = (tiles + 1) * FRUSTUM_ENTRIES;
-                    const SetupGrid grid = setup_grid(K, fast_div((uint32_t)K), hw[0], hw[1], wanted ? tiles : 0);
+                    const SetupGrid grid = setup_grid(K, fast_div((uint32_t)K), hw[0], hw[1], wanted ? tiles : 0, n);
                     const int rays = ray_stride(hw[0]) + ray_stride(hw[1]);
-                    const int blocks = setup_blocks(grid, n);
+                    const int blocks = setup_blocks(grid);
                     std::vector<int> table((size_t)K * rays, 0), entry((size_t)K * per, 0), agent(n, 0);
                     if (sizeof(float) * 4 * entry.size() != frusta_bytes(K, hw[0], hw[1])) return std::printf("%d entries do not fill the table\n", (int)entry.size()), 1;
                     int idle = 0;
