@@ -130,7 +130,7 @@ __device__ __forceinline__ void frusta_setup(const RigParams& R, int k, int i, c
 // thread, since a block per camera that goes through them is the longest chain of a call of a few views of many pixels, and the divisions that find
 // an entry by numbers fixed per call.  One view, class and depth, a block per camera for both / for the tables / an entry per thread: an empty
 // map at 2 160 x 3 840 111 / 21.2 / 18.5 us, a town at 2 160 x 3 840 124 / 35.1 / 31.6 (colours 132 / 43.2 / 39.2), one tile with eight agents
-// 8.75 / 9.11 / 8.70 on the GPU alone.
+// 8.8 / 9.1 / 8.8 on the GPU alone.
 __global__ void __launch_bounds__(SETUP_THREADS) setup_kernel(const __grid_constant__ AgentArgs G, const __grid_constant__ RigParams R,
                                                               const __grid_constant__ RigTables T, uint32_t* overflow) {
     launch_dependents();
